@@ -18,9 +18,9 @@ cudaError_t launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st)
 cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uint32_t* wq, unsigned long long* cum, int32_t* samples,
                                   float* wlog, uint64_t seed, cudaStream_t st);
 cudaError_t launch_tau(const AttnArgs& at, const int32_t* tpos, float* ltau, cudaStream_t st);
-cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout,
-                            float* delta, float* dq, float* dk, float* dv, void* dq_final, int dq_mode, float scale, int* status, cudaStream_t st);
-cudaError_t launch_to_bf16(const float* src, void* dst, size_t count, cudaStream_t st);
+cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout, float2* stat, int* sched,
+                            float* dq, float* dk, float* dv, float scale, int* status, cudaStream_t st);
+cudaError_t launch_to_bf16(const float* src, void* dq, void* dk, void* dv, size_t count, cudaStream_t st);
 
 namespace {
 
@@ -88,7 +88,7 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
 
 struct Plan {
   size_t q16, k16, v16, q16lo, k16lo, ids, hist, offs, perm_q, perm_k, rank_k, samples, tpos, ltau, vwq, vcum, swlog, wnodes, sched, part_o, part_lse, total;
-  size_t delta, gacc;   // backward only: <dO, O> per row; fp32 gradient accumulators (bf16 gradients only)
+  size_t stat, gacc;    // backward only: (-lse, -<dO, O>) per row; fp32 gradient accumulators (bf16 gradients only)
 };
 
 // backward: 0 forward plan; 1 backward with fp32 gradients (accumulated in place); 2 backward with bf16 gradients
@@ -122,7 +122,7 @@ Plan make_plan(const Geometry& g, int is_fp32, int backward = 0, bool capped = f
   const size_t part_rows = (g.L && !backward) ? (size_t)g.G * g.n + lvl_rows : 0;
   pl.part_o = take(part_rows * g.d * (part_bf16 ? 2 : 4));
   pl.part_lse = take(part_rows * 4);
-  pl.delta = take(backward ? (size_t)g.G * g.n * 4 : 0);
+  pl.stat = take(backward ? (size_t)g.G * g.n * 8 : 0);
   pl.gacc = take(backward == 2 ? (size_t)3 * g.G * g.n * g.d * 4 : 0);
   pl.total = off + kAlign;
   return pl;
@@ -416,18 +416,12 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     float* dq = g32 ? reinterpret_cast<float*>(bw->dq) : acc;
     float* dk = g32 ? reinterpret_cast<float*>(bw->dk) : acc + elems;
     float* dv = g32 ? reinterpret_cast<float*>(bw->dv) : acc + 2 * elems;
-    StageScope sc(st, HYPERATTN_STAGE_BACKWARD, 2 + (g32 ? 0 : 3));
-    // without the causal recursion every query row belongs to one tile: the kernel writes dQ in its final type
-    const int dq_mode = a.direct ? (g32 ? 1 : 2) : 0;
-    if (!dq_mode) HA_CHECK(cudaMemsetAsync(dq, 0, elems * 4, st));
-    HA_CHECK(cudaMemsetAsync(dk, 0, elems * 4, st));
-    HA_CHECK(cudaMemsetAsync(dv, 0, elems * 4, st));
-    HA_CHECK(launch_backward(a, p.out, out_fp32, p.lse, bw->dout, reinterpret_cast<float*>(base + pl.delta), dq, dk, dv, bw->dq, dq_mode, scale, ws.status, st));
-    if (!g32) {
-      if (!dq_mode) HA_CHECK(launch_to_bf16(dq, bw->dq, elems, st));
-      HA_CHECK(launch_to_bf16(dk, bw->dk, elems, st));
-      HA_CHECK(launch_to_bf16(dv, bw->dv, elems, st));
-    }
+    StageScope sc(st, HYPERATTN_STAGE_BACKWARD, 2 + (g32 ? 0 : 1));
+    if (g32) for (float* x : {dq, dk, dv}) HA_CHECK(cudaMemsetAsync(x, 0, elems * 4, st));
+    else HA_CHECK(cudaMemsetAsync(acc, 0, 3 * elems * 4, st));
+    HA_CHECK(launch_backward(a, p.out, out_fp32, p.lse, bw->dout, reinterpret_cast<float2*>(base + pl.stat), reinterpret_cast<int*>(base + pl.sched),
+                             dq, dk, dv, scale, ws.status, st));
+    if (!g32) HA_CHECK(launch_to_bf16(acc, bw->dq, bw->dk, bw->dv, elems, st));
     return HYPERATTN_OK;
   }
   if (capped) {

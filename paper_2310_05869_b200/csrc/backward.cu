@@ -10,518 +10,770 @@
 // The merge of the causal recursion needs no derivative of its own: the merged output is one
 // softmax over everything a row sees, so every tile of every level uses the FINAL lse and delta.
 //
-// One CTA per query tile of the forward schedule (same row tables, same sort and samples), key
-// tiles of 128, all five products on the tcgen05 tensor cores with accumulators in TMEM (see
-// bwd_tc_kernel); the three gradients are accumulated in fp32 with global reductions (a key
-// tile is shared by every query tile that samples it, a query row by every level it appears in).
-#include <cuda.h>
-#include "attn_common.cuh"
+// A work item is a tile of 128 KEYS and a run of query tiles (steps): the key tiles of a leaf against the query tiles from the
+// diagonal on, a key tile of a sorted block against the block's query tiles, a tile of a node's sampled keys against a chunk of the
+// node's query tiles.  dK and dV of the item stay in TMEM over its steps and leave once, by fp32 reductions; dQ leaves after every
+// step.  (The other way round - query tiles stay, dK and dV leave after every step - is twice the reductions and was what
+// the kernel's first version did, one phase after the other: 10 500 clocks per 128 x 128 tile at d = 64, 17 400 at d = 128.)
+// Per step, all five products on the tcgen05 tensor cores, keys in the TMEM lanes of the first two:
+//     S^T  = K Q^T,  dP^T = V dO^T      operands in 128-byte-swizzled shared memory, K-major
+//     P^T  -> TMEM (bf16), dS^T -> shared memory (bf16, [key][query])          two warpgroups, 64 query columns each
+//     dV  += P^T dO      A from TMEM, B = dO [query][d] MN-major
+//     dK  += dS^T Q      A K-major, B = Q MN-major
+//     dQ   = dS K        A = the same dS^T tile read MN-major, B = K [key][d] MN-major
+// What bounds it: the tensor pipe needs 1700 (d = 64) / 2700 (d = 128) clocks per step, the exponentials 1024; scores, hand-over,
+// exponentials, hand-over are one chain of about 2200.  d = 64: the next step's S^T and dP^T are issued before this step's three
+// gradient products, which then run while the warpgroups are busy with the next step; d = 128 has not the TMEM columns (P^T goes over S^T,
+// dQ over dP^T), so there dQ comes first and leaves TMEM while dV, the next S^T and dK are multiplied.
+//
+// Warp roles (512 threads): warps 0-3 and 4-7 P and dS; warps 8-11 dQ, dK and dV to global memory; warp 12 MMA issue (one
+// thread; the warp also allocates TMEM); warp 13 Q, dO and the row statistics; warp 14 K and V; warp 15 item descriptors.
+// Every wait is bounded: on a timeout the CTA raises the device status word, drains its copies, frees its TMEM and returns.
+#include "tc_util.cuh"
 
 namespace hyperattn {
-
-bool encode_rows_map(CUtensorMap* m, const void* base, size_t rows, int d, int box_rows);   // attn_tc.cu
-
 namespace {
 
-// K and V as [G * n rows x d] bf16 tensors, 128-byte swizzle, box = 64 columns x 128 rows: key tiles of
-// consecutive rows (causal leaves, unsorted nodes) arrive by TMA instead of through the load/store unit,
-// which the reductions keep busy
+constexpr int kThreads = 512;
+constexpr int kDescs = 3;              // item descriptors in flight
+constexpr int kTileK = 128;            // keys per item, query rows per step
+
+// tensor maps of Q, K, V, dO as [G n x d] bf16 tensors, 128-byte swizzle, box = 64 columns x 128 rows: tiles of consecutive rows
 struct alignas(64) BwdMaps {
-  CUtensorMap k, v;
+  CUtensorMap q, k, v, dout;
 };
-
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src));
-}
-__device__ __forceinline__ void st_shared_zero16(uint32_t dst) {
-  asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};\n" ::"r"(dst), "r"(0));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
-__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
-  __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t*>(&t);
-}
-// byte offset of 16-byte chunk c of row `row` in a [ROWS x 64k] bf16 tile: slabs of [ROWS x 128 B], 128-byte swizzle
-template <int ROWS>
-__device__ __forceinline__ uint32_t tile_off(int row, int c) {
-  return (uint32_t)((c >> 3) * (ROWS * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4));
-}
-template <int D, int ROWS, class RowFn>
-__device__ __forceinline__ void gather_tile(uint32_t dst, const __nv_bfloat16* src, RowFn rowfn, int tid) {
-  constexpr int CPR = D / 8;
-#pragma unroll
-  for (int i = 0; i < ROWS * CPR / 256; ++i) {
-    const int c = tid + i * 256;
-    const int row = c / CPR, cc = c % CPR;
-    const int gr = rowfn(row);
-    const uint32_t d = dst + tile_off<ROWS>(row, cc);
-    if (gr >= 0) cp_async16(d, src + (size_t)gr * D + cc * 8);
-    else st_shared_zero16(d);
-  }
-}
 
 struct BwdArgs {
-  AttnArgs a;
+  AttnArgs a;                  // geometry, permutations, samples
   const __nv_bfloat16* dout;   // [G, n, D]
-  const float* lse;            // [G, n] final log-sum-exp of the forward pass (natural log)
-  const float* delta;          // [G, n] <dO_i, O_i>
-  float *dq, *dk, *dv;         // [G, n, D] fp32 accumulators, zeroed before the launch
-  void* dq_final;              // dq_mode 1 / 2: dQ rows are written here directly (fp32 / bf16) instead of accumulated
-  int dq_mode;                 // 0: a query row collects from several tiles (causal recursion): fp32 reductions into dq
+  const float2* stat;          // [G, n] (-lse log2 e, -<dO, O>) of the rows
+  float *dq, *dk, *dv;         // [G, n, D] fp32 accumulators, zero at launch
   float scale;
-  int table_keys;              // key columns of a node tile's row tables (block and samples, each padded to whole tiles)
+  int* sched;                  // work counter of the launch, zero at launch
+  // items: the key tiles of the leaves, then level by level those of the nodes
+  int leaf_ktiles, n_leaf_items;
+  int level_item_start[kMaxLevels + 1];
+  int block_ktiles, smp_ktiles;          // key tiles per sorted block, per sample set
+  int chunk;                             // query tiles of a sampled item
+  int total_items;
 };
 
-// delta_i = <dO_i, O_i>: one warp per row
-template <int D, bool OUT_FP32>
-__global__ void __launch_bounds__(256) delta_kernel(const __nv_bfloat16* __restrict__ dout, const void* __restrict__ out,
-                                                    float* __restrict__ delta, size_t rows) {
-  const size_t row = (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= rows) return;
-  float acc = 0.f;
-  for (int c = lane; c < D; c += 32) {
-    const float o = OUT_FP32 ? reinterpret_cast<const float*>(out)[row * D + c]
-                             : __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(out)[row * D + c]);
-    acc += o * __bfloat162float(dout[row * D + c]);
-  }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) delta[row] = acc;
-}
-
-// ---------------------------------------------------------------------------------------------
-// One CTA per query tile, key tiles of 128, all five
-// products on the 5th-generation tensor cores with operands in 128-byte-swizzled shared memory:
-//     S  = Q K^T       A = Q  [query][d]   K-major,  B = K  [key][d]   K-major      -> TMEM cols   0..127
-//     dP = dO V^T      A = dO [query][d]   K-major,  B = V  [key][d]   K-major      -> TMEM cols 128..255
-//     dQ += dS K       A = dS [query][key] K-major,  B = K  [key][d]   MN-major     -> TMEM cols 256..256+d
-//     dV  = P^T dO     A = P  [query][key] MN-major, B = dO [query][d]  MN-major     -> over S's columns
-//     dK  = dS^T Q     A = dS [query][key] MN-major, B = Q  [query][d]  MN-major     -> over dP's columns
-// 512 threads: threads t, t + 128, t + 256 and t + 384 share TMEM lane t mod 128 - query row t when P
-// and dS are formed (each takes 32 of the tile's 128 key columns), key row t when dV and dK leave
-// TMEM (the 2 d / 32 pieces of 32 columns are dealt round to the four groups of 128 threads).  Sixteen
-// warps instead of eight hide a little more latency (2-3 % per call).  The phases of a key tile run one after the other (loads, S
-// and dP, P and dS, the three gradient products, reductions): correct first, overlapped later.
-constexpr int TKB = 128;   // keys per tile
-constexpr unsigned long long kBwdWaitNs = 2000000000ull;
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// bounded wait: false after two seconds (the caller raises the status word and winds down)
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity) {
-  unsigned long long t0 = 0;
-  for (unsigned it = 0;; ++it) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-                 : "=r"(ok) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
-    if (ok) return true;
-    if ((it & 63u) == 63u) {
-      const unsigned long long now = global_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > kBwdWaitNs) return false;
-    }
-  }
-}
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t acc) {
-  asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
-               "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}\n"
-               ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc) : "memory");
-}
-// packed fp32 pairs (two lanes per instruction)
-__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
-  uint64_t d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(__float_as_uint(lo)), "r"(__float_as_uint(hi)));
-  return d;
-}
-__device__ __forceinline__ uint64_t pk2u(uint32_t lo, uint32_t hi) {
-  uint64_t d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
-  return d;
-}
-__device__ __forceinline__ void upk2(uint64_t v, float& lo, float& hi) {
-  uint32_t a, b;
-  asm("mov.b64 {%0, %1}, %2;" : "=r"(a), "=r"(b) : "l"(v));
-  lo = __uint_as_float(a); hi = __uint_as_float(b);
-}
-__device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t fadd2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-               "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-               "\ttcgen05.wait::ld.sync.aligned;\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                 "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                 "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                 "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-               : "r"(taddr) : "memory");
-}
-// two loads in flight, one wait
-__device__ __forceinline__ void tmem_ld32_pair(uint32_t ta, uint32_t (&a)[32], uint32_t tb, uint32_t (&b)[32]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-               "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-               : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]),
-                 "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15]),
-                 "=r"(a[16]), "=r"(a[17]), "=r"(a[18]), "=r"(a[19]), "=r"(a[20]), "=r"(a[21]), "=r"(a[22]), "=r"(a[23]),
-                 "=r"(a[24]), "=r"(a[25]), "=r"(a[26]), "=r"(a[27]), "=r"(a[28]), "=r"(a[29]), "=r"(a[30]), "=r"(a[31])
-               : "r"(ta) : "memory");
-  tmem_ld32(tb, b);     // (its wait covers both loads)
-#pragma unroll
-  for (int i = 0; i < 32; ++i) asm volatile("" : "+r"(a[i]));    // no use of a[] may be scheduled above the wait
-}
-
-constexpr int kBwdThreads = 512;   // four threads per TMEM lane: 32 of a tile's 128 columns each
-
-template <int D>
-struct SmemTc {
-  static constexpr int kQ = 128 * D * 2;              // Q, dO, K, V tiles: [128 rows x D]
-  static constexpr int kP = 128 * TKB * 2;            // P, dS: [128 queries x 128 keys]
-  static constexpr int kOffQ = 0, kOffdO = kQ, kOffK = 2 * kQ, kOffV = 3 * kQ, kOffP = 4 * kQ, kOffdS = 4 * kQ + kP;
-  static constexpr int kOffMisc = 4 * kQ + 2 * kP;    // mbarrier, TMEM address, abort flag
-  static constexpr int kOffRow = kOffMisc + 64;       // s_qrow [128]
-  static constexpr int kFixed = kOffRow + 128 * 4;    // + 8 bytes per key column of the row tables
+// what every role needs to know about a work item; made once, by the descriptor warp
+struct BwdItem {
+  int kind;              // 0 consecutive keys and queries, 1 sorted block, 2 samples; -1: the list is exhausted
+  int seg, steps;
+  int causal;            // the first step's tile lies on the diagonal
+  int nkeys;             // keys of the tile that exist
+  int k0;                // kind 0: first key row; else: first key row of the node (segment-relative)
+  int q0;                // kind 0: first query row; else: first query row of the node (segment-relative)
+  int qend;              // kind 0: end of the query rows
+  int tn0;               // else: query tile (in sorted order) of the first step
+  int nq_node;
+  float wlog;            // log2 of the weight of the tile's columns
+  size_t slice;          // slice offset in perm_q / rank_k
+  size_t kidx;           // kind 1: the tile's first entry of perm_k; kind 2: of the samples
 };
 
-template <int D>
-__global__ void __launch_bounds__(kBwdThreads, 1) bwd_tc_kernel(const __grid_constant__ BwdArgs b, const __grid_constant__ BwdMaps maps, int* status) {
-  extern __shared__ __align__(1024) uint8_t smem[];
-  using SM = SmemTc<D>;
+__device__ __forceinline__ bool decode_item(const BwdArgs& b, int item, BwdItem& t) {
   const AttnArgs& a = b.a;
   const Geometry& g = a.g;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int row = tid & 127, part = tid >> 7;            // TMEM lane / tile row of this thread; which quarter of the work it takes
-  const TileDesc t = decode_tile(a, blockIdx.x);
-  if (t.nq <= 0) return;
-
-  const uint32_t ubase = smem_u32(smem);
-  const uint32_t uQ = ubase + SM::kOffQ, udO = ubase + SM::kOffdO, uK = ubase + SM::kOffK, uV = ubase + SM::kOffV;
-  const uint32_t uP = ubase + SM::kOffP, udS = ubase + SM::kOffdS;
-  const uint32_t bar = ubase + SM::kOffMisc;
-  const uint32_t bar_kv = ubase + SM::kOffMisc + 8;       // K and V tile of consecutive rows landed (TMA)
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + SM::kOffMisc + 16);
-  volatile int* s_abort = reinterpret_cast<volatile int*>(smem + SM::kOffMisc + 32);
-  int* s_qrow = reinterpret_cast<int*>(smem + SM::kOffRow);
-  int* s_kidx = s_qrow + 128;                                    // [table_keys]
-  float* s_kbias = reinterpret_cast<float*>(s_kidx + b.table_keys);
-
-  const size_t seg_row0 = (size_t)t.seg * g.n;
-  const __nv_bfloat16* qs = a.q + seg_row0 * D;
-  const __nv_bfloat16* ks = a.k + seg_row0 * D;
-  const __nv_bfloat16* vs = a.v + seg_row0 * D;
-  const __nv_bfloat16* dos = b.dout + seg_row0 * D;
-
-  // ---- row tables: key columns padded to whole tiles of 128 ----------------------------------
-  int nkeys;
-  if (t.mode == 1) {
-    const int bpad = (g.b + TKB - 1) / TKB * TKB, mpad = (g.m + TKB - 1) / TKB * TKB;
-    nkeys = bpad + mpad;
-    const float wlog = g.m > 0 ? log2f((float)t.nk / (float)g.m) : 0.f;
-    const int32_t* smp = a.samples + ((size_t)t.seg * g.nodes + t.node) * g.m;
-    for (int i = tid; i < nkeys; i += kBwdThreads) {
-      int idx = -1; float bias = -INFINITY;
-      if (i < bpad) {
-        if (i < block_len(t.nk, g.b, t.beta)) { idx = t.k0 + a.perm_k[t.slice + (size_t)t.beta * g.b + i]; bias = 0.f; }
-      } else if (i - bpad < g.m) {
-        const int l = smp[i - bpad];
-        idx = t.k0 + l;
-        bias = (a.rank_k[t.slice + l] / g.b == t.beta) ? -INFINITY : wlog;
-      }
-      s_kidx[i] = idx; s_kbias[i] = bias;
-    }
-    if (tid < 128) s_qrow[tid] = tid < t.nq ? t.qnode0 + a.perm_q[t.slice + t.spos0 + tid] : -1;
-  } else {
-    const int lim = t.causal ? min(t.nk, t.qk_off + t.nq) : t.nk;
-    nkeys = (lim + TKB - 1) / TKB * TKB;
-    if (tid < 128) s_qrow[tid] = tid < t.nq ? t.q0 + tid : -1;
+  t.causal = 0; t.wlog = 0.f; t.slice = t.kidx = 0; t.tn0 = t.nq_node = t.qend = 0;
+  if (item < b.n_leaf_items) {
+    // leaf after leaf, heaviest key tile (the first: every query tile sees it) first; the CTAs that run at the same time work on
+    // a few neighbouring leaves and find each other's rows - and dQ accumulators - in L2
+    const int kt = item % b.leaf_ktiles, rem = item / b.leaf_ktiles;
+    t.seg = rem / a.leaves_per_seg;
+    const int leaf0 = (rem % a.leaves_per_seg) * g.leaf;
+    t.kind = 0;
+    t.nkeys = min(kTileK, g.leaf - kt * kTileK);
+    t.k0 = leaf0 + kt * kTileK;
+    t.causal = a.dense_causal;
+    t.q0 = a.dense_causal ? t.k0 : leaf0;
+    t.qend = leaf0 + g.leaf;
+    t.steps = (t.qend - t.q0 + kTileQ - 1) / kTileQ;
+    return true;
   }
+  int level = 0;
+  while (level + 1 < g.levels && item >= b.level_item_start[level + 1]) ++level;
+  int idx = item - b.level_item_start[level];
+  int s, q0n, k0n;
+  node_rows(g, level, 0, s, q0n, k0n);
+  const int nodes_lvl = g.causal ? (1 << level) : 1;
+  if (!a.level_sorted[level]) {
+    const int kts = (s + kTileK - 1) / kTileK;
+    const int kt = idx % kts; idx /= kts;
+    t.seg = idx / nodes_lvl;
+    node_rows(g, level, idx % nodes_lvl, s, q0n, k0n);
+    t.kind = 0;
+    t.nkeys = min(kTileK, s - kt * kTileK);
+    t.k0 = k0n + kt * kTileK;
+    t.q0 = q0n; t.qend = q0n + s;
+    t.steps = (s + kTileQ - 1) / kTileQ;
+    return true;
+  }
+  const int blocks = node_blocks(s, g.b), tiles_node = blocks * a.tiles_per_block;
+  const int chunks = (tiles_node + b.chunk - 1) / b.chunk;
+  const int smp_items = b.smp_ktiles * chunks, per_node = smp_items + blocks * b.block_ktiles;
+  int x = idx % per_node; idx /= per_node;
+  const int j = idx % nodes_lvl;
+  t.seg = idx / nodes_lvl;
+  node_rows(g, level, j, s, q0n, k0n);
+  t.k0 = k0n; t.q0 = q0n; t.nq_node = s;
+  t.slice = ((size_t)level * g.G + t.seg) * g.nl + (g.causal ? (size_t)j * s : 0);
+  if (x < smp_items) {
+    const int st = x % b.smp_ktiles, node = g.causal ? (1 << level) - 1 + j : 0;
+    t.kind = 2;
+    t.nkeys = min(kTileK, g.m - st * kTileK);
+    t.kidx = ((size_t)t.seg * g.nodes + node) * g.m + st * kTileK;
+    t.tn0 = (x / b.smp_ktiles) * b.chunk;
+    t.steps = min(b.chunk, tiles_node - t.tn0);
+    t.wlog = log2f((float)s / (float)g.m);
+  } else {
+    x -= smp_items;
+    const int kt = x % b.block_ktiles, beta = x / b.block_ktiles, len = block_len(s, g.b, beta);
+    t.kind = 1;
+    t.nkeys = min(kTileK, len - kt * kTileK);
+    t.kidx = t.slice + (size_t)beta * g.b + kt * kTileK;
+    t.tn0 = beta * a.tiles_per_block;
+    t.steps = (len + kTileQ - 1) / kTileQ;
+    if (t.nkeys <= 0) return false;                     // (a short last block has fewer key tiles)
+  }
+  return true;
+}
+
+// query tile of a step: its rows, and where they start (kind 0: row of the segment; else: sorted position of the node)
+struct StepRows { int first, nq, beta; };
+__device__ __forceinline__ StepRows step_rows(const BwdArgs& b, const BwdItem& t, int s) {
+  StepRows r;
+  if (t.kind == 0) { r.first = t.q0 + s * kTileQ; r.nq = min(kTileQ, t.qend - r.first); r.beta = -1; return r; }
+  const int tn = t.tn0 + s, tpb = b.a.tiles_per_block;
+  r.beta = tn / tpb;
+  const int sub = tn - r.beta * tpb;
+  r.first = r.beta * b.a.g.b + sub * kTileQ;
+  r.nq = max(0, min(kTileQ, block_len(t.nq_node, b.a.g.b, r.beta) - sub * kTileQ));
+  return r;
+}
+
+template <int D>
+struct Cfg {
+  static constexpr int kTile = 128 * D * 2;           // bytes of a [128 rows x D] tile
+  static constexpr int NKV = D == 64 ? 2 : 1;         // K / V buffers (an item each)
+  static constexpr int NDO = D == 64 ? 2 : 1;         // dO buffers (a step each); Q: two
+  static constexpr int NDS = D == 64 ? 2 : 1;         // dS buffers
+  static constexpr int kOffKV = 0;
+  static constexpr int kOffQ = kOffKV + NKV * 2 * kTile;
+  static constexpr int kOffDO = kOffQ + 2 * kTile;
+  static constexpr int kOffDS = kOffDO + NDO * kTile;
+  static constexpr int kOffStage = kOffDS + NDS * 128 * 128 * 2;    // results on their way out: 8 KB per warp
+  static constexpr int kStageWarp = D == 64 ? 4096 : 8192;
+  static constexpr int kOffStat = kOffStage + 4 * kStageWarp;       // float [2 steps][-lse2 | -delta][128]
+  static constexpr int kOffDesc = kOffStat + 2 * 2 * 128 * 4;
+  static constexpr int kDescBytes = (sizeof(BwdItem) + 15) / 16 * 16;
+  static constexpr int kOffBar = kOffDesc + kDescs * kDescBytes;
+  static constexpr int kNumBar = 2 * NKV + 20 + 2 * kDescs;
+  static constexpr int kOffMisc = kOffBar + 8 * kNumBar;
+  static constexpr int kTotal = kOffMisc + 16;
+  static_assert(kTotal <= 232448, "shared memory");
+  // TMEM columns.  d = 64: S^T | dP^T | P^T | dV | dK | dQ.  d = 128: S^T (P^T over it) | dP^T (dQ over it) | dV | dK.
+  static constexpr int kColS = 0, kColDP = 128;
+  static constexpr int kColP = D == 64 ? 256 : 0;
+  static constexpr int kPHalf = D == 64 ? 32 : 64;    // columns from the first 64 queries' P^T to the other 64's
+  static constexpr int kColDV = D == 64 ? 320 : 256, kColDK = 384, kColDQ = D == 64 ? 448 : 128;
+};
+
+// (-lse log2 e, -<dO, O>) of every row: D / 8 lanes per row, 16 bytes of dO and O each (HBM-bound)
+template <int D, bool OUT_FP32>
+__global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__ dout, const void* __restrict__ out, const float* __restrict__ lse,
+                                                       float2* __restrict__ stat, size_t rows, int* sched) {
+  constexpr int LPR = D / 8;
+  const size_t c = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (c == 0) *sched = 0;
+  const size_t row = c / LPR;
+  float acc = 0.f;
+  if (row < rows) {
+    const uint4 x = __ldcs(dout + c);
+    const uint32_t xd[4] = {x.x, x.y, x.z, x.w};
+    float o[8];
+    if (OUT_FP32) {
+      const float4 a0 = __ldcs(reinterpret_cast<const float4*>(out) + 2 * c), a1 = __ldcs(reinterpret_cast<const float4*>(out) + 2 * c + 1);
+      o[0] = a0.x; o[1] = a0.y; o[2] = a0.z; o[3] = a0.w; o[4] = a1.x; o[5] = a1.y; o[6] = a1.z; o[7] = a1.w;
+    } else {
+      const uint4 y = __ldcs(reinterpret_cast<const uint4*>(out) + c);
+      const uint32_t yd[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) { o[2 * e] = __uint_as_float(yd[e] << 16); o[2 * e + 1] = __uint_as_float(yd[e] & 0xffff0000u); }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      acc = fmaf(o[2 * e], __uint_as_float(xd[e] << 16), acc);
+      acc = fmaf(o[2 * e + 1], __uint_as_float(xd[e] & 0xffff0000u), acc);
+    }
+  }
+#pragma unroll
+  for (int o = LPR / 2; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (row < rows && c % LPR == 0) stat[row] = make_float2(-lse[row] * 1.4426950408889634f, -acc);
+}
+
+template <int D>
+__global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant__ BwdArgs b, const __grid_constant__ BwdMaps maps, int* status) {
+  using C = Cfg<D>;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
+  volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
+  const uint32_t ubase = smem_u32(smem);
+  const uint32_t bar0 = ubase + C::kOffBar;
+  // (pairs of barriers are used in turn by the steps; a waiter that is a step behind never meets a phase twice)
+  auto bar_qfull = [&](uint32_t g) { return bar0 + 8 * (g & 1); };                // Q of a step landed
+  auto bar_qfree = [&](uint32_t g) { return bar0 + 8 * (2 + (g & 1)); };          // dK of the step multiplied: Q, statistics free
+  auto bar_stat = [&](uint32_t g) { return bar0 + 8 * (4 + (g & 1)); };           // row statistics of a step written
+  auto bar_dofull = [&](uint32_t g) { return bar0 + 8 * (6 + g % C::NDO); };      // dO landed
+  auto bar_dofree = [&](uint32_t g) { return bar0 + 8 * (8 + g % C::NDO); };      // dV multiplied: dO and P free
+  auto bar_dq = [&](uint32_t g) { return bar0 + 8 * (10 + (g & 1)); };            // dQ multiplied: in TMEM, dS free
+  const uint32_t bar_s = bar0 + 8 * 12, bar_dp = bar0 + 8 * 13;                   // S^T, dP^T written
+  const uint32_t bar_h = bar0 + 8 * 14;                                           // P and dS written (S^T and dP^T have been read)
+  const uint32_t bar_dqfree = bar0 + 8 * 15;                                      // dQ has left TMEM
+  const uint32_t bar_acc = bar0 + 8 * 16, bar_accfree = bar0 + 8 * 17;            // dK, dV of the item complete; have left TMEM
+  auto bar_kv = [&](int it) { return bar0 + 8 * (20 + it % C::NKV); };            // K and V of an item landed
+  auto bar_kvfree = [&](int it) { return bar0 + 8 * (20 + C::NKV + it % C::NKV); };
+  auto bar_dfull = [&](int it) { return bar0 + 8 * (20 + 2 * C::NKV + it % kDescs); };
+  auto bar_dfree = [&](int it) { return bar0 + 8 * (20 + 2 * C::NKV + kDescs + it % kDescs); };
+
+  const AttnArgs& a = b.a;
+  const Geometry& g = a.g;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+  if (tid == 0) *s_abort = *reinterpret_cast<volatile int*>(status);
+  __syncthreads();
+  if (*s_abort) return;                                 // (a launch in which some wait already timed out drains quickly)
+  __syncthreads();
   if (tid == 0) {
-    *s_abort = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_kv) : "memory");
+    for (int x = 0; x < 2; ++x) { mbar_init(bar_qfull(x), 32); mbar_init(bar_qfree(x), 1); mbar_init(bar_stat(x), 1); mbar_init(bar_dq(x), 1); }
+    for (int x = 0; x < C::NDO; ++x) { mbar_init(bar_dofull(x), 32); mbar_init(bar_dofree(x), 1); }
+    mbar_init(bar_s, 1); mbar_init(bar_dp, 1); mbar_init(bar_h, 8); mbar_init(bar_dqfree, 4); mbar_init(bar_acc, 1); mbar_init(bar_accfree, 4);
+    for (int x = 0; x < C::NKV; ++x) { mbar_init(bar_kv(x), 32); mbar_init(bar_kvfree(x), 1); }
+    for (int x = 0; x < kDescs; ++x) { mbar_init(bar_dfull(x), 1); mbar_init(bar_dfree(x), 15); }   // 8 + 4 warps, issuer, two loaders
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  constexpr int kTmemCols = 512;                       // S 128 | dP 128 | dQ D  (power of two)
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(kTmemCols) : "memory");
+  if (warp == 12) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tc_fence_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  tc_fence_after();
   const uint32_t tmem = *s_tmem;
-  const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-  constexpr uint32_t colS = 0, colDP = 128, colDQ = 256;
-
-  const int my_qrow = s_qrow[row];
-  // (a padding row gets lse = +inf, so that all its weights are zero)
-  const float lse2 = my_qrow >= 0 ? b.lse[seg_row0 + my_qrow] * 1.4426950408889634f : INFINITY;
-  const float delta = my_qrow >= 0 ? b.delta[seg_row0 + my_qrow] : 0.f;
-
-  auto krow_of = [&](int i) {          // segment-relative key row of key column i, -1: padding
-    if (t.mode == 1) return s_kidx[i];
-    return i < t.nk ? t.k0 + i : -1;
+  auto desc_of = [&](int it) -> const BwdItem& { return *reinterpret_cast<const BwdItem*>(smem + C::kOffDesc + (it % kDescs) * C::kDescBytes); };
+  auto wait_desc = [&](int it) { return wait_fast<1>(bar_dfull(it), (it / kDescs) & 1, s_abort, status); };
+  // key row (segment-relative) of key r of an item's tile, r < nkeys
+  auto key_row = [&](const BwdItem& t, int r) -> int {
+    if (t.kind == 0) return t.k0 + r;
+    return t.k0 + __ldg((t.kind == 1 ? a.perm_k : a.samples) + t.kidx + r);
   };
-  constexpr int CPR = D / 8;
-  auto gather_rows = [&](uint32_t dst, const __nv_bfloat16* src, auto rowfn) {
-#pragma unroll
-    for (int i = 0; i < 128 * CPR / kBwdThreads; ++i) {
-      const int c = tid + i * kBwdThreads;
-      const int r = c / CPR, cc = c % CPR;
-      const int gr = rowfn(r);
-      const uint32_t d = dst + tile_off<128>(r, cc);
-      if (gr >= 0) cp_async16(d, src + (size_t)gr * D + cc * 8);
-      else st_shared_zero16(d);
-    }
-  };
-  gather_rows(uQ, qs, [&](int r) { return s_qrow[r]; });
-  gather_rows(udO, dos, [&](int r) { return s_qrow[r]; });
 
-  // descriptors: low word = start >> 4 | (leading byte offset >> 4) << 16, high word = stride 1024 B | version | 128-byte swizzle
-  constexpr uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
-  constexpr uint32_t kSlab = 128 * 128;                // bytes of one [128 rows x 64 columns] slab
-  constexpr uint32_t idesc_base = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
-  constexpr uint32_t idesc_s = idesc_base | ((128u >> 3) << 17);                              // K-major x K-major, N = 128
-  constexpr uint32_t idesc_dq = idesc_base | (1u << 16) | (((uint32_t)D >> 3) << 17);          // K-major x MN-major, N = D
-  constexpr uint32_t idesc_t = idesc_base | (1u << 15) | (1u << 16) | (((uint32_t)D >> 3) << 17);   // MN-major x MN-major, N = D
-  auto kmajor = [&](uint32_t base, int ks) { return ((base + (ks >> 2) * kSlab + (ks & 3) * 32) >> 4) | (1u << 16); };
-  auto mnmajor = [&](uint32_t base, int kk) { return ((base + kk * 2048) >> 4) | ((kSlab >> 4) << 16); };
-
-  // Rows leave TMEM one per thread, but a reduction instruction whose lanes hit 32 different rows costs
-  // the L2 32 half-filled sectors: the warp's 32 rows x 32 columns pass through a 4 KB slice of shared
-  // memory (the P tile's, idle at that point; chunks XOR-swizzled by row) and go out with eight lanes
-  // per row, four rows per instruction.
-  const uint32_t ustage = uP + warp * 4096;
-  auto reduce_rows = [&](const uint32_t (&r)[32], float f, float* base, int grow, int c0, int store) {
-    const int lane = tid & 31;
-#pragma unroll
-    for (int c = 0; c < 8; ++c)
-      asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(ustage + lane * 128 + ((c ^ (lane & 7)) << 4)),
-                   "f"(__uint_as_float(r[4 * c]) * f), "f"(__uint_as_float(r[4 * c + 1]) * f),
-                   "f"(__uint_as_float(r[4 * c + 2]) * f), "f"(__uint_as_float(r[4 * c + 3]) * f) : "memory");
-    __syncwarp();
-#pragma unroll
-    for (int it = 0; it < 8; ++it) {
-      const int rr = 4 * it + (lane >> 3), c = lane & 7;
-      const int gr = __shfl_sync(0xffffffffu, grow, rr);
-      float4 v;
-      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                   : "r"(ustage + rr * 128 + ((c ^ (rr & 7)) << 4)) : "memory");
-      if (gr >= 0) {
-        const size_t el = (seg_row0 + gr) * D + c0 + 4 * c;
-        if (store == 0) atomicAdd(reinterpret_cast<float4*>(base + el), v);
-        else if (store == 1) *reinterpret_cast<float4*>(base + el) = v;
-        else *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(base) + el) = make_uint2(pack2(v.x, v.y), pack2(v.z, v.w));
-      }
-    }
-    __syncwarp();
-  };
-  const int ntiles = nkeys / TKB;
-  uint32_t phase = 0;
+  // Every role walks the same items and steps at its own pace; gs counts steps over all items.
+  uint32_t gs = 0;
   bool ok = true;
-  const bool dense = t.mode != 1;
-  auto load_kv = [&](int kt) {
-    if (dense) {
-      // consecutive rows: one TMA box per 64 columns (rows past the key range are masked, rows past the tensor are zeros)
-      if (tid == 0) {
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_kv), "r"((uint32_t)(2 * SM::kQ)) : "memory");
-        const int y = (int)seg_row0 + t.k0 + kt * TKB;
-#pragma unroll
-        for (int sl = 0; sl < D / 64; ++sl) {
-          asm volatile("cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                       ::"r"(uK + sl * kSlab), "l"(&maps.k), "r"(sl * 64), "r"(y), "r"(bar_kv) : "memory");
-          asm volatile("cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                       ::"r"(uV + sl * kSlab), "l"(&maps.v), "r"(sl * 64), "r"(y), "r"(bar_kv) : "memory");
-        }
-      }
-    } else {
-      gather_rows(uK, ks, [&](int r) { return krow_of(kt * TKB + r); });
-      gather_rows(uV, vs, [&](int r) { return krow_of(kt * TKB + r); });
-    }
-    cp_async_commit();
-  };
-  if (ntiles > 0) load_kv(0);
-  for (int kt = 0; kt < ntiles; ++kt) {
-    // ---- this tile's K and V (requested while the previous tile's dV and dK left TMEM) ----------
-    cp_async_wait<0>();
-    if (dense && !mbar_wait_bounded(bar_kv, kt & 1)) *s_abort = 1;
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    // ---- S = Q K^T, dP = dO V^T ----------------------------------------------------------------
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-      for (int s = 0; s < D / 16; ++s) mma_ss(tmem + colS, kmajor(uQ, s), kmajor(uK, s), desc_hi, idesc_s, s > 0);
-#pragma unroll
-      for (int s = 0; s < D / 16; ++s) mma_ss(tmem + colDP, kmajor(udO, s), kmajor(uV, s), desc_hi, idesc_s, s > 0);
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-    }
-    if (!mbar_wait_bounded(bar, phase)) *s_abort = 1;
-    phase ^= 1;
-    __syncthreads();
-    if (*s_abort) { ok = false; break; }
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // ---- P = C o exp(s - lse), dS = P (dP - delta): thread = query row ---------------------------
+  if (warp < 8) {
+    // ================= P and dS: thread = key, warpgroup h: query columns 64 h .. 64 h + 63 ==================
+    const int h = warp >> 2, row = tid & 127;
+    const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint64_t sc2 = pack_f2(a.scale_log2, a.scale_log2);
+    for (int it = 0; ok; ++it) {
+      ok = __all_sync(0xffffffffu, wait_desc(it));
+      if (!ok) break;
+      const BwdItem& t = desc_of(it);
+      if (t.kind < 0) break;
+      const bool exists = row < t.nkeys;
+      const int kind = t.kind, steps = t.steps, causal = t.causal;
+      int kblk = -2;                                    // sampled keys: the sorted block the key lies in (its entries there are masked)
+      if (kind == 2 && exists) kblk = __ldg(a.rank_k + t.slice + __ldg(a.samples + t.kidx + row)) / g.b;
 #pragma unroll 1
-    for (int c0 = 32 * part; c0 < 32 * part + 32; c0 += 32) {
-      uint32_t rs[32], rd[32];
-      tmem_ld32_pair(lane_addr + colS + c0, rs, lane_addr + colDP + c0, rd);
-      uint32_t pp[16], dd[16];
-      const int colbase = kt * TKB + c0;
-      // dense tiles need the mask only where the tile crosses the diagonal or the end of the keys
-      const bool dense_mask = t.mode != 1 && (colbase + 32 > t.nk || (t.causal && colbase + 31 > t.qk_off));
-      const uint64_t sc2 = pk2(a.scale_log2, a.scale_log2), nlse2 = pk2(-lse2, -lse2), ndel2 = pk2(-delta, -delta);
+      for (int s = 0; s < steps; ++s, ++gs) {
+        // entries that do not count: keys that do not exist, sampled keys of the query tile's own block, above the diagonal
+        bool dead = !exists;
+        if (kind == 2) dead = dead || kblk == (t.tn0 + s) / a.tiles_per_block;
+        const bool diag = causal && s == 0;
+        const bool masked = diag || __any_sync(0xffffffffu, dead);
+        ok = wait_fast<2>(bar_stat(gs), (gs >> 1) & 1, s_abort, status) && wait_fast<3>(bar_s, gs & 1, s_abort, status) &&
+             wait_fast<4>(bar_dp, gs & 1, s_abort, status);
+        // the products of the steps before that still read P and dS
+        if (D == 64) {
+          if (gs > 0) ok = ok && wait_fast<5>(bar_dofree(gs - 1), ((gs - 1) / C::NDO) & 1, s_abort, status);
+          if (gs > 1) ok = ok && wait_fast<6>(bar_dq(gs), ((gs >> 1) - 1) & 1, s_abort, status);
+        }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        const float* st_l = reinterpret_cast<const float*>(smem + C::kOffStat) + (gs & 1) * 256 + 64 * h;
+        const uint32_t uds = ubase + C::kOffDS + (gs % C::NDS) * (128 * 128 * 2) + h * (128 * 128);      // this warpgroup's 64 columns
+#pragma unroll 1
+        for (int c = 0; c < 2; ++c) {
+          uint32_t rs[32], rd[32];
+          tmem_ld32_issue(lane_addr + C::kColS + 64 * h + 32 * c, rs);
+          tmem_ld32_issue(lane_addr + C::kColDP + 64 * h + 32 * c, rd);
+          tmem_ld32_wait(rs);
+          tmem_ld32_wait(rd);
+          if (masked) {
+            const int first = dead ? 128 : (diag ? row - 64 * h - 32 * c : 0);      // columns below it do not count
 #pragma unroll
-      for (int e = 0; e < 32; e += 4) {
-        float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (t.mode == 1) bias = *reinterpret_cast<const float4*>(s_kbias + colbase + e);
-        const uint64_t off2[2] = {t.mode == 1 ? fadd2(pk2(bias.x, bias.y), nlse2) : nlse2, t.mode == 1 ? fadd2(pk2(bias.z, bias.w), nlse2) : nlse2};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          float x0, x1, p0, p1, d0, d1;
-          upk2(ffma2(pk2u(rs[e + 2 * h], rs[e + 2 * h + 1]), sc2, off2[h]), x0, x1);
-          if (dense_mask) {
-            const int col = colbase + e + 2 * h;
-            if (col >= t.nk || (t.causal && col > t.qk_off + row)) x0 = -INFINITY;
-            if (col + 1 >= t.nk || (t.causal && col + 1 > t.qk_off + row)) x1 = -INFINITY;
+            for (int e = 0; e < 32; ++e)
+              if (e < first) rs[e] = 0xff800000u;
           }
-          asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p0) : "f"(x0));
-          asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p1) : "f"(x1));
-          upk2(fmul2(pk2(p0, p1), fadd2(pk2u(rd[e + 2 * h], rd[e + 2 * h + 1]), ndel2)), d0, d1);
-          pp[(e >> 1) + h] = pack2(p0, p1);
-          dd[(e >> 1) + h] = pack2(d0, d1);
+          uint32_t pp[16];
+#pragma unroll
+          for (int e = 0; e < 32; e += 8) {
+            uint32_t dd[4];
+#pragma unroll
+            for (int x = 0; x < 8; x += 4) {
+              const float4 nl = *reinterpret_cast<const float4*>(st_l + 32 * c + e + x), nd = *reinterpret_cast<const float4*>(st_l + 128 + 32 * c + e + x);
+              const uint64_t nl2[2] = {pack_f2(nl.x, nl.y), pack_f2(nl.z, nl.w)}, nd2[2] = {pack_f2(nd.x, nd.y), pack_f2(nd.z, nd.w)};
+#pragma unroll
+              for (int y = 0; y < 2; ++y) {
+                const int i0 = e + x + 2 * y;
+                float x0, x1, d0, d1;
+                unpack_f2(ffma2(pack_u2(rs[i0], rs[i0 + 1]), sc2, nl2[y]), x0, x1);
+                const float p0 = ex2(x0), p1 = ex2(x1);
+                unpack_f2(fmul2(pack_f2(p0, p1), fadd2(pack_u2(rd[i0], rd[i0 + 1]), nd2[y])), d0, d1);
+                pp[i0 >> 1] = pack2(p0, p1);
+                dd[(x >> 1) + y] = pack2(d0, d1);
+              }
+            }
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(uds + row * 128 + (((4 * c + (e >> 3)) ^ (row & 7)) << 4)),
+                         "r"(dd[0]), "r"(dd[1]), "r"(dd[2]), "r"(dd[3]) : "memory");
+          }
+          // (d = 128: P goes over the scores of this warpgroup that have been read)
+          tmem_st16(lane_addr + C::kColP + C::kPHalf * h + 16 * c, pp);
         }
+        tmem_wait_st();
+        tc_fence_before();
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_h);
       }
-      // row `tid`, key columns c0 .. c0+31 = 16-byte chunks c0/8 .. c0/8+3 of the [query][key] tiles
-#pragma unroll
-      for (int q4 = 0; q4 < 4; ++q4) {
-        const uint32_t off = tile_off<128>(row, c0 / 8 + q4);
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(uP + off), "r"(pp[4 * q4]), "r"(pp[4 * q4 + 1]), "r"(pp[4 * q4 + 2]), "r"(pp[4 * q4 + 3]) : "memory");
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(udS + off), "r"(dd[4 * q4]), "r"(dd[4 * q4 + 1]), "r"(dd[4 * q4 + 2]), "r"(dd[4 * q4 + 3]) : "memory");
-      }
+      if (!ok) break;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_dfree(it));
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    // ---- dQ += dS K, dV = P^T dO, dK = dS^T Q -------------------------------------------------------
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-      for (int kk = 0; kk < TKB / 16; ++kk) mma_ss(tmem + colDQ, kmajor(udS, kk), mnmajor(uK, kk), desc_hi, idesc_dq, (kt > 0 || kk > 0) ? 1u : 0u);
-#pragma unroll
-      for (int kk = 0; kk < 128 / 16; ++kk) mma_ss(tmem + colS, mnmajor(uP, kk), mnmajor(udO, kk), desc_hi, idesc_t, kk > 0);
-#pragma unroll
-      for (int kk = 0; kk < 128 / 16; ++kk) mma_ss(tmem + colDP, mnmajor(udS, kk), mnmajor(uQ, kk), desc_hi, idesc_t, kk > 0);
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-    }
-    if (!mbar_wait_bounded(bar, phase)) *s_abort = 1;
-    phase ^= 1;
-    __syncthreads();
-    if (*s_abort) { ok = false; break; }
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // ---- dV and dK of this key tile leave TMEM: thread = key row ----------------------------------
-    {
-      const int kr = krow_of(kt * TKB + row);
-      // every product that read K and V has finished: the next tile's rows can come in meanwhile
-      if (kt + 1 < ntiles) load_kv(kt + 1);
-      // 2 * D / 32 pieces of 32 columns (dV first, then dK), every fourth one to each group of 128 threads
+  } else if (warp < 12) {
+    // ================= dQ after every step, dK and dV after every item: out of TMEM, into the fp32 accumulators ==================
+    // Rows leave TMEM one per thread, but a reduction instruction whose lanes hit 32 different rows costs the L2 32 half-filled
+    // sectors: a warp's 32 rows x 32 columns pass through shared memory (chunks XOR-swizzled by row) and go out with eight
+    // lanes per row, four rows per instruction.
+    const int row = tid - 256;
+    const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t stage = ubase + C::kOffStage + (warp & 3) * C::kStageWarp;
+    constexpr int NP = C::kStageWarp / 4096;            // 32-column pieces staged together
+    auto out_rows = [&](uint32_t taddr, float f, float* base, size_t seg_row0, int grow, uint32_t bar_done) {
 #pragma unroll 1
-      for (int piece = part; piece < 2 * (D / 32); piece += 4) {
-        const bool is_dk = piece >= D / 32;
-        const int c0 = (piece % (D / 32)) * 32;
-        uint32_t r[32];
-        tmem_ld32(lane_addr + (is_dk ? colDP : colS) + c0, r);
-        reduce_rows(r, is_dk ? b.scale : 1.f, is_dk ? b.dk : b.dv, kr, c0, 0);
+      for (int c0 = 0; c0 < D; c0 += 32 * NP) {
+#pragma unroll 1
+        for (int p = 0; p < NP; ++p) {
+          uint32_t r[32];
+          tmem_ld32_issue(taddr + c0 + 32 * p, r);
+          tmem_ld32_wait(r);
+#pragma unroll
+          for (int c = 0; c < 8; ++c)
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stage + p * 4096 + lane * 128 + ((c ^ (lane & 7)) << 4)),
+                         "f"(__uint_as_float(r[4 * c]) * f), "f"(__uint_as_float(r[4 * c + 1]) * f),
+                         "f"(__uint_as_float(r[4 * c + 2]) * f), "f"(__uint_as_float(r[4 * c + 3]) * f) : "memory");
+        }
+        if (c0 + 32 * NP == D && bar_done) {            // everything has left TMEM
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_done);
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int p = 0; p < NP; ++p) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const int rr = 4 * q + (lane >> 3), c = lane & 7;
+            const int gr = __shfl_sync(0xffffffffu, grow, rr);
+            float4 v;
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                         : "r"(stage + p * 4096 + rr * 128 + ((c ^ (rr & 7)) << 4)) : "memory");
+            if (gr >= 0) atomicAdd(reinterpret_cast<float4*>(base + (seg_row0 + gr) * D + c0 + 32 * p + 4 * c), v);
+          }
+        }
+        __syncwarp();
+      }
+    };
+    for (int it = 0; ok; ++it) {
+      ok = __all_sync(0xffffffffu, wait_desc(it));
+      if (!ok) break;
+      const BwdItem& t = desc_of(it);
+      if (t.kind < 0) break;
+      const size_t seg_row0 = (size_t)t.seg * g.n;
+      const int kr = row < t.nkeys ? key_row(t, row) : -1;
+      const int steps = t.steps;
+#pragma unroll 1
+      for (int s = 0; s < steps; ++s, ++gs) {
+        const StepRows sr = step_rows(b, t, s);
+        int qr = -1;
+        if (row < sr.nq) qr = t.kind == 0 ? sr.first + row : t.q0 + __ldg(a.perm_q + t.slice + sr.first + row);
+        ok = __all_sync(0xffffffffu, wait_fast<7>(bar_dq(gs), (gs >> 1) & 1, s_abort, status));
+        if (!ok) break;
+        tc_fence_after();
+        out_rows(lane_addr + C::kColDQ, b.scale, b.dq, seg_row0, qr, bar_dqfree);
+      }
+      if (!ok) break;
+      ok = __all_sync(0xffffffffu, wait_fast<8>(bar_acc, it & 1, s_abort, status));
+      if (!ok) break;
+      tc_fence_after();
+      out_rows(lane_addr + C::kColDV, 1.f, b.dv, seg_row0, kr, 0);
+      out_rows(lane_addr + C::kColDK, b.scale, b.dk, seg_row0, kr, bar_accfree);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_dfree(it));
+    }
+  } else if (warp == 12) {
+    // ================= MMA issue (one lane) ==================
+    if (lane == 0) {
+      // descriptors: low word = start >> 4 | (leading byte offset >> 4) << 16, high word = stride 1024 B | version | 128-byte swizzle
+      constexpr uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+      constexpr uint32_t kSlab = 128 * 128;             // bytes of one [128 rows x 64 columns] slab
+      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
+      constexpr uint32_t idesc_s = idesc | ((128u >> 3) << 17);                                            // K-major x K-major, N = 128
+      constexpr uint32_t idesc_n = idesc | (1u << 16) | (((uint32_t)D >> 3) << 17);                        // K-major (or TMEM) x MN-major, N = D
+      constexpr uint32_t idesc_t = idesc | (1u << 15) | (1u << 16) | (((uint32_t)D >> 3) << 17);           // MN-major x MN-major, N = D
+      auto kmajor = [&](uint32_t off, int ks) { return ((ubase + off + (ks >> 2) * kSlab + (ks & 3) * 32) >> 4) | (1u << 16); };
+      auto mnmajor = [&](uint32_t off, int kk) { return ((ubase + off + kk * 2048) >> 4) | ((kSlab >> 4) << 16); };
+      uint32_t kv = 0;                                  // where the item's K and V lie
+      auto score = [&](uint32_t gq) {                   // S^T of step gq
+        ok = ok && wait_fast<9>(bar_qfull(gq), (gq >> 1) & 1, s_abort, status);
+        if (!ok) return;
+        fence_async_smem();
+        tc_fence_after();
+        const uint32_t q = C::kOffQ + (gq & 1) * C::kTile;
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColS, kmajor(kv, ks), kmajor(q, ks), desc_hi, idesc_s, ks > 0);
+        umma_commit(bar_s);
+      };
+      auto dscore = [&](uint32_t gq) {                  // dP^T
+        ok = ok && wait_fast<10>(bar_dofull(gq), (gq / C::NDO) & 1, s_abort, status);
+        if (!ok) return;
+        fence_async_smem();
+        tc_fence_after();
+        const uint32_t o = C::kOffDO + (gq % C::NDO) * C::kTile;
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColDP, kmajor(kv + C::kTile, ks), kmajor(o, ks), desc_hi, idesc_s, ks > 0);
+        umma_commit(bar_dp);
+      };
+      for (int it = 0; ok; ++it) {
+        ok = wait_desc(it);
+        if (!ok) break;
+        const BwdItem& t = desc_of(it);
+        if (t.kind < 0) break;
+        const int steps = t.steps;
+        kv = C::kOffKV + (it % C::NKV) * 2 * C::kTile;
+        ok = wait_fast<11>(bar_kv(it), (it / C::NKV) & 1, s_abort, status);
+        if (!ok) break;
+        if (D == 128 && gs > 0) ok = wait_fast<12>(bar_dqfree, (gs - 1) & 1, s_abort, status);
+        score(gs);
+        dscore(gs);
+#pragma unroll 1
+        for (int s = 0; s < steps && ok; ++s, ++gs) {
+          ok = wait_fast<13>(bar_h, gs & 1, s_abort, status);
+          if (!ok) break;
+          tc_fence_after();
+          const bool more = s + 1 < steps;
+          const uint32_t q = C::kOffQ + (gs & 1) * C::kTile, o = C::kOffDO + (gs % C::NDO) * C::kTile, ds = C::kOffDS + (gs % C::NDS) * (128 * 128 * 2);
+          auto grad_v = [&]() {
+            if (s == 0 && it > 0) ok = ok && wait_fast<14>(bar_accfree, (it - 1) & 1, s_abort, status);
+            if (!ok) return;
+            tc_fence_after();
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk)
+              mma_ts2(tmem + C::kColDV, tmem + C::kColP + (kk >> 2) * C::kPHalf + (kk & 3) * 8, mnmajor(o, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
+            umma_commit(bar_dofree(gs));
+          };
+          auto grad_k = [&]() {
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) mma_ss2(tmem + C::kColDK, kmajor(ds, kk), mnmajor(q, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
+            umma_commit(bar_qfree(gs));
+          };
+          auto grad_q = [&]() {
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) mma_ss2(tmem + C::kColDQ, mnmajor(ds, kk), mnmajor(kv, kk), desc_hi, idesc_t, kk > 0);
+            umma_commit(bar_dq(gs));
+          };
+          if (D == 64) {
+            if (more) { score(gs + 1); dscore(gs + 1); }
+            if (!ok) break;
+            grad_v();
+            if (!ok) break;
+            grad_k();
+            if (!more) umma_commit(bar_acc);
+            if (gs > 0) ok = wait_fast<12>(bar_dqfree, (gs - 1) & 1, s_abort, status);
+            if (!ok) break;
+            tc_fence_after();
+            grad_q();
+          } else {
+            grad_q();
+            grad_v();
+            if (!ok) break;
+            if (more) score(gs + 1);
+            if (!ok) break;
+            grad_k();
+            if (!more) umma_commit(bar_acc);
+            else {
+              ok = wait_fast<12>(bar_dqfree, gs & 1, s_abort, status);
+              dscore(gs + 1);
+            }
+          }
+        }
+        if (!ok) break;
+        umma_commit(bar_kvfree(it));
+        mbar_arrive(bar_dfree(it));
       }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();   // S / dP columns and the K, V, P, dS tiles are free again
-  }
-  // ---- dQ: thread = query row (a row collects from every level it appears in) ---------------------
-  if (ok && ntiles > 0) {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    __syncwarp();
+  } else if (warp < 15) {
+    // ================= loaders: warp 13 Q, dO and row statistics of every step, warp 14 K and V of every item ==================
+    // Tiles of consecutive rows: lane 0 issues TMA boxes.  Others: rows gathered in 16-byte chunks, lane -> chunk cc of row
+    // k RPI + crow of instruction k; lane l holds the row numbers of rows l, l + 32, ..., handed round by shuffles.
+    constexpr int CPR = D / 8, RPI = 32 / CPR, NSW = 8 / RPI;
+    const int cc = lane % CPR, crow = lane / CPR;
+    uint32_t sw[NSW];                                    // byte offset of (row k RPI + crow, chunk cc) is k RPI 128 + sw[k % NSW]
+#pragma unroll
+    for (int k = 0; k < NSW; ++k) sw[k] = (uint32_t)((cc >> 3) * (128 * 128) + crow * 128 + (((cc & 7) ^ ((k * RPI + crow) & 7)) << 4));
+    auto gather = [&](uint32_t dst, const __nv_bfloat16* base, const int (&v)[4], uint32_t bar) {
+      const char* src = reinterpret_cast<const char*>(base) + cc * 16;
+#pragma unroll
+      for (int k = 0; k < 128 / RPI; ++k) {
+        const int rw = __shfl_sync(0xffffffffu, v[k * RPI / 32], (k * RPI & 31) + crow);
+        cp_async16(dst + k * RPI * 128 + sw[k % NSW], src + (size_t)(uint32_t)rw * (D * 2));
+      }
+      cp_async_arrive_noinc(bar);
+    };
+    auto boxes = [&](uint32_t dst, const CUtensorMap* map, int y, uint32_t bar) {
+#pragma unroll
+      for (int sl = 0; sl < D / 64; ++sl) tma_tile(dst + sl * (128 * 128), map, sl * 64, y, bar);
+    };
+    if (warp == 13) {
+      for (int it = 0; ok; ++it) {
+        ok = __all_sync(0xffffffffu, wait_desc(it));
+        if (!ok) break;
+        const BwdItem& t = desc_of(it);
+        if (t.kind < 0) break;
+        const int steps = t.steps, seg_row0 = t.seg * g.n;
+        const float wlog = t.wlog;
+        // row numbers and statistics of a step's query rows (rows that do not exist: the node's first row, with weights of zero)
+        int vn[4];
+        float2 sn[4];
+        auto rows_of = [&](int s) {
+          const StepRows sr = step_rows(b, t, s);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int r = lane + 32 * u;
+            const bool in = r < sr.nq;
+            int x = t.q0;
+            if (in) x = t.kind == 0 ? sr.first + r : t.q0 + __ldg(a.perm_q + t.slice + sr.first + r);
+            vn[u] = seg_row0 + x;
+            sn[u] = in ? __ldg(b.stat + vn[u]) : make_float2(-INFINITY, 0.f);
+          }
+        };
+        rows_of(0);
 #pragma unroll 1
-    for (int c0 = 32 * part; c0 < D; c0 += 128) {
-      uint32_t r[32];
-      tmem_ld32(lane_addr + colDQ + c0, r);
-      // (without the causal recursion a query row belongs to exactly one tile: its dQ is final)
-      reduce_rows(r, b.scale, b.dq_mode ? reinterpret_cast<float*>(b.dq_final) : b.dq, my_qrow, c0, b.dq_mode);
+        for (int s = 0; s < steps; ++s, ++gs) {
+          const int v[4] = {vn[0], vn[1], vn[2], vn[3]};
+          if (gs > 1) {
+            ok = __all_sync(0xffffffffu, wait_fast<16>(bar_qfree(gs), ((gs >> 1) - 1) & 1, s_abort, status));
+            if (!ok) break;
+          }
+          float* st = reinterpret_cast<float*>(smem + C::kOffStat) + (gs & 1) * 256;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) { st[lane + 32 * u] = sn[u].x + wlog; st[128 + lane + 32 * u] = sn[u].y; }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_stat(gs));
+          const uint32_t dq = ubase + C::kOffQ + (gs & 1) * C::kTile, dd = ubase + C::kOffDO + (gs % C::NDO) * C::kTile;
+          const bool dense = t.kind == 0;
+          const int y = seg_row0 + t.q0 + s * kTileQ;
+          if (dense) {
+            if (lane == 0) { mbar_expect_tx(bar_qfull(gs), C::kTile); boxes(dq, &maps.q, y, bar_qfull(gs)); }
+            __syncwarp();
+            mbar_arrive(bar_qfull(gs));
+          } else gather(dq, a.q, v, bar_qfull(gs));
+          if (s + 1 < steps) rows_of(s + 1);               // (in flight while this step's copies are issued)
+          if (gs >= C::NDO) {
+            ok = __all_sync(0xffffffffu, wait_fast<17>(bar_dofree(gs), (gs / C::NDO - 1) & 1, s_abort, status));
+            if (!ok) break;
+          }
+          if (dense) {
+            if (lane == 0) { mbar_expect_tx(bar_dofull(gs), C::kTile); boxes(dd, &maps.dout, y, bar_dofull(gs)); }
+            __syncwarp();
+            mbar_arrive(bar_dofull(gs));
+          } else gather(dd, b.dout, v, bar_dofull(gs));
+        }
+        if (!ok) break;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_dfree(it));
+      }
+      cp_async_commit();
+      cp_async_wait_all();
+      // (nothing may be in flight into shared memory when the CTA exits - trivially true unless it is giving up)
+      if (!ok) for (int x = 0; x < 2; ++x) { mbar_drain(bar_qfull(x), 0); mbar_drain(bar_qfull(x), 1); mbar_drain(bar_dofull(x % C::NDO), 0); mbar_drain(bar_dofull(x % C::NDO), 1); }
+    } else {
+      int it = 0;
+      for (; ok; ++it) {
+        ok = __all_sync(0xffffffffu, wait_desc(it));
+        if (!ok) break;
+        const BwdItem& t = desc_of(it);
+        if (t.kind < 0) break;
+        const uint32_t dst = ubase + C::kOffKV + (it % C::NKV) * 2 * C::kTile, bar = bar_kv(it);
+        const int seg_row0 = t.seg * g.n;
+        int v[4];
+        if (t.kind != 0) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[u] = seg_row0 + key_row(t, min(lane + 32 * u, t.nkeys - 1));     // (keys that do not exist: the last one)
+        }
+        if (it >= C::NKV) {
+          ok = __all_sync(0xffffffffu, wait_fast<18>(bar_kvfree(it), (it / C::NKV - 1) & 1, s_abort, status));
+          if (!ok) break;
+        }
+        if (t.kind == 0) {
+          if (lane == 0) {
+            mbar_expect_tx(bar, 2 * C::kTile);
+            boxes(dst, &maps.k, seg_row0 + t.k0, bar);
+            boxes(dst + C::kTile, &maps.v, seg_row0 + t.k0, bar);
+          }
+          __syncwarp();
+          mbar_arrive(bar);
+        } else {
+          const char* srck = reinterpret_cast<const char*>(a.k) + cc * 16;
+#pragma unroll
+          for (int k = 0; k < 128 / RPI; ++k) {
+            const int rw = __shfl_sync(0xffffffffu, v[k * RPI / 32], (k * RPI & 31) + crow);
+            cp_async16(dst + k * RPI * 128 + sw[k % NSW], srck + (size_t)(uint32_t)rw * (D * 2));
+          }
+          gather(dst + C::kTile, a.v, v, bar);            // (its arrival covers both tiles' copies)
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_dfree(it));
+      }
+      cp_async_commit();
+      cp_async_wait_all();
+      if (!ok) for (int x = 0; x < C::NKV; ++x) { mbar_drain(bar_kv(x), 0); mbar_drain(bar_kv(x), 1); }
+    }
+  } else {
+    // ================= item descriptors ==================
+    // Work items are handed out by a counter in global memory, in list order (heavy first); the first gridDim.x need none.
+    int item = blockIdx.x;
+    for (int it = 0; ok; ++it) {
+      BwdItem t;
+      for (;; ) {
+        if (it > 0 || item < 0) {
+          if (lane == 0) item = gridDim.x + atomicAdd(b.sched, 1);
+          item = __shfl_sync(0xffffffffu, item, 0);
+        }
+        if (item >= b.total_items) { t.kind = -1; break; }
+        if (decode_item(b, item, t)) break;
+        item = -1;
+      }
+      if (it >= kDescs) {
+        ok = __all_sync(0xffffffffu, wait_fast<19>(bar_dfree(it), (it / kDescs - 1) & 1, s_abort, status));
+        if (!ok) break;
+      }
+      if (lane == 0) {
+        *reinterpret_cast<BwdItem*>(smem + C::kOffDesc + (it % kDescs) * C::kDescBytes) = t;
+        mbar_arrive(bar_dfull(it));
+      }
+      __syncwarp();
+      if (t.kind < 0) break;
     }
   }
-  if (!ok && tid == 0) atomicOr(status, 1 << 30);      // a bounded wait gave up
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+
+  // ---- teardown ------------------------------------------------------------------------------------
+  tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  if (warp == 12) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
   }
 }
 
-__global__ void to_bf16_kernel(const float4* __restrict__ src, uint2* __restrict__ dst, size_t count4) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count4; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 v = src[i];
-    dst[i] = make_uint2(pack2(v.x, v.y), pack2(v.z, v.w));
+// the three fp32 accumulators (one after the other) rounded to bf16: 32 bytes in, 16 out per thread and pass
+__global__ void __launch_bounds__(256) to_bf16_kernel(const float4* __restrict__ src, uint4* __restrict__ dq, uint4* __restrict__ dk, uint4* __restrict__ dv, size_t count8) {
+  uint4* dst = blockIdx.y == 0 ? dq : (blockIdx.y == 1 ? dk : dv);
+  src += (size_t)blockIdx.y * count8 * 2;
+  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < count8; i += (size_t)gridDim.x * 256) {
+    const float4 x = __ldcs(src + 2 * i), y = __ldcs(src + 2 * i + 1);
+    __stcs(dst + i, make_uint4(pack2(x.x, x.y), pack2(x.z, x.w), pack2(y.x, y.y), pack2(y.z, y.w)));
   }
 }
 
 }  // namespace
 
-// a: the forward schedule (tile list, permutations, samples); dq/dk/dv accumulators must be zero
-cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout,
-                            float* delta, float* dq, float* dk, float* dv, void* dq_final, int dq_mode, float scale, int* status, cudaStream_t st) {
-  const size_t rows = (size_t)a.g.G * a.g.n;
-  const __nv_bfloat16* d16 = reinterpret_cast<const __nv_bfloat16*>(dout);
-  const int dgrid = (int)((rows + 7) / 8);
-  if (a.g.d == 64) {
-    if (out_fp32) delta_kernel<64, true><<<dgrid, 256, 0, st>>>(d16, out, delta, rows);
-    else delta_kernel<64, false><<<dgrid, 256, 0, st>>>(d16, out, delta, rows);
-  } else {
-    if (out_fp32) delta_kernel<128, true><<<dgrid, 256, 0, st>>>(d16, out, delta, rows);
-    else delta_kernel<128, false><<<dgrid, 256, 0, st>>>(d16, out, delta, rows);
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || a.total_tiles == 0) return e;
-  BwdArgs b;
-  b.a = a; b.dout = d16; b.lse = lse; b.delta = delta; b.dq = dq; b.dk = dk; b.dv = dv; b.dq_final = dq_final; b.dq_mode = dq_mode; b.scale = scale;
+// a: the forward schedule (permutations, samples, tile geometry); the accumulators dq, dk, dv must be zero
+cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout, float2* stat, int* sched,
+                            float* dq, float* dk, float* dv, float scale, int* status, cudaStream_t st) {
+  const Geometry& g = a.g;
+  const size_t rows = (size_t)g.G * g.n;
   if (rows > 0x7fffffffull) return cudaErrorInvalidValue;            // TMA row coordinates are 32-bit
+  {
+    const unsigned grid = (unsigned)((rows * (g.d / 8) + 255) / 256);
+    const uint4* d4 = reinterpret_cast<const uint4*>(dout);
+    if (g.d == 64) {
+      if (out_fp32) row_stat_kernel<64, true><<<grid, 256, 0, st>>>(d4, out, lse, stat, rows, sched);
+      else row_stat_kernel<64, false><<<grid, 256, 0, st>>>(d4, out, lse, stat, rows, sched);
+    } else {
+      if (out_fp32) row_stat_kernel<128, true><<<grid, 256, 0, st>>>(d4, out, lse, stat, rows, sched);
+      else row_stat_kernel<128, false><<<grid, 256, 0, st>>>(d4, out, lse, stat, rows, sched);
+    }
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cudaErrorUnknown;
+  BwdArgs b;
+  b.a = a; b.dout = reinterpret_cast<const __nv_bfloat16*>(dout); b.stat = stat; b.dq = dq; b.dk = dk; b.dv = dv; b.scale = scale; b.sched = sched;
+  b.leaf_ktiles = a.n_leaf_tiles ? (g.leaf + kTileK - 1) / kTileK : 0;
+  b.block_ktiles = (g.b + kTileK - 1) / kTileK;
+  b.smp_ktiles = (g.m + kTileK - 1) / kTileK;
+  // Sampled items take at most 16 query tiles (their dK and dV leave once per item) and fewer where that leaves less than
+  // about six items for an SM.
+  long long steps = 0;
+  for (int l = 0; l < g.levels; ++l) {
+    int s, q0, k0;
+    node_rows(g, l, 0, s, q0, k0);
+    if (a.level_sorted[l]) steps += (long long)(g.causal ? (1 << l) : 1) * g.G * node_blocks(s, g.b) * a.tiles_per_block * (b.smp_ktiles + b.block_ktiles);
+  }
+  if (b.leaf_ktiles) steps += (long long)a.leaves_per_seg * g.G * b.leaf_ktiles * (a.dense_causal ? (b.leaf_ktiles + 1) / 2 : b.leaf_ktiles);
+  const long long want = steps / (6LL * sms);
+  b.chunk = (int)(want < 2 ? 2 : (want > 16 ? 16 : want));
+  long long items = b.leaf_ktiles ? (long long)g.G * a.leaves_per_seg * b.leaf_ktiles : 0;
+  b.n_leaf_items = (int)items;
+  for (int l = 0; l < g.levels; ++l) {
+    int s, q0, k0;
+    node_rows(g, l, 0, s, q0, k0);
+    b.level_item_start[l] = (int)items;
+    long long per_node = (s + kTileK - 1) / kTileK;
+    if (a.level_sorted[l]) {
+      const int blocks = node_blocks(s, g.b), tiles_node = blocks * a.tiles_per_block;
+      per_node = (long long)b.smp_ktiles * ((tiles_node + b.chunk - 1) / b.chunk) + (long long)blocks * b.block_ktiles;
+    }
+    items += per_node * (g.causal ? (1 << l) : 1) * g.G;
+    if (items > 0x7fffffffLL) return cudaErrorInvalidValue;
+  }
+  b.level_item_start[g.levels] = (int)items;
+  b.total_items = (int)items;
+  if (items == 0) return cudaSuccess;
   BwdMaps maps;
-  if (!encode_rows_map(&maps.k, a.k, rows, a.g.d, 128) || !encode_rows_map(&maps.v, a.v, rows, a.g.d, 128)) return cudaErrorInvalidValue;
-  b.table_keys = a.g.sorted ? (a.g.b + TKB - 1) / TKB * TKB + (a.g.m + TKB - 1) / TKB * TKB : 0;
-  if (b.table_keys > kMaxNodeKeys) return cudaErrorInvalidValue;
+  if (!encode_rows_map(&maps.q, a.q, rows, g.d, 128) || !encode_rows_map(&maps.k, a.k, rows, g.d, 128) ||
+      !encode_rows_map(&maps.v, a.v, rows, g.d, 128) || !encode_rows_map(&maps.dout, dout, rows, g.d, 128)) return cudaErrorInvalidValue;
   auto go = [&](auto kernel, int smem_bytes) {
-    cudaError_t e2 = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes + kMaxNodeKeys * 8);
-    if (e2 != cudaSuccess) return e2;
-    kernel<<<a.total_tiles, kBwdThreads, smem_bytes + b.table_keys * 8, st>>>(b, maps, status);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    if (e != cudaSuccess) return e;
+    kernel<<<items < sms ? (unsigned)items : (unsigned)sms, kThreads, smem_bytes, st>>>(b, maps, status);      // persistent: one CTA per SM
     return cudaGetLastError();
   };
-  if (a.g.d == 64) return go(bwd_tc_kernel<64>, SmemTc<64>::kFixed);
-  return go(bwd_tc_kernel<128>, SmemTc<128>::kFixed);
+  return g.d == 64 ? go(bwd_kernel<64>, Cfg<64>::kTotal) : go(bwd_kernel<128>, Cfg<128>::kTotal);
 }
 
-cudaError_t launch_to_bf16(const float* src, void* dst, size_t count, cudaStream_t st) {
-  const size_t count4 = count / 4;
-  int blocks = (int)((count4 + 255) / 256);
-  if (blocks > 148 * 16) blocks = 148 * 16;
-  if (blocks < 1) blocks = 1;
-  to_bf16_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const float4*>(src), reinterpret_cast<uint2*>(dst), count4);
+// src: dq, dk, dv one after the other, count entries each (a multiple of 8)
+cudaError_t launch_to_bf16(const float* src, void* dq, void* dk, void* dv, size_t count, cudaStream_t st) {
+  const size_t count8 = count / 8, want = (count8 + 255) / 256;
+  const dim3 grid((unsigned)(want < 148 * 16 ? want : 148 * 16), 3);
+  to_bf16_kernel<<<grid, 256, 0, st>>>(reinterpret_cast<const float4*>(src), reinterpret_cast<uint4*>(dq), reinterpret_cast<uint4*>(dk), reinterpret_cast<uint4*>(dv), count8);
   return cudaGetLastError();
 }
 

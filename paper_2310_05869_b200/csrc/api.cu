@@ -15,7 +15,7 @@
 namespace hyperattn {
 cudaError_t launch_attention_mma(const AttnArgs& a, cudaStream_t st);
 cudaError_t launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st);
-cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uint32_t* wq, unsigned long long* cum, int32_t* samples,
+cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uint32_t* wq, unsigned long long* sums, unsigned long long* cum, int32_t* samples,
                                   float* wlog, uint64_t seed, cudaStream_t st);
 cudaError_t launch_tau(const AttnArgs& at, const int32_t* tpos, float* ltau, cudaStream_t st);
 cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout, float2* stat, int* sched,
@@ -79,15 +79,19 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
     const int bpad = (g.b + 127) / 128 * 128, mpad = (g.m + 127) / 128 * 128;
     if (2 * bpad + mpad > kMaxNodeKeys) return HYPERATTN_UNSUPPORTED_SHAPE;
   }
-  g.chunks_per_unit = (g.unit + kSortChunk - 1) / kSortChunk;
+  // Chunks of 2048 rows, halved (down to 256) while a side's hash would leave SMs without a CTA: three CTAs of the hash per SM
+  // are resident, and below that the longest chunk is the whole time (32 heads of 4096 rows: MEASURED_HASH).
+  g.chunk = kSortChunk;
+  while (g.chunk > 256 && (long long)g.G * ((g.npad / g.unit) * ((g.unit + g.chunk - 1) / g.chunk) + (g.causal ? (g.npad / g.unit) : 1) * ((g.unit_k + g.chunk - 1) / g.chunk)) < 444) g.chunk /= 2;
+  g.chunks_per_unit = (g.unit + g.chunk - 1) / g.chunk;
   g.chunks_per_seg = (g.npad / g.unit) * g.chunks_per_unit;
-  g.chunks_per_unit_k = (g.unit_k + kSortChunk - 1) / kSortChunk;
+  g.chunks_per_unit_k = (g.unit_k + g.chunk - 1) / g.chunk;
   g.chunks_per_seg_k = g.causal ? g.chunks_per_seg : g.chunks_per_unit_k;
   return HYPERATTN_OK;
 }
 
 struct Plan {
-  size_t q16, k16, v16, q16lo, k16lo, ids, hist, offs, perm_q, perm_k, rank_k, samples, tpos, ltau, vwq, vcum, swlog, wnodes, sched, part_o, part_lse, total;
+  size_t q16, k16, v16, q16lo, k16lo, ids, hist, offs, perm_q, perm_k, rank_k, samples, tpos, ltau, vwq, vsum, vcum, swlog, wnodes, sched, part_o, part_lse, total;
   size_t stat, gacc;    // backward only: (-lse, -<dO, O>) per row; fp32 gradient accumulators (bf16 gradients only)
 };
 
@@ -117,6 +121,7 @@ Plan make_plan(const Geometry& g, int is_fp32, int backward = 0, bool capped = f
   pl.tpos = take(capped ? (size_t)g.G * g.nodes * g.m * 4 : 0);
   pl.ltau = take(capped ? (size_t)g.G * g.nodes * 4 : 0);
   pl.vwq = take(vnorm ? (size_t)g.G * g.nk * 4 : 0);
+  pl.vsum = take(vnorm ? (size_t)g.G * ((g.nk + 255) / 256) * 8 : 0);
   pl.vcum = take(vnorm ? (size_t)g.G * ((size_t)g.nk + 1) * 8 : 0);
   pl.swlog = take(vnorm ? (size_t)g.G * g.nodes * g.m * 4 : 0);
   const size_t part_rows = (g.L && !backward) ? (size_t)g.G * g.n + lvl_rows : 0;
@@ -290,6 +295,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
   ws.part_o = base + pl.part_o;
   ws.part_bf16 = part_bf16;
   ws.part_lse = reinterpret_cast<float*>(base + pl.part_lse);
+  ws.sched = reinterpret_cast<int*>(base + pl.sched);
   ws.status = ds.status;
 
   const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.f / std::sqrt((float)p.d);
@@ -301,11 +307,9 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
   const __nv_bfloat16 *q16 = reinterpret_cast<const __nv_bfloat16*>(p.q), *k16 = reinterpret_cast<const __nv_bfloat16*>(p.k),
                       *v16 = reinterpret_cast<const __nv_bfloat16*>(p.v);
   if (is_fp32) {
-    StageScope sc(st, HYPERATTN_STAGE_CONVERT, 3);
-    const size_t cnt = (size_t)g.G * g.n * g.d, cnt_k = (size_t)g.G * g.nk * g.d;
-    HA_CHECK(launch_convert(reinterpret_cast<const float*>(p.q), ws.q16, ws.q16lo, cnt, st));
-    HA_CHECK(launch_convert(reinterpret_cast<const float*>(p.k), ws.k16, ws.k16lo, cnt_k, st));
-    HA_CHECK(launch_convert(reinterpret_cast<const float*>(p.v), ws.v16, nullptr, cnt_k, st));
+    StageScope sc(st, HYPERATTN_STAGE_CONVERT, 1);
+    HA_CHECK(launch_convert(reinterpret_cast<const float*>(p.q), reinterpret_cast<const float*>(p.k), reinterpret_cast<const float*>(p.v), ws,
+                            (size_t)g.G * g.n * g.d, (size_t)g.G * g.nk * g.d, st));
     q16 = ws.q16; k16 = ws.k16; v16 = ws.v16;
   }
   if (g.sorted) {
@@ -335,7 +339,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     }
     if (vnorm) {
       StageScope sc(st, HYPERATTN_STAGE_SAMPLE, 3);
-      HA_CHECK(launch_vnorm_sampling(g, v16, reinterpret_cast<uint32_t*>(base + pl.vwq), reinterpret_cast<unsigned long long*>(base + pl.vcum),
+      HA_CHECK(launch_vnorm_sampling(g, v16, reinterpret_cast<uint32_t*>(base + pl.vwq), reinterpret_cast<unsigned long long*>(base + pl.vsum), reinterpret_cast<unsigned long long*>(base + pl.vcum),
                                      ws.samples, reinterpret_cast<float*>(base + pl.swlog), p.seed, st));
       if (dbg && dbg->sample_log2w)
         HA_CHECK(cudaMemcpyAsync(dbg->sample_log2w, base + pl.swlog, (size_t)g.G * g.nodes * g.m * 4, cudaMemcpyDeviceToDevice, st));
@@ -396,13 +400,12 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     tiles += per_node * nodes_lvl * g.G;
     if (tiles > 0x7fffffffLL) return HYPERATTN_UNSUPPORTED_SHAPE;
     a.level_pair_start[l] = (int)pairs;
-    // two query tiles share a CTA when they share their block's keys (even tiles per block),
-    // or when a block is a single tile; other block sizes run one tile per CTA (a pair that
-    // straddles two larger blocks would make each tile's issuer skip more key tiles of the
-    // other's block than the stage ring holds, which the ring's release order does not allow)
-    // (a single query tile per group only pairs up when the groups' key blocks are short as well: with fewer
-    // queries than keys a group of at most 128 queries can face a key block of many tiles)
-    a.level_paired[l] = !a.level_sorted[l] || a.tiles_per_block % 2 == 0 || (a.tiles_per_block == 1 && g.b <= kTileQ);
+    // Two query tiles share a CTA when they share their block's keys (even tiles per block).  Pairs that straddle
+    // two blocks walk both blocks' key tiles, each tile's issuer skipping the other's: it releases the K stages of the tiles it
+    // skips before the V stages, so a block's tiles and one more have to fit the ring of 8 (d = 64) or 4 (d = 128) stages.  Beyond that
+    // one tile per CTA, which leaves half of its softmax warps idle (50 000 queries against 131 072 keys, groups of 98 queries and
+    // blocks of 256 keys: 218 us unpaired, MEASURED_PAIR us paired).
+    a.level_paired[l] = !a.level_sorted[l] || a.tiles_per_block % 2 == 0 || (g.b + 63) / 64 + 1 <= (g.d == 64 ? 8 : 4);
     pairs += (a.level_paired[l] ? (per_node + 1) / 2 : per_node) * nodes_lvl * g.G;
   }
   a.level_start[g.levels] = (int)tiles;
@@ -419,7 +422,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     StageScope sc(st, HYPERATTN_STAGE_BACKWARD, 2 + (g32 ? 0 : 1));
     if (g32) for (float* x : {dq, dk, dv}) HA_CHECK(cudaMemsetAsync(x, 0, elems * 4, st));
     else HA_CHECK(cudaMemsetAsync(acc, 0, 3 * elems * 4, st));
-    HA_CHECK(launch_backward(a, p.out, out_fp32, p.lse, bw->dout, reinterpret_cast<float2*>(base + pl.stat), reinterpret_cast<int*>(base + pl.sched),
+    HA_CHECK(launch_backward(a, p.out, out_fp32, p.lse, bw->dout, reinterpret_cast<float2*>(base + pl.stat), ws.sched,
                              dq, dk, dv, scale, ws.status, st));
     if (!g32) HA_CHECK(launch_to_bf16(acc, bw->dq, bw->dk, bw->dv, elems, st));
     return HYPERATTN_OK;
@@ -436,8 +439,8 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     // bf16 inputs: tcgen05 path; fp32 inputs: split-bf16 logits on the warp-level MMA path
     if (is_fp32) HA_CHECK(launch_attention_mma(a, st));
     else {
-      a.sched = reinterpret_cast<int*>(base + pl.sched);
-      HA_CHECK(cudaMemsetAsync(a.sched, 0, 4, st));
+      a.sched = ws.sched;
+      if (!g.sorted) HA_CHECK(cudaMemsetAsync(a.sched, 0, 4, st));       // (else the sort scan has zeroed it)
       HA_CHECK(launch_attention_tc(a, ws.status, st));
     }
   }

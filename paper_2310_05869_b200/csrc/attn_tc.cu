@@ -762,9 +762,11 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
                 asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}" : "+f"(lrta), "+f"(lrtb) : "r"(w));
               p[e >> 1] = w;
               if constexpr (PRECISE) {
-                // what the rounding to bf16 left over, as a second bf16 number (infinite weights leave none)
-                const float r0 = p0 - __uint_as_float(w << 16), r1 = p1 - __uint_as_float(w & 0xffff0000u);
-                const uint32_t wl = pack2(r0 == r0 ? r0 : 0.f, r1 == r1 ? r1 : 0.f);
+                // what the rounding to bf16 left over, as a second bf16 number (an infinite weight leaves NaN here, but it
+                // also makes the tile's sum infinite, and the tile is exponentiated again)
+                float r0, r1;
+                unpack_f2(fadd2(pack_f2(p0, p1), pack_f2(-__uint_as_float(w << 16), -__uint_as_float(w & 0xffff0000u))), r0, r1);
+                const uint32_t wl = pack2(r0, r1);
                 if constexpr (!C::kOnes)
                   asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}" : "+f"(lrta), "+f"(lrtb) : "r"(wl));
                 plo[e >> 1] = wl;

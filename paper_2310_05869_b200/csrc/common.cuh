@@ -8,7 +8,7 @@
 
 namespace hyperattn {
 
-constexpr int kSortChunk = 2048;      // rows per histogram / scatter chunk
+constexpr int kSortChunk = 2048;      // most rows per histogram / scatter chunk
 constexpr int kBuckets = 256;         // 2^r with r <= 8
 constexpr int kTileQ = 128;           // query rows per attention tile
 constexpr int kMaxLevelsMerge = 24;   // deepest causal recursion supported
@@ -45,7 +45,7 @@ constexpr uint32_t kDomainDirections = 1, kDomainSamples = 2, kDomainRowSubset =
 
 // ---- geometry of one forward call, shared by all stages --------------------------------
 // "unit" = the largest row range that never straddles a recursion node: a causal leaf of n0
-// rows, or the whole segment.  Units are cut into chunks of at most kSortChunk rows; one
+// rows, or the whole segment.  Units are cut into chunks of `chunk` rows; one
 // hash CTA produces the ids and the 256-bin histogram of one chunk, one scatter CTA places it.
 struct Geometry {
   int G, n, d;         // n: query rows per segment
@@ -58,6 +58,7 @@ struct Geometry {
   int causal;          // 1: causal with L >= 1 levels or a single causal leaf
   int L;               // number of recursion levels with off-diagonal nodes (0: none)
   int leaf;            // rows per exact leaf (n if L == 0)
+  int chunk;           // rows per chunk: kSortChunk, or less where the problem is small (a multiple of 256)
   int unit;            // rows per unit (query side; both sides of a causal call)
   int chunks_per_unit;
   int chunks_per_seg;  // (npad / unit) * chunks_per_unit
@@ -119,10 +120,12 @@ struct Workspace {
   float* ltau;                     // capped row sums: [G, nodes] log2 of the largest unmasked probe row sum
   void* part_o; float* part_lse;   // causal partials: leaf [G,n,(d)] then per level [G,nl,(d)]; rows of fp32 or bf16
   int part_bf16;
+  int* sched;                      // work counter of the attention launch: zeroed by the sort scan
   int* status;                     // device status word
 };
 
-cudaError_t launch_convert(const float* src, __nv_bfloat16* hi, __nv_bfloat16* lo, size_t count, cudaStream_t st);
+// fp32 inputs of count_q (q) and count_k (k, v) entries to the workspace's bf16 copies
+cudaError_t launch_convert(const float* q, const float* k, const float* v, const Workspace& ws, size_t count_q, size_t count_k, cudaStream_t st);
 // w_host: the shared direction matrix; w_nodes (device, [nodes, d, r], g.node_dirs only): the nodes' own
 cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_fp32, const float* w_host,
                         const Workspace& ws, unsigned long long* near_zero, cudaStream_t st, int side_mask = 3,

@@ -52,6 +52,7 @@ struct HashArgs {
   unsigned long long* near_zero;
   int G, r;
   int side_mask;          // bit s set: side s is hashed
+  int chunk;              // rows per chunk
   int n[2];               // rows per segment of either side
   int unit[2], chunks_per_unit[2], chunks_per_seg[2];
   // directions of every recursion node's own (causal calls): the grid covers every level; a chunk belongs to
@@ -74,8 +75,8 @@ __device__ __forceinline__ ChunkPos chunk_of_cta(const HashArgs& a, int cta) {
   c.chunk = cta % a.chunks_per_seg[c.side];
   c.seg = cta / a.chunks_per_seg[c.side];
   const int unit_idx = c.chunk / a.chunks_per_unit[c.side], cu = c.chunk % a.chunks_per_unit[c.side];
-  c.row0 = unit_idx * a.unit[c.side] + cu * kSortChunk;
-  c.rows = max(0, min(min(kSortChunk, a.unit[c.side] - cu * kSortChunk), a.n[c.side] - c.row0));
+  c.row0 = unit_idx * a.unit[c.side] + cu * a.chunk;
+  c.rows = max(0, min(min(a.chunk, a.unit[c.side] - cu * a.chunk), a.n[c.side] - c.row0));
   if (a.w_nodes) {
     // level l: nodes of 2 u units, u = 2^(L - 1 - l); queries live in the second half, keys in the first
     const int u = 1 << (a.L - 1 - c.level);
@@ -93,8 +94,8 @@ __device__ __forceinline__ size_t hist_base(const HashArgs& a, const ChunkPos& c
   return c.level * a.hist_level_stride + ((c.side ? (size_t)a.G * a.chunks_per_seg[0] : 0) + (size_t)c.seg * a.chunks_per_seg[c.side] + c.chunk) * kBuckets;
 }
 
-// One CTA = one chunk (<= kSortChunk rows of one side of one segment).  Each warp walks over
-// groups of 16 rows; the loads of the next group are issued before the MMAs of the current
+// One CTA = one chunk (<= a.chunk rows of one side of one segment).  Each warp walks over
+// groups of 16 rows; the loads of the next group are issued between the MMAs of the current
 // one, and the direction fragments live in shared memory (one 8-byte read per MMA) instead
 // of 48 registers, so that two to four CTAs fit an SM and ~128 KB of loads are in flight.
 template <int D>
@@ -117,16 +118,17 @@ __global__ void __launch_bounds__(256, D == 64 ? 4 : 3) hash_bf16_kernel(const _
   const char* base = reinterpret_cast<const char*>(a.x[side]) + ((size_t)seg * a.n[side] + row0) * (D * 2);
   unsigned nz = 0;
   const int groups = (rows + 15) >> 4;
+  // The 16-byte chunks of a lane's two rows are asked for again (for the warp's next group) as soon as they have been
+  // multiplied: no second set of registers, and no spills at d = 128.
   uint4 xa[CPL], xb[CPL];
-  auto load_group = [&](int grp, uint4 (&pa)[CPL], uint4 (&pb)[CPL]) {
+  auto load_chunk = [&](int grp, int h) {
     const int ra = grp * 16 + gid, rb = ra + 8;
-#pragma unroll
-    for (int h = 0; h < CPL; ++h) {
-      pa[h] = (grp < groups && ra < rows) ? ldg_stream(base + (size_t)ra * (D * 2) + (tig + 4 * h) * 16) : make_uint4(0, 0, 0, 0);
-      pb[h] = (grp < groups && rb < rows) ? ldg_stream(base + (size_t)rb * (D * 2) + (tig + 4 * h) * 16) : make_uint4(0, 0, 0, 0);
-    }
+    const char* pa = base + (size_t)ra * (D * 2) + (tig + 4 * h) * 16;
+    xa[h] = ra < rows ? ldg_stream(pa) : make_uint4(0, 0, 0, 0);
+    xb[h] = rb < rows ? ldg_stream(pa + 8 * (D * 2)) : make_uint4(0, 0, 0, 0);
   };
-  load_group(warp, xa, xb);                           // the first rows are on their way while the fragments are built
+#pragma unroll
+  for (int h = 0; h < CPL; ++h) load_chunk(warp, h);  // the first rows are on their way while the fragments are built
 
   // Direction fragments.  k-slot (step s, half h, element e) of lane (gid, tig) holds
   // coordinate 8*(tig + 4*(s>>1)) + 2*(2*(s&1) + h) + e; column gid is direction gid.
@@ -157,8 +159,6 @@ __global__ void __launch_bounds__(256, D == 64 ? 4 : 3) hash_bf16_kernel(const _
 
   for (int grp = warp; grp < groups; grp += 8) {
     const int ra = grp * 16 + gid, rb = ra + 8;
-    uint4 na[CPL], nb[CPL];
-    load_group(grp + 8, na, nb);                      // in flight while this group is multiplied
     float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int s = 0; s < KS; ++s) {
@@ -172,6 +172,7 @@ __global__ void __launch_bounds__(256, D == 64 ? 4 : 3) hash_bf16_kernel(const _
       mma_bf16_16816(lo, af, w3.x, w3.y);
       mma_bf16_16816(lo, af, w2.x, w2.y);
       mma_bf16_16816(hi, af, w1.x, w1.y);
+      if (s & 1) load_chunk(grp + 8, s >> 1);         // (rows past the end are not read)
     }
     // lane holds p[row gid][2tig], p[gid][2tig+1], p[gid+8][2tig], p[gid+8][2tig+1]
     float p[4];
@@ -187,8 +188,6 @@ __global__ void __launch_bounds__(256, D == 64 ? 4 : 3) hash_bf16_kernel(const _
     gb |= __shfl_xor_sync(0xffffffffu, gb, 1); gb |= __shfl_xor_sync(0xffffffffu, gb, 2);
     if (tig == 0 && ra < rows) { const uint32_t id = gray_rank8(ga); s_ids[ra] = (uint8_t)id; atomicAdd(&s_hist[id], 1u); }
     if (tig == 1 && rb < rows) { const uint32_t id = gray_rank8(gb); s_ids[rb] = (uint8_t)id; atomicAdd(&s_hist[id], 1u); }
-#pragma unroll
-    for (int h = 0; h < CPL; ++h) { xa[h] = na[h]; xb[h] = nb[h]; }
   }
   if (a.near_zero) {
 #pragma unroll
@@ -206,75 +205,92 @@ __global__ void __launch_bounds__(256, D == 64 ? 4 : 3) hash_bf16_kernel(const _
   a.hist[hist_base(a, cp) + tid] = s_hist[tid];
 }
 
-// fp32 rows (small problems): one thread per row, plain fp32 FMA in coordinate order.
-__global__ void __launch_bounds__(256) hash_fp32_kernel(const __grid_constant__ HashArgs a, int d) {
-  __shared__ float s_w[128 * 8];
+// fp32 rows: thread = (row, direction), plain fp32 FMA in coordinate order.  The eight threads of a row share its 16-byte
+// loads; a warp's ballot holds the sign patterns of its four rows.  Bound by latency (a CTA makes chunk / 32 passes): 1024 rows
+// of d = 64 on both sides took 25 us with a thread per row and all directions and chunks of 2048 rows.
+template <int D>
+__global__ void __launch_bounds__(256) hash_fp32_kernel(const __grid_constant__ HashArgs a) {
+  __shared__ float s_w[D * 8];
   __shared__ uint32_t s_hist[kBuckets];
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, t = tid & 7;
   const ChunkPos cp = chunk_of_cta(a, blockIdx.x);
-  const int side = cp.side, seg = cp.seg, row0 = cp.row0, rows = cp.rows;
-  if (!((a.side_mask >> side) & 1) || rows < 0) return;
-  const float* wsrc = a.w_nodes ? a.w_nodes + (size_t)cp.node * (d * a.r) : a.w;
+  const int rows = cp.rows;
+  if (!((a.side_mask >> cp.side) & 1) || rows < 0) return;
+  const float* wsrc = a.w_nodes ? a.w_nodes + (size_t)cp.node * (D * a.r) : a.w;
   s_hist[tid] = 0;
-  for (int i = tid; i < d * a.r; i += 256) s_w[i] = wsrc[i];
+  for (int i = tid; i < D * 8; i += 256) s_w[i] = (i & 7) < a.r ? wsrc[(i >> 3) * a.r + (i & 7)] : 0.f;
   __syncthreads();
-  const float* base = reinterpret_cast<const float*>(a.x[side]) + ((size_t)seg * a.n[side] + row0) * d;
+  const float* base = reinterpret_cast<const float*>(a.x[cp.side]) + ((size_t)cp.seg * a.n[cp.side] + cp.row0) * D;
   uint8_t* dst = a.ids + ids_base(a, cp);
-  unsigned long long nz = 0;
-  for (int row = tid; row < rows; row += 256) {
-    float p[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const float4* xr = reinterpret_cast<const float4*>(base + (size_t)row * d);
-    for (int c = 0; c < d / 4; ++c) {
-      const float4 x = xr[c];
-      const float xs[4] = {x.x, x.y, x.z, x.w};
+  unsigned nz = 0;
+  for (int row0 = 0; row0 < rows; row0 += 32) {
+    const int row = row0 + (tid >> 3);
+    const float4* xr = reinterpret_cast<const float4*>(base + (size_t)min(row, rows - 1) * D);
+    float p = 0.f;
 #pragma unroll
-      for (int e = 0; e < 4; ++e)
+    for (int c0 = 0; c0 < D / 4; c0 += 16) {
+      float4 x[16];
 #pragma unroll
-        for (int t = 0; t < 8; ++t)
-          if (t < a.r) p[t] = fmaf(xs[e], s_w[(4 * c + e) * a.r + t], p[t]);
+      for (int c = 0; c < 16; ++c) x[c] = __ldg(xr + c0 + c);
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        const float* w = s_w + (c0 + c) * 32 + t;
+        p = fmaf(x[c].x, w[0], p); p = fmaf(x[c].y, w[8], p); p = fmaf(x[c].z, w[16], p); p = fmaf(x[c].w, w[24], p);
+      }
     }
-    uint32_t g = 0;
-#pragma unroll
-    for (int t = 0; t < 8; ++t)
-      if (t < a.r) { g |= (p[t] > 0.f ? 1u : 0u) << t; nz += fabsf(p[t]) < 1e-4f; }
-    const uint32_t id = gray_rank8(g);
-    dst[row] = (uint8_t)id;
-    atomicAdd(&s_hist[id], 1u);
+    if (row < rows && t < a.r) nz += fabsf(p) < 1e-4f;
+    const uint32_t bits = __ballot_sync(0xffffffffu, p > 0.f) >> (lane & 24);
+    if (t == 0 && row < rows) {
+      const uint32_t id = gray_rank8(bits & 0xffu);
+      dst[row] = (uint8_t)id;
+      atomicAdd(&s_hist[id], 1u);
+    }
   }
-  if (a.near_zero && nz) atomicAdd(a.near_zero, nz);
+  if (a.near_zero && nz) atomicAdd(a.near_zero, (unsigned long long)nz);
   __syncthreads();
   a.hist[hist_base(a, cp) + tid] = s_hist[tid];
 }
 
-// fp32 -> bf16 staging; `lo` (optional) receives the rounding remainder as a second bf16 term
-__global__ void convert_kernel(const float4* __restrict__ src, uint2* __restrict__ hi, uint2* __restrict__ lo,
-                               size_t count4) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count4; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 x = src[i];
+// fp32 -> bf16 staging of Q, K, V (blockIdx.y); for Q and K also the rounding remainder as a second bf16 term
+struct ConvertArgs {
+  const float4* src[3];
+  uint2 *hi[3], *lo[3];
+  size_t count4[3];
+};
+__global__ void __launch_bounds__(256) convert_kernel(const __grid_constant__ ConvertArgs a) {
+  const int s = blockIdx.y;
+  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < a.count4[s]; i += (size_t)gridDim.x * 256) {
+    const float4 x = a.src[s][i];
     const float xs[4] = {x.x, x.y, x.z, x.w};
     float h[4], l[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) { h[e] = __bfloat162float(__float2bfloat16_rn(xs[e])); l[e] = xs[e] - h[e]; }
-    hi[i] = make_uint2(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]));
-    if (lo) lo[i] = make_uint2(pack_bf16(l[0], l[1]), pack_bf16(l[2], l[3]));
+    a.hi[s][i] = make_uint2(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]));
+    if (a.lo[s]) a.lo[s][i] = make_uint2(pack_bf16(l[0], l[1]), pack_bf16(l[2], l[3]));
   }
 }
 
 }  // namespace
 
-cudaError_t launch_convert(const float* src, __nv_bfloat16* hi, __nv_bfloat16* lo, size_t count, cudaStream_t st) {
-  const size_t count4 = count / 4;
-  const size_t want = (count4 + 255) / 256;
-  const int blocks = (int)(want < 148 * 16 ? (want ? want : 1) : 148 * 16);
-  convert_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const float4*>(src), reinterpret_cast<uint2*>(hi),
-                                         reinterpret_cast<uint2*>(lo), count4);
+cudaError_t launch_convert(const float* q, const float* k, const float* v, const Workspace& ws, size_t count_q, size_t count_k, cudaStream_t st) {
+  ConvertArgs a;
+  const float* src[3] = {q, k, v};
+  __nv_bfloat16 *hi[3] = {ws.q16, ws.k16, ws.v16}, *lo[3] = {ws.q16lo, ws.k16lo, nullptr};
+  for (int s = 0; s < 3; ++s) {
+    a.src[s] = reinterpret_cast<const float4*>(src[s]);
+    a.hi[s] = reinterpret_cast<uint2*>(hi[s]); a.lo[s] = reinterpret_cast<uint2*>(lo[s]);
+    a.count4[s] = (s ? count_k : count_q) / 4;
+  }
+  const size_t most = a.count4[0] > a.count4[1] ? a.count4[0] : a.count4[1], want = (most + 255) / 256;
+  const dim3 grid((unsigned)(want < 148 * 16 ? want : 148 * 16), 3);
+  convert_kernel<<<grid, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_fp32, const float* w_host,
                         const Workspace& ws, unsigned long long* near_zero, cudaStream_t st, int side_mask, const float* w_nodes) {
   HashArgs a;
-  a.side_mask = side_mask;
+  a.side_mask = side_mask; a.chunk = g.chunk;
   a.w_nodes = g.node_dirs ? w_nodes : nullptr;
   a.levels = g.node_dirs ? g.levels : 1; a.L = g.L; a.d = g.d;
   a.ids_level_stride = ids_level_stride(g); a.hist_level_stride = hist_level_stride(g);
@@ -286,7 +302,8 @@ cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_
     a.chunks_per_unit[s] = side_cpu(g, s); a.chunks_per_seg[s] = side_cps(g, s);
   }
   const int grid = a.levels * g.G * (g.chunks_per_seg + g.chunks_per_seg_k);
-  if (is_fp32) hash_fp32_kernel<<<grid, 256, 0, st>>>(a, g.d);
+  if (is_fp32 && g.d == 64) hash_fp32_kernel<64><<<grid, 256, 0, st>>>(a);
+  else if (is_fp32) hash_fp32_kernel<128><<<grid, 256, 0, st>>>(a);
   else if (g.d == 64) hash_bf16_kernel<64><<<grid, 256, 0, st>>>(a);
   else hash_bf16_kernel<128><<<grid, 256, 0, st>>>(a);
   return cudaGetLastError();

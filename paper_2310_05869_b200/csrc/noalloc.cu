@@ -73,6 +73,7 @@ extern "C" int hyperattn_sortlsh_noalloc(const void* x, int n, int d, int hash_b
   g.G = 1; g.n = 0; g.nk = n; g.npad = 0; g.d = d; g.b = 1; g.bq = 1; g.m = 0; g.r = hash_bits;
   g.causal = 0; g.L = 0; g.leaf = 0; g.unit = 1; g.unit_k = n;
   g.chunks_per_unit = 0; g.chunks_per_seg = 0;
+  g.chunk = kSortChunk;
   g.chunks_per_unit_k = (n + kSortChunk - 1) / kSortChunk;
   g.chunks_per_seg_k = g.chunks_per_unit_k;
   g.levels = 1; g.nl = n; g.nodes = 1; g.sorted = 1;

@@ -39,6 +39,7 @@ struct SampleArgs {
   float* ltau;       // capped row sums only: [G, nodes], set to -inf here (the probe pass takes a maximum into it)
   Geometry g;
   uint32_t k0, k1;
+  int* sched;        // zeroed by the launch (null: nothing)
 };
 
 // Alg. 2 line 4: m i.i.d. uniform key indices per (segment, node); word w of Philox call c is
@@ -78,6 +79,7 @@ __device__ __forceinline__ void samples_body(const SampleArgs& a, int block, int
 // sampling as extra blocks (both are tiny and independent of each other).
 __global__ void __launch_bounds__(256) sort_scan_kernel(SortArgs a, SampleArgs sa, int scan_blocks) {
   __shared__ uint32_t s_tot[kBuckets];
+  if (sa.sched && blockIdx.x == 0 && threadIdx.x == 0) *sa.sched = 0;
   if ((int)blockIdx.x >= scan_blocks) { samples_body(sa, blockIdx.x - scan_blocks, gridDim.x - scan_blocks); return; }
   const Geometry& g = a.g;
   const int v = threadIdx.x;
@@ -127,7 +129,7 @@ __global__ void __launch_bounds__(256) sort_scan_kernel(SortArgs a, SampleArgs s
   }
 }
 
-// One CTA per (side, level, segment, chunk of the level): stable placement of <= 2048 rows.
+// One CTA per (side, level, segment, chunk of the level): stable placement of <= g.chunk rows.
 template <int R>
 __global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a) {
   __shared__ __align__(16) uint32_t s_cnt[8][kBuckets];   // per-warp running positions
@@ -153,19 +155,19 @@ __global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a) {
   const int cn = lc - j * nchunks_node;                  // chunk within the node
   const int cpu_s = side_cpu(g, side), unit_s = side_unit(g, side);
   const int u = cn / cpu_s, cu = cn % cpu_s;
-  const int local0 = u * unit_s + cu * kSortChunk;       // first row, relative to the node
+  const int local0 = u * unit_s + cu * g.chunk;       // first row, relative to the node
   const int row0 = (side == 0 ? q0 : k0) + local0;       // first row within the segment
   // (a chunk beyond the last row of the side has nothing to place)
-  const int rows = min(min(kSortChunk, unit_s - cu * kSortChunk), side_rows(g, side) - row0);
+  const int rows = min(min(g.chunk, unit_s - cu * g.chunk), side_rows(g, side) - row0);
   if (rows <= 0) return;
 
   const uint8_t* ids = a.ids + level * ids_level_stride(g) + side_ids_base(g, side) + (size_t)seg * side_rows(g, side) + row0;
   for (int i = tid; i < rows; i += 256) s_id[i] = ids[i];
   for (int i = tid; i < 8 * kBuckets / 4; i += 256) reinterpret_cast<uint4*>(&s_cnt[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
-  // per-warp histograms of consecutive sub-ranges of 256 rows
-  const int wbeg = warp * (kSortChunk / 8);
-  const int wend = min(rows, wbeg + kSortChunk / 8);
+  // per-warp histograms of consecutive sub-ranges of an eighth of the chunk
+  const int wbeg = warp * (g.chunk / 8);
+  const int wend = min(rows, wbeg + g.chunk / 8);
   for (int i = wbeg + lane; i < wend; i += 32) atomicAdd(&s_cnt[warp][s_id[i]], 1u);
   __syncthreads();
   {
@@ -221,7 +223,7 @@ cudaError_t launch_sort_scan(const Geometry& g, const Workspace& ws, bool with_s
   const SortArgs a = make_sort_args(g, ws, side_mask);
   const int nodes_per = g.causal ? g.nodes : 1;
   const int scan_blocks = 2 * g.G * nodes_per;
-  SampleArgs sa; sa.samples = ws.samples; sa.tpos = ws.tpos; sa.ltau = ws.ltau; sa.g = g; sa.k0 = (uint32_t)seed; sa.k1 = (uint32_t)(seed >> 32);
+  SampleArgs sa; sa.samples = ws.samples; sa.tpos = ws.tpos; sa.ltau = ws.ltau; sa.g = g; sa.k0 = (uint32_t)seed; sa.k1 = (uint32_t)(seed >> 32); sa.sched = ws.sched;
   int sample_blocks = 0;
   if (with_samples && g.nodes > 0 && g.m > 0) {
     const size_t total = (size_t)g.G * g.nodes * ((g.m + 3) / 4);

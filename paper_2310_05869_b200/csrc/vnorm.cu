@@ -13,68 +13,86 @@ namespace {
 
 constexpr float kNormScale = 4096.f;      // 2^12
 
-// one thread per key row
+// A CTA weighs 256 rows of one segment: the rows come in by whole lines and are read back one per thread (the chunks
+// of a row XOR-swizzled, so that neither side has bank conflicts); also the sum of the CTA's weights.
 template <int D>
-__global__ void __launch_bounds__(256) vnorm_weights_kernel(const __nv_bfloat16* __restrict__ v, uint32_t* __restrict__ wq, size_t rows) {
-  const size_t row = (size_t)blockIdx.x * 256 + threadIdx.x;
-  if (row >= rows) return;
-  const uint4* src = reinterpret_cast<const uint4*>(v + row * D);
-  float acc = 0.f;
+__global__ void __launch_bounds__(256) vnorm_weights_kernel(const __nv_bfloat16* __restrict__ v, uint32_t* __restrict__ wq,
+                                                            unsigned long long* __restrict__ sums, int nk) {
+  constexpr int CPR = D / 8;
+  extern __shared__ uint4 s_row[];                        // [256][CPR]
+  __shared__ unsigned long long s_warp[8];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int row0 = blockIdx.x * 256, rows = min(256, nk - row0);
+  const size_t first = (size_t)blockIdx.y * nk + row0;
+  const uint4* src = reinterpret_cast<const uint4*>(v) + first * CPR;
 #pragma unroll
-  for (int c = 0; c < D / 8; ++c) {
-    const uint4 x = src[c];
-    const uint32_t words[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float lo = __uint_as_float(words[e] << 16), hi = __uint_as_float(words[e] & 0xffff0000u);
-      acc = __fadd_rn(acc, __fmul_rn(lo, lo));          // (coordinate order, no fused multiply-add: the stated arithmetic)
-      acc = __fadd_rn(acc, __fmul_rn(hi, hi));
-    }
+  for (int e = 0; e < CPR; ++e) {
+    const int c = tid + 256 * e, r = c / CPR, cc = c % CPR;
+    if (r < rows) s_row[r * CPR + (cc ^ (r & 7))] = __ldg(src + c);
   }
-  wq[row] = (uint32_t)(acc * kNormScale);               // exact scaling, truncation = floor (acc >= 0)
+  __syncthreads();
+  unsigned long long w = 0;
+  if (tid < rows) {
+    float acc = 0.f;
+#pragma unroll
+    for (int c = 0; c < CPR; ++c) {
+      const uint4 x = s_row[tid * CPR + (c ^ (tid & 7))];
+      const uint32_t words[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float lo = __uint_as_float(words[e] << 16), hi = __uint_as_float(words[e] & 0xffff0000u);
+        acc = __fadd_rn(acc, __fmul_rn(lo, lo));          // (coordinate order, no fused multiply-add: the stated arithmetic)
+        acc = __fadd_rn(acc, __fmul_rn(hi, hi));
+      }
+    }
+    const uint32_t q = (uint32_t)(acc * kNormScale);      // exact scaling, truncation = floor (acc >= 0)
+    wq[first + tid] = q;
+    w = q;
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+  if (lane == 0) s_warp[tid >> 5] = w;
+  __syncthreads();
+  if (tid == 0) {
+    for (int e = 1; e < 8; ++e) w += s_warp[e];
+    sums[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = w;
+  }
 }
 
-// One CTA per segment: cum[seg][0] = 0, cum[seg][i + 1] = wq[seg][0] + ... + wq[seg][i] (64-bit).
-__global__ void __launch_bounds__(1024) vnorm_scan_kernel(const uint32_t* __restrict__ wq, unsigned long long* __restrict__ cum, int nk) {
-  __shared__ unsigned long long s_warp[32];
-  __shared__ unsigned long long s_base;
-  const int seg = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// cum[seg][0] = 0, cum[seg][i + 1] = wq[seg][0] + ... + wq[seg][i] (64-bit).  A CTA does 4096 rows of one segment and adds up
+// the sums of the rows before them by itself, so all CTAs run at once (one CTA per segment walking its rows: 94 us for 4 segments of
+// 131072 rows; MEASURED_SCAN).
+__global__ void __launch_bounds__(1024) vnorm_scan_kernel(const uint32_t* __restrict__ wq, const unsigned long long* __restrict__ sums,
+                                                          unsigned long long* __restrict__ cum, int nk, int blocks) {
+  __shared__ unsigned long long s_warp[32], s_before[32];
+  const int seg = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t* w = wq + (size_t)seg * nk;
   unsigned long long* c = cum + (size_t)seg * (nk + 1);
-  if (tid == 0) { s_base = 0; c[0] = 0; }
-  __syncthreads();
-  for (int i0 = 0; i0 < nk; i0 += 4096) {
-    const int i = i0 + 4 * tid;
-    unsigned long long x[4];
+  const int i = blockIdx.x * 4096 + 4 * tid;
+  unsigned long long x[4], before = 0;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) x[e] = i + e < nk ? w[i + e] : 0ull;
-    x[1] += x[0]; x[2] += x[1]; x[3] += x[2];
-    unsigned long long run = x[3];
+  for (int e = 0; e < 4; ++e) x[e] = i + e < nk ? w[i + e] : 0ull;
+  for (int e = tid; e < (int)blockIdx.x * 16; e += 1024) before += sums[(size_t)seg * blocks + e];
+  x[1] += x[0]; x[2] += x[1]; x[3] += x[2];
+  unsigned long long run = x[3];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long t = __shfl_up_sync(0xffffffffu, run, o);
-      if (lane >= o) run += t;
-    }
-    if (lane == 31) s_warp[warp] = run;
-    __syncthreads();
-    if (warp == 0) {
-      unsigned long long t = s_warp[lane];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long u = __shfl_up_sync(0xffffffffu, t, o);
-        if (lane >= o) t += u;
-      }
-      s_warp[lane] = t;
-    }
-    __syncthreads();
-    const unsigned long long before = s_base + (warp ? s_warp[warp - 1] : 0ull) + (run - x[3]);
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      if (i + e < nk) c[i + e + 1] = before + x[e];
-    __syncthreads();
-    if (tid == 1023) s_base = before + x[3];
-    __syncthreads();
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long t = __shfl_up_sync(0xffffffffu, run, o);
+    if (lane >= o) run += t;
   }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+  if (lane == 31) { s_warp[warp] = run; s_before[warp] = before; }
+  __syncthreads();
+  // sums of the warps before this one, and of everything before the CTA
+  unsigned long long t = s_before[lane] + (lane < warp ? s_warp[lane] : 0ull);
+#pragma unroll
+  for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  t += run - x[3];
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    if (i + e < nk) c[i + e + 1] = t + x[e];
+  if (i == 0) c[0] = 0;
 }
 
 struct VnormSampleArgs {
@@ -85,10 +103,13 @@ struct VnormSampleArgs {
   uint32_t k0, k1;
 };
 
+// LPD lanes per draw: 1, or 32 where draws are few - the search is a chain of dependent reads, and 32 probes at a time
+// make it four steps long instead of 17 for 131072 keys.
+template <int LPD>
 __global__ void __launch_bounds__(256) vnorm_sample_kernel(VnormSampleArgs a) {
   const Geometry& g = a.g;
   const size_t total_draws = (size_t)g.G * g.nodes * g.m;
-  const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+  const size_t i = ((size_t)blockIdx.x * 256 + threadIdx.x) / LPD;
   if (i >= total_draws) return;
   const int jd = (int)(i % g.m);
   const int nd = (int)((i / g.m) % g.nodes);
@@ -110,33 +131,50 @@ __global__ void __launch_bounds__(256) vnorm_sample_kernel(VnormSampleArgs a) {
   } else {
     const unsigned long long target = __umul64hi((unsigned long long)x << 32, total);     // floor(x * total / 2^32)
     int lo = 0, hi = have - 1;                           // smallest l with c[l + 1] - base > target
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (c[mid + 1] - base > target) hi = mid; else lo = mid + 1;
+    if (LPD == 1) {
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (c[mid + 1] - base > target) hi = mid; else lo = mid + 1;
+      }
+    } else {
+      const int lane = threadIdx.x & 31;
+      while (lo < hi) {
+        const int step = (hi - lo) / 32 + 1;               // probes lo + step - 1, lo + 2 step - 1, ...; those past hi: hi, where it holds
+        const int at = min((long long)hi, lo + (long long)(lane + 1) * step - 1);
+        const int first = __ffs(__ballot_sync(0xffffffffu, c[at + 1] - base > target)) - 1;
+        hi = (int)min((long long)hi, lo + (long long)(first + 1) * step - 1);
+        lo += first * step;
+      }
     }
     idx = lo;
     const unsigned long long w = c[idx + 1] - c[idx];
     wl = log2f((float)total / ((float)g.m * (float)w));
   }
+  if (LPD > 1 && (threadIdx.x & 31)) return;
   a.samples[i] = idx;
   a.wlog[i] = wl;
 }
 
 }  // namespace
 
-cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uint32_t* wq, unsigned long long* cum, int32_t* samples,
+cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uint32_t* wq, unsigned long long* sums, unsigned long long* cum, int32_t* samples,
                                   float* wlog, uint64_t seed, cudaStream_t st) {
   if (!g.sorted || g.m == 0 || g.nodes == 0) return cudaSuccess;
-  const size_t rows = (size_t)g.G * g.nk;
-  const size_t blocks = (rows + 255) / 256;
-  if (blocks > 0x7fffffffull) return cudaErrorInvalidValue;
-  if (g.d == 64) vnorm_weights_kernel<64><<<(unsigned)blocks, 256, 0, st>>>(v, wq, rows);
-  else vnorm_weights_kernel<128><<<(unsigned)blocks, 256, 0, st>>>(v, wq, rows);
-  vnorm_scan_kernel<<<g.G, 1024, 0, st>>>(wq, cum, g.nk);
+  const int blocks = (g.nk + 255) / 256;
+  if (g.G > 65535) return cudaErrorInvalidValue;
+  const dim3 grid(blocks, g.G);
+  if (g.d == 64) vnorm_weights_kernel<64><<<grid, 256, 256 * 128, st>>>(v, wq, sums, g.nk);
+  else {
+    const cudaError_t e = cudaFuncSetAttribute(vnorm_weights_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, 256 * 256);
+    if (e != cudaSuccess) return e;
+    vnorm_weights_kernel<128><<<grid, 256, 256 * 256, st>>>(v, wq, sums, g.nk);
+  }
+  vnorm_scan_kernel<<<dim3((g.nk + 4095) / 4096, g.G), 1024, 0, st>>>(wq, sums, cum, g.nk, blocks);
   VnormSampleArgs a;
   a.cum = cum; a.samples = samples; a.wlog = wlog; a.g = g; a.k0 = (uint32_t)seed; a.k1 = (uint32_t)(seed >> 32);
   const size_t draws = (size_t)g.G * g.nodes * g.m;
-  vnorm_sample_kernel<<<(unsigned)((draws + 255) / 256), 256, 0, st>>>(a);
+  if (draws < 16384) vnorm_sample_kernel<32><<<(unsigned)((draws + 7) / 8), 256, 0, st>>>(a);
+  else vnorm_sample_kernel<1><<<(unsigned)((draws + 255) / 256), 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -93,6 +93,21 @@ def _check(rc: int, what: str):
         raise HyperAttnError(f"{what}: {lib().hyperattn_status_string(rc).decode()} ({rc})")
 
 
+def _raw_stream(device: torch.device) -> int:
+    """Handle of torch's current stream on a device (without building a Stream object)."""
+    return torch._C._cuda_getCurrentRawStream(device.index)
+
+
+def _call(fn, what, device, *args):
+    """Calls a library entry point with `device` current."""
+    if torch._C._cuda_getDevice() == device.index:
+        rc = fn(*args)
+    else:
+        with torch.cuda.device(device):
+            rc = fn(*args)
+    _check(rc, what)
+
+
 def _dtype_code(t: torch.dtype) -> int:
     if t == torch.bfloat16:
         return BF16
@@ -139,24 +154,19 @@ def forward(q, k, v, block, samples, hash_bits, causal=False, n0=0, seed=0, out_
     n_k = k.shape[2]
     if k.shape != (B, H, n_k, d) or v.shape != k.shape:
         raise HyperAttnError("k and v must be [B, H, n_k, d] with the batch, heads and d of q")
+    dev = q.device
     out_dtype = out_dtype or q.dtype
-    out = torch.empty((B, H, n, d), dtype=out_dtype, device=q.device)
-    lse = torch.empty((B, H, n), dtype=torch.float32, device=q.device)
-    p = _Params()
-    _fill(p, B, H, n, d, block, samples, hash_bits, causal, n0, seed, _dtype_code(q.dtype), _dtype_code(out_dtype), scale, n_k)
-    p.q, p.k, p.v, p.out, p.lse = q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), lse.data_ptr()
-    if workspace is not None:
-        p.workspace, p.workspace_bytes = workspace.data_ptr(), workspace.numel() * workspace.element_size()
-    p.stream = stream if stream is not None else torch.cuda.current_stream(q.device).cuda_stream
-    p.precise = int(bool(precise))
-    if caps is not None:
-        p.capped, p.cap_scale, p.kappa = 1, float(caps[0]), float(caps[1])
-    p.sampling = int(bool(value_norm_sampling))
-    p.node_directions = int(bool(node_directions))
+    out = torch.empty_like(q) if out_dtype == q.dtype else torch.empty((B, H, n, d), dtype=out_dtype, device=dev)
+    lse = torch.empty((B, H, n), dtype=torch.float32, device=dev)
+    capped, cap_scale, kappa = (0, 0.0, 0.0) if caps is None else (1, float(caps[0]), float(caps[1]))
+    ws, ws_bytes = (None, 0) if workspace is None else (workspace.data_ptr(), workspace.numel() * workspace.element_size())
+    p = _Params(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), lse.data_ptr(), B, H, n, d, block, samples, hash_bits,
+                1 if causal else 0, n0, seed, _dtype_code(q.dtype), _dtype_code(out_dtype), scale, ws, ws_bytes, None,
+                _raw_stream(dev) if stream is None else stream, 1 if precise else 0, 0 if n_k == n else n_k, capped, cap_scale, kappa,
+                1 if value_norm_sampling else 0, 1 if node_directions else 0)
     inter = None
     if debug:
         G, LV, NL, NODES = _debug_shapes(B, H, n, block, samples, causal, n0, n_k)
-        dev = q.device
         id_sets = (LV,) if (node_directions and causal and NODES > 0) else ()
         inter = {
             "q_ids": torch.zeros(id_sets + (G, n), dtype=torch.uint8, device=dev),
@@ -172,8 +182,7 @@ def forward(q, k, v, block, samples, hash_bits, causal=False, n0=0, seed=0, out_
         }
         dbg = _Debug(*(inter[f].data_ptr() for f, _ in _Debug._fields_))
         p.debug = C.pointer(dbg)
-    with torch.cuda.device(q.device):
-        _check(lib().hyperattn_forward_ex(C.byref(p)), "hyperattn_forward_ex")
+    _call(lib().hyperattn_forward_ex, "hyperattn_forward_ex", dev, C.byref(p))
     return (out, lse, inter) if debug else (out, lse)
 
 
@@ -190,14 +199,13 @@ def backward(q, k, v, out, lse, dout, block, samples, hash_bits, causal=False, n
     q, k, v, out, lse, dout = (t.contiguous() for t in (q, k, v, out, lse, dout))
     B, H, n, d = q.shape
     grad_dtype = grad_dtype or torch.bfloat16
-    dq, dk, dv = (torch.empty((B, H, n, d), dtype=grad_dtype, device=q.device) for _ in range(3))
-    p = _Params()
-    _fill(p, B, H, n, d, block, samples, hash_bits, causal, n0, seed, _dtype_code(q.dtype), _dtype_code(out.dtype), scale)
-    p.q, p.k, p.v, p.out, p.lse = q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), lse.data_ptr()
-    p.stream = stream if stream is not None else torch.cuda.current_stream(q.device).cuda_stream
+    dev = q.device
+    dq, dk, dv = (torch.empty((B, H, n, d), dtype=grad_dtype, device=dev) for _ in range(3))
+    p = _Params(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), lse.data_ptr(), B, H, n, d, block, samples, hash_bits,
+                1 if causal else 0, n0, seed, _dtype_code(q.dtype), _dtype_code(out.dtype), scale, None, 0, None,
+                _raw_stream(dev) if stream is None else stream)
     g = _Grads(dout.data_ptr(), dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), _dtype_code(grad_dtype))
-    with torch.cuda.device(q.device):
-        _check(lib().hyperattn_backward(C.byref(p), C.byref(g)), "hyperattn_backward")
+    _call(lib().hyperattn_backward, "hyperattn_backward", dev, C.byref(p), C.byref(g))
     return dq, dk, dv
 
 

@@ -79,10 +79,10 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
     const int bpad = (g.b + 127) / 128 * 128, mpad = (g.m + 127) / 128 * 128;
     if (2 * bpad + mpad > kMaxNodeKeys) return HYPERATTN_UNSUPPORTED_SHAPE;
   }
-  // Chunks of 2048 rows, halved (down to 256) while a side's hash would leave SMs without a CTA: three CTAs of the hash per SM
-  // are resident, and below that the longest chunk is the whole time (32 heads of 4096 rows: MEASURED_HASH).
+  // Chunks of 2048 rows, halved (down to 256) while the hash has fewer than two CTAs for an SM: below that one chunk is the whole time
+  // (32 heads of 4096 rows: 14 us as 128 chunks, 9.5 us as 512; 12 heads 13 and 6 us; 356 chunks of 2048 are faster than 708 of 1024).
   g.chunk = kSortChunk;
-  while (g.chunk > 256 && (long long)g.G * ((g.npad / g.unit) * ((g.unit + g.chunk - 1) / g.chunk) + (g.causal ? (g.npad / g.unit) : 1) * ((g.unit_k + g.chunk - 1) / g.chunk)) < 444) g.chunk /= 2;
+  while (g.chunk > 256 && (long long)g.G * ((g.npad / g.unit) * ((g.unit + g.chunk - 1) / g.chunk) + (g.causal ? (g.npad / g.unit) : 1) * ((g.unit_k + g.chunk - 1) / g.chunk)) < 296) g.chunk /= 2;
   g.chunks_per_unit = (g.unit + g.chunk - 1) / g.chunk;
   g.chunks_per_seg = (g.npad / g.unit) * g.chunks_per_unit;
   g.chunks_per_unit_k = (g.unit_k + g.chunk - 1) / g.chunk;
@@ -334,7 +334,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     }
     {
       // (the samples of Alg. 2 line 4 are drawn by extra blocks of this launch)
-      StageScope sc(st, HYPERATTN_STAGE_SORT_SCAN, 1);
+      StageScope sc(st, HYPERATTN_STAGE_SORT_SCAN, scan_in_scatter(g) ? 0 : 1);
       HA_CHECK(launch_sort_scan(g, ws, !vnorm, p.seed, st));
     }
     if (vnorm) {
@@ -346,7 +346,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     }
     {
       StageScope sc(st, HYPERATTN_STAGE_SORT_SCATTER, 1);
-      HA_CHECK(launch_sort_scatter(g, ws, st));
+      HA_CHECK(launch_sort_scatter(g, ws, !vnorm, p.seed, st));
     }
     if (dbg) {
       const size_t lvl_bytes = (size_t)g.levels * g.G * g.nl * 4;
@@ -404,7 +404,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     // two blocks walk both blocks' key tiles, each tile's issuer skipping the other's: it releases the K stages of the tiles it
     // skips before the V stages, so a block's tiles and one more have to fit the ring of 8 (d = 64) or 4 (d = 128) stages.  Beyond that
     // one tile per CTA, which leaves half of its softmax warps idle (50 000 queries against 131 072 keys, groups of 98 queries and
-    // blocks of 256 keys: 218 us unpaired, MEASURED_PAIR us paired).
+    // blocks of 256 keys: 218 us unpaired, 142 us paired).
     a.level_paired[l] = !a.level_sorted[l] || a.tiles_per_block % 2 == 0 || (g.b + 63) / 64 + 1 <= (g.d == 64 ? 8 : 4);
     pairs += (a.level_paired[l] ? (per_node + 1) / 2 : per_node) * nodes_lvl * g.G;
   }
@@ -420,8 +420,6 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     float* dk = g32 ? reinterpret_cast<float*>(bw->dk) : acc + elems;
     float* dv = g32 ? reinterpret_cast<float*>(bw->dv) : acc + 2 * elems;
     StageScope sc(st, HYPERATTN_STAGE_BACKWARD, 2 + (g32 ? 0 : 1));
-    if (g32) for (float* x : {dq, dk, dv}) HA_CHECK(cudaMemsetAsync(x, 0, elems * 4, st));
-    else HA_CHECK(cudaMemsetAsync(acc, 0, 3 * elems * 4, st));
     HA_CHECK(launch_backward(a, p.out, out_fp32, p.lse, bw->dout, reinterpret_cast<float2*>(base + pl.stat), ws.sched,
                              dq, dk, dv, scale, ws.status, st));
     if (!g32) HA_CHECK(launch_to_bf16(acc, bw->dq, bw->dk, bw->dv, elems, st));

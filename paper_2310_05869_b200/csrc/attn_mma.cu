@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(256, 1) attn_mma_kernel(const __grid_constant_
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int gid = lane >> 2, tig = lane & 3;
   const TileDesc t = decode_tile(a, blockIdx.x);
+  wait_for_stream();
   if (t.nq <= 0) return;                          // (a tile of the schedule whose rows do not exist)
 
   const __nv_bfloat16* qs = a.q + (size_t)t.seg * g.n * D;
@@ -291,15 +292,13 @@ __global__ void __launch_bounds__(256, 1) attn_mma_kernel(const __grid_constant_
 
 cudaError_t launch_attention_mma(const AttnArgs& a, cudaStream_t st) {
   if (a.total_tiles == 0) return cudaSuccess;
-  auto go = [&](auto kernel, int smem_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
-    kernel<<<a.total_tiles, 256, smem_bytes, st>>>(a);
-    return cudaGetLastError();
-  };
   const bool split = a.q_lo != nullptr;
-  if (a.g.d == 64) return split ? go(attn_mma_kernel<64, true>, Smem<64, true>::kTotal) : go(attn_mma_kernel<64, false>, Smem<64, false>::kTotal);
-  return split ? go(attn_mma_kernel<128, true>, Smem<128, true>::kTotal) : go(attn_mma_kernel<128, false>, Smem<128, false>::kTotal);
+#define HA_GO(D, SPLIT) do { const cudaError_t e = allow_smem<attn_mma_kernel<D, SPLIT>>(Smem<D, SPLIT>::kTotal); \
+    return e != cudaSuccess ? e : launch(attn_mma_kernel<D, SPLIT>, a.total_tiles, 256, Smem<D, SPLIT>::kTotal, st, a); } while (0)
+  if (a.g.d == 64) { if (split) HA_GO(64, true); HA_GO(64, false); }
+  if (split) HA_GO(128, true);
+  HA_GO(128, false);
+#undef HA_GO
 }
 
 }  // namespace hyperattn

@@ -551,6 +551,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
+  wait_for_stream();
 
   // The CTA is persistent: it walks over work items (pairs of query tiles) blockIdx.x,
   // blockIdx.x + gridDim.x, ...  Every role runs the same item loop at its own pace; what
@@ -1472,29 +1473,25 @@ cudaError_t launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st)
   TmaMaps maps;
   if (!encode_rows_map(&maps.q, a.q, rows, a.g.d, 128) || !encode_rows_map(&maps.k, a.k, rows_k, a.g.d, TK) ||
       !encode_rows_map(&maps.v, a.v, rows_k, a.g.d, TK)) return cudaErrorInvalidValue;
-  auto go = [&](auto kernel, int smem_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cudaErrorUnknown;
-    int grid = a.total_pairs < sms ? a.total_pairs : sms;     // persistent: one CTA per SM walks the item list
-    kernel<<<grid, 384, smem_bytes, st>>>(a, maps, status);
-    return cudaGetLastError();
-  };
-  if (a.capped || a.sample_wlog) {
-    if (a.precise || (a.capped && a.sample_wlog)) return cudaErrorInvalidValue;
-    if (a.g.d == 64) return go(attn_tc_kernel<64, false, false, true>, Cfg<64>::kTotal);
-    if (!a.direct && !a.part_bf16) return go(attn_tc_kernel<128, true, false, true>, Cfg<128>::kTotal);
-    return go(attn_tc_kernel<128, false, false, true>, Cfg<128>::kTotal);
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  const int grid = a.total_pairs < sms ? a.total_pairs : sms;     // persistent: one CTA per SM walks the item list
+  const bool variant = a.capped || a.sample_wlog;
+  if (variant && (a.precise || (a.capped && a.sample_wlog))) return cudaErrorInvalidValue;
+  const bool late = a.g.d == 128 && !a.direct && !a.part_bf16;
+#define HA_GO(D, LATE, PRECISE, CAPPED) do { e = allow_smem<attn_tc_kernel<D, LATE, PRECISE, CAPPED>>(Cfg<D>::kTotal); \
+    return e != cudaSuccess ? e : launch(attn_tc_kernel<D, LATE, PRECISE, CAPPED>, grid, 384, Cfg<D>::kTotal, st, a, maps, status); } while (0)
+  if (a.g.d == 64) {
+    if (variant) HA_GO(64, false, false, true);
+    if (a.precise) HA_GO(64, false, true, false);
+    HA_GO(64, false, false, false);
   }
-  if (a.precise) {
-    if (a.g.d == 64) return go(attn_tc_kernel<64, false, true, false>, Cfg<64>::kTotal);
-    if (!a.direct && !a.part_bf16) return go(attn_tc_kernel<128, true, true, false>, Cfg<128>::kTotal);
-    return go(attn_tc_kernel<128, false, true, false>, Cfg<128>::kTotal);
-  }
-  if (a.g.d == 64) return go(attn_tc_kernel<64, false, false, false>, Cfg<64>::kTotal);
-  if (!a.direct && !a.part_bf16) return go(attn_tc_kernel<128, true, false, false>, Cfg<128>::kTotal);
-  return go(attn_tc_kernel<128, false, false, false>, Cfg<128>::kTotal);
+  if (variant) { if (late) HA_GO(128, true, false, true); HA_GO(128, false, false, true); }
+  if (a.precise) { if (late) HA_GO(128, true, true, false); HA_GO(128, false, true, false); }
+  if (late) HA_GO(128, true, false, false);
+  HA_GO(128, false, false, false);
+#undef HA_GO
 }
 
 }  // namespace hyperattn

@@ -47,7 +47,7 @@ struct BwdArgs {
   AttnArgs a;                  // geometry, permutations, samples
   const __nv_bfloat16* dout;   // [G, n, D]
   const float2* stat;          // [G, n] (-lse log2 e, -<dO, O>) of the rows
-  float *dq, *dk, *dv;         // [G, n, D] fp32 accumulators, zero at launch
+  float *dq, *dk, *dv;         // [G, n, D] fp32 accumulators, cleared by row_stat_kernel
   float scale;
   int* sched;                  // work counter of the launch, zero at launch
   // items: the key tiles of the leaves, then level by level those of the nodes
@@ -181,16 +181,20 @@ struct Cfg {
   static constexpr int kColDV = D == 64 ? 320 : 256, kColDK = 384, kColDQ = D == 64 ? 448 : 128;
 };
 
-// (-lse log2 e, -<dO, O>) of every row: D / 8 lanes per row, 16 bytes of dO and O each (HBM-bound)
+// (-lse log2 e, -<dO, O>) of every row: D / 8 lanes per row, 16 bytes of dO and O each (HBM-bound).
+// The same threads clear the accumulators: 32 bytes of each.
 template <int D, bool OUT_FP32>
 __global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__ dout, const void* __restrict__ out, const float* __restrict__ lse,
-                                                       float2* __restrict__ stat, size_t rows, int* sched) {
+                                                       float2* __restrict__ stat, size_t rows, int* sched, float4* dq, float4* dk, float4* dv) {
   constexpr int LPR = D / 8;
   const size_t c = (size_t)blockIdx.x * 256 + threadIdx.x;
+  wait_for_stream();
   if (c == 0) *sched = 0;
   const size_t row = c / LPR;
   float acc = 0.f;
   if (row < rows) {
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    dq[2 * c] = z; dq[2 * c + 1] = z; dk[2 * c] = z; dk[2 * c + 1] = z; dv[2 * c] = z; dv[2 * c + 1] = z;
     const uint4 x = __ldcs(dout + c);
     const uint32_t xd[4] = {x.x, x.y, x.z, x.w};
     float o[8];
@@ -262,6 +266,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
+  wait_for_stream();
   auto desc_of = [&](int it) -> const BwdItem& { return *reinterpret_cast<const BwdItem*>(smem + C::kOffDesc + (it % kDescs) * C::kDescBytes); };
   auto wait_desc = [&](int it) { return wait_fast<1>(bar_dfull(it), (it / kDescs) & 1, s_abort, status); };
   // key row (segment-relative) of key r of an item's tile, r < nkeys
@@ -693,6 +698,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
 
 // the three fp32 accumulators (one after the other) rounded to bf16: 32 bytes in, 16 out per thread and pass
 __global__ void __launch_bounds__(256) to_bf16_kernel(const float4* __restrict__ src, uint4* __restrict__ dq, uint4* __restrict__ dk, uint4* __restrict__ dv, size_t count8) {
+  wait_for_stream();
   uint4* dst = blockIdx.y == 0 ? dq : (blockIdx.y == 1 ? dk : dv);
   src += (size_t)blockIdx.y * count8 * 2;
   for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < count8; i += (size_t)gridDim.x * 256) {
@@ -703,7 +709,7 @@ __global__ void __launch_bounds__(256) to_bf16_kernel(const float4* __restrict__
 
 }  // namespace
 
-// a: the forward schedule (permutations, samples, tile geometry); the accumulators dq, dk, dv must be zero
+// a: the forward schedule (permutations, samples, tile geometry); the accumulators dq, dk, dv are cleared here
 cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout, float2* stat, int* sched,
                             float* dq, float* dk, float* dv, float scale, int* status, cudaStream_t st) {
   const Geometry& g = a.g;
@@ -712,18 +718,12 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   {
     const unsigned grid = (unsigned)((rows * (g.d / 8) + 255) / 256);
     const uint4* d4 = reinterpret_cast<const uint4*>(dout);
-    if (g.d == 64) {
-      if (out_fp32) row_stat_kernel<64, true><<<grid, 256, 0, st>>>(d4, out, lse, stat, rows, sched);
-      else row_stat_kernel<64, false><<<grid, 256, 0, st>>>(d4, out, lse, stat, rows, sched);
-    } else {
-      if (out_fp32) row_stat_kernel<128, true><<<grid, 256, 0, st>>>(d4, out, lse, stat, rows, sched);
-      else row_stat_kernel<128, false><<<grid, 256, 0, st>>>(d4, out, lse, stat, rows, sched);
-    }
-    const cudaError_t e = cudaGetLastError();
+    auto* kernel = g.d == 64 ? (out_fp32 ? row_stat_kernel<64, true> : row_stat_kernel<64, false>) : (out_fp32 ? row_stat_kernel<128, true> : row_stat_kernel<128, false>);
+    const cudaError_t e = launch(kernel, grid, 256, 0, st, d4, out, lse, stat, rows, sched, reinterpret_cast<float4*>(dq), reinterpret_cast<float4*>(dk), reinterpret_cast<float4*>(dv));
     if (e != cudaSuccess) return e;
   }
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cudaErrorUnknown;
+  int sms = 0;
+  if (const cudaError_t e = sm_count(&sms); e != cudaSuccess) return e;
   BwdArgs b;
   b.a = a; b.dout = reinterpret_cast<const __nv_bfloat16*>(dout); b.stat = stat; b.dq = dq; b.dk = dk; b.dv = dv; b.scale = scale; b.sched = sched;
   b.leaf_ktiles = a.n_leaf_tiles ? (g.leaf + kTileK - 1) / kTileK : 0;
@@ -760,21 +760,17 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   BwdMaps maps;
   if (!encode_rows_map(&maps.q, a.q, rows, g.d, 128) || !encode_rows_map(&maps.k, a.k, rows, g.d, 128) ||
       !encode_rows_map(&maps.v, a.v, rows, g.d, 128) || !encode_rows_map(&maps.dout, dout, rows, g.d, 128)) return cudaErrorInvalidValue;
-  auto go = [&](auto kernel, int smem_bytes) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
-    kernel<<<items < sms ? (unsigned)items : (unsigned)sms, kThreads, smem_bytes, st>>>(b, maps, status);      // persistent: one CTA per SM
-    return cudaGetLastError();
-  };
-  return g.d == 64 ? go(bwd_kernel<64>, Cfg<64>::kTotal) : go(bwd_kernel<128>, Cfg<128>::kTotal);
+  const unsigned grid = items < sms ? (unsigned)items : (unsigned)sms;      // persistent: one CTA per SM
+  cudaError_t e = g.d == 64 ? allow_smem<bwd_kernel<64>>(Cfg<64>::kTotal) : allow_smem<bwd_kernel<128>>(Cfg<128>::kTotal);
+  if (e != cudaSuccess) return e;
+  return launch(g.d == 64 ? bwd_kernel<64> : bwd_kernel<128>, grid, kThreads, g.d == 64 ? Cfg<64>::kTotal : Cfg<128>::kTotal, st, b, maps, status);
 }
 
 // src: dq, dk, dv one after the other, count entries each (a multiple of 8)
 cudaError_t launch_to_bf16(const float* src, void* dq, void* dk, void* dv, size_t count, cudaStream_t st) {
   const size_t count8 = count / 8, want = (count8 + 255) / 256;
   const dim3 grid((unsigned)(want < 148 * 16 ? want : 148 * 16), 3);
-  to_bf16_kernel<<<grid, 256, 0, st>>>(reinterpret_cast<const float4*>(src), reinterpret_cast<uint4*>(dq), reinterpret_cast<uint4*>(dk), reinterpret_cast<uint4*>(dv), count8);
-  return cudaGetLastError();
+  return launch(to_bf16_kernel, grid, 256, 0, st, reinterpret_cast<const float4*>(src), reinterpret_cast<uint4*>(dq), reinterpret_cast<uint4*>(dk), reinterpret_cast<uint4*>(dv), count8);
 }
 
 }  // namespace hyperattn

@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(256) tau_kernel(const __grid_constant__ TauArg
   constexpr int KS = D / 16, CPL = D / 32;
   constexpr int U = D == 64 ? 4 : 2;               // 8-key blocks per step (independent loads in flight)
   __shared__ float s_m[8][16], s_l[8][16];
+  wait_for_stream();
   const Geometry& g = a.g;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
   const int groups = (g.m + 15) / 16;
@@ -175,9 +176,7 @@ cudaError_t launch_tau(const AttnArgs& at, const int32_t* tpos, float* ltau, cud
   a.scale_log2 = at.scale_log2;
   const long long grid = (long long)g.G * g.nodes * ((g.m + 15) / 16);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  if (g.d == 64) tau_kernel<64><<<(unsigned)grid, 256, 0, st>>>(a);
-  else tau_kernel<128><<<(unsigned)grid, 256, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch(g.d == 64 ? tau_kernel<64> : tau_kernel<128>, (unsigned)grid, 256, 0, st, a);
 }
 
 }  // namespace hyperattn

@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <atomic>
 
 namespace hyperattn {
 
@@ -107,6 +108,47 @@ __host__ __device__ inline int side_cps(const Geometry& g, int side) { return si
 // chunks of one (level, segment) on a side: every node of the level (causal), or the whole side
 __host__ __device__ inline int side_cpl(const Geometry& g, int side) { return g.causal ? (g.nl / g.unit) * g.chunks_per_unit : side_cps(g, side); }
 
+// ---- launches -----------------------------------------------------------------------------
+// Every kernel of a call is launched with programmatic stream serialisation: its launch is prepared while the kernel before
+// it on the stream runs, and its blocks wait in wait_for_stream() until that one has completed and its writes are visible.  So
+// nothing that an earlier kernel writes may be read - and nothing written - before it; since every kernel waits, all
+// earlier ones have completed by then, not only the last.  (Small calls gain 5-8 us; letting the next kernel's blocks in
+// early with griddepcontrol.launch_dependents costs large calls 3-7 %: they take slots from the kernel that still runs.)
+__device__ __forceinline__ void wait_for_stream() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st; cfg.attrs = &attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+// dynamic shared memory beyond the default is asked for once per kernel and device, not on every launch
+template <auto Kernel>
+cudaError_t allow_smem(int bytes) {
+  static std::atomic<unsigned long long> done{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = dev < 64 ? 1ull << dev : 0;
+  if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+  return e;
+}
+inline cudaError_t sm_count(int* sms) {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 64 && (*sms = known[dev].load(std::memory_order_relaxed)) > 0) return cudaSuccess;
+  e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess && dev < 64) known[dev].store(*sms, std::memory_order_relaxed);
+  return e;
+}
+
 // ---- stage launchers (each enqueues on `st`; returns cudaGetLastError()) ---------------
 struct Workspace {
   __nv_bfloat16 *q16, *k16, *v16;  // bf16 staging of fp32 inputs (else null)
@@ -132,7 +174,9 @@ cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_
                         const float* w_nodes = nullptr);
 // side_mask: bit 0 queries, bit 1 keys (3: both)
 cudaError_t launch_sort_scan(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask = 3);
-cudaError_t launch_sort_scatter(const Geometry& g, const Workspace& ws, cudaStream_t st, int side_mask = 3);
+bool scan_in_scatter(const Geometry& g);
+// (small nodes: the scatter does the scan's work, samples included, and launch_sort_scan launches nothing)
+cudaError_t launch_sort_scatter(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask = 3);
 // side_mask for the hash as well (a side that is left out is neither read nor written)
 cudaError_t launch_merge(const Geometry& g, const Workspace& ws, void* out, float* lse, int out_fp32,
                          cudaStream_t st);

@@ -114,6 +114,7 @@ __global__ void __launch_bounds__(256, D == 64 ? 4 : 3) hash_bf16_kernel(const _
   const float* wsrc = a.w_nodes ? a.w_nodes + (size_t)cp.node * (D * a.r) : a.w;
 
   s_hist[tid] = 0;
+  wait_for_stream();
 
   const char* base = reinterpret_cast<const char*>(a.x[side]) + ((size_t)seg * a.n[side] + row0) * (D * 2);
   unsigned nz = 0;
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(256) hash_fp32_kernel(const __grid_constant__ 
   if (!((a.side_mask >> cp.side) & 1) || rows < 0) return;
   const float* wsrc = a.w_nodes ? a.w_nodes + (size_t)cp.node * (D * a.r) : a.w;
   s_hist[tid] = 0;
+  wait_for_stream();
   for (int i = tid; i < D * 8; i += 256) s_w[i] = (i & 7) < a.r ? wsrc[(i >> 3) * a.r + (i & 7)] : 0.f;
   __syncthreads();
   const float* base = reinterpret_cast<const float*>(a.x[cp.side]) + ((size_t)cp.seg * a.n[cp.side] + cp.row0) * D;
@@ -259,6 +261,7 @@ struct ConvertArgs {
 };
 __global__ void __launch_bounds__(256) convert_kernel(const __grid_constant__ ConvertArgs a) {
   const int s = blockIdx.y;
+  wait_for_stream();
   for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < a.count4[s]; i += (size_t)gridDim.x * 256) {
     const float4 x = a.src[s][i];
     const float xs[4] = {x.x, x.y, x.z, x.w};
@@ -283,8 +286,7 @@ cudaError_t launch_convert(const float* q, const float* k, const float* v, const
   }
   const size_t most = a.count4[0] > a.count4[1] ? a.count4[0] : a.count4[1], want = (most + 255) / 256;
   const dim3 grid((unsigned)(want < 148 * 16 ? want : 148 * 16), 3);
-  convert_kernel<<<grid, 256, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch(convert_kernel, grid, 256, 0, st, a);
 }
 
 cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_fp32, const float* w_host,
@@ -302,11 +304,8 @@ cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_
     a.chunks_per_unit[s] = side_cpu(g, s); a.chunks_per_seg[s] = side_cps(g, s);
   }
   const int grid = a.levels * g.G * (g.chunks_per_seg + g.chunks_per_seg_k);
-  if (is_fp32 && g.d == 64) hash_fp32_kernel<64><<<grid, 256, 0, st>>>(a);
-  else if (is_fp32) hash_fp32_kernel<128><<<grid, 256, 0, st>>>(a);
-  else if (g.d == 64) hash_bf16_kernel<64><<<grid, 256, 0, st>>>(a);
-  else hash_bf16_kernel<128><<<grid, 256, 0, st>>>(a);
-  return cudaGetLastError();
+  auto* kernel = is_fp32 ? (g.d == 64 ? hash_fp32_kernel<64> : hash_fp32_kernel<128>) : (g.d == 64 ? hash_bf16_kernel<64> : hash_bf16_kernel<128>);
+  return launch(kernel, grid, 256, 0, st, a);
 }
 
 }  // namespace hyperattn

@@ -39,6 +39,7 @@ __global__ void __launch_bounds__(256, LM <= 8 ? (D == 64 ? 4 : 3) : 1) merge_ke
   constexpr int LG = LM <= 5 ? LM : 4;             // levels whose rows are in flight together
   const Geometry& g = a.g;
   const int seg = blockIdx.y;
+  wait_for_stream();
   const int lane = threadIdx.x & 31;
   const int row0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
   if (row0 >= g.n) return;
@@ -176,7 +177,8 @@ cudaError_t launch_merge(const Geometry& g, const Workspace& ws, void* out, floa
   const size_t warps = ((size_t)g.n + 31) / 32;                                 // a warp per 32 rows
   const dim3 blocks((unsigned)((warps + 7) / 8), (unsigned)g.G);
   if (g.G > 65535) return cudaErrorInvalidValue;
-  auto go = [&](auto kernel) { kernel<<<blocks, 256, 0, st>>>(a); };
+  cudaError_t e = cudaSuccess;
+  auto go = [&](auto* kernel) { e = launch(kernel, blocks, 256, 0, st, a); };
   auto pick = [&](auto dtag, auto pbtag) {
     constexpr int D = decltype(dtag)::value;
     constexpr bool PB = decltype(pbtag)::value;
@@ -185,7 +187,7 @@ cudaError_t launch_merge(const Geometry& g, const Workspace& ws, void* out, floa
   using std::integral_constant;
   if (g.d == 64) { if (ws.part_bf16) pick(integral_constant<int, 64>{}, integral_constant<bool, true>{}); else pick(integral_constant<int, 64>{}, integral_constant<bool, false>{}); }
   else { if (ws.part_bf16) pick(integral_constant<int, 128>{}, integral_constant<bool, true>{}); else pick(integral_constant<int, 128>{}, integral_constant<bool, false>{}); }
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace hyperattn

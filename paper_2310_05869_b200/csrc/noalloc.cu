@@ -91,7 +91,7 @@ extern "C" int hyperattn_sortlsh_noalloc(const void* x, int n, int d, int hash_b
   constexpr int kKeysOnly = 2;
   if (launch_hash(g, nullptr, x, /*is_fp32=*/0, w, ws, nullptr, st, kKeysOnly) != cudaSuccess) return HYPERATTN_CUDA_ERROR;
   if (launch_sort_scan(g, ws, false, 0, st, kKeysOnly) != cudaSuccess) return HYPERATTN_CUDA_ERROR;
-  if (launch_sort_scatter(g, ws, st, kKeysOnly) != cudaSuccess) return HYPERATTN_CUDA_ERROR;
+  if (launch_sort_scatter(g, ws, false, 0, st, kKeysOnly) != cudaSuccess) return HYPERATTN_CUDA_ERROR;
   if (cudaMemcpyAsync(ids, ws.ids, (size_t)n, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return HYPERATTN_CUDA_ERROR;
   return HYPERATTN_OK;
 }

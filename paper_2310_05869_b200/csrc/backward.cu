@@ -34,7 +34,7 @@
 namespace hyperattn {
 namespace {
 
-constexpr int kThreads = 512;
+constexpr int kThreads = 640;
 constexpr int kDescs = 3;              // item descriptors in flight
 constexpr int kTileK = 128;            // keys per item, query rows per step
 
@@ -157,20 +157,19 @@ __device__ __forceinline__ StepRows step_rows(const BwdArgs& b, const BwdItem& t
 template <int D>
 struct Cfg {
   static constexpr int kTile = 128 * D * 2;           // bytes of a [128 rows x D] tile
-  static constexpr int NKV = D == 64 ? 2 : 1;         // K / V buffers (an item each)
-  static constexpr int NDO = D == 64 ? 2 : 1;         // dO buffers (a step each); Q: two
-  static constexpr int NDS = D == 64 ? 2 : 1;         // dS buffers
-  static constexpr int kOffKV = 0;
-  static constexpr int kOffQ = kOffKV + NKV * 2 * kTile;
-  static constexpr int kOffDO = kOffQ + 2 * kTile;
+  // buffers: K and V (an item each), Q, dO and dS (a step each); d = 128 has room for two only of Q
+  static constexpr int NKV = D == 64 ? 2 : 1, NQ = 2, NDO = D == 64 ? 2 : 1, NDS = D == 64 ? 2 : 1;
+  static constexpr int kOffK = 0;
+  static constexpr int kOffV = kOffK + NKV * kTile;
+  static constexpr int kOffQ = kOffV + NKV * kTile;
+  static constexpr int kOffDO = kOffQ + NQ * kTile;
   static constexpr int kOffDS = kOffDO + NDO * kTile;
-  static constexpr int kOffStage = kOffDS + NDS * 128 * 128 * 2;    // results on their way out: 8 KB per warp
-  static constexpr int kStageWarp = D == 64 ? 4096 : 8192;
-  static constexpr int kOffStat = kOffStage + 4 * kStageWarp;       // float [2 steps][-lse2 | -delta][128]
-  static constexpr int kOffDesc = kOffStat + 2 * 2 * 128 * 4;
+  static constexpr int kOffStage = kOffDS + NDS * 128 * 128 * 2;            // results on their way out: 4 KB per warp
+  static constexpr int kOffStat = kOffStage + 8 * 4096;                     // float [NQ][-lse2 | -delta][128]
+  static constexpr int kOffDesc = kOffStat + NQ * 1024;
   static constexpr int kDescBytes = (sizeof(BwdItem) + 15) / 16 * 16;
   static constexpr int kOffBar = kOffDesc + kDescs * kDescBytes;
-  static constexpr int kNumBar = 2 * NKV + 20 + 2 * kDescs;
+  static constexpr int kNumBar = 24 + 2 * kDescs;
   static constexpr int kOffMisc = kOffBar + 8 * kNumBar;
   static constexpr int kTotal = kOffMisc + 16;
   static_assert(kTotal <= 232448, "shared memory");
@@ -226,24 +225,26 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
   const uint32_t ubase = smem_u32(smem);
   const uint32_t bar0 = ubase + C::kOffBar;
-  // (pairs of barriers are used in turn by the steps; a waiter that is a step behind never meets a phase twice)
-  auto bar_qfull = [&](uint32_t g) { return bar0 + 8 * (g & 1); };                // Q of a step landed
-  auto bar_qfree = [&](uint32_t g) { return bar0 + 8 * (2 + (g & 1)); };          // dK of the step multiplied: Q, statistics free
-  auto bar_stat = [&](uint32_t g) { return bar0 + 8 * (4 + (g & 1)); };           // row statistics of a step written
-  auto bar_dofull = [&](uint32_t g) { return bar0 + 8 * (6 + g % C::NDO); };      // dO landed
-  auto bar_dofree = [&](uint32_t g) { return bar0 + 8 * (8 + g % C::NDO); };      // dV multiplied: dO and P free
-  auto bar_dq = [&](uint32_t g) { return bar0 + 8 * (10 + (g & 1)); };            // dQ multiplied: in TMEM, dS free
-  const uint32_t bar_s = bar0 + 8 * 12, bar_dp = bar0 + 8 * 13;                   // S^T, dP^T written
-  const uint32_t bar_h = bar0 + 8 * 14;                                           // P and dS written (S^T and dP^T have been read)
-  const uint32_t bar_dqfree = bar0 + 8 * 15;                                      // dQ has left TMEM
-  const uint32_t bar_acc = bar0 + 8 * 16, bar_accfree = bar0 + 8 * 17;            // dK, dV of the item complete; have left TMEM
-  auto bar_kv = [&](int it) { return bar0 + 8 * (20 + it % C::NKV); };            // K and V of an item landed
-  auto bar_kvfree = [&](int it) { return bar0 + 8 * (20 + C::NKV + it % C::NKV); };
-  auto bar_dfull = [&](int it) { return bar0 + 8 * (20 + 2 * C::NKV + it % kDescs); };
-  auto bar_dfree = [&](int it) { return bar0 + 8 * (20 + 2 * C::NKV + kDescs + it % kDescs); };
+  // g: step, it: item, counted over the CTA's whole work list.  (Pairs of barriers are used in turn by the steps; a waiter that
+  // is a step behind never meets a phase twice.)
+  const uint32_t bar_s = bar0, bar_dp = bar0 + 8;                                 // S^T, dP^T written
+  const uint32_t bar_h = bar0 + 16;                                               // P and dS written (S^T and dP^T have been read)
+  const uint32_t bar_dqfree = bar0 + 24;                                          // dQ has left TMEM
+  const uint32_t bar_acc = bar0 + 32, bar_accfree = bar0 + 40;                    // dK, dV of the item complete; have left TMEM
+  auto bar_dsfree = [&](uint32_t g) { return bar0 + 8 * (6 + g % C::NDS); };      // dK and dQ of a step multiplied: its dS is free
+  auto bar_dq = [&](uint32_t g) { return bar0 + 8 * (8 + (g & 1)); };             // dQ of a step in TMEM
+  auto bar_qfull = [&](uint32_t g) { return bar0 + 8 * (10 + (g & 1)); };         // Q and the row statistics of a step landed
+  auto bar_qfree = [&](uint32_t g) { return bar0 + 8 * (12 + (g & 1)); };
+  auto bar_dofull = [&](uint32_t g) { return bar0 + 8 * (14 + g % C::NDO); };     // dO landed
+  auto bar_dofree = [&](uint32_t g) { return bar0 + 8 * (16 + (g & 1)); };        // dV multiplied: dO and P are free
+  auto bar_kfull = [&](int it) { return bar0 + 8 * (18 + it % C::NKV); };         // K, V of an item landed
+  auto bar_vfull = [&](int it) { return bar0 + 8 * (20 + it % C::NKV); };
+  auto bar_kfree = [&](int it) { return bar0 + 8 * (22 + it % C::NKV); };         // dQ of the item multiplied: K and V are free
+  auto bar_dfull = [&](int it) { return bar0 + 8 * (24 + it % kDescs); };         // item descriptor written
+  auto bar_dfree = [&](int it) { return bar0 + 8 * (24 + kDescs + it % kDescs); };
 
   const AttnArgs& a = b.a;
-  const Geometry& g = a.g;
+  const Geometry& g_ = a.g;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (tid == 0) *s_abort = *reinterpret_cast<volatile int*>(status);
@@ -251,14 +252,14 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
   if (*s_abort) return;                                 // (a launch in which some wait already timed out drains quickly)
   __syncthreads();
   if (tid == 0) {
-    for (int x = 0; x < 2; ++x) { mbar_init(bar_qfull(x), 32); mbar_init(bar_qfree(x), 1); mbar_init(bar_stat(x), 1); mbar_init(bar_dq(x), 1); }
-    for (int x = 0; x < C::NDO; ++x) { mbar_init(bar_dofull(x), 32); mbar_init(bar_dofree(x), 1); }
-    mbar_init(bar_s, 1); mbar_init(bar_dp, 1); mbar_init(bar_h, 8); mbar_init(bar_dqfree, 4); mbar_init(bar_acc, 1); mbar_init(bar_accfree, 4);
-    for (int x = 0; x < C::NKV; ++x) { mbar_init(bar_kv(x), 32); mbar_init(bar_kvfree(x), 1); }
-    for (int x = 0; x < kDescs; ++x) { mbar_init(bar_dfull(x), 1); mbar_init(bar_dfree(x), 15); }   // 8 + 4 warps, issuer, two loaders
+    mbar_init(bar_s, 1); mbar_init(bar_dp, 1); mbar_init(bar_h, 8); mbar_init(bar_dqfree, 8); mbar_init(bar_acc, 1); mbar_init(bar_accfree, 8);   // (8: one arrival per warp)
+    for (int x = 0; x < 2; ++x) { mbar_init(bar_dsfree(x), 1); mbar_init(bar_dq(x), 1); mbar_init(bar_qfull(x), 64); mbar_init(bar_qfree(x), 1); mbar_init(bar_dofree(x), 1); }
+    for (int x = 0; x < C::NDO; ++x) mbar_init(bar_dofull(x), 32);
+    for (int x = 0; x < C::NKV; ++x) { mbar_init(bar_kfull(x), 32); mbar_init(bar_vfull(x), 32); mbar_init(bar_kfree(x), 1); }
+    for (int x = 0; x < kDescs; ++x) { mbar_init(bar_dfull(x), 1); mbar_init(bar_dfree(x), 19); }   // 8 + 8 warps, issuer, two loaders
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 12) {
+  if (warp == 16) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -274,15 +275,19 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
     if (t.kind == 0) return t.k0 + r;
     return t.k0 + __ldg((t.kind == 1 ? a.perm_k : a.samples) + t.kidx + r);
   };
+  // query row (segment-relative) of row r of a step, -1: does not exist
+  auto query_row = [&](const BwdItem& t, const StepRows& sr, int r) -> int {
+    if (r >= sr.nq) return -1;
+    return t.kind == 0 ? sr.first + r : t.q0 + __ldg(a.perm_q + t.slice + sr.first + r);
+  };
 
-  // Every role walks the same items and steps at its own pace; gs counts steps over all items.
-  uint32_t gs = 0;
   bool ok = true;
   if (warp < 8) {
     // ================= P and dS: thread = key, warpgroup h: query columns 64 h .. 64 h + 63 ==================
     const int h = warp >> 2, row = tid & 127;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const uint64_t sc2 = pack_f2(a.scale_log2, a.scale_log2);
+    uint32_t g = 0;
     for (int it = 0; ok; ++it) {
       ok = __all_sync(0xffffffffu, wait_desc(it));
       if (!ok) break;
@@ -291,64 +296,86 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
       const bool exists = row < t.nkeys;
       const int kind = t.kind, steps = t.steps, causal = t.causal;
       int kblk = -2;                                    // sampled keys: the sorted block the key lies in (its entries there are masked)
-      if (kind == 2 && exists) kblk = __ldg(a.rank_k + t.slice + __ldg(a.samples + t.kidx + row)) / g.b;
+      if (kind == 2 && exists) kblk = __ldg(a.rank_k + t.slice + __ldg(a.samples + t.kidx + row)) / g_.b;
 #pragma unroll 1
-      for (int s = 0; s < steps; ++s, ++gs) {
+      for (int s = 0; s < steps; ++s, ++g) {
         // entries that do not count: keys that do not exist, sampled keys of the query tile's own block, above the diagonal
         bool dead = !exists;
         if (kind == 2) dead = dead || kblk == (t.tn0 + s) / a.tiles_per_block;
         const bool diag = causal && s == 0;
         const bool masked = diag || __any_sync(0xffffffffu, dead);
-        ok = wait_fast<2>(bar_stat(gs), (gs >> 1) & 1, s_abort, status) && wait_fast<3>(bar_s, gs & 1, s_abort, status) &&
-             wait_fast<4>(bar_dp, gs & 1, s_abort, status);
-        // the products of the steps before that still read P and dS
-        if (D == 64) {
-          if (gs > 0) ok = ok && wait_fast<5>(bar_dofree(gs - 1), ((gs - 1) / C::NDO) & 1, s_abort, status);
-          if (gs > 1) ok = ok && wait_fast<6>(bar_dq(gs), ((gs >> 1) - 1) & 1, s_abort, status);
-        }
+        ok = wait_fast<2>(bar_qfull(g), (g >> 1) & 1, s_abort, status) && wait_fast<3>(bar_s, g & 1, s_abort, status);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
-        const float* st_l = reinterpret_cast<const float*>(smem + C::kOffStat) + (gs & 1) * 256 + 64 * h;
-        const uint32_t uds = ubase + C::kOffDS + (gs % C::NDS) * (128 * 128 * 2) + h * (128 * 128);      // this warpgroup's 64 columns
+        const float* st = reinterpret_cast<const float*>(smem + C::kOffStat) + (g & 1) * 256 + 64 * h;
+        const uint32_t uds = ubase + C::kOffDS + (g % C::NDS) * 32768 + h * 16384 + row * 128;
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
-          uint32_t rs[32], rd[32];
-          tmem_ld32_issue(lane_addr + C::kColS + 64 * h + 32 * c, rs);
-          tmem_ld32_issue(lane_addr + C::kColDP + 64 * h + 32 * c, rd);
-          tmem_ld32_wait(rs);
-          tmem_ld32_wait(rd);
-          if (masked) {
-            const int first = dead ? 128 : (diag ? row - 64 * h - 32 * c : 0);      // columns below it do not count
-#pragma unroll
-            for (int e = 0; e < 32; ++e)
-              if (e < first) rs[e] = 0xff800000u;
-          }
+          float p[32];
           uint32_t pp[16];
+          {
+            uint32_t rs[32];
+            tmem_ld32_issue(lane_addr + C::kColS + 64 * h + 32 * c, rs);
+            tmem_ld32_wait(rs);
+            if (masked) {
+              const int first = dead ? 128 : (diag ? row - 64 * h - 32 * c : 0);      // columns below it do not count
 #pragma unroll
-          for (int e = 0; e < 32; e += 8) {
-            uint32_t dd[4];
-#pragma unroll
-            for (int x = 0; x < 8; x += 4) {
-              const float4 nl = *reinterpret_cast<const float4*>(st_l + 32 * c + e + x), nd = *reinterpret_cast<const float4*>(st_l + 128 + 32 * c + e + x);
-              const uint64_t nl2[2] = {pack_f2(nl.x, nl.y), pack_f2(nl.z, nl.w)}, nd2[2] = {pack_f2(nd.x, nd.y), pack_f2(nd.z, nd.w)};
-#pragma unroll
-              for (int y = 0; y < 2; ++y) {
-                const int i0 = e + x + 2 * y;
-                float x0, x1, d0, d1;
-                unpack_f2(ffma2(pack_u2(rs[i0], rs[i0 + 1]), sc2, nl2[y]), x0, x1);
-                const float p0 = ex2(x0), p1 = ex2(x1);
-                unpack_f2(fmul2(pack_f2(p0, p1), fadd2(pack_u2(rd[i0], rd[i0 + 1]), nd2[y])), d0, d1);
-                pp[i0 >> 1] = pack2(p0, p1);
-                dd[(x >> 1) + y] = pack2(d0, d1);
-              }
+              for (int e = 0; e < 32; ++e)
+                if (e < first) rs[e] = 0xff800000u;
             }
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(uds + row * 128 + (((4 * c + (e >> 3)) ^ (row & 7)) << 4)),
-                         "r"(dd[0]), "r"(dd[1]), "r"(dd[2]), "r"(dd[3]) : "memory");
+#pragma unroll
+            for (int e = 0; e < 32; e += 4) {
+              const float4 nl = *reinterpret_cast<const float4*>(st + 32 * c + e);
+              float x0, x1, x2, x3;
+              unpack_f2(ffma2(pack_u2(rs[e], rs[e + 1]), sc2, pack_f2(nl.x, nl.y)), x0, x1);
+              unpack_f2(ffma2(pack_u2(rs[e + 2], rs[e + 3]), sc2, pack_f2(nl.z, nl.w)), x2, x3);
+              p[e] = ex2(x0); p[e + 1] = ex2(x1); p[e + 2] = ex2(x2); p[e + 3] = ex2(x3);
+              pp[e >> 1] = pack2(p[e], p[e + 1]); pp[(e >> 1) + 1] = pack2(p[e + 2], p[e + 3]);
+            }
           }
-          // (d = 128: P goes over the scores of this warpgroup that have been read)
-          tmem_st16(lane_addr + C::kColP + C::kPHalf * h + 16 * c, pp);
+          // d = 128: P goes over scores of this warpgroup that have been read
+          if (D == 128) tmem_st16(lane_addr + C::kColP + C::kPHalf * h + 16 * c, pp);
+          if (c == 0) {
+            ok = wait_fast<4>(bar_dp, g & 1, s_abort, status);
+            if (g >= C::NDS) ok = ok && wait_fast<5>(bar_dsfree(g), (g / C::NDS - 1) & 1, s_abort, status);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+          }
+#pragma unroll
+          for (int c2 = 0; c2 < 32; c2 += 16) {
+            uint32_t rd[16];
+            tmem_ld16_issue(lane_addr + C::kColDP + 64 * h + 32 * c + c2, rd);
+            tmem_ld16_wait(rd);
+#pragma unroll
+            for (int e = 0; e < 16; e += 8) {
+              uint32_t dd[4];
+#pragma unroll
+              for (int x = 0; x < 8; x += 4) {
+                const float4 nd = *reinterpret_cast<const float4*>(st + 128 + 32 * c + c2 + e + x);
+                const int i0 = c2 + e + x;
+                float d0, d1, d2, d3;
+                unpack_f2(fmul2(pack_f2(p[i0], p[i0 + 1]), fadd2(pack_u2(rd[e + x], rd[e + x + 1]), pack_f2(nd.x, nd.y))), d0, d1);
+                unpack_f2(fmul2(pack_f2(p[i0 + 2], p[i0 + 3]), fadd2(pack_u2(rd[e + x + 2], rd[e + x + 3]), pack_f2(nd.z, nd.w))), d2, d3);
+                dd[x >> 1] = pack2(d0, d1); dd[(x >> 1) + 1] = pack2(d2, d3);
+              }
+              // (no memory clobber: the reads of the statistics may move across; what follows is ordered by the fences below)
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(uds + (((4 * c + ((c2 + e) >> 3)) ^ (row & 7)) << 4)),
+                           "r"(dd[0]), "r"(dd[1]), "r"(dd[2]), "r"(dd[3]));
+            }
+          }
+          if (D == 64) {
+            // (P of the step before is read by the dV product until here at most)
+            if (c == 0 && g > 0) {
+              ok = __all_sync(0xffffffffu, wait_fast<6>(bar_dofree(g - 1), ((g - 1) >> 1) & 1, s_abort, status));
+              if (!ok) break;
+              tc_fence_after();
+            }
+            tmem_st16(lane_addr + C::kColP + C::kPHalf * h + 16 * c, pp);
+          }
         }
+        if (!ok) break;
         tmem_wait_st();
         tc_fence_before();
         fence_async_smem();
@@ -359,64 +386,66 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_dfree(it));
     }
-  } else if (warp < 12) {
-    // ================= dQ after every step, dK and dV after every item: out of TMEM, into the fp32 accumulators ==================
-    // Rows leave TMEM one per thread, but a reduction instruction whose lanes hit 32 different rows costs the L2 32 half-filled
-    // sectors: a warp's 32 rows x 32 columns pass through shared memory (chunks XOR-swizzled by row) and go out with eight
-    // lanes per row, four rows per instruction.
-    const int row = tid - 256;
+  } else if (warp < 16) {
+    // ================= results, fp32 reductions into the accumulators: dQ after every step, dK and dV after every item; warpgroup
+    // r takes half of the columns ==================
+    const int r_ = (warp - 8) >> 2, row = tid & 127;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t stage = ubase + C::kOffStage + (warp & 3) * C::kStageWarp;
-    constexpr int NP = C::kStageWarp / 4096;            // 32-column pieces staged together
+    constexpr int NC = D / 2;                           // columns of a result that this warpgroup takes
+    // A reduction instruction whose lanes hit 32 different rows costs the L2 32 half-filled sectors: a warp's 32 rows x 32
+    // columns pass through shared memory (chunks XOR-swizzled by row) and go out with eight lanes per row, four rows per instruction.
+    const uint32_t stage = ubase + C::kOffStage + (warp - 8) * 4096;
     auto out_rows = [&](uint32_t taddr, float f, float* base, size_t seg_row0, int grow, uint32_t bar_done) {
-#pragma unroll 1
-      for (int c0 = 0; c0 < D; c0 += 32 * NP) {
-#pragma unroll 1
-        for (int p = 0; p < NP; ++p) {
-          uint32_t r[32];
-          tmem_ld32_issue(taddr + c0 + 32 * p, r);
-          tmem_ld32_wait(r);
+      uint32_t r[NC];
 #pragma unroll
-          for (int c = 0; c < 8; ++c)
-            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stage + p * 4096 + lane * 128 + ((c ^ (lane & 7)) << 4)),
-                         "f"(__uint_as_float(r[4 * c]) * f), "f"(__uint_as_float(r[4 * c + 1]) * f),
-                         "f"(__uint_as_float(r[4 * c + 2]) * f), "f"(__uint_as_float(r[4 * c + 3]) * f) : "memory");
-        }
-        if (c0 + 32 * NP == D && bar_done) {            // everything has left TMEM
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_done);
-        }
+      for (int p = 0; p < NC / 32; ++p) tmem_ld32_issue(taddr + NC * r_ + 32 * p, *reinterpret_cast<uint32_t(*)[32]>(r + 32 * p));
+#pragma unroll
+      for (int p = 0; p < NC / 32; ++p) tmem_ld32_wait(*reinterpret_cast<uint32_t(*)[32]>(r + 32 * p));
+      if (bar_done) {                                   // it has left TMEM
+        tc_fence_before();
         __syncwarp();
-#pragma unroll 1
-        for (int p = 0; p < NP; ++p) {
+        if (lane == 0) mbar_arrive(bar_done);
+      }
+      const int c = lane & 7;
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int rr = 4 * q + (lane >> 3), c = lane & 7;
-            const int gr = __shfl_sync(0xffffffffu, grow, rr);
-            float4 v;
-            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                         : "r"(stage + p * 4096 + rr * 128 + ((c ^ (rr & 7)) << 4)) : "memory");
-            if (gr >= 0) atomicAdd(reinterpret_cast<float4*>(base + (seg_row0 + gr) * D + c0 + 32 * p + 4 * c), v);
+      for (int p = 0; p < NC / 32; ++p) {
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((x ^ (lane & 7)) << 4)),
+                       "f"(__uint_as_float(r[32 * p + 4 * x]) * f), "f"(__uint_as_float(r[32 * p + 4 * x + 1]) * f),
+                       "f"(__uint_as_float(r[32 * p + 4 * x + 2]) * f), "f"(__uint_as_float(r[32 * p + 4 * x + 3]) * f) : "memory");
+        __syncwarp();
+#pragma unroll
+        for (int q0 = 0; q0 < 8; q0 += 4) {
+          float4 v[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int rr = 4 * (q0 + q) + (lane >> 3);
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[q].x), "=f"(v[q].y), "=f"(v[q].z), "=f"(v[q].w)
+                         : "r"(stage + rr * 128 + ((c ^ (rr & 7)) << 4)) : "memory");
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int gr = __shfl_sync(0xffffffffu, grow, 4 * (q0 + q) + (lane >> 3));
+            if (gr >= 0) atomicAdd(reinterpret_cast<float4*>(base + (seg_row0 + gr) * D + NC * r_ + 32 * p + 4 * c), v[q]);
           }
         }
         __syncwarp();
       }
     };
+    uint32_t g = 0;
     for (int it = 0; ok; ++it) {
       ok = __all_sync(0xffffffffu, wait_desc(it));
       if (!ok) break;
       const BwdItem& t = desc_of(it);
       if (t.kind < 0) break;
-      const size_t seg_row0 = (size_t)t.seg * g.n;
+      const size_t seg_row0 = (size_t)t.seg * g_.n;
       const int kr = row < t.nkeys ? key_row(t, row) : -1;
       const int steps = t.steps;
 #pragma unroll 1
-      for (int s = 0; s < steps; ++s, ++gs) {
-        const StepRows sr = step_rows(b, t, s);
-        int qr = -1;
-        if (row < sr.nq) qr = t.kind == 0 ? sr.first + row : t.q0 + __ldg(a.perm_q + t.slice + sr.first + row);
-        ok = __all_sync(0xffffffffu, wait_fast<7>(bar_dq(gs), (gs >> 1) & 1, s_abort, status));
+      for (int s = 0; s < steps; ++s, ++g) {
+        const int qr = query_row(t, step_rows(b, t, s), row);
+        ok = __all_sync(0xffffffffu, wait_fast<7>(bar_dq(g), (g >> 1) & 1, s_abort, status));
         if (!ok) break;
         tc_fence_after();
         out_rows(lane_addr + C::kColDQ, b.scale, b.dq, seg_row0, qr, bar_dqfree);
@@ -430,7 +459,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_dfree(it));
     }
-  } else if (warp == 12) {
+  } else if (warp == 16) {
     // ================= MMA issue (one lane) ==================
     if (lane == 0) {
       // descriptors: low word = start >> 4 | (leading byte offset >> 4) << 16, high word = stride 1024 B | version | 128-byte swizzle
@@ -440,174 +469,201 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
       constexpr uint32_t idesc_s = idesc | ((128u >> 3) << 17);                                            // K-major x K-major, N = 128
       constexpr uint32_t idesc_n = idesc | (1u << 16) | (((uint32_t)D >> 3) << 17);                        // K-major (or TMEM) x MN-major, N = D
       constexpr uint32_t idesc_t = idesc | (1u << 15) | (1u << 16) | (((uint32_t)D >> 3) << 17);           // MN-major x MN-major, N = D
-      auto kmajor = [&](uint32_t off, int ks) { return ((ubase + off + (ks >> 2) * kSlab + (ks & 3) * 32) >> 4) | (1u << 16); };
-      auto mnmajor = [&](uint32_t off, int kk) { return ((ubase + off + kk * 2048) >> 4) | ((kSlab >> 4) << 16); };
-      uint32_t kv = 0;                                  // where the item's K and V lie
-      auto score = [&](uint32_t gq) {                   // S^T of step gq
-        ok = ok && wait_fast<9>(bar_qfull(gq), (gq >> 1) & 1, s_abort, status);
+      const uint32_t base = ubase >> 4;
+      auto kmajor = [&](uint32_t off, int ks) { return base + ((off + (ks >> 2) * kSlab + (ks & 3) * 32) >> 4) + (1u << 16); };
+      auto mnmajor = [&](uint32_t off, int kk) { return base + ((off + kk * 2048) >> 4) + ((kSlab >> 4) << 16); };
+      // Scores run a step ahead of the gradients, across item boundaries.  gs, gp: next step of S and dP; its / itp: its item;
+      // ls / lp: steps left in it.
+      uint32_t gs = 0, gp = 0, g = 0;
+      int its = -1, itp = -1, ls = 0, lp = 0;
+      bool ends = false;
+      // whether S (dP) of the next step could be issued without waiting
+      auto s_ready = [&]() {
+        if (ls == 0) {
+          if (!mbar_test(bar_dfull(its + 1), ((its + 1) / kDescs) & 1)) return false;
+          if (desc_of(its + 1).kind < 0 || !mbar_test(bar_kfull(its + 1), ((its + 1) / C::NKV) & 1)) return false;
+        }
+        return mbar_test(bar_qfull(gs), (gs >> 1) & 1);
+      };
+      auto issue_s = [&]() {
+        if (ls == 0) {
+          ++its;
+          ok = ok && wait_desc(its);
+          if (!ok) return;
+          if (desc_of(its).kind < 0) { ends = true; return; }
+          ls = desc_of(its).steps;
+          ok = wait_fast<9>(bar_kfull(its), (its / C::NKV) & 1, s_abort, status);
+        }
+        ok = ok && wait_fast<10>(bar_qfull(gs), (gs >> 1) & 1, s_abort, status);
         if (!ok) return;
         fence_async_smem();
         tc_fence_after();
-        const uint32_t q = C::kOffQ + (gq & 1) * C::kTile;
+        const uint32_t k = C::kOffK + (its % C::NKV) * C::kTile, q = C::kOffQ + (gs & 1) * C::kTile;
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColS, kmajor(kv, ks), kmajor(q, ks), desc_hi, idesc_s, ks > 0);
+        for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColS, kmajor(k, ks), kmajor(q, ks), desc_hi, idesc_s, ks > 0);
         umma_commit(bar_s);
+        ++gs; --ls;
       };
-      auto dscore = [&](uint32_t gq) {                  // dP^T
-        ok = ok && wait_fast<10>(bar_dofull(gq), (gq / C::NDO) & 1, s_abort, status);
+      // (dP only ever follows S of the same step: its item is known)
+      auto p_ready = [&]() {
+        if (gp >= gs) return false;
+        if (lp == 0 && !mbar_test(bar_vfull(itp + 1), ((itp + 1) / C::NKV) & 1)) return false;
+        if (D == 128 && gp > 0 && !mbar_test(bar_dqfree, (gp - 1) & 1)) return false;
+        return mbar_test(bar_dofull(gp), (gp / C::NDO) & 1);
+      };
+      auto issue_p = [&]() {
+        if (lp == 0) {
+          ++itp;
+          lp = desc_of(itp).steps;
+          ok = ok && wait_fast<11>(bar_vfull(itp), (itp / C::NKV) & 1, s_abort, status);
+        }
+        // (d = 128: dQ of the step before lies there)
+        if (D == 128 && gp > 0) ok = ok && wait_fast<12>(bar_dqfree, (gp - 1) & 1, s_abort, status);
+        ok = ok && wait_fast<13>(bar_dofull(gp), (gp / C::NDO) & 1, s_abort, status);
         if (!ok) return;
         fence_async_smem();
         tc_fence_after();
-        const uint32_t o = C::kOffDO + (gq % C::NDO) * C::kTile;
+        const uint32_t v = C::kOffV + (itp % C::NKV) * C::kTile, o = C::kOffDO + (gp % C::NDO) * C::kTile;
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColDP, kmajor(kv + C::kTile, ks), kmajor(o, ks), desc_hi, idesc_s, ks > 0);
+        for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColDP, kmajor(v, ks), kmajor(o, ks), desc_hi, idesc_s, ks > 0);
         umma_commit(bar_dp);
+        ++gp; --lp;
       };
-      for (int it = 0; ok; ++it) {
-        ok = wait_desc(it);
-        if (!ok) break;
-        const BwdItem& t = desc_of(it);
-        if (t.kind < 0) break;
-        const int steps = t.steps;
-        kv = C::kOffKV + (it % C::NKV) * 2 * C::kTile;
-        ok = wait_fast<11>(bar_kv(it), (it / C::NKV) & 1, s_abort, status);
-        if (!ok) break;
-        if (D == 128 && gs > 0) ok = wait_fast<12>(bar_dqfree, (gs - 1) & 1, s_abort, status);
-        score(gs);
-        dscore(gs);
+      issue_s();
+      if (ok && !ends) issue_p();
+      for (int it = 0; ok && !ends; ++it) {
+        const int steps = desc_of(it).steps;
+        const uint32_t kt = C::kOffK + (it % C::NKV) * C::kTile;
 #pragma unroll 1
-        for (int s = 0; s < steps && ok; ++s, ++gs) {
-          ok = wait_fast<13>(bar_h, gs & 1, s_abort, status);
+        for (int s = 0; s < steps && ok; ++s, ++g) {
+          ok = wait_fast<14>(bar_h, g & 1, s_abort, status);
           if (!ok) break;
           tc_fence_after();
-          const bool more = s + 1 < steps;
-          const uint32_t q = C::kOffQ + (gs & 1) * C::kTile, o = C::kOffDO + (gs % C::NDO) * C::kTile, ds = C::kOffDS + (gs % C::NDS) * (128 * 128 * 2);
+          const bool last = s + 1 == steps;
+          const uint32_t q = C::kOffQ + (g & 1) * C::kTile, o = C::kOffDO + (g % C::NDO) * C::kTile, ds = C::kOffDS + (g % C::NDS) * (128 * 128 * 2);
           auto grad_v = [&]() {
-            if (s == 0 && it > 0) ok = ok && wait_fast<14>(bar_accfree, (it - 1) & 1, s_abort, status);
+            if (s == 0 && it > 0) {
+              ok = ok && wait_fast<15>(bar_accfree, (it - 1) & 1, s_abort, status);
+              tc_fence_after();
+            }
             if (!ok) return;
-            tc_fence_after();
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk)
               mma_ts2(tmem + C::kColDV, tmem + C::kColP + (kk >> 2) * C::kPHalf + (kk & 3) * 8, mnmajor(o, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
-            umma_commit(bar_dofree(gs));
+            umma_commit(bar_dofree(g));
           };
           auto grad_k = [&]() {
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) mma_ss2(tmem + C::kColDK, kmajor(ds, kk), mnmajor(q, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
-            umma_commit(bar_qfree(gs));
+            umma_commit(bar_qfree(g));
+            if (last) umma_commit(bar_acc);
           };
           auto grad_q = [&]() {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) mma_ss2(tmem + C::kColDQ, mnmajor(ds, kk), mnmajor(kv, kk), desc_hi, idesc_t, kk > 0);
-            umma_commit(bar_dq(gs));
+            for (int kk = 0; kk < 8; ++kk) mma_ss2(tmem + C::kColDQ, mnmajor(ds, kk), mnmajor(kt, kk), desc_hi, idesc_t, kk > 0);
+            umma_commit(bar_dq(g));
+            if (last) umma_commit(bar_kfree(it));
           };
           if (D == 64) {
-            if (more) { score(gs + 1); dscore(gs + 1); }
-            if (!ok) break;
+            if (s_ready()) issue_s();
+            if (ok && p_ready()) issue_p();
             grad_v();
             if (!ok) break;
             grad_k();
-            if (!more) umma_commit(bar_acc);
-            if (gs > 0) ok = wait_fast<12>(bar_dqfree, (gs - 1) & 1, s_abort, status);
+            if (g > 0) ok = wait_fast<12>(bar_dqfree, (g - 1) & 1, s_abort, status);
             if (!ok) break;
             tc_fence_after();
             grad_q();
+            umma_commit(bar_dsfree(g));
           } else {
-            grad_q();
             grad_v();
             if (!ok) break;
-            if (more) score(gs + 1);
+            grad_q();
+            if (s_ready()) issue_s();
             if (!ok) break;
             grad_k();
-            if (!more) umma_commit(bar_acc);
-            else {
-              ok = wait_fast<12>(bar_dqfree, gs & 1, s_abort, status);
-              dscore(gs + 1);
-            }
+            umma_commit(bar_dsfree(g));
           }
+          if (ok && gs == g + 1) issue_s();
+          if (ok && !ends && gp == g + 1) issue_p();
         }
-        if (!ok) break;
-        umma_commit(bar_kvfree(it));
-        mbar_arrive(bar_dfree(it));
+        if (ok) mbar_arrive(bar_dfree(it));
       }
     }
     __syncwarp();
-  } else if (warp < 15) {
-    // ================= loaders: warp 13 Q, dO and row statistics of every step, warp 14 K and V of every item ==================
+  } else {
+    // ================= loaders: warp 17 Q and row statistics, warp 18 dO, warp 19 items, K and V ==================
     // Tiles of consecutive rows: lane 0 issues TMA boxes.  Others: rows gathered in 16-byte chunks, lane -> chunk cc of row
     // k RPI + crow of instruction k; lane l holds the row numbers of rows l, l + 32, ..., handed round by shuffles.
     constexpr int CPR = D / 8, RPI = 32 / CPR, NSW = 8 / RPI;
     const int cc = lane % CPR, crow = lane / CPR;
-    uint32_t sw[NSW];                                    // byte offset of (row k RPI + crow, chunk cc) is k RPI 128 + sw[k % NSW]
+    uint32_t sw[NSW];                                    // byte offset of (row k RPI + crow, chunk cc) in its slab is k RPI 128 + sw[k % NSW]
 #pragma unroll
-    for (int k = 0; k < NSW; ++k) sw[k] = (uint32_t)((cc >> 3) * (128 * 128) + crow * 128 + (((cc & 7) ^ ((k * RPI + crow) & 7)) << 4));
-    auto gather = [&](uint32_t dst, const __nv_bfloat16* base, const int (&v)[4], uint32_t bar) {
+    for (int k = 0; k < NSW; ++k) sw[k] = (uint32_t)(crow * 128 + (((cc & 7) ^ ((k * RPI + crow) & 7)) << 4));
+    auto gather = [&](uint32_t dst, const __nv_bfloat16* base, auto& v, uint32_t bar) {
+      constexpr int ROWS = 32 * (sizeof(v) / sizeof(v[0]));
       const char* src = reinterpret_cast<const char*>(base) + cc * 16;
+      const uint32_t d = dst + (cc >> 3) * (ROWS * 128);
 #pragma unroll
-      for (int k = 0; k < 128 / RPI; ++k) {
+      for (int k = 0; k < ROWS / RPI; ++k) {
         const int rw = __shfl_sync(0xffffffffu, v[k * RPI / 32], (k * RPI & 31) + crow);
-        cp_async16(dst + k * RPI * 128 + sw[k % NSW], src + (size_t)(uint32_t)rw * (D * 2));
+        cp_async16(d + k * RPI * 128 + sw[k % NSW], src + (size_t)(uint32_t)rw * (D * 2));
       }
       cp_async_arrive_noinc(bar);
     };
-    auto boxes = [&](uint32_t dst, const CUtensorMap* map, int y, uint32_t bar) {
+    auto boxes = [&](uint32_t dst, int rows, const CUtensorMap* map, int y, uint32_t bar) {
+      if (lane == 0) {
+        mbar_expect_tx(bar, rows * D * 2);
 #pragma unroll
-      for (int sl = 0; sl < D / 64; ++sl) tma_tile(dst + sl * (128 * 128), map, sl * 64, y, bar);
+        for (int sl = 0; sl < D / 64; ++sl) tma_tile(dst + sl * rows * 128, map, sl * 64, y, bar);
+      }
+      __syncwarp();
+      mbar_arrive(bar);
     };
-    if (warp == 13) {
+    if (warp < 19) {
+      const bool is_q = warp == 17;
+      const int nbuf = is_q ? C::NQ : C::NDO;
+      uint32_t g = 0;
       for (int it = 0; ok; ++it) {
         ok = __all_sync(0xffffffffu, wait_desc(it));
         if (!ok) break;
         const BwdItem& t = desc_of(it);
         if (t.kind < 0) break;
-        const int steps = t.steps, seg_row0 = t.seg * g.n;
+        const int steps = t.steps, seg_row0 = t.seg * g_.n;
+        const bool dense = t.kind == 0;
         const float wlog = t.wlog;
         // row numbers and statistics of a step's query rows (rows that do not exist: the node's first row, with weights of zero)
         int vn[4];
         float2 sn[4];
-        auto rows_of = [&](int s) {
-          const StepRows sr = step_rows(b, t, s);
+        auto rows_of = [&](int x) {
+          const StepRows sr = step_rows(b, t, x);
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const int r = lane + 32 * u;
-            const bool in = r < sr.nq;
-            int x = t.q0;
-            if (in) x = t.kind == 0 ? sr.first + r : t.q0 + __ldg(a.perm_q + t.slice + sr.first + r);
-            vn[u] = seg_row0 + x;
-            sn[u] = in ? __ldg(b.stat + vn[u]) : make_float2(-INFINITY, 0.f);
+            const int qr = query_row(t, sr, lane + 32 * u);
+            vn[u] = seg_row0 + (qr >= 0 ? qr : t.q0);
+            if (is_q) sn[u] = qr >= 0 ? __ldg(b.stat + vn[u]) : make_float2(-INFINITY, 0.f);
           }
         };
-        rows_of(0);
+        if (is_q || !dense) rows_of(0);
 #pragma unroll 1
-        for (int s = 0; s < steps; ++s, ++gs) {
-          const int v[4] = {vn[0], vn[1], vn[2], vn[3]};
-          if (gs > 1) {
-            ok = __all_sync(0xffffffffu, wait_fast<16>(bar_qfree(gs), ((gs >> 1) - 1) & 1, s_abort, status));
+        for (int x = 0; x < steps; ++x, ++g) {
+          int v[4] = {vn[0], vn[1], vn[2], vn[3]};
+          const uint32_t bar = is_q ? bar_qfull(g) : bar_dofull(g);
+          const uint32_t dst = ubase + (is_q ? C::kOffQ + (g % C::NQ) * C::kTile : C::kOffDO + (g % C::NDO) * C::kTile);
+          if (g >= (uint32_t)nbuf) {
+            const uint32_t last = g - nbuf;              // (the step that used the buffer before)
+            ok = __all_sync(0xffffffffu, wait_fast<16>(is_q ? bar_qfree(last) : bar_dofree(last), (last >> 1) & 1, s_abort, status));
             if (!ok) break;
           }
-          float* st = reinterpret_cast<float*>(smem + C::kOffStat) + (gs & 1) * 256;
+          if (is_q) {
+            float* st = reinterpret_cast<float*>(smem + C::kOffStat) + (g % C::NQ) * 256;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) { st[lane + 32 * u] = sn[u].x + wlog; st[128 + lane + 32 * u] = sn[u].y; }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_stat(gs));
-          const uint32_t dq = ubase + C::kOffQ + (gs & 1) * C::kTile, dd = ubase + C::kOffDO + (gs % C::NDO) * C::kTile;
-          const bool dense = t.kind == 0;
-          const int y = seg_row0 + t.q0 + s * kTileQ;
-          if (dense) {
-            if (lane == 0) { mbar_expect_tx(bar_qfull(gs), C::kTile); boxes(dq, &maps.q, y, bar_qfull(gs)); }
-            __syncwarp();
-            mbar_arrive(bar_qfull(gs));
-          } else gather(dq, a.q, v, bar_qfull(gs));
-          if (s + 1 < steps) rows_of(s + 1);               // (in flight while this step's copies are issued)
-          if (gs >= C::NDO) {
-            ok = __all_sync(0xffffffffu, wait_fast<17>(bar_dofree(gs), (gs / C::NDO - 1) & 1, s_abort, status));
-            if (!ok) break;
+            for (int u = 0; u < 4; ++u) { st[lane + 32 * u] = sn[u].x + wlog; st[128 + lane + 32 * u] = sn[u].y; }
+            mbar_arrive(bar);
           }
-          if (dense) {
-            if (lane == 0) { mbar_expect_tx(bar_dofull(gs), C::kTile); boxes(dd, &maps.dout, y, bar_dofull(gs)); }
-            __syncwarp();
-            mbar_arrive(bar_dofull(gs));
-          } else gather(dd, b.dout, v, bar_dofull(gs));
+          if (dense) boxes(dst, 128, is_q ? &maps.q : &maps.dout, seg_row0 + t.q0 + x * 128, bar);
+          else gather(dst, is_q ? a.q : b.dout, v, bar);
+          if (x + 1 < steps && (is_q || !dense)) rows_of(x + 1);
         }
         if (!ok) break;
         __syncwarp();
@@ -616,81 +672,56 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
       cp_async_commit();
       cp_async_wait_all();
       // (nothing may be in flight into shared memory when the CTA exits - trivially true unless it is giving up)
-      if (!ok) for (int x = 0; x < 2; ++x) { mbar_drain(bar_qfull(x), 0); mbar_drain(bar_qfull(x), 1); mbar_drain(bar_dofull(x % C::NDO), 0); mbar_drain(bar_dofull(x % C::NDO), 1); }
+      if (!ok)
+        for (int x = 0; x < nbuf; ++x) { mbar_drain(is_q ? bar_qfull(x) : bar_dofull(x), 0); mbar_drain(is_q ? bar_qfull(x) : bar_dofull(x), 1); }
     } else {
-      int it = 0;
-      for (; ok; ++it) {
-        ok = __all_sync(0xffffffffu, wait_desc(it));
-        if (!ok) break;
-        const BwdItem& t = desc_of(it);
+      // Work items are handed out by a counter in global memory, in list order (heavy first); the first gridDim.x need none.
+      int item = blockIdx.x;
+      for (int it = 0; ok; ++it) {
+        BwdItem t;
+        for (;;) {
+          if (it > 0 || item < 0) {
+            if (lane == 0) item = gridDim.x + atomicAdd(b.sched, 1);
+            item = __shfl_sync(0xffffffffu, item, 0);
+          }
+          if (item >= b.total_items) { t.kind = -1; break; }
+          if (decode_item(b, item, t)) break;
+          item = -1;
+        }
+        if (it >= kDescs) {
+          ok = __all_sync(0xffffffffu, wait_fast<17>(bar_dfree(it), (it / kDescs - 1) & 1, s_abort, status));
+          if (!ok) break;
+        }
+        if (lane == 0) {
+          *reinterpret_cast<BwdItem*>(smem + C::kOffDesc + (it % kDescs) * C::kDescBytes) = t;
+          mbar_arrive(bar_dfull(it));
+        }
+        __syncwarp();
         if (t.kind < 0) break;
-        const uint32_t dst = ubase + C::kOffKV + (it % C::NKV) * 2 * C::kTile, bar = bar_kv(it);
-        const int seg_row0 = t.seg * g.n;
-        int v[4];
+        const uint32_t dk = ubase + C::kOffK + (it % C::NKV) * C::kTile, dv = ubase + C::kOffV + (it % C::NKV) * C::kTile;
+        const int seg_row0 = t.seg * g_.n;
+        int v[4] = {0, 0, 0, 0};
         if (t.kind != 0) {
 #pragma unroll
           for (int u = 0; u < 4; ++u) v[u] = seg_row0 + key_row(t, min(lane + 32 * u, t.nkeys - 1));     // (keys that do not exist: the last one)
         }
-        if (it >= C::NKV) {
-          ok = __all_sync(0xffffffffu, wait_fast<18>(bar_kvfree(it), (it / C::NKV - 1) & 1, s_abort, status));
-          if (!ok) break;
-        }
-        if (t.kind == 0) {
-          if (lane == 0) {
-            mbar_expect_tx(bar, 2 * C::kTile);
-            boxes(dst, &maps.k, seg_row0 + t.k0, bar);
-            boxes(dst + C::kTile, &maps.v, seg_row0 + t.k0, bar);
-          }
-          __syncwarp();
-          mbar_arrive(bar);
-        } else {
-          const char* srck = reinterpret_cast<const char*>(a.k) + cc * 16;
-#pragma unroll
-          for (int k = 0; k < 128 / RPI; ++k) {
-            const int rw = __shfl_sync(0xffffffffu, v[k * RPI / 32], (k * RPI & 31) + crow);
-            cp_async16(dst + k * RPI * 128 + sw[k % NSW], srck + (size_t)(uint32_t)rw * (D * 2));
-          }
-          gather(dst + C::kTile, a.v, v, bar);            // (its arrival covers both tiles' copies)
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_dfree(it));
+        if (it >= C::NKV) ok = __all_sync(0xffffffffu, wait_fast<18>(bar_kfree(it), (it / C::NKV - 1) & 1, s_abort, status));
+        if (!ok) break;
+        if (t.kind == 0) boxes(dk, 128, &maps.k, seg_row0 + t.k0, bar_kfull(it));
+        else gather(dk, a.k, v, bar_kfull(it));
+        if (t.kind == 0) boxes(dv, 128, &maps.v, seg_row0 + t.k0, bar_vfull(it));
+        else gather(dv, a.v, v, bar_vfull(it));
       }
       cp_async_commit();
       cp_async_wait_all();
-      if (!ok) for (int x = 0; x < C::NKV; ++x) { mbar_drain(bar_kv(x), 0); mbar_drain(bar_kv(x), 1); }
-    }
-  } else {
-    // ================= item descriptors ==================
-    // Work items are handed out by a counter in global memory, in list order (heavy first); the first gridDim.x need none.
-    int item = blockIdx.x;
-    for (int it = 0; ok; ++it) {
-      BwdItem t;
-      for (;; ) {
-        if (it > 0 || item < 0) {
-          if (lane == 0) item = gridDim.x + atomicAdd(b.sched, 1);
-          item = __shfl_sync(0xffffffffu, item, 0);
-        }
-        if (item >= b.total_items) { t.kind = -1; break; }
-        if (decode_item(b, item, t)) break;
-        item = -1;
-      }
-      if (it >= kDescs) {
-        ok = __all_sync(0xffffffffu, wait_fast<19>(bar_dfree(it), (it / kDescs - 1) & 1, s_abort, status));
-        if (!ok) break;
-      }
-      if (lane == 0) {
-        *reinterpret_cast<BwdItem*>(smem + C::kOffDesc + (it % kDescs) * C::kDescBytes) = t;
-        mbar_arrive(bar_dfull(it));
-      }
-      __syncwarp();
-      if (t.kind < 0) break;
+      if (!ok) for (int x = 0; x < C::NKV; ++x) for (int y = 0; y < 2; ++y) { mbar_drain(bar_kfull(x), y); mbar_drain(bar_vfull(x), y); }
     }
   }
 
   // ---- teardown ------------------------------------------------------------------------------------
   tc_fence_before();
   __syncthreads();
-  if (warp == 12) {
+  if (warp == 16) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
   }

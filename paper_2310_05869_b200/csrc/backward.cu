@@ -34,7 +34,6 @@
 namespace hyperattn {
 namespace {
 
-constexpr int kThreads = 640;
 constexpr int kDescs = 3;              // item descriptors in flight
 constexpr int kTileK = 128;            // keys per item, query rows per step
 
@@ -156,6 +155,8 @@ __device__ __forceinline__ StepRows step_rows(const BwdArgs& b, const BwdItem& t
 
 template <int D>
 struct Cfg {
+  // warps: P and dS (SW of them, 128 / (SW / 4) query columns each), results, then issue, Q, dO, items
+  static constexpr int SW = D == 64 ? 16 : 8, kThreads = 32 * (SW + 12);
   static constexpr int kTile = 128 * D * 2;           // bytes of a [128 rows x D] tile
   // buffers: K and V (an item each), Q, dO and dS (a step each); d = 128 has room for two only of Q
   static constexpr int NKV = D == 64 ? 2 : 1, NQ = 2, NDO = D == 64 ? 2 : 1, NDS = D == 64 ? 2 : 1;
@@ -217,8 +218,13 @@ __global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__
   if (row < rows && c % LPR == 0) stat[row] = make_float2(-lse[row] * 1.4426950408889634f, -acc);
 }
 
+template <int SITE>
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
+  return __all_sync(0xffffffffu, wait_fast<SITE>(bar, parity, abort_flag, status)) != 0;
+}
+
 template <int D>
-__global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant__ BwdArgs b, const __grid_constant__ BwdMaps maps, int* status) {
+__global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_constant__ BwdArgs b, const __grid_constant__ BwdMaps maps, int* status) {
   using C = Cfg<D>;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
@@ -245,28 +251,29 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
 
   const AttnArgs& a = b.a;
   const Geometry& g_ = a.g;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);       // (known to be the same for the whole warp)
 
   if (tid == 0) *s_abort = *reinterpret_cast<volatile int*>(status);
   __syncthreads();
   if (*s_abort) return;                                 // (a launch in which some wait already timed out drains quickly)
   __syncthreads();
   if (tid == 0) {
-    mbar_init(bar_s, 1); mbar_init(bar_dp, 1); mbar_init(bar_h, 8); mbar_init(bar_dqfree, 8); mbar_init(bar_acc, 1); mbar_init(bar_accfree, 8);   // (8: one arrival per warp)
+    mbar_init(bar_s, 1); mbar_init(bar_dp, 1); mbar_init(bar_h, C::SW); mbar_init(bar_dqfree, 8); mbar_init(bar_acc, 1); mbar_init(bar_accfree, 8);   // (8: one arrival per warp)
     for (int x = 0; x < 2; ++x) { mbar_init(bar_dsfree(x), 1); mbar_init(bar_dq(x), 1); mbar_init(bar_qfull(x), 64); mbar_init(bar_qfree(x), 1); mbar_init(bar_dofree(x), 1); }
     for (int x = 0; x < C::NDO; ++x) mbar_init(bar_dofull(x), 32);
     for (int x = 0; x < C::NKV; ++x) { mbar_init(bar_kfull(x), 32); mbar_init(bar_vfull(x), 32); mbar_init(bar_kfree(x), 1); }
-    for (int x = 0; x < kDescs; ++x) { mbar_init(bar_dfull(x), 1); mbar_init(bar_dfree(x), 19); }   // 8 + 8 warps, issuer, two loaders
+    for (int x = 0; x < kDescs; ++x) { mbar_init(bar_dfull(x), 1); mbar_init(bar_dfree(x), C::SW + 11); }   // P and results warps, issuer, two loaders
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 16) {
+  if (warp == C::SW + 8) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *s_tmem;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *s_tmem, 0);
   wait_for_stream();
   auto desc_of = [&](int it) -> const BwdItem& { return *reinterpret_cast<const BwdItem*>(smem + C::kOffDesc + (it % kDescs) * C::kDescBytes); };
   auto wait_desc = [&](int it) { return wait_fast<1>(bar_dfull(it), (it / kDescs) & 1, s_abort, status); };
@@ -282,10 +289,12 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
   };
 
   bool ok = true;
-  if (warp < 8) {
-    // ================= P and dS: thread = key, warpgroup h: query columns 64 h .. 64 h + 63 ==================
-    const int h = warp >> 2, row = tid & 127;
+  if (warp < C::SW) {
+    // ================= P and dS: thread = key, warpgroup q: query columns W q .. W q + W - 1, in two chunks ==================
+    constexpr int W = 128 / (C::SW / 4), CW = W / 2;
+    const int row = tid & 127, col0 = (warp >> 2) * W;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t p_addr = lane_addr + C::kColP + C::kPHalf * (col0 >> 6) + (col0 & 63) / 2;
     const uint64_t sc2 = pack_f2(a.scale_log2, a.scale_log2);
     uint32_t g = 0;
     for (int it = 0; ok; ++it) {
@@ -308,34 +317,39 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
-        const float* st = reinterpret_cast<const float*>(smem + C::kOffStat) + (g & 1) * 256 + 64 * h;
-        const uint32_t uds = ubase + C::kOffDS + (g % C::NDS) * 32768 + h * 16384 + row * 128;
+        const float* st = reinterpret_cast<const float*>(smem + C::kOffStat) + (g & 1) * 256 + col0;
+        const uint32_t uds = ubase + C::kOffDS + (g % C::NDS) * 32768 + (col0 >> 6) * 16384 + row * 128;
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
-          float p[32];
-          uint32_t pp[16];
-          {
-            uint32_t rs[32];
-            tmem_ld32_issue(lane_addr + C::kColS + 64 * h + 32 * c, rs);
-            tmem_ld32_wait(rs);
-            if (masked) {
-              const int first = dead ? 128 : (diag ? row - 64 * h - 32 * c : 0);      // columns below it do not count
+          float p[CW];
+          uint32_t pp[CW / 2];
 #pragma unroll
-              for (int e = 0; e < 32; ++e)
+          for (int c2 = 0; c2 < CW; c2 += 16) {
+            uint32_t rs[16];
+            tmem_ld16_issue(lane_addr + C::kColS + col0 + CW * c + c2, rs);
+            tmem_ld16_wait(rs);
+            if (masked) {
+              const int first = dead ? 128 : (diag ? row - col0 - CW * c - c2 : 0);      // columns below it do not count
+#pragma unroll
+              for (int e = 0; e < 16; ++e)
                 if (e < first) rs[e] = 0xff800000u;
             }
 #pragma unroll
-            for (int e = 0; e < 32; e += 4) {
-              const float4 nl = *reinterpret_cast<const float4*>(st + 32 * c + e);
+            for (int e = 0; e < 16; e += 4) {
+              const float4 nl = *reinterpret_cast<const float4*>(st + CW * c + c2 + e);
+              const int i0 = c2 + e;
               float x0, x1, x2, x3;
               unpack_f2(ffma2(pack_u2(rs[e], rs[e + 1]), sc2, pack_f2(nl.x, nl.y)), x0, x1);
               unpack_f2(ffma2(pack_u2(rs[e + 2], rs[e + 3]), sc2, pack_f2(nl.z, nl.w)), x2, x3);
-              p[e] = ex2(x0); p[e + 1] = ex2(x1); p[e + 2] = ex2(x2); p[e + 3] = ex2(x3);
-              pp[e >> 1] = pack2(p[e], p[e + 1]); pp[(e >> 1) + 1] = pack2(p[e + 2], p[e + 3]);
+              p[i0] = ex2(x0); p[i0 + 1] = ex2(x1); p[i0 + 2] = ex2(x2); p[i0 + 3] = ex2(x3);
+              pp[i0 >> 1] = pack2(p[i0], p[i0 + 1]); pp[(i0 >> 1) + 1] = pack2(p[i0 + 2], p[i0 + 3]);
             }
           }
+          auto put_p = [&]() {
+            if constexpr (CW == 32) tmem_st16(p_addr + 16 * c, pp); else tmem_st8(p_addr + 8 * c, pp);
+          };
           // d = 128: P goes over scores of this warpgroup that have been read
-          if (D == 128) tmem_st16(lane_addr + C::kColP + C::kPHalf * h + 16 * c, pp);
+          if (D == 128) put_p();
           if (c == 0) {
             ok = wait_fast<4>(bar_dp, g & 1, s_abort, status);
             if (g >= C::NDS) ok = ok && wait_fast<5>(bar_dsfree(g), (g / C::NDS - 1) & 1, s_abort, status);
@@ -344,16 +358,16 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
             tc_fence_after();
           }
 #pragma unroll
-          for (int c2 = 0; c2 < 32; c2 += 16) {
+          for (int c2 = 0; c2 < CW; c2 += 16) {
             uint32_t rd[16];
-            tmem_ld16_issue(lane_addr + C::kColDP + 64 * h + 32 * c + c2, rd);
+            tmem_ld16_issue(lane_addr + C::kColDP + col0 + CW * c + c2, rd);
             tmem_ld16_wait(rd);
 #pragma unroll
             for (int e = 0; e < 16; e += 8) {
               uint32_t dd[4];
 #pragma unroll
               for (int x = 0; x < 8; x += 4) {
-                const float4 nd = *reinterpret_cast<const float4*>(st + 128 + 32 * c + c2 + e + x);
+                const float4 nd = *reinterpret_cast<const float4*>(st + 128 + CW * c + c2 + e + x);
                 const int i0 = c2 + e + x;
                 float d0, d1, d2, d3;
                 unpack_f2(fmul2(pack_f2(p[i0], p[i0 + 1]), fadd2(pack_u2(rd[e + x], rd[e + x + 1]), pack_f2(nd.x, nd.y))), d0, d1);
@@ -361,7 +375,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
                 dd[x >> 1] = pack2(d0, d1); dd[(x >> 1) + 1] = pack2(d2, d3);
               }
               // (no memory clobber: the reads of the statistics may move across; what follows is ordered by the fences below)
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(uds + (((4 * c + ((c2 + e) >> 3)) ^ (row & 7)) << 4)),
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(uds + (((((col0 & 63) + CW * c + c2 + e) >> 3) ^ (row & 7)) << 4)),
                            "r"(dd[0]), "r"(dd[1]), "r"(dd[2]), "r"(dd[3]));
             }
           }
@@ -372,7 +386,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
               if (!ok) break;
               tc_fence_after();
             }
-            tmem_st16(lane_addr + C::kColP + C::kPHalf * h + 16 * c, pp);
+            put_p();
           }
         }
         if (!ok) break;
@@ -386,15 +400,15 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_dfree(it));
     }
-  } else if (warp < 16) {
+  } else if (warp < C::SW + 8) {
     // ================= results, fp32 reductions into the accumulators: dQ after every step, dK and dV after every item; warpgroup
     // r takes half of the columns ==================
-    const int r_ = (warp - 8) >> 2, row = tid & 127;
+    const int r_ = (warp - C::SW) >> 2, row = tid & 127;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     constexpr int NC = D / 2;                           // columns of a result that this warpgroup takes
     // A reduction instruction whose lanes hit 32 different rows costs the L2 32 half-filled sectors: a warp's 32 rows x 32
     // columns pass through shared memory (chunks XOR-swizzled by row) and go out with eight lanes per row, four rows per instruction.
-    const uint32_t stage = ubase + C::kOffStage + (warp - 8) * 4096;
+    const uint32_t stage = ubase + C::kOffStage + (warp - C::SW) * 4096;
     auto out_rows = [&](uint32_t taddr, float f, float* base, size_t seg_row0, int grow, uint32_t bar_done) {
       uint32_t r[NC];
 #pragma unroll
@@ -459,9 +473,15 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_dfree(it));
     }
-  } else if (warp == 16) {
-    // ================= MMA issue (one lane) ==================
-    if (lane == 0) {
+  } else if (warp == C::SW + 8) {
+    // ================= MMA issue ==================
+    // The whole warp walks through this code together and one elected lane issues: descriptors and addresses are then made of
+    // uniform registers, which the instructions take directly (a lone lane's have to be moved there one by one).
+    {
+      const bool el = elect_one();
+      auto uni = [&](int x) { return __shfl_sync(0xffffffffu, x, 0); };
+      auto utest = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_test(bar, parity)) != 0; };
+      auto uwait_desc = [&](int it) { return __all_sync(0xffffffffu, wait_desc(it)) != 0; };
       // descriptors: low word = start >> 4 | (leading byte offset >> 4) << 16, high word = stride 1024 B | version | 128-byte swizzle
       constexpr uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
       constexpr uint32_t kSlab = 128 * 128;             // bytes of one [128 rows x 64 columns] slab
@@ -480,89 +500,99 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
       // whether S (dP) of the next step could be issued without waiting
       auto s_ready = [&]() {
         if (ls == 0) {
-          if (!mbar_test(bar_dfull(its + 1), ((its + 1) / kDescs) & 1)) return false;
-          if (desc_of(its + 1).kind < 0 || !mbar_test(bar_kfull(its + 1), ((its + 1) / C::NKV) & 1)) return false;
+          if (!utest(bar_dfull(its + 1), ((its + 1) / kDescs) & 1)) return false;
+          if (uni(desc_of(its + 1).kind) < 0 || !utest(bar_kfull(its + 1), ((its + 1) / C::NKV) & 1)) return false;
         }
-        return mbar_test(bar_qfull(gs), (gs >> 1) & 1);
+        return utest(bar_qfull(gs), (gs >> 1) & 1);
       };
       auto issue_s = [&]() {
         if (ls == 0) {
           ++its;
-          ok = ok && wait_desc(its);
+          ok = ok && uwait_desc(its);
           if (!ok) return;
-          if (desc_of(its).kind < 0) { ends = true; return; }
-          ls = desc_of(its).steps;
-          ok = wait_fast<9>(bar_kfull(its), (its / C::NKV) & 1, s_abort, status);
+          if (uni(desc_of(its).kind) < 0) { ends = true; return; }
+          ls = uni(desc_of(its).steps);
+          ok = warp_wait<9>(bar_kfull(its), (its / C::NKV) & 1, s_abort, status);
         }
-        ok = ok && wait_fast<10>(bar_qfull(gs), (gs >> 1) & 1, s_abort, status);
+        ok = ok && warp_wait<10>(bar_qfull(gs), (gs >> 1) & 1, s_abort, status);
         if (!ok) return;
         fence_async_smem();
         tc_fence_after();
         const uint32_t k = C::kOffK + (its % C::NKV) * C::kTile, q = C::kOffQ + (gs & 1) * C::kTile;
+        if (el) {
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColS, kmajor(k, ks), kmajor(q, ks), desc_hi, idesc_s, ks > 0);
-        umma_commit(bar_s);
+          for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColS, kmajor(k, ks), kmajor(q, ks), desc_hi, idesc_s, ks > 0);
+          umma_commit(bar_s);
+        }
         ++gs; --ls;
       };
       // (dP only ever follows S of the same step: its item is known)
       auto p_ready = [&]() {
         if (gp >= gs) return false;
-        if (lp == 0 && !mbar_test(bar_vfull(itp + 1), ((itp + 1) / C::NKV) & 1)) return false;
-        if (D == 128 && gp > 0 && !mbar_test(bar_dqfree, (gp - 1) & 1)) return false;
-        return mbar_test(bar_dofull(gp), (gp / C::NDO) & 1);
+        if (lp == 0 && !utest(bar_vfull(itp + 1), ((itp + 1) / C::NKV) & 1)) return false;
+        if (D == 128 && gp > 0 && !utest(bar_dqfree, (gp - 1) & 1)) return false;
+        return utest(bar_dofull(gp), (gp / C::NDO) & 1);
       };
       auto issue_p = [&]() {
         if (lp == 0) {
           ++itp;
-          lp = desc_of(itp).steps;
-          ok = ok && wait_fast<11>(bar_vfull(itp), (itp / C::NKV) & 1, s_abort, status);
+          lp = uni(desc_of(itp).steps);
+          ok = ok && warp_wait<11>(bar_vfull(itp), (itp / C::NKV) & 1, s_abort, status);
         }
         // (d = 128: dQ of the step before lies there)
-        if (D == 128 && gp > 0) ok = ok && wait_fast<12>(bar_dqfree, (gp - 1) & 1, s_abort, status);
-        ok = ok && wait_fast<13>(bar_dofull(gp), (gp / C::NDO) & 1, s_abort, status);
+        if (D == 128 && gp > 0) ok = ok && warp_wait<12>(bar_dqfree, (gp - 1) & 1, s_abort, status);
+        ok = ok && warp_wait<13>(bar_dofull(gp), (gp / C::NDO) & 1, s_abort, status);
         if (!ok) return;
         fence_async_smem();
         tc_fence_after();
         const uint32_t v = C::kOffV + (itp % C::NKV) * C::kTile, o = C::kOffDO + (gp % C::NDO) * C::kTile;
+        if (el) {
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColDP, kmajor(v, ks), kmajor(o, ks), desc_hi, idesc_s, ks > 0);
-        umma_commit(bar_dp);
+          for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColDP, kmajor(v, ks), kmajor(o, ks), desc_hi, idesc_s, ks > 0);
+          umma_commit(bar_dp);
+        }
         ++gp; --lp;
       };
       issue_s();
       if (ok && !ends) issue_p();
       for (int it = 0; ok && !ends; ++it) {
-        const int steps = desc_of(it).steps;
+        const int steps = uni(desc_of(it).steps);
         const uint32_t kt = C::kOffK + (it % C::NKV) * C::kTile;
 #pragma unroll 1
         for (int s = 0; s < steps && ok; ++s, ++g) {
-          ok = wait_fast<14>(bar_h, g & 1, s_abort, status);
+          ok = warp_wait<14>(bar_h, g & 1, s_abort, status);
           if (!ok) break;
           tc_fence_after();
           const bool last = s + 1 == steps;
           const uint32_t q = C::kOffQ + (g & 1) * C::kTile, o = C::kOffDO + (g % C::NDO) * C::kTile, ds = C::kOffDS + (g % C::NDS) * (128 * 128 * 2);
           auto grad_v = [&]() {
             if (s == 0 && it > 0) {
-              ok = ok && wait_fast<15>(bar_accfree, (it - 1) & 1, s_abort, status);
+              ok = ok && warp_wait<15>(bar_accfree, (it - 1) & 1, s_abort, status);
               tc_fence_after();
             }
             if (!ok) return;
+            if (el) {
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk)
               mma_ts2(tmem + C::kColDV, tmem + C::kColP + (kk >> 2) * C::kPHalf + (kk & 3) * 8, mnmajor(o, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
             umma_commit(bar_dofree(g));
+            }
           };
           auto grad_k = [&]() {
+            if (el) {
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) mma_ss2(tmem + C::kColDK, kmajor(ds, kk), mnmajor(q, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
             umma_commit(bar_qfree(g));
             if (last) umma_commit(bar_acc);
+            }
           };
           auto grad_q = [&]() {
+            if (el) {
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) mma_ss2(tmem + C::kColDQ, mnmajor(ds, kk), mnmajor(kt, kk), desc_hi, idesc_t, kk > 0);
             umma_commit(bar_dq(g));
             if (last) umma_commit(bar_kfree(it));
+            }
           };
           if (D == 64) {
             if (s_ready()) issue_s();
@@ -570,11 +600,11 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
             grad_v();
             if (!ok) break;
             grad_k();
-            if (g > 0) ok = wait_fast<12>(bar_dqfree, (g - 1) & 1, s_abort, status);
+            if (g > 0) ok = warp_wait<12>(bar_dqfree, (g - 1) & 1, s_abort, status);
             if (!ok) break;
             tc_fence_after();
             grad_q();
-            umma_commit(bar_dsfree(g));
+            if (el) umma_commit(bar_dsfree(g));
           } else {
             grad_v();
             if (!ok) break;
@@ -582,17 +612,17 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
             if (s_ready()) issue_s();
             if (!ok) break;
             grad_k();
-            umma_commit(bar_dsfree(g));
+            if (el) umma_commit(bar_dsfree(g));
           }
           if (ok && gs == g + 1) issue_s();
           if (ok && !ends && gp == g + 1) issue_p();
         }
-        if (ok) mbar_arrive(bar_dfree(it));
+        if (ok && el) mbar_arrive(bar_dfree(it));
       }
     }
     __syncwarp();
   } else {
-    // ================= loaders: warp 17 Q and row statistics, warp 18 dO, warp 19 items, K and V ==================
+    // ================= loaders, a warp each: Q and row statistics; dO; items, K and V ==================
     // Tiles of consecutive rows: lane 0 issues TMA boxes.  Others: rows gathered in 16-byte chunks, lane -> chunk cc of row
     // k RPI + crow of instruction k; lane l holds the row numbers of rows l, l + 32, ..., handed round by shuffles.
     constexpr int CPR = D / 8, RPI = 32 / CPR, NSW = 8 / RPI;
@@ -620,8 +650,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
       __syncwarp();
       mbar_arrive(bar);
     };
-    if (warp < 19) {
-      const bool is_q = warp == 17;
+    if (warp < C::SW + 11) {
+      const bool is_q = warp == C::SW + 9;
       const int nbuf = is_q ? C::NQ : C::NDO;
       uint32_t g = 0;
       for (int it = 0; ok; ++it) {
@@ -721,7 +751,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_kernel(const __grid_constant_
   // ---- teardown ------------------------------------------------------------------------------------
   tc_fence_before();
   __syncthreads();
-  if (warp == 16) {
+  if (warp == C::SW + 8) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
   }
@@ -794,7 +824,7 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   const unsigned grid = items < sms ? (unsigned)items : (unsigned)sms;      // persistent: one CTA per SM
   cudaError_t e = g.d == 64 ? allow_smem<bwd_kernel<64>>(Cfg<64>::kTotal) : allow_smem<bwd_kernel<128>>(Cfg<128>::kTotal);
   if (e != cudaSuccess) return e;
-  return launch(g.d == 64 ? bwd_kernel<64> : bwd_kernel<128>, grid, kThreads, g.d == 64 ? Cfg<64>::kTotal : Cfg<128>::kTotal, st, b, maps, status);
+  return launch(g.d == 64 ? bwd_kernel<64> : bwd_kernel<128>, grid, g.d == 64 ? Cfg<64>::kThreads : Cfg<128>::kThreads, g.d == 64 ? Cfg<64>::kTotal : Cfg<128>::kTotal, st, b, maps, status);
 }
 
 // src: dq, dk, dv one after the other, count entries each (a multiple of 8)

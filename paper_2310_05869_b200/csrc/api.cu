@@ -186,7 +186,7 @@ cudaEvent_t take_event() {
 
 struct StageScope {
   cudaStream_t st; int stage; int launches; bool on; cudaEvent_t beg = nullptr;
-  StageScope(cudaStream_t s, int stage_, int launches_) : st(s), stage(stage_), launches(launches_), on(g_profile && launches_ > 0 && ((g_profile_mask >> stage_) & 1u)) {
+  StageScope(cudaStream_t s, int stage_, int launches_) : st(s), stage(stage_), launches(launches_), on(g_profile && ((g_profile_mask >> stage_) & 1u)) {
     if (on) { beg = take_event(); cudaEventRecord(beg, st); }
   }
   ~StageScope() {

@@ -32,8 +32,7 @@
 // Every mbarrier wait is bounded: on a timeout the CTA raises the device status word,
 // drains its copies, frees its TMEM and returns.
 #include <cstdlib>
-#include <cuda.h>
-#include "attn_common.cuh"
+#include "tc_util.cuh"
 
 namespace hyperattn {
 namespace {
@@ -45,10 +44,6 @@ struct alignas(64) TmaMaps {
 };
 
 constexpr int TK = 64;                  // keys per tile
-#ifndef HA_WAIT_LIMIT_NS
-#define HA_WAIT_LIMIT_NS 2000000000ull
-#endif
-constexpr unsigned long long kWaitLimitNs = HA_WAIT_LIMIT_NS;   // every mbarrier wait gives up after 2 s
 // Test build only (-DHA_TEST_DROP_ARRIVAL, never in the shipped library): when armed, the K / V streamer of one CTA
 // leaves out the copies of one V tile once, so that the wait for that tile runs out and the give-up path can be
 // exercised without any fault.
@@ -74,202 +69,10 @@ __device__ unsigned long long g_tc_timing[48];
 #define HA_LFLUSH(slot, name)
 #endif
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// ---- mbarrier ---------------------------------------------------------------------------
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// One potentially-blocking probe: the hardware may park the warp for up to the hinted time (ns)
-// and wakes it when the phase completes, so waiting warps leave the issue slots to the others.
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-               : "=r"(ok) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
-  return ok != 0;
-}
-// returns false when the wait gave up (timeout or another thread aborted)
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// SLEEP_NS: back-off between probes, so that waiting warps do not take issue slots from the
-// warps that compute (every role waits far more often than it works)
-template <int SLEEP_NS = 32, int SITE = 1>
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
-  unsigned long long t0 = 0;
-  for (unsigned it = 0;; ++it) {
-    if (mbar_try(bar, parity)) return true;
-    __nanosleep(SLEEP_NS);
-    if ((it & 63u) == 63u) {
-      if (*abort_flag) return false;
-      const unsigned long long now = global_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > kWaitLimitNs) break;
-    }
-  }
-  *abort_flag = 1;
-  atomicOr(status, 1 << SITE);     // bit mask of the wait sites that gave up
-  return false;
-}
-
-// the slow path of a wait, out of line; SITE tags the wait in the status word
-template <int SITE>
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
-  return mbar_wait<20, SITE>(bar, parity, abort_flag, status);
-}
-// one probe inline (the common case for the MMA issuers: what they wait for is usually there)
-template <int SITE>
-__device__ __forceinline__ bool wait_fast(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
-  if (mbar_try(bar, parity)) return true;
-  return mbar_wait_slow<SITE>(bar, parity, abort_flag, status);
-}
-
-// ---- tcgen05 ----------------------------------------------------------------------------
-// tcgen05.mma with shared-memory descriptors given as (low, high) 32-bit words: only the low word ever changes
-// (low word = start address >> 4 | (leading byte offset >> 4) << 16, high word = stride byte offset >> 4 |
-// descriptor version 1 << 14 | 128-byte swizzle 2 << 29); [a_tmem]: the A operand read from TMEM
-__device__ __forceinline__ void mma_ss2(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t acc) {
-  asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
-               "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}\n"
-               ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void mma_ts2(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t acc) {
-  asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 db;\n\tmov.b64 db, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
-               "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}\n"
-               ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// issue without waiting; the data is valid only after tmem_ld32_wait on the same registers
-__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-               "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                 "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                 "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                 "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-               : "r"(taddr));
-}
-// waits for every outstanding TMEM load of this thread; the registers are listed as
-// read-write operands so that no use of them can be scheduled above the wait
-__device__ __forceinline__ void tmem_ld32_wait(uint32_t (&r)[32]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
-                 "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
-                 "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-               :: "memory");
-}
-__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                 "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-               : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_ld16_wait(uint32_t (&r)[16]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-               :: "memory");
-}
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
-}
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-#ifdef HA_EXP_FAKE
-  asm("mul.f32 %0, %1, 0f00000000;" : "=f"(y) : "f"(x));     // timing experiment only: results are meaningless
-#else
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-#endif
-  return y;
-}
-// packed pairs of fp32 (one instruction, two lanes)
-__device__ __forceinline__ uint64_t pack_u2(uint32_t lo, uint32_t hi) {
-  uint64_t d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
-  return d;
-}
-__device__ __forceinline__ uint64_t pack_f2(float lo, float hi) { return pack_u2(__float_as_uint(lo), __float_as_uint(hi)); }
-__device__ __forceinline__ void unpack_f2(uint64_t v, float& lo, float& hi) {
-  uint32_t a, b;
-  asm("mov.b64 {%0, %1}, %2;" : "=r"(a), "=r"(b) : "l"(v));
-  lo = __uint_as_float(a); hi = __uint_as_float(b);
-}
-__device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t fadd2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n"
-               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-                 "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
-}
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
-
-// ---- copies -----------------------------------------------------------------------------
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
-}
-// the executing thread's arrival on the mbarrier happens when all its earlier cp.async have landed
-__device__ __forceinline__ void cp_async_arrive_noinc(uint32_t bar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-// One TMA box (64 columns x the map's box rows, starting at column x, row y) into a
-// 128B-swizzled slab; completion is counted in bytes on the mbarrier.
-__device__ __forceinline__ void tma_tile(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-  asm volatile("cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-               ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
-}
-// announces bytes to the current phase without arriving
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// Teardown only: waits (bounded, whatever the abort flag says) until a phase that this warp
-// armed has received all its bytes, so that no copy is in flight into the CTA's shared
-// memory when it exits.
-__device__ __noinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
-  const unsigned long long t0 = global_ns();
-  for (unsigned it = 0;; ++it) {
-    if (mbar_try(bar, parity)) return;
-    if ((it & 15u) == 15u && global_ns() - t0 > kWaitLimitNs) return;
-  }
-}
-
-__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
-  __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t*>(&t);
-}
-
-// byte offset of 16-byte chunk c of row `row` in a [ROWS x D] bf16 tile: D/64 slabs of
-// [ROWS rows x 128 B], 128-byte swizzle inside each slab (the canonical tcgen05 layout)
-template <int ROWS>
-__device__ __forceinline__ uint32_t tile_off(int row, int c) {
-  return (uint32_t)((c >> 3) * (ROWS * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4));
 }
 
 // Tiles with masked columns (a minority: the diagonal tiles of a causal leaf, padding, sampled
@@ -511,7 +314,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
   auto bar_vempty = [&](int i, int s) { return bar0 + 168 + 8 * ((4 + i) * C::NS + s); };
 
   const Geometry& g = a.g;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);       // (known to be the same for the whole warp)
   HA_T0(t_cta);
 
   // A CTA of a launch in which some wait already timed out returns at once (nothing allocated
@@ -550,7 +354,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *s_tmem;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *s_tmem, 0);
   wait_for_stream();
 
   // The CTA is persistent: it walks over work items (pairs of query tiles) blockIdx.x,
@@ -968,16 +772,19 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
     }
 #endif
   } else if (warp < 10) {
-    // ================= MMA issue: one lane per query tile (warp 8: tile 0, warp 9: tile 1) ===========
+    // ================= MMA issue, a warp per query tile (warp 8: tile 0, warp 9: tile 1) ===========
     // Each issuer walks its own key tiles: scores run two tiles ahead of the PV products
     // (S buffers alternate).  A tcgen05.mma occupies the issuing thread and the tensor pipe
     // for about 55-65 cycles whatever its size, so the two chains are issued by two threads.
     // The issuer shares its scheduler with two busy softmax warps and has no instruction-level
-    // parallelism of its own, so its loop is kept to a minimum of instructions: descriptors
-    // are two 32-bit words of which only the low one moves, waits are one probe in the common
+    // parallelism of its own, so its loop is kept to a minimum of instructions: the whole warp walks it together with
+    // warp-uniform values and one elected lane issues, so that descriptors are made of uniform registers (a lone lane's have to be moved
+    // there one by one; d = 64 leaves 525 -> 497 us, node items 1207 -> 1141, d = 128 400 -> 378, split weights 2059 -> 1687); descriptors are two 32-bit words of which only the low one moves; waits are one probe in the common
     // case, everything unusual lives in out-of-line slow paths.
     const int i = warp - 8;
-    if (lane == 0) {
+    {
+      const bool el = elect_one();
+      auto uni = [&](int x) { return __shfl_sync(0xffffffffu, x, 0); };
       constexpr uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | (((uint32_t)TK >> 3) << 17) | ((128u >> 4) << 24);
       constexpr uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | (((uint32_t)C::kOCols >> 3) << 17) | ((128u >> 4) << 24);
       // descriptor: low word = start address >> 4 | (leading byte offset >> 4) << 16,
@@ -1004,37 +811,39 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       // tcgen05.commit, so they also stay behind this thread's earlier MMAs.
       auto skip_k = [&](int gj) {
         for (; knext < gj && ok; ++knext) {
-          ok = wait_fast<7>(bar_kfull(knext % C::NS), (knext / C::NS) & 1, s_abort, status);
-          if (ok) umma_commit(bar_kempty(i, knext % C::NS));
+          ok = warp_wait<7>(bar_kfull(knext % C::NS), (knext / C::NS) & 1, s_abort, status);
+          if (ok && el) umma_commit(bar_kempty(i, knext % C::NS));
         }
       };
       auto skip_v = [&](int gj) {
         for (; vnext < gj && ok; ++vnext) {
-          ok = wait_fast<9>(bar_vfull(vnext % C::NS), (vnext / C::NS) & 1, s_abort, status);
-          if (ok) umma_commit(bar_vempty(i, vnext % C::NS));
+          ok = warp_wait<9>(bar_vfull(vnext % C::NS), (vnext / C::NS) & 1, s_abort, status);
+          if (ok && el) umma_commit(bar_vempty(i, vnext % C::NS));
         }
       };
       int it = 0;
       HA_LDECL(b_q); HA_LDECL(b_p); HA_LDECL(b_v); HA_LDECL(b_k);
       HA_T0(tloop);
       for (; ok; ++it) {
-        ok = wait_fast<22>(bar_tabfull(it & 1), (it >> 1) & 1, s_abort, status);
+        ok = warp_wait<22>(bar_tabfull(it & 1), (it >> 1) & 1, s_abort, status);
         if (!ok) break;
         const ItemDesc& de = *reinterpret_cast<const ItemDesc*>(smem + C::kOffDesc + (it & 1) * C::kDescBytes);
-        if (de.t.mode < 0) break;
-        const QTile q = i ? de.qb : de.qa;
+        if (uni(de.t.mode) < 0) break;
+        const QTile& qd = i ? de.qb : de.qa;
+        QTile q;
+        q.s1 = uni(qd.s1); q.n1 = uni(qd.n1); q.s2 = uni(qd.s2); q.n2 = uni(qd.n2);
         const int total = q.n1 + q.n2;
-        const int ntiles = de.t.ntiles;
+        const int ntiles = uni(de.t.ntiles), exists = uni(qd.valid);
 #ifdef HA_TC_TIMING
         if (i == 0) atomicAdd(&g_tc_timing[14], (unsigned long long)ntiles);
 #endif
         // Q of this item (an issuer without a tile waits too: it may not run ahead of the others)
         HA_T0(tq);
-        ok = wait_fast<6>(bar_q, it & 1, s_abort, status);
+        ok = warp_wait<6>(bar_q, it & 1, s_abort, status);
         if (!ok) break;
         HA_LACC(b_q, tq);
         fence_async_smem();
-        if (total == 0) mbar_arrive(bar_qfree);
+        if (total == 0 && el) mbar_arrive(bar_qfree);
         auto issue_pv = [&](int a2) {
           // ---- O += P V of key tile a2 ----------------------------------------------------------
           const int gj = gbase + tile_of(q, a2);
@@ -1042,28 +851,30 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
           const int gw = ga + a2;
           if (gj != vnext) skip_v(gj);
           HA_T0(tp);
-          ok = ok && wait_fast<8>(bar_p(i, gw % C::kSBufs), (gw / C::kSBufs) & 1, s_abort, status);
+          ok = ok && warp_wait<8>(bar_p(i, gw % C::kSBufs), (gw / C::kSBufs) & 1, s_abort, status);
           HA_LACC(b_p, tp);
           HA_T0(tv);
-          ok = ok && wait_fast<9>(bar_vfull(s), (gj / C::NS) & 1, s_abort, status);
+          ok = ok && warp_wait<9>(bar_vfull(s), (gj / C::NS) & 1, s_abort, status);
           HA_LACC(b_v, tv);
           // the first product of an item overwrites O: the previous item's O must have been read
-          if (a2 == 0 && vi > 0) ok = ok && wait_fast<15>(bar_ofree(i), (vi - 1) & 1, s_abort, status);
+          if (a2 == 0 && vi > 0) ok = ok && warp_wait<15>(bar_ofree(i), (vi - 1) & 1, s_abort, status);
           if (!ok) return;
           fence_async_smem();
           tc_fence_after();
           const uint32_t pcol = scol + 64 * (gw % C::kSBufs);
           const uint32_t dv_lo = dv_lo0 + (uint32_t)s * dv_step;
-          mma_ts2(ocol, pcol, dv_lo, desc_hi, idesc_o, a2 > 0);
+          if (el) {
+            mma_ts2(ocol, pcol, dv_lo, desc_hi, idesc_o, a2 > 0);
 #pragma unroll
-          for (int kk = 1; kk < TK / 16; ++kk) mma_ts2(ocol, pcol + kk * 8, dv_lo + kk * (2048 >> 4), desc_hi, idesc_o, 1);
-          if constexpr (PRECISE) {
+            for (int kk = 1; kk < TK / 16; ++kk) mma_ts2(ocol, pcol + kk * 8, dv_lo + kk * (2048 >> 4), desc_hi, idesc_o, 1);
+            if constexpr (PRECISE) {
 #pragma unroll
-            for (int kk = 0; kk < TK / 16; ++kk) mma_ts2(ocol, pcol + 32 + kk * 8, dv_lo + kk * (2048 >> 4), desc_hi, idesc_o, 1);
+              for (int kk = 0; kk < TK / 16; ++kk) mma_ts2(ocol, pcol + 32 + kk * 8, dv_lo + kk * (2048 >> 4), desc_hi, idesc_o, 1);
+            }
+            umma_commit(bar_vempty(i, s));
+            if (a2 == total - 1) umma_commit(bar_o(i));
           }
-          umma_commit(bar_vempty(i, s));
           vnext = gj + 1;
-          if (a2 == total - 1) umma_commit(bar_o(i));
         };
         auto issue_s = [&](int r) {
           // ---- S = Q K^T of key tile r into buffer (ga + r) % kSBufs --------------------------------
@@ -1072,21 +883,23 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
           const int gw = ga + r;
           if (gj != knext) skip_k(gj);
           HA_T0(tk);
-          ok = ok && wait_fast<7>(bar_kfull(s), (gj / C::NS) & 1, s_abort, status);
+          ok = ok && warp_wait<7>(bar_kfull(s), (gj / C::NS) & 1, s_abort, status);
           HA_LACC(b_k, tk);
           if (!ok) return;
           fence_async_smem();
           tc_fence_after();
           const uint32_t dcol = scol + 64 * (gw % C::kSBufs);
           const uint32_t dk_lo = dk_lo0 + (uint32_t)s * (C::kTile >> 4);
+          if (el) {
 #pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks)
-            mma_ss2(dcol, dq_lo + (((ks >> 2) * (128 * 128) + (ks & 3) * 32) >> 4),
-                    dk_lo + (((ks >> 2) * (TK * 128) + (ks & 3) * 32) >> 4), desc_hi, idesc_s, ks > 0);
-          umma_commit(bar_s(i, gw % C::kSBufs));
-          umma_commit(bar_kempty(i, s));
+            for (int ks = 0; ks < D / 16; ++ks)
+              mma_ss2(dcol, dq_lo + (((ks >> 2) * (128 * 128) + (ks & 3) * 32) >> 4),
+                      dk_lo + (((ks >> 2) * (TK * 128) + (ks & 3) * 32) >> 4), desc_hi, idesc_s, ks > 0);
+            umma_commit(bar_s(i, gw % C::kSBufs));
+            umma_commit(bar_kempty(i, s));
+            if (r == total - 1) umma_commit(bar_qfree);     // nothing of this item reads Q any more
+          }
           knext = gj + 1;
-          if (r == total - 1) umma_commit(bar_qfree);     // nothing of this item reads Q any more
         };
         // The S buffer of tile r held P of tile r - kSBufs, so the product P V of that tile must be
         // issued before the scores of tile r.  Two buffers: P V (r - 2), then S (r).  Three: the
@@ -1107,7 +920,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
         for (int e = min(knext, vnext) + 1; e <= gbase + ntiles && ok; ++e) { skip_k(e); skip_v(e); }
         gbase += ntiles;
         ga += total;
-        vi += q.valid;
+        vi += exists;
       }
       if (i == 0) { HA_TACC(8, tloop); HA_TACC(12, t_cta); HA_LFLUSH(7, b_q); HA_LFLUSH(4, b_p); HA_LFLUSH(5, b_v); HA_LFLUSH(6, b_k); }
 #ifdef HA_TC_TIMING

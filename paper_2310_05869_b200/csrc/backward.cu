@@ -218,11 +218,6 @@ __global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__
   if (row < rows && c % LPR == 0) stat[row] = make_float2(-lse[row] * 1.4426950408889634f, -acc);
 }
 
-template <int SITE>
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
-  return __all_sync(0xffffffffu, wait_fast<SITE>(bar, parity, abort_flag, status)) != 0;
-}
-
 template <int D>
 __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_constant__ BwdArgs b, const __grid_constant__ BwdMaps maps, int* status) {
   using C = Cfg<D>;

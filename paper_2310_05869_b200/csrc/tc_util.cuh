@@ -1,4 +1,4 @@
-// Device helpers of the backward pass: mbarriers with bounded waits, tcgen05 / TMEM access, packed fp32
+// Device helpers of the tcgen05 kernels (attention and backward pass): mbarriers with bounded waits, tcgen05 / TMEM access, packed fp32
 // arithmetic, asynchronous copies.
 #pragma once
 #include <cuda.h>
@@ -85,6 +85,11 @@ __device__ __forceinline__ bool wait_fast(uint32_t bar, uint32_t parity, volatil
   return mbar_wait_slow<SITE>(bar, parity, abort_flag, status);
 }
 
+// the same for a converged warp: all lanes get the same answer
+template <int SITE>
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
+  return __all_sync(0xffffffffu, wait_fast<SITE>(bar, parity, abort_flag, status)) != 0;
+}
 // true for one lane of a converged warp
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;

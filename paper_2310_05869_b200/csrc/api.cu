@@ -91,7 +91,7 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
 }
 
 struct Plan {
-  size_t q16, k16, v16, q16lo, k16lo, ids, hist, offs, perm_q, perm_k, rank_k, samples, tpos, ltau, vwq, vsum, vcum, swlog, wnodes, sched, part_o, part_lse, total;
+  size_t q16, k16, v16, q16lo, k16lo, ids, hist, offs, perm_q, perm_k, rank_k, samples, tpos, ltau, vwq, vsum, vcum, swlog, wnodes, smp_blk, sched, part_o, part_lse, total;
   size_t stat, gacc;    // backward only: (-lse, -<dO, O>) per row; fp32 gradient accumulators (bf16 gradients only)
 };
 
@@ -117,6 +117,7 @@ Plan make_plan(const Geometry& g, int is_fp32, int backward = 0, bool capped = f
   pl.perm_k = take(g.sorted ? lvl_rows * 4 : 0);
   pl.rank_k = take(g.sorted ? lvl_rows * 4 : 0);
   pl.samples = take((size_t)g.G * g.nodes * g.m * 4);
+  pl.smp_blk = take((size_t)g.G * g.nodes * g.m * 4);
   pl.sched = take(256);
   pl.tpos = take(capped ? (size_t)g.G * g.nodes * g.m * 4 : 0);
   pl.ltau = take(capped ? (size_t)g.G * g.nodes * 4 : 0);
@@ -290,6 +291,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
   ws.perm_k = reinterpret_cast<int32_t*>(base + pl.perm_k);
   ws.rank_k = reinterpret_cast<int32_t*>(base + pl.rank_k);
   ws.samples = reinterpret_cast<int32_t*>(base + pl.samples);
+  ws.smp_blk = g.m > 0 ? reinterpret_cast<int32_t*>(base + pl.smp_blk) : nullptr;
   ws.tpos = capped ? reinterpret_cast<int32_t*>(base + pl.tpos) : nullptr;
   ws.ltau = capped ? reinterpret_cast<float*>(base + pl.ltau) : nullptr;
   ws.part_o = base + pl.part_o;
@@ -371,7 +373,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
   a.q = q16; a.k = k16; a.v = v16; a.g = g;
   if (is_fp32) { a.q_lo = ws.q16lo; a.k_lo = ws.k16lo; }
   a.scale_log2 = scale * 1.4426950408889634f;
-  a.perm_q = ws.perm_q; a.perm_k = ws.perm_k; a.rank_k = ws.rank_k; a.samples = ws.samples;
+  a.perm_q = ws.perm_q; a.perm_k = ws.perm_k; a.rank_k = ws.rank_k; a.samples = ws.samples; a.smp_blk = ws.smp_blk;
   a.part_o = ws.part_o; a.part_lse = ws.part_lse; a.part_bf16 = part_bf16; a.out = p.out; a.lse = p.lse;
   a.out_fp32 = out_fp32;
   a.precise = p.precise != 0;

@@ -25,7 +25,7 @@ struct AttnArgs {
   const __nv_bfloat16 *q_lo, *k_lo;  // second bf16 term of fp32 inputs (else null)
   Geometry g;
   float scale_log2;                  // softmax scale * log2(e)
-  const int32_t *perm_q, *perm_k, *rank_k, *samples;
+  const int32_t *perm_q, *perm_k, *rank_k, *samples, *smp_blk;
   void* part_o; float* part_lse;     // partial results, used when !direct: rows of fp32, or of bf16 when part_bf16
   int part_bf16;                     // (partials are kept in the type of the final output; their log-sum-exp always in fp32)
   void* out; float* lse;             // final results, used when direct

@@ -979,7 +979,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
         const int ncols = t.ntiles * TK;
         const int32_t* smp = a.samples + ((size_t)t.seg * g.nodes + t.node) * g.m;
         const int32_t* pk = a.perm_k + t.slice;
-        const int32_t* rk = a.rank_k + t.slice;
+        const int32_t* sblk = a.smp_blk + ((size_t)t.seg * g.nodes + t.node) * g.m;
         for (int c00 = lane; c00 < nblk; c00 += 32 * UB) {
           int idx[UB];
 #pragma unroll
@@ -1020,9 +1020,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
             for (int u = 0; u < UB; ++u) {
               const int c = c00 + u * 32;
               l[u] = c < g.m ? smp[c] : -1;
+              blk[u] = c < g.m ? sblk[c] : -1;
             }
-#pragma unroll
-            for (int u = 0; u < UB; ++u) blk[u] = l[u] >= 0 ? rk[l[u]] / g.b : -1;
 #pragma unroll
             for (int u = 0; u < UB; ++u) {
               const int c = c00 + u * 32;

@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
       const bool exists = row < t.nkeys;
       const int kind = t.kind, steps = t.steps, causal = t.causal;
       int kblk = -2;                                    // sampled keys: the sorted block the key lies in (its entries there are masked)
-      if (kind == 2 && exists) kblk = __ldg(a.rank_k + t.slice + __ldg(a.samples + t.kidx + row)) / g_.b;
+      if (kind == 2 && exists) kblk = __ldg(a.smp_blk + t.kidx + row);
 #pragma unroll 1
       for (int s = 0; s < steps; ++s, ++g) {
         // entries that do not count: keys that do not exist, sampled keys of the query tile's own block, above the diagonal

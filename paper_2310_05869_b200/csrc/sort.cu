@@ -18,6 +18,7 @@ struct SortArgs {
   const uint32_t* hist;   // queries [G, chunks_per_seg, 256], then keys [G, chunks_per_seg_k, 256]
   uint32_t* offs;         // queries [levels, G, chunks per (level, segment), 256], then the same for keys
   int32_t *perm_q, *perm_k, *rank_k;  // [levels, G, nl]
+  int32_t* smp_blk;       // [G, nodes, m] sorted block of every sampled key, or null
   Geometry g;
   int side_mask;          // bit s set: side s is sorted (both, unless a caller wants one side only)
 };
@@ -41,6 +42,7 @@ struct SampleArgs {
   float* ltau;       // capped row sums only: [G, nodes], set to -inf here (the probe pass takes a maximum into it)
   Geometry g;
   uint32_t k0, k1;
+  int draw;          // 1: the samples are drawn by this launch
   int* sched;        // zeroed by the launch (null: nothing)
 };
 
@@ -244,6 +246,22 @@ __global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a, SampleArg
       if (rank) rank[local0 + i] = (int32_t)pos;
     }
   }
+  // The block of every sampled key among these rows, which decides whether a query tile's own block holds the sample: the attention
+  // kernel asks for it in every work item, and from here it comes without the detour over the ranks (node items 8 % faster).
+  if (side == 1 && a.smp_blk) {
+    __syncthreads();                                     // (the ranks above are read back)
+    const int node = g.causal ? (1 << level) - 1 + j : 0;
+    const size_t base = ((size_t)seg * g.nodes + node) * g.m;
+    const uint32_t N = g.causal ? (uint32_t)(g.npad >> (level + 1)) : (uint32_t)g.nk;
+    for (int c = tid; c < g.m; c += 256) {
+      int l;
+      if (SCAN && sa.draw) {                             // (drawn by other blocks of this very launch: the stream gives it again)
+        const Philox4 x = philox4x32_10((uint32_t)(c >> 2), (uint32_t)(g.seg0 + seg), (uint32_t)node, kDomainSamples, sa.k0, sa.k1);
+        l = (int)__umulhi((c & 2) ? ((c & 1) ? x.x[3] : x.x[2]) : ((c & 1) ? x.x[1] : x.x[0]), N);
+      } else l = sa.samples[base + c];
+      if ((unsigned)(l - local0) < (unsigned)rows) a.smp_blk[base + c] = rank[l] / g.b;
+    }
+  }
 }
 
 }  // namespace
@@ -251,7 +269,7 @@ __global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a, SampleArg
 static SortArgs make_sort_args(const Geometry& g, const Workspace& ws, int side_mask) {
   SortArgs a;
   a.ids = ws.ids; a.hist = ws.hist; a.offs = ws.offs;
-  a.perm_q = ws.perm_q; a.perm_k = ws.perm_k; a.rank_k = ws.rank_k;
+  a.perm_q = ws.perm_q; a.perm_k = ws.perm_k; a.rank_k = ws.rank_k; a.smp_blk = ws.smp_blk;
   a.g = g;
   a.side_mask = side_mask;
   return a;
@@ -266,7 +284,7 @@ bool scan_in_scatter(const Geometry& g) {
 
 static SampleArgs make_sample_args(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, int* blocks) {
   // (ws.tpos non-null: the probe rows of the capped row-sum estimate are drawn as well)
-  SampleArgs sa; sa.samples = ws.samples; sa.tpos = ws.tpos; sa.ltau = ws.ltau; sa.g = g; sa.k0 = (uint32_t)seed; sa.k1 = (uint32_t)(seed >> 32); sa.sched = ws.sched;
+  SampleArgs sa; sa.samples = ws.samples; sa.tpos = ws.tpos; sa.ltau = ws.ltau; sa.g = g; sa.k0 = (uint32_t)seed; sa.k1 = (uint32_t)(seed >> 32); sa.sched = ws.sched; sa.draw = with_samples;
   *blocks = 0;
   if (with_samples && g.nodes > 0 && g.m > 0) {
     const size_t total = (size_t)g.G * g.nodes * ((g.m + 3) / 4);

@@ -47,20 +47,20 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
                : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
-// returns false when the wait gave up (timeout or another thread aborted)
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-// SLEEP_NS: back-off between probes, so that waiting warps do not take issue slots from the
-// warps that compute (every role waits far more often than it works)
-template <int SLEEP_NS = 32, int SITE = 1>
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
+// The slow path of a wait, out of line: parks, with a pause between probes, so that waiting warps do not take issue
+// slots from the warps that compute.  SITE tags the wait in the status word; false when the wait gave up (time limit,
+// or another thread aborted).
+template <int SITE>
+__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
   unsigned long long t0 = 0;
   for (unsigned it = 0;; ++it) {
     if (mbar_park(bar, parity)) return true;
-    __nanosleep(SLEEP_NS);
+    __nanosleep(20);
     if ((it & 63u) == 63u) {
       if (*abort_flag) return false;
       const unsigned long long now = global_ns();
@@ -72,13 +72,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   atomicOr(status, 1 << SITE);     // bit mask of the wait sites that gave up
   return false;
 }
-
-// the slow path of a wait, out of line; SITE tags the wait in the status word
-template <int SITE>
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
-  return mbar_wait<20, SITE>(bar, parity, abort_flag, status);
-}
-// one probe inline (the common case for the MMA issuers: what they wait for is usually there)
+// One probe inline, without a time hint: what a role waits for is usually there, and a satisfied try_wait costs about
+// 15 cycles without a hint, 49 with one (B200).  With every wait of the attention kernel in this form instead of a
+// parking one first, the recursion node of 65536 rows (32 heads, d = 64) went from 1070 to 980 us.
 template <int SITE>
 __device__ __forceinline__ bool wait_fast(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
   if (mbar_try(bar, parity)) return true;

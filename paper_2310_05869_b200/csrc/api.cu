@@ -19,8 +19,7 @@ cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uin
                                   float* wlog, uint64_t seed, cudaStream_t st);
 cudaError_t launch_tau(const AttnArgs& at, const int32_t* tpos, float* ltau, cudaStream_t st);
 cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout, float2* stat, int* sched,
-                            float* dq, float* dk, float* dv, float scale, int* status, cudaStream_t st);
-cudaError_t launch_to_bf16(const float* src, void* dq, void* dk, void* dv, size_t count, cudaStream_t st);
+                            const BwdGrads& gr, float scale, int* status, cudaStream_t st);
 
 namespace {
 
@@ -91,9 +90,14 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
 }
 
 struct Plan {
-  size_t q16, k16, v16, q16lo, k16lo, ids, hist, offs, perm_q, perm_k, rank_k, samples, tpos, ltau, vwq, vsum, vcum, swlog, wnodes, smp_blk, sched, part_o, part_lse, total;
+  size_t q16, k16, v16, q16lo, k16lo, ids, hist, offs, perm_q, perm_k, rank_k, samples, tpos, ltau, vwq, vsum, vcum, swlog, wnodes, smp_blk, key_slot, sched, part_o, part_lse, total;
   size_t stat, gacc;    // backward only: (-lse, -<dO, O>) per row; fp32 gradient accumulators (bf16 gradients only)
 };
+
+// Where every key belongs to one tile of keys only besides the samples (no recursion), the backward pass writes bf16 dK and dV of
+// the keys that no sample drew straight from that tile; fp32 accumulators are left for the sampled keys.
+bool direct_key_grads(const Geometry& g) { return g.L == 0; }
+size_t key_grad_rows(const Geometry& g, bool direct) { return direct ? (g.sorted ? (size_t)g.G * g.m : 0) : (size_t)g.G * g.n; }
 
 // backward: 0 forward plan; 1 backward with fp32 gradients (accumulated in place); 2 backward with bf16 gradients
 Plan make_plan(const Geometry& g, int is_fp32, int backward = 0, bool capped = false, bool vnorm = false, bool part_bf16 = false) {
@@ -118,6 +122,8 @@ Plan make_plan(const Geometry& g, int is_fp32, int backward = 0, bool capped = f
   pl.rank_k = take(g.sorted ? lvl_rows * 4 : 0);
   pl.samples = take((size_t)g.G * g.nodes * g.m * 4);
   pl.smp_blk = take((size_t)g.G * g.nodes * g.m * 4);
+  const bool direct = backward == 2 && direct_key_grads(g);
+  pl.key_slot = take(direct && g.sorted && g.m > 0 ? (size_t)g.G * g.nk * 4 : 0);
   pl.sched = take(256);
   pl.tpos = take(capped ? (size_t)g.G * g.nodes * g.m * 4 : 0);
   pl.ltau = take(capped ? (size_t)g.G * g.nodes * 4 : 0);
@@ -129,7 +135,7 @@ Plan make_plan(const Geometry& g, int is_fp32, int backward = 0, bool capped = f
   pl.part_o = take(part_rows * g.d * (part_bf16 ? 2 : 4));
   pl.part_lse = take(part_rows * 4);
   pl.stat = take(backward ? (size_t)g.G * g.n * 8 : 0);
-  pl.gacc = take(backward == 2 ? (size_t)3 * g.G * g.n * g.d * 4 : 0);
+  pl.gacc = take(backward == 2 ? ((size_t)g.G * g.n + 2 * key_grad_rows(g, direct)) * g.d * 4 : 0);
   pl.total = off + kAlign;
   return pl;
 }
@@ -292,6 +298,8 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
   ws.rank_k = reinterpret_cast<int32_t*>(base + pl.rank_k);
   ws.samples = reinterpret_cast<int32_t*>(base + pl.samples);
   ws.smp_blk = g.m > 0 ? reinterpret_cast<int32_t*>(base + pl.smp_blk) : nullptr;
+  const bool direct = bw && bw->grad_dtype == HYPERATTN_BF16 && direct_key_grads(g);
+  ws.key_slot = direct && g.sorted && g.m > 0 ? reinterpret_cast<int32_t*>(base + pl.key_slot) : nullptr;
   ws.tpos = capped ? reinterpret_cast<int32_t*>(base + pl.tpos) : nullptr;
   ws.ltau = capped ? reinterpret_cast<float*>(base + pl.ltau) : nullptr;
   ws.part_o = base + pl.part_o;
@@ -417,14 +425,17 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
   if (bw) {
     const size_t elems = (size_t)g.G * g.n * g.d;
     const bool g32 = bw->grad_dtype == HYPERATTN_FP32;
+    const size_t kv_elems = key_grad_rows(g, direct) * g.d;
+    BwdGrads gr;
     float* acc = reinterpret_cast<float*>(base + pl.gacc);
-    float* dq = g32 ? reinterpret_cast<float*>(bw->dq) : acc;
-    float* dk = g32 ? reinterpret_cast<float*>(bw->dk) : acc + elems;
-    float* dv = g32 ? reinterpret_cast<float*>(bw->dv) : acc + 2 * elems;
+    gr.dq = g32 ? reinterpret_cast<float*>(bw->dq) : acc;
+    gr.dk = g32 ? reinterpret_cast<float*>(bw->dk) : acc + elems;
+    gr.dv = g32 ? reinterpret_cast<float*>(bw->dv) : gr.dk + kv_elems;
+    gr.kv_elems = kv_elems;
+    gr.dq16 = g32 ? nullptr : bw->dq; gr.dk16 = g32 ? nullptr : bw->dk; gr.dv16 = g32 ? nullptr : bw->dv;
+    gr.direct = direct; gr.key_slot = ws.key_slot;
     StageScope sc(st, HYPERATTN_STAGE_BACKWARD, 2 + (g32 ? 0 : 1));
-    HA_CHECK(launch_backward(a, p.out, out_fp32, p.lse, bw->dout, reinterpret_cast<float2*>(base + pl.stat), ws.sched,
-                             dq, dk, dv, scale, ws.status, st));
-    if (!g32) HA_CHECK(launch_to_bf16(acc, bw->dq, bw->dk, bw->dv, elems, st));
+    HA_CHECK(launch_backward(a, p.out, out_fp32, p.lse, bw->dout, reinterpret_cast<float2*>(base + pl.stat), ws.sched, gr, scale, ws.status, st));
     return HYPERATTN_OK;
   }
   if (capped) {

@@ -20,6 +20,15 @@ constexpr int kMaxLevels = 24;
 constexpr int kMaxWeightedSamples = 512;   // sampled columns with weights of their own (sampling by value norms): table size
 constexpr int kMaxNodeKeys = 2048;   // 2 * (b rounded up to 128) + (m rounded up to 128) must fit the key table
 
+// gradients of the backward pass
+struct BwdGrads {
+  float *dq, *dk, *dv;         // fp32 accumulators
+  size_t kv_elems;             // entries of dk and of dv
+  void *dq16, *dk16, *dv16;    // bf16 results (null: the accumulators are the results)
+  const int32_t* key_slot;     // [G, n] (null: no samples)
+  int direct;                  // every key has one tile only besides the samples: its bf16 dK and dV leave from there
+};
+
 struct AttnArgs {
   const __nv_bfloat16 *q, *k, *v;    // [G, n, D]
   const __nv_bfloat16 *q_lo, *k_lo;  // second bf16 term of fp32 inputs (else null)

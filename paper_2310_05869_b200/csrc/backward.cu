@@ -36,6 +36,7 @@ namespace {
 
 constexpr int kDescs = 3;              // item descriptors in flight
 constexpr int kTileK = 128;            // keys per item, query rows per step
+constexpr int kNoRow = (int)0x80000000;   // (rows are numbered below 2^31 - 1)
 
 // tensor maps of Q, K, V, dO as [G n x d] bf16 tensors, 128-byte swizzle, box = 64 columns x 128 rows: tiles of consecutive rows
 struct alignas(64) BwdMaps {
@@ -46,7 +47,10 @@ struct BwdArgs {
   AttnArgs a;                  // geometry, permutations, samples
   const __nv_bfloat16* dout;   // [G, n, D]
   const float2* stat;          // [G, n] (-lse log2 e, -<dO, O>) of the rows
-  float *dq, *dk, *dv;         // [G, n, D] fp32 accumulators, cleared by row_stat_kernel
+  float *dq, *dk, *dv;         // fp32 accumulators, cleared by row_stat_kernel: [G, n, D]; direct: dk and dv [G, m, D], of the samples
+  __nv_bfloat16 *dk16, *dv16;  // direct: dK and dV of the keys without samples
+  const int32_t* key_slot;     // direct: [G, n] the sample that stands for a key, -1: none (null: none for any)
+  int direct;
   float scale;
   int* sched;                  // work counter of the launch, zero at launch
   // items: the key tiles of the leaves, then level by level those of the nodes
@@ -185,16 +189,17 @@ struct Cfg {
 // The same threads clear the accumulators: 32 bytes of each.
 template <int D, bool OUT_FP32>
 __global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__ dout, const void* __restrict__ out, const float* __restrict__ lse,
-                                                       float2* __restrict__ stat, size_t rows, int* sched, float4* dq, float4* dk, float4* dv) {
+                                                       float2* __restrict__ stat, size_t rows, int* sched, float4* dq, float4* dk, float4* dv, size_t kv_rows) {
   constexpr int LPR = D / 8;
   const size_t c = (size_t)blockIdx.x * 256 + threadIdx.x;
   wait_for_stream();
   if (c == 0) *sched = 0;
   const size_t row = c / LPR;
   float acc = 0.f;
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (size_t i = c; i < kv_rows * LPR; i += (size_t)gridDim.x * 256) { dk[2 * i] = z; dk[2 * i + 1] = z; dv[2 * i] = z; dv[2 * i + 1] = z; }
   if (row < rows) {
-    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-    dq[2 * c] = z; dq[2 * c + 1] = z; dk[2 * c] = z; dk[2 * c + 1] = z; dv[2 * c] = z; dv[2 * c + 1] = z;
+    dq[2 * c] = z; dq[2 * c + 1] = z;
     const uint4 x = __ldcs(dout + c);
     const uint32_t xd[4] = {x.x, x.y, x.z, x.w};
     float o[8];
@@ -404,7 +409,8 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
     // A reduction instruction whose lanes hit 32 different rows costs the L2 32 half-filled sectors: a warp's 32 rows x 32
     // columns pass through shared memory (chunks XOR-swizzled by row) and go out with eight lanes per row, four rows per instruction.
     const uint32_t stage = ubase + C::kOffStage + (warp - C::SW) * 4096;
-    auto out_rows = [&](uint32_t taddr, float f, float* base, size_t seg_row0, int grow, uint32_t bar_done) {
+    // grow: accumulator row of this thread's lane, < 0: none.  DIRECT: ~row of the bf16 result instead.
+    auto out_rows = [&](auto direct, uint32_t taddr, float f, float* base, __nv_bfloat16* base16, int grow, uint32_t bar_done) {
       uint32_t r[NC];
 #pragma unroll
       for (int p = 0; p < NC / 32; ++p) tmem_ld32_issue(taddr + NC * r_ + 32 * p, *reinterpret_cast<uint32_t(*)[32]>(r + 32 * p));
@@ -436,7 +442,9 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const int gr = __shfl_sync(0xffffffffu, grow, 4 * (q0 + q) + (lane >> 3));
-            if (gr >= 0) atomicAdd(reinterpret_cast<float4*>(base + (seg_row0 + gr) * D + NC * r_ + 32 * p + 4 * c), v[q]);
+            if (gr >= 0) atomicAdd(reinterpret_cast<float4*>(base + (size_t)gr * D + NC * r_ + 32 * p + 4 * c), v[q]);
+            else if (decltype(direct)::value && gr != kNoRow)
+              *reinterpret_cast<uint2*>(base16 + (size_t)~gr * D + NC * r_ + 32 * p + 4 * c) = make_uint2(pack2(v[q].x, v[q].y), pack2(v[q].z, v[q].w));
           }
         }
         __syncwarp();
@@ -448,8 +456,15 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
       if (!ok) break;
       const BwdItem& t = desc_of(it);
       if (t.kind < 0) break;
-      const size_t seg_row0 = (size_t)t.seg * g_.n;
-      const int kr = row < t.nkeys ? key_row(t, row) : -1;
+      const int seg_row0 = t.seg * g_.n;
+      int kr = kNoRow;
+      if (row < t.nkeys) {
+        kr = seg_row0 + key_row(t, row);
+        if (b.direct) {                                 // the key's tile has all of its gradient, or the sample's row collects it
+          const int slot = t.kind != 0 && b.key_slot ? __ldg(b.key_slot + kr) : -1;
+          kr = slot >= 0 ? t.seg * g_.m + slot : ~kr;
+        }
+      }
       const int steps = t.steps;
 #pragma unroll 1
       for (int s = 0; s < steps; ++s, ++g) {
@@ -457,14 +472,14 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
         ok = __all_sync(0xffffffffu, wait_fast<7>(bar_dq(g), (g >> 1) & 1, s_abort, status));
         if (!ok) break;
         tc_fence_after();
-        out_rows(lane_addr + C::kColDQ, b.scale, b.dq, seg_row0, qr, bar_dqfree);
+        out_rows(std::false_type{}, lane_addr + C::kColDQ, b.scale, b.dq, nullptr, qr >= 0 ? seg_row0 + qr : kNoRow, bar_dqfree);
       }
       if (!ok) break;
       ok = __all_sync(0xffffffffu, wait_fast<8>(bar_acc, it & 1, s_abort, status));
       if (!ok) break;
       tc_fence_after();
-      out_rows(lane_addr + C::kColDV, 1.f, b.dv, seg_row0, kr, 0);
-      out_rows(lane_addr + C::kColDK, b.scale, b.dk, seg_row0, kr, bar_accfree);
+      out_rows(std::true_type{}, lane_addr + C::kColDV, 1.f, b.dv, b.dv16, kr, 0);
+      out_rows(std::true_type{}, lane_addr + C::kColDK, b.scale, b.dk, b.dk16, kr, bar_accfree);
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_dfree(it));
     }
@@ -752,22 +767,38 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
   }
 }
 
-// the three fp32 accumulators (one after the other) rounded to bf16: 32 bytes in, 16 out per thread and pass
-__global__ void __launch_bounds__(256) to_bf16_kernel(const float4* __restrict__ src, uint4* __restrict__ dq, uint4* __restrict__ dk, uint4* __restrict__ dv, size_t count8) {
+// fp32 accumulators rounded to bf16, 32 bytes in and 16 out per thread and pass: blockIdx.y 0: dQ, 1 and 2: dK and dV, all rows
+// or (direct) the samples' rows, each to the key that it stands for.
+struct ToBf16Args {
+  const float4* src[3];
+  uint4* dst[3];
+  size_t count8[3];
+  const int32_t *key_slot, *samples;     // direct (else null)
+  int n, m, lg_lpr;                      // lg_lpr: log2 of the 16-byte pieces of a row
+};
+__global__ void __launch_bounds__(256) to_bf16_kernel(const __grid_constant__ ToBf16Args a) {
   wait_for_stream();
-  uint4* dst = blockIdx.y == 0 ? dq : (blockIdx.y == 1 ? dk : dv);
-  src += (size_t)blockIdx.y * count8 * 2;
-  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < count8; i += (size_t)gridDim.x * 256) {
-    const float4 x = __ldcs(src + 2 * i), y = __ldcs(src + 2 * i + 1);
-    __stcs(dst + i, make_uint4(pack2(x.x, x.y), pack2(x.z, x.w), pack2(y.x, y.y), pack2(y.z, y.w)));
+  const int y = blockIdx.y;
+  const float4* __restrict__ src = a.src[y];
+  uint4* __restrict__ dst = a.dst[y];
+  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < a.count8[y]; i += (size_t)gridDim.x * 256) {
+    size_t o = i;
+    if (y > 0 && a.key_slot) {
+      const int slot = (int)(i >> a.lg_lpr), seg = slot / a.m;
+      const size_t row = (size_t)seg * a.n + a.samples[slot];
+      if (a.key_slot[row] != slot - seg * a.m) continue;                  // (another draw of the same key stands for it)
+      o = (row << a.lg_lpr) + (i & ((1u << a.lg_lpr) - 1));
+    }
+    const float4 x = __ldcs(src + 2 * i), y4 = __ldcs(src + 2 * i + 1);
+    __stcs(dst + o, make_uint4(pack2(x.x, x.y), pack2(x.z, x.w), pack2(y4.x, y4.y), pack2(y4.z, y4.w)));
   }
 }
 
 }  // namespace
 
-// a: the forward schedule (permutations, samples, tile geometry); the accumulators dq, dk, dv are cleared here
+// a: the forward schedule (permutations, samples, tile geometry); the accumulators of gr are cleared here
 cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout, float2* stat, int* sched,
-                            float* dq, float* dk, float* dv, float scale, int* status, cudaStream_t st) {
+                            const BwdGrads& gr, float scale, int* status, cudaStream_t st) {
   const Geometry& g = a.g;
   const size_t rows = (size_t)g.G * g.n;
   if (rows > 0x7fffffffull) return cudaErrorInvalidValue;            // TMA row coordinates are 32-bit
@@ -775,13 +806,16 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
     const unsigned grid = (unsigned)((rows * (g.d / 8) + 255) / 256);
     const uint4* d4 = reinterpret_cast<const uint4*>(dout);
     auto* kernel = g.d == 64 ? (out_fp32 ? row_stat_kernel<64, true> : row_stat_kernel<64, false>) : (out_fp32 ? row_stat_kernel<128, true> : row_stat_kernel<128, false>);
-    const cudaError_t e = launch(kernel, grid, 256, 0, st, d4, out, lse, stat, rows, sched, reinterpret_cast<float4*>(dq), reinterpret_cast<float4*>(dk), reinterpret_cast<float4*>(dv));
+    const cudaError_t e = launch(kernel, grid, 256, 0, st, d4, out, lse, stat, rows, sched, reinterpret_cast<float4*>(gr.dq), reinterpret_cast<float4*>(gr.dk),
+                                 reinterpret_cast<float4*>(gr.dv), gr.kv_elems / g.d);
     if (e != cudaSuccess) return e;
   }
   int sms = 0;
   if (const cudaError_t e = sm_count(&sms); e != cudaSuccess) return e;
   BwdArgs b;
-  b.a = a; b.dout = reinterpret_cast<const __nv_bfloat16*>(dout); b.stat = stat; b.dq = dq; b.dk = dk; b.dv = dv; b.scale = scale; b.sched = sched;
+  b.a = a; b.dout = reinterpret_cast<const __nv_bfloat16*>(dout); b.stat = stat; b.scale = scale; b.sched = sched;
+  b.dq = gr.dq; b.dk = gr.dk; b.dv = gr.dv;
+  b.dk16 = reinterpret_cast<__nv_bfloat16*>(gr.dk16); b.dv16 = reinterpret_cast<__nv_bfloat16*>(gr.dv16); b.key_slot = gr.key_slot; b.direct = gr.direct;
   b.leaf_ktiles = a.n_leaf_tiles ? (g.leaf + kTileK - 1) / kTileK : 0;
   b.block_ktiles = (g.b + kTileK - 1) / kTileK;
   b.smp_ktiles = (g.m + kTileK - 1) / kTileK;
@@ -819,14 +853,16 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   const unsigned grid = items < sms ? (unsigned)items : (unsigned)sms;      // persistent: one CTA per SM
   cudaError_t e = g.d == 64 ? allow_smem<bwd_kernel<64>>(Cfg<64>::kTotal) : allow_smem<bwd_kernel<128>>(Cfg<128>::kTotal);
   if (e != cudaSuccess) return e;
-  return launch(g.d == 64 ? bwd_kernel<64> : bwd_kernel<128>, grid, g.d == 64 ? Cfg<64>::kThreads : Cfg<128>::kThreads, g.d == 64 ? Cfg<64>::kTotal : Cfg<128>::kTotal, st, b, maps, status);
-}
-
-// src: dq, dk, dv one after the other, count entries each (a multiple of 8)
-cudaError_t launch_to_bf16(const float* src, void* dq, void* dk, void* dv, size_t count, cudaStream_t st) {
-  const size_t count8 = count / 8, want = (count8 + 255) / 256;
-  const dim3 grid((unsigned)(want < 148 * 16 ? want : 148 * 16), 3);
-  return launch(to_bf16_kernel, grid, 256, 0, st, reinterpret_cast<const float4*>(src), reinterpret_cast<uint4*>(dq), reinterpret_cast<uint4*>(dk), reinterpret_cast<uint4*>(dv), count8);
+  e = launch(g.d == 64 ? bwd_kernel<64> : bwd_kernel<128>, grid, g.d == 64 ? Cfg<64>::kThreads : Cfg<128>::kThreads, g.d == 64 ? Cfg<64>::kTotal : Cfg<128>::kTotal, st, b, maps, status);
+  if (e != cudaSuccess || !gr.dq16) return e;
+  ToBf16Args c;
+  const size_t elems[3] = {rows * g.d, gr.kv_elems, gr.kv_elems};
+  const float* src[3] = {gr.dq, gr.dk, gr.dv};
+  void* dst[3] = {gr.dq16, gr.dk16, gr.dv16};
+  for (int y = 0; y < 3; ++y) { c.src[y] = reinterpret_cast<const float4*>(src[y]); c.dst[y] = reinterpret_cast<uint4*>(dst[y]); c.count8[y] = elems[y] / 8; }
+  c.key_slot = gr.direct ? gr.key_slot : nullptr; c.samples = a.samples; c.n = g.n; c.m = g.m; c.lg_lpr = g.d == 64 ? 3 : 4;
+  const size_t blocks = (c.count8[0] + 255) / 256;
+  return launch(to_bf16_kernel, dim3((unsigned)(blocks < 148 * 16 ? blocks : 148 * 16), gr.kv_elems ? 3 : 1), 256, 0, st, c);
 }
 
 }  // namespace hyperattn

@@ -159,6 +159,7 @@ struct Workspace {
   int32_t *perm_q, *perm_k, *rank_k;  // [levels, G, nl]
   int32_t* samples;                // [G, nodes, m]
   int32_t* smp_blk;                // [G, nodes, m] sorted block that the sampled key lies in (null: not wanted)
+  int32_t* key_slot;               // [G, nk] one of the samples that drew the key, -1: none did (one node only; null: not wanted)
   int32_t* tpos;                   // capped row sums: [G, nodes, m] probe positions (else null)
   float* ltau;                     // capped row sums: [G, nodes] log2 of the largest unmasked probe row sum
   void* part_o; float* part_lse;   // causal partials: leaf [G,n,(d)] then per level [G,nl,(d)]; rows of fp32 or bf16

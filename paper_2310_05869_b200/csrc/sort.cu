@@ -19,6 +19,7 @@ struct SortArgs {
   uint32_t* offs;         // queries [levels, G, chunks per (level, segment), 256], then the same for keys
   int32_t *perm_q, *perm_k, *rank_k;  // [levels, G, nl]
   int32_t* smp_blk;       // [G, nodes, m] sorted block of every sampled key, or null
+  int32_t* key_slot;      // [G, nk] one of the samples that drew the key, or -1 (null: not wanted)
   Geometry g;
   int side_mask;          // bit s set: side s is sorted (both, unless a caller wants one side only)
 };
@@ -244,6 +245,7 @@ __global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a, SampleArg
     if (act) {
       perm[pos] = local0 + i;
       if (rank) rank[local0 + i] = (int32_t)pos;
+      if (side == 1 && a.key_slot) a.key_slot[(size_t)seg * g.nk + local0 + i] = -1;
     }
   }
   // The block of every sampled key among these rows, which decides whether a query tile's own block holds the sample: the attention
@@ -259,7 +261,10 @@ __global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a, SampleArg
         const Philox4 x = philox4x32_10((uint32_t)(c >> 2), (uint32_t)(g.seg0 + seg), (uint32_t)node, kDomainSamples, sa.k0, sa.k1);
         l = (int)__umulhi((c & 2) ? ((c & 1) ? x.x[3] : x.x[2]) : ((c & 1) ? x.x[1] : x.x[0]), N);
       } else l = sa.samples[base + c];
-      if ((unsigned)(l - local0) < (unsigned)rows) a.smp_blk[base + c] = rank[l] / g.b;
+      if ((unsigned)(l - local0) < (unsigned)rows) {
+        a.smp_blk[base + c] = rank[l] / g.b;
+        if (a.key_slot) a.key_slot[(size_t)seg * g.nk + l] = c;      // (a key drawn more than once: any of its draws, the last to write)
+      }
     }
   }
 }
@@ -269,7 +274,7 @@ __global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a, SampleArg
 static SortArgs make_sort_args(const Geometry& g, const Workspace& ws, int side_mask) {
   SortArgs a;
   a.ids = ws.ids; a.hist = ws.hist; a.offs = ws.offs;
-  a.perm_q = ws.perm_q; a.perm_k = ws.perm_k; a.rank_k = ws.rank_k; a.smp_blk = ws.smp_blk;
+  a.perm_q = ws.perm_q; a.perm_k = ws.perm_k; a.rank_k = ws.rank_k; a.smp_blk = ws.smp_blk; a.key_slot = ws.key_slot;
   a.g = g;
   a.side_mask = side_mask;
   return a;

@@ -663,51 +663,79 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
     if (warp < C::SW + 11) {
       const bool is_q = warp == C::SW + 9;
       const int nbuf = is_q ? C::NQ : C::NDO;
-      uint32_t g = 0;
-      for (int it = 0; ok; ++it) {
-        ok = __all_sync(0xffffffffu, wait_desc(it));
-        if (!ok) break;
-        const BwdItem& t = desc_of(it);
-        if (t.kind < 0) break;
-        const int steps = t.steps, seg_row0 = t.seg * g_.n;
-        const bool dense = t.kind == 0;
-        const float wlog = t.wlog;
-        // row numbers and statistics of a step's query rows (rows that do not exist: the node's first row, with weights of zero)
-        int vn[4];
-        float2 sn[4];
-        auto rows_of = [&](int x) {
-          const StepRows sr = step_rows(b, t, x);
+      // Row numbers are asked for two steps ahead and statistics one, across items: under this kernel's load a dependent read takes
+      // 2000 clocks, and in line with the copies two of them are longer than a step (PREFETCH_FIGURES).
+      struct Step {
+        int rel[4];                                      // row lane + 32 u of the query tile, relative to base (rows that do not exist: 0)
+        int base, nq;                                    // nq: rows that exist
+        int y;                                           // tiles of consecutive rows: the first (else -1)
+        float wlog;
+      };
+      Step s0, s1;                                       // this step, the next
+      float2 n0[4];                                      // statistics of this step
+      int have = 0, pit = 0, ps = 0;                     // steps asked for; item and step to ask for next
+      bool end = false;
+      auto ask = [&](Step& d) {
+        const BwdItem& t = desc_of(pit);
+        const StepRows sr = step_rows(b, t, ps);
+        d.base = t.seg * g_.n + t.q0; d.nq = sr.nq; d.wlog = t.wlog;
+        d.y = t.kind == 0 ? t.seg * g_.n + sr.first : -1;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int qr = query_row(t, sr, lane + 32 * u);
-            vn[u] = seg_row0 + (qr >= 0 ? qr : t.q0);
-            if (is_q) sn[u] = qr >= 0 ? __ldg(b.stat + vn[u]) : make_float2(-INFINITY, 0.f);
-          }
-        };
-        if (is_q || !dense) rows_of(0);
-#pragma unroll 1
-        for (int x = 0; x < steps; ++x, ++g) {
-          int v[4] = {vn[0], vn[1], vn[2], vn[3]};
-          const uint32_t bar = is_q ? bar_qfull(g) : bar_dofull(g);
-          const uint32_t dst = ubase + (is_q ? C::kOffQ + (g % C::NQ) * C::kTile : C::kOffDO + (g % C::NDO) * C::kTile);
-          if (g >= (uint32_t)nbuf) {
-            const uint32_t last = g - nbuf;              // (the step that used the buffer before)
-            ok = __all_sync(0xffffffffu, wait_fast<16>(is_q ? bar_qfree(last) : bar_dofree(last), (last >> 1) & 1, s_abort, status));
-            if (!ok) break;
-          }
-          if (is_q) {
-            float* st = reinterpret_cast<float*>(smem + C::kOffStat) + (g % C::NQ) * 256;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) { st[lane + 32 * u] = sn[u].x + wlog; st[128 + lane + 32 * u] = sn[u].y; }
-            mbar_arrive(bar);
-          }
-          if (dense) boxes(dst, 128, is_q ? &maps.q : &maps.dout, seg_row0 + t.q0 + x * 128, bar);
-          else gather(dst, is_q ? a.q : b.dout, v, bar);
-          if (x + 1 < steps && (is_q || !dense)) rows_of(x + 1);
+        for (int u = 0; u < 4; ++u) {
+          const int r = lane + 32 * u;
+          d.rel[u] = r < sr.nq ? (t.kind == 0 ? sr.first - t.q0 + r : __ldg(a.perm_q + t.slice + sr.first + r)) : 0;
         }
-        if (!ok) break;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_dfree(it));
+        ++have;
+        if (++ps == t.steps) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_dfree(pit));
+          ps = 0; ++pit;
+        }
+      };
+      // the next step, if its item is known by now
+      auto more = [&]() {
+        if (end) return false;
+        if (ps == 0) {
+          if (!__all_sync(0xffffffffu, mbar_test(bar_dfull(pit), (pit / kDescs) & 1))) return false;
+          if (desc_of(pit).kind < 0) { end = true; return false; }
+        }
+        return true;
+      };
+      auto stats = [&]() {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) n0[u] = lane + 32 * u < s0.nq ? __ldg(b.stat + s0.base + s0.rel[u]) : make_float2(-INFINITY, 0.f);
+      };
+      for (uint32_t g = 0; ok; ++g) {
+        if (have == 0) {
+          if (!end && ps == 0) ok = __all_sync(0xffffffffu, wait_desc(pit));
+          if (!ok || !more()) break;
+          ask(s0);
+          if (is_q) stats();
+        }
+        if (more()) ask(s1);
+        const uint32_t bar = is_q ? bar_qfull(g) : bar_dofull(g);
+        const uint32_t dst = ubase + (is_q ? C::kOffQ + (g % C::NQ) * C::kTile : C::kOffDO + (g % C::NDO) * C::kTile);
+        if (g >= (uint32_t)nbuf) {
+          const uint32_t last = g - nbuf;                // (the step that used the buffer before)
+          ok = __all_sync(0xffffffffu, wait_fast<16>(is_q ? bar_qfree(last) : bar_dofree(last), (last >> 1) & 1, s_abort, status));
+          if (!ok) break;
+        }
+        if (is_q) {
+          float* st = reinterpret_cast<float*>(smem + C::kOffStat) + (g % C::NQ) * 256;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) { st[lane + 32 * u] = n0[u].x + s0.wlog; st[128 + lane + 32 * u] = n0[u].y; }
+          mbar_arrive(bar);
+        }
+        if (s0.y >= 0) boxes(dst, 128, is_q ? &maps.q : &maps.dout, s0.y, bar);
+        else {
+          int v[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[u] = s0.base + s0.rel[u];
+          gather(dst, is_q ? a.q : b.dout, v, bar);
+        }
+        s0 = s1;
+        --have;
+        if (is_q && have > 0) stats();
       }
       cp_async_commit();
       cp_async_wait_all();

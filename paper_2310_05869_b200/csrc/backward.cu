@@ -12,8 +12,9 @@
 //
 // A work item is a tile of 128 KEYS and a run of query tiles (steps): the key tiles of a leaf against the query tiles from the
 // diagonal on, a key tile of a sorted block against the block's query tiles, a tile of a node's sampled keys against a chunk of the
-// node's query tiles.  dK and dV of the item stay in TMEM over its steps and leave once, by fp32 reductions; dQ leaves after every
-// step.  (The other way round - query tiles stay, dK and dV leave after every step - is twice the reductions and was what
+// node's query tiles.  dK and dV of the item stay in TMEM over its steps and leave once: by fp32 reductions, or, without recursion
+// and for keys that are not sampled, which no other item adds to, as bf16 results (32 heads x 32768 rows, d = 128: accumulators that need not
+// be cleared, added to and converted, 1934 -> 1416 us); dQ leaves after every step.  (The other way round - query tiles stay, dK and dV leave after every step - is twice the reductions and was what
 // the kernel's first version did, one phase after the other: 10 500 clocks per 128 x 128 tile at d = 64, 17 400 at d = 128.)
 // Per step, all five products on the tcgen05 tensor cores, keys in the TMEM lanes of the first two:
 //     S^T  = K Q^T,  dP^T = V dO^T      operands in 128-byte-swizzled shared memory, K-major
@@ -21,13 +22,18 @@
 //     dV  += P^T dO      A from TMEM, B = dO [query][d] MN-major
 //     dK  += dS^T Q      A K-major, B = Q MN-major
 //     dQ   = dS K        A = the same dS^T tile read MN-major, B = K [key][d] MN-major
-// What bounds it: the tensor pipe needs 1700 (d = 64) / 2700 (d = 128) clocks per step, the exponentials 1024; scores, hand-over,
-// exponentials, hand-over are one chain of about 2200.  d = 64: the next step's S^T and dP^T are issued before this step's three
-// gradient products, which then run while the warpgroups are busy with the next step; d = 128 has not the TMEM columns (P^T goes over S^T,
-// dQ over dP^T), so there dQ comes first and leaves TMEM while dV, the next S^T and dK are multiplied.
+// d = 64: a step's two halves of 64 queries are two chains - scores, hand-over, exponentials, hand-over - that P warpgroups 0 and 1 work
+// through independently, half a step apart, with S^T, dP^T, P^T, dV, dK and dQ side by side in TMEM; the tensor pipe needs about 2000
+// clocks per step, the exponentials 1024.  d = 128 has not the TMEM columns (P^T goes over S^T, dQ over dP^T): one chain, in
+// which dQ comes before dK so that it leaves TMEM while dK and the next S^T are multiplied.
+// What bounds it: a step takes 4000 (causal leaves) to 5000 clocks (sorted blocks), of which no single unit is busy for half; the
+// load and store unit is the fullest (gathered copies, dS, results through shared memory, reductions at 25 bytes per clock), and
+// everything else in a chain waits behind it.  Time, us, of the whole pass, one chain -> two: 131072 rows, 32 heads 3335 -> 3025;
+// causal leaves of 4096 rows, 128 heads 1167 -> 1098; 12 heads x 4096 rows 59 -> 56 (d = 64; two chains at d = 128 are 10 % slower in the
+// leaves).  16 P warps instead of 8 force 64 registers a thread and are slower (3160).
 //
-// Warp roles (512 threads): warps 0-3 and 4-7 P and dS; warps 8-11 dQ, dK and dV to global memory; warp 12 MMA issue (one
-// thread; the warp also allocates TMEM); warp 13 Q, dO and the row statistics; warp 14 K and V; warp 15 item descriptors.
+// Warp roles (672 threads): warps 0-7 P and dS; 8-15 dQ, dK and dV to global memory; 16 issue of S^T and dP^T (the warp also allocates
+// TMEM); 17 issue of the gradient products; 18 item descriptors, K and V; 19 Q and the row statistics; 20 dO.
 // Every wait is bounded: on a timeout the CTA raises the device status word, drains its copies, frees its TMEM and returns.
 #include "tc_util.cuh"
 
@@ -159,8 +165,8 @@ __device__ __forceinline__ StepRows step_rows(const BwdArgs& b, const BwdItem& t
 
 template <int D>
 struct Cfg {
-  // warps: P and dS (SW of them, 128 / (SW / 4) query columns each), results, then issue, Q, dO, items
-  static constexpr int SW = D == 64 ? 16 : 8, kThreads = 32 * (SW + 12);
+  // warps: P and dS (SW of them, 128 / (SW / 4) query columns each), results (RW), issue of scores, of gradients, items, Q, dO; NH: chains
+  static constexpr int SW = 8, RW = 8, NH = D == 64 ? 2 : 1, kThreads = 32 * (SW + RW + 5);
   static constexpr int kTile = 128 * D * 2;           // bytes of a [128 rows x D] tile
   // buffers: K and V (an item each), Q, dO and dS (a step each); d = 128 has room for two only of Q
   static constexpr int NKV = D == 64 ? 2 : 1, NQ = 2, NDO = D == 64 ? 2 : 1, NDS = D == 64 ? 2 : 1;
@@ -170,11 +176,11 @@ struct Cfg {
   static constexpr int kOffDO = kOffQ + NQ * kTile;
   static constexpr int kOffDS = kOffDO + NDO * kTile;
   static constexpr int kOffStage = kOffDS + NDS * 128 * 128 * 2;            // results on their way out: 4 KB per warp
-  static constexpr int kOffStat = kOffStage + 8 * 4096;                     // float [NQ][-lse2 | -delta][128]
+  static constexpr int kOffStat = kOffStage + RW * 4096;                     // float [NQ][-lse2 | -delta][128]
   static constexpr int kOffDesc = kOffStat + NQ * 1024;
   static constexpr int kDescBytes = (sizeof(BwdItem) + 15) / 16 * 16;
   static constexpr int kOffBar = kOffDesc + kDescs * kDescBytes;
-  static constexpr int kNumBar = 24 + 2 * kDescs;
+  static constexpr int kNumBar = 27 + 2 * kDescs;
   static constexpr int kOffMisc = kOffBar + 8 * kNumBar;
   static constexpr int kTotal = kOffMisc + 16;
   static_assert(kTotal <= 232448, "shared memory");
@@ -233,21 +239,22 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
   const uint32_t bar0 = ubase + C::kOffBar;
   // g: step, it: item, counted over the CTA's whole work list.  (Pairs of barriers are used in turn by the steps; a waiter that
   // is a step behind never meets a phase twice.)
-  const uint32_t bar_s = bar0, bar_dp = bar0 + 8;                                 // S^T, dP^T written
-  const uint32_t bar_h = bar0 + 16;                                               // P and dS written (S^T and dP^T have been read)
-  const uint32_t bar_dqfree = bar0 + 24;                                          // dQ has left TMEM
-  const uint32_t bar_acc = bar0 + 32, bar_accfree = bar0 + 40;                    // dK, dV of the item complete; have left TMEM
-  auto bar_dsfree = [&](uint32_t g) { return bar0 + 8 * (6 + g % C::NDS); };      // dK and dQ of a step multiplied: its dS is free
-  auto bar_dq = [&](uint32_t g) { return bar0 + 8 * (8 + (g & 1)); };             // dQ of a step in TMEM
+  // x: half of the step's queries, 64 columns of S^T and dP^T
+  auto bar_s = [&](int x) { return bar0 + 8 * (0 + x); };                         // S^T of the half written
+  auto bar_dp = [&](int x) { return bar0 + 8 * (2 + x); };                        // dP^T of the half written
+  auto bar_h = [&](int x) { return bar0 + 8 * (4 + x); };                         // P and dS of the half written (S^T and dP^T have been read)
+  auto bar_pfree = [&](int x) { return bar0 + 8 * (6 + x); };                     // dV of the half multiplied: its P is free
+  auto bar_dq = [&](uint32_t g) { return bar0 + 8 * (8 + (g & 1)); };             // dQ of a step in TMEM: all its products are done, its dS is free
   auto bar_qfull = [&](uint32_t g) { return bar0 + 8 * (10 + (g & 1)); };         // Q and the row statistics of a step landed
   auto bar_qfree = [&](uint32_t g) { return bar0 + 8 * (12 + (g & 1)); };
   auto bar_dofull = [&](uint32_t g) { return bar0 + 8 * (14 + g % C::NDO); };     // dO landed
-  auto bar_dofree = [&](uint32_t g) { return bar0 + 8 * (16 + (g & 1)); };        // dV multiplied: dO and P are free
+  auto bar_dofree = [&](uint32_t g) { return bar0 + 8 * (16 + (g & 1)); };        // dV multiplied: dO is free
   auto bar_kfull = [&](int it) { return bar0 + 8 * (18 + it % C::NKV); };         // K, V of an item landed
   auto bar_vfull = [&](int it) { return bar0 + 8 * (20 + it % C::NKV); };
   auto bar_kfree = [&](int it) { return bar0 + 8 * (22 + it % C::NKV); };         // dQ of the item multiplied: K and V are free
-  auto bar_dfull = [&](int it) { return bar0 + 8 * (24 + it % kDescs); };         // item descriptor written
-  auto bar_dfree = [&](int it) { return bar0 + 8 * (24 + kDescs + it % kDescs); };
+  const uint32_t bar_dqfree = bar0 + 8 * 24, bar_acc = bar0 + 8 * 25, bar_accfree = bar0 + 8 * 26;   // dQ has left TMEM; dK, dV of the item complete; have left TMEM
+  auto bar_dfull = [&](int it) { return bar0 + 8 * (27 + it % kDescs); };         // item descriptor written
+  auto bar_dfree = [&](int it) { return bar0 + 8 * (27 + kDescs + it % kDescs); };
 
   const AttnArgs& a = b.a;
   const Geometry& g_ = a.g;
@@ -259,14 +266,14 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
   if (*s_abort) return;                                 // (a launch in which some wait already timed out drains quickly)
   __syncthreads();
   if (tid == 0) {
-    mbar_init(bar_s, 1); mbar_init(bar_dp, 1); mbar_init(bar_h, C::SW); mbar_init(bar_dqfree, 8); mbar_init(bar_acc, 1); mbar_init(bar_accfree, 8);   // (8: one arrival per warp)
-    for (int x = 0; x < 2; ++x) { mbar_init(bar_dsfree(x), 1); mbar_init(bar_dq(x), 1); mbar_init(bar_qfull(x), 64); mbar_init(bar_qfree(x), 1); mbar_init(bar_dofree(x), 1); }
+    mbar_init(bar_dqfree, C::RW); mbar_init(bar_acc, 1); mbar_init(bar_accfree, C::RW);   // (one arrival per warp)
+    for (int x = 0; x < 2; ++x) { mbar_init(bar_s(x), 1); mbar_init(bar_dp(x), 1); mbar_init(bar_h(x), C::SW / C::NH); mbar_init(bar_pfree(x), 1); mbar_init(bar_dq(x), 1); mbar_init(bar_qfull(x), 64); mbar_init(bar_qfree(x), 1); mbar_init(bar_dofree(x), 1); }
     for (int x = 0; x < C::NDO; ++x) mbar_init(bar_dofull(x), 32);
     for (int x = 0; x < C::NKV; ++x) { mbar_init(bar_kfull(x), 32); mbar_init(bar_vfull(x), 32); mbar_init(bar_kfree(x), 1); }
-    for (int x = 0; x < kDescs; ++x) { mbar_init(bar_dfull(x), 1); mbar_init(bar_dfree(x), C::SW + 11); }   // P and results warps, issuer, two loaders
+    for (int x = 0; x < kDescs; ++x) { mbar_init(bar_dfull(x), 1); mbar_init(bar_dfree(x), C::SW + C::RW + 4); }   // P and results warps, two issuers, loaders of Q and dO
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == C::SW + 8) {
+  if (warp == C::SW + C::RW) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -292,7 +299,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
   if (warp < C::SW) {
     // ================= P and dS: thread = key, warpgroup q: query columns W q .. W q + W - 1, in two chunks ==================
     constexpr int W = 128 / (C::SW / 4), CW = W / 2;
-    const int row = tid & 127, col0 = (warp >> 2) * W;
+    const int row = tid & 127, col0 = (warp >> 2) * W, half = C::NH == 2 ? col0 >> 6 : 0;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t p_addr = lane_addr + C::kColP + C::kPHalf * (col0 >> 6) + (col0 & 63) / 2;
     const uint64_t sc2 = pack_f2(a.scale_log2, a.scale_log2);
@@ -313,7 +320,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
         if (kind == 2) dead = dead || kblk == (t.tn0 + s) / a.tiles_per_block;
         const bool diag = causal && s == 0;
         const bool masked = diag || __any_sync(0xffffffffu, dead);
-        ok = wait_fast<2>(bar_qfull(g), (g >> 1) & 1, s_abort, status) && wait_fast<3>(bar_s, g & 1, s_abort, status);
+        ok = wait_fast<2>(bar_qfull(g), (g >> 1) & 1, s_abort, status) && wait_fast<3>(bar_s(half), g & 1, s_abort, status);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
@@ -351,8 +358,9 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
           // d = 128: P goes over scores of this warpgroup that have been read
           if (D == 128) put_p();
           if (c == 0) {
-            ok = wait_fast<4>(bar_dp, g & 1, s_abort, status);
-            if (g >= C::NDS) ok = ok && wait_fast<5>(bar_dsfree(g), (g / C::NDS - 1) & 1, s_abort, status);
+            ok = wait_fast<4>(bar_dp(half), g & 1, s_abort, status);
+            // (dS of the step that used the buffer before has been multiplied; the last of its products is dQ or, d = 128, dK)
+            if (g >= C::NDS) ok = ok && wait_fast<5>(D == 64 ? bar_dq(g - C::NDS) : bar_qfree(g - C::NDS), ((g - C::NDS) >> 1) & 1, s_abort, status);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
@@ -382,7 +390,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
           if (D == 64) {
             // (P of the step before is read by the dV product until here at most)
             if (c == 0 && g > 0) {
-              ok = __all_sync(0xffffffffu, wait_fast<6>(bar_dofree(g - 1), ((g - 1) >> 1) & 1, s_abort, status));
+              ok = __all_sync(0xffffffffu, wait_fast<6>(bar_pfree(half), (g - 1) & 1, s_abort, status));
               if (!ok) break;
               tc_fence_after();
             }
@@ -394,41 +402,39 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
         tc_fence_before();
         fence_async_smem();
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_h);
+        if (lane == 0) mbar_arrive(bar_h(half));
       }
       if (!ok) break;
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_dfree(it));
     }
-  } else if (warp < C::SW + 8) {
+  } else if (warp < C::SW + C::RW) {
     // ================= results, fp32 reductions into the accumulators: dQ after every step, dK and dV after every item; warpgroup
     // r takes half of the columns ==================
     const int r_ = (warp - C::SW) >> 2, row = tid & 127;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    constexpr int NC = D / 2;                           // columns of a result that this warpgroup takes
+    constexpr int NC = D * 4 / C::RW;                // columns of a result that this warpgroup takes
     // A reduction instruction whose lanes hit 32 different rows costs the L2 32 half-filled sectors: a warp's 32 rows x 32
     // columns pass through shared memory (chunks XOR-swizzled by row) and go out with eight lanes per row, four rows per instruction.
     const uint32_t stage = ubase + C::kOffStage + (warp - C::SW) * 4096;
     // grow: accumulator row of this thread's lane, < 0: none.  DIRECT: ~row of the bf16 result instead.
     auto out_rows = [&](auto direct, uint32_t taddr, float f, float* base, __nv_bfloat16* base16, int grow, uint32_t bar_done) {
-      uint32_t r[NC];
-#pragma unroll
-      for (int p = 0; p < NC / 32; ++p) tmem_ld32_issue(taddr + NC * r_ + 32 * p, *reinterpret_cast<uint32_t(*)[32]>(r + 32 * p));
-#pragma unroll
-      for (int p = 0; p < NC / 32; ++p) tmem_ld32_wait(*reinterpret_cast<uint32_t(*)[32]>(r + 32 * p));
-      if (bar_done) {                                   // it has left TMEM
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_done);
-      }
       const int c = lane & 7;
 #pragma unroll
       for (int p = 0; p < NC / 32; ++p) {
+        uint32_t r[32];
+        tmem_ld32_issue(taddr + NC * r_ + 32 * p, r);
+        tmem_ld32_wait(r);
+        if (p == NC / 32 - 1 && bar_done) {             // it has left TMEM
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_done);
+        }
 #pragma unroll
         for (int x = 0; x < 8; ++x)
           asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((x ^ (lane & 7)) << 4)),
-                       "f"(__uint_as_float(r[32 * p + 4 * x]) * f), "f"(__uint_as_float(r[32 * p + 4 * x + 1]) * f),
-                       "f"(__uint_as_float(r[32 * p + 4 * x + 2]) * f), "f"(__uint_as_float(r[32 * p + 4 * x + 3]) * f) : "memory");
+                       "f"(__uint_as_float(r[4 * x]) * f), "f"(__uint_as_float(r[4 * x + 1]) * f),
+                       "f"(__uint_as_float(r[4 * x + 2]) * f), "f"(__uint_as_float(r[4 * x + 3]) * f) : "memory");
         __syncwarp();
 #pragma unroll
         for (int q0 = 0; q0 < 8; q0 += 4) {
@@ -483,149 +489,123 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_dfree(it));
     }
-  } else if (warp == C::SW + 8) {
-    // ================= MMA issue ==================
+  } else if (warp < C::SW + C::RW + 2) {
+    // ================= MMA issue, a warp for the scores and one for the gradients ==================
     // The whole warp walks through this code together and one elected lane issues: descriptors and addresses are then made of
     // uniform registers, which the instructions take directly (a lone lane's have to be moved there one by one).
-    {
-      const bool el = elect_one();
-      auto uni = [&](int x) { return __shfl_sync(0xffffffffu, x, 0); };
-      auto utest = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_test(bar, parity)) != 0; };
-      auto uwait_desc = [&](int it) { return __all_sync(0xffffffffu, wait_desc(it)) != 0; };
-      // descriptors: low word = start >> 4 | (leading byte offset >> 4) << 16, high word = stride 1024 B | version | 128-byte swizzle
-      constexpr uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
-      constexpr uint32_t kSlab = 128 * 128;             // bytes of one [128 rows x 64 columns] slab
-      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
-      constexpr uint32_t idesc_s = idesc | ((128u >> 3) << 17);                                            // K-major x K-major, N = 128
-      constexpr uint32_t idesc_n = idesc | (1u << 16) | (((uint32_t)D >> 3) << 17);                        // K-major (or TMEM) x MN-major, N = D
-      constexpr uint32_t idesc_t = idesc | (1u << 15) | (1u << 16) | (((uint32_t)D >> 3) << 17);           // MN-major x MN-major, N = D
-      const uint32_t base = ubase >> 4;
-      auto kmajor = [&](uint32_t off, int ks) { return base + ((off + (ks >> 2) * kSlab + (ks & 3) * 32) >> 4) + (1u << 16); };
-      auto mnmajor = [&](uint32_t off, int kk) { return base + ((off + kk * 2048) >> 4) + ((kSlab >> 4) << 16); };
-      // Scores run a step ahead of the gradients, across item boundaries.  gs, gp: next step of S and dP; its / itp: its item;
-      // ls / lp: steps left in it.
-      uint32_t gs = 0, gp = 0, g = 0;
-      int its = -1, itp = -1, ls = 0, lp = 0;
-      bool ends = false;
-      // whether S (dP) of the next step could be issued without waiting
-      auto s_ready = [&]() {
-        if (ls == 0) {
-          if (!utest(bar_dfull(its + 1), ((its + 1) / kDescs) & 1)) return false;
-          if (uni(desc_of(its + 1).kind) < 0 || !utest(bar_kfull(its + 1), ((its + 1) / C::NKV) & 1)) return false;
-        }
-        return utest(bar_qfull(gs), (gs >> 1) & 1);
-      };
-      auto issue_s = [&]() {
-        if (ls == 0) {
-          ++its;
-          ok = ok && uwait_desc(its);
-          if (!ok) return;
-          if (uni(desc_of(its).kind) < 0) { ends = true; return; }
-          ls = uni(desc_of(its).steps);
-          ok = warp_wait<9>(bar_kfull(its), (its / C::NKV) & 1, s_abort, status);
-        }
-        ok = ok && warp_wait<10>(bar_qfull(gs), (gs >> 1) & 1, s_abort, status);
-        if (!ok) return;
-        fence_async_smem();
-        tc_fence_after();
-        const uint32_t k = C::kOffK + (its % C::NKV) * C::kTile, q = C::kOffQ + (gs & 1) * C::kTile;
-        if (el) {
-#pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColS, kmajor(k, ks), kmajor(q, ks), desc_hi, idesc_s, ks > 0);
-          umma_commit(bar_s);
-        }
-        ++gs; --ls;
-      };
-      // (dP only ever follows S of the same step: its item is known)
-      auto p_ready = [&]() {
-        if (gp >= gs) return false;
-        if (lp == 0 && !utest(bar_vfull(itp + 1), ((itp + 1) / C::NKV) & 1)) return false;
-        if (D == 128 && gp > 0 && !utest(bar_dqfree, (gp - 1) & 1)) return false;
-        return utest(bar_dofull(gp), (gp / C::NDO) & 1);
-      };
-      auto issue_p = [&]() {
-        if (lp == 0) {
-          ++itp;
-          lp = uni(desc_of(itp).steps);
-          ok = ok && warp_wait<11>(bar_vfull(itp), (itp / C::NKV) & 1, s_abort, status);
-        }
-        // (d = 128: dQ of the step before lies there)
-        if (D == 128 && gp > 0) ok = ok && warp_wait<12>(bar_dqfree, (gp - 1) & 1, s_abort, status);
-        ok = ok && warp_wait<13>(bar_dofull(gp), (gp / C::NDO) & 1, s_abort, status);
-        if (!ok) return;
-        fence_async_smem();
-        tc_fence_after();
-        const uint32_t v = C::kOffV + (itp % C::NKV) * C::kTile, o = C::kOffDO + (gp % C::NDO) * C::kTile;
-        if (el) {
-#pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColDP, kmajor(v, ks), kmajor(o, ks), desc_hi, idesc_s, ks > 0);
-          umma_commit(bar_dp);
-        }
-        ++gp; --lp;
-      };
-      issue_s();
-      if (ok && !ends) issue_p();
-      for (int it = 0; ok && !ends; ++it) {
+    const bool el = elect_one();
+    auto uni = [&](int x) { return __shfl_sync(0xffffffffu, x, 0); };
+    // descriptors: low word = start >> 4 | (leading byte offset >> 4) << 16, high word = stride 1024 B | version | 128-byte swizzle
+    constexpr uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+    constexpr uint32_t kSlab = 128 * 128;               // bytes of one [128 rows x 64 columns] slab
+    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
+    constexpr uint32_t idesc_s = idesc | (((128u / C::NH) >> 3) << 17);                                  // K-major x K-major, N = 128 / NH
+    constexpr uint32_t idesc_n = idesc | (1u << 16) | (((uint32_t)D >> 3) << 17);                        // K-major (or TMEM) x MN-major, N = D
+    constexpr uint32_t idesc_t = idesc | (1u << 15) | (1u << 16) | (((uint32_t)D >> 3) << 17);           // MN-major x MN-major, N = D
+    const uint32_t base = ubase >> 4;
+    auto kmajor = [&](uint32_t off, int ks) { return base + ((off + (ks >> 2) * kSlab + (ks & 3) * 32) >> 4) + (1u << 16); };
+    auto mnmajor = [&](uint32_t off, int kk) { return base + ((off + kk * 2048) >> 4) + ((kSlab >> 4) << 16); };
+    uint32_t g = 0;
+    if (warp == C::SW + C::RW) {
+      // S^T and dP^T of a half, as soon as the half's warps have read the step before
+      for (int it = 0; ok; ++it) {
+        ok = __all_sync(0xffffffffu, wait_desc(it)) != 0;
+        if (!ok || uni(desc_of(it).kind) < 0) break;
         const int steps = uni(desc_of(it).steps);
-        const uint32_t kt = C::kOffK + (it % C::NKV) * C::kTile;
+        const uint32_t k = C::kOffK + (it % C::NKV) * C::kTile, v = C::kOffV + (it % C::NKV) * C::kTile;
+        ok = warp_wait<9>(bar_kfull(it), (it / C::NKV) & 1, s_abort, status);
 #pragma unroll 1
         for (int s = 0; s < steps && ok; ++s, ++g) {
-          ok = warp_wait<14>(bar_h, g & 1, s_abort, status);
-          if (!ok) break;
-          tc_fence_after();
-          const bool last = s + 1 == steps;
-          const uint32_t q = C::kOffQ + (g & 1) * C::kTile, o = C::kOffDO + (g % C::NDO) * C::kTile, ds = C::kOffDS + (g % C::NDS) * (128 * 128 * 2);
-          auto grad_v = [&]() {
-            if (s == 0 && it > 0) {
-              ok = ok && warp_wait<15>(bar_accfree, (it - 1) & 1, s_abort, status);
-              tc_fence_after();
+          const uint32_t q = C::kOffQ + (g & 1) * C::kTile, o = C::kOffDO + (g % C::NDO) * C::kTile;
+          ok = warp_wait<10>(bar_qfull(g), (g >> 1) & 1, s_abort, status);
+          auto scores = [&](int x) {
+            if (g > 0) ok = ok && warp_wait<14>(D == 64 ? bar_h(x) : bar_pfree(x), (g - 1) & 1, s_abort, status);   // (d = 128: P lies over the scores)
+            if (!ok) return;
+            if (x == 0) fence_async_smem();
+            tc_fence_after();
+            if (el) {
+#pragma unroll
+              for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColS + 64 * x, kmajor(k, ks), kmajor(q + x * 8192, ks), desc_hi, idesc_s, ks > 0);
+              umma_commit(bar_s(x));
+            }
+          };
+          auto dprob = [&](int x) {
+            if (x == 0) {
+              if (s == 0) ok = ok && warp_wait<11>(bar_vfull(it), (it / C::NKV) & 1, s_abort, status);
+              ok = ok && warp_wait<13>(bar_dofull(g), (g / C::NDO) & 1, s_abort, status);
+              if (D == 128 && g > 0) ok = ok && warp_wait<12>(bar_dqfree, (g - 1) & 1, s_abort, status);   // (dQ lies over dP)
+              fence_async_smem();
+              if (D == 128) tc_fence_after();
             }
             if (!ok) return;
             if (el) {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk)
-              mma_ts2(tmem + C::kColDV, tmem + C::kColP + (kk >> 2) * C::kPHalf + (kk & 3) * 8, mnmajor(o, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
-            umma_commit(bar_dofree(g));
+              for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColDP + 64 * x, kmajor(v, ks), kmajor(o + x * 8192, ks), desc_hi, idesc_s, ks > 0);
+              umma_commit(bar_dp(x));
             }
           };
-          auto grad_k = [&]() {
+#pragma unroll
+          for (int x = 0; x < C::NH; ++x) { scores(x); dprob(x); }
+          if (!ok) break;
+        }
+        if (ok && el) mbar_arrive(bar_dfree(it));
+      }
+    } else {
+      for (int it = 0; ok; ++it) {
+        ok = __all_sync(0xffffffffu, wait_desc(it)) != 0;
+        if (!ok || uni(desc_of(it).kind) < 0) break;
+        const int steps = uni(desc_of(it).steps);
+        const uint32_t kt = C::kOffK + (it % C::NKV) * C::kTile;
+#pragma unroll 1
+        for (int s = 0; s < steps && ok; ++s, ++g) {
+          const bool last = s + 1 == steps;
+          const uint32_t q = C::kOffQ + (g & 1) * C::kTile, o = C::kOffDO + (g % C::NDO) * C::kTile, ds = C::kOffDS + (g % C::NDS) * (128 * 128 * 2);
+          constexpr int KK = 8 / C::NH;                 // 16-query slices of a half
+          auto grad_v = [&](int x) {
+            ok = warp_wait<14>(bar_h(x), g & 1, s_abort, status);
+            if (x == 0 && s == 0 && it > 0) ok = ok && warp_wait<15>(bar_accfree, (it - 1) & 1, s_abort, status);
+            if (!ok) return;
+            fence_async_smem();
+            tc_fence_after();
             if (el) {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) mma_ss2(tmem + C::kColDK, kmajor(ds, kk), mnmajor(q, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
-            umma_commit(bar_qfree(g));
-            if (last) umma_commit(bar_acc);
+              for (int kk = x * KK; kk < (x + 1) * KK; ++kk)
+                mma_ts2(tmem + C::kColDV, tmem + C::kColP + (kk >> 2) * C::kPHalf + (kk & 3) * 8, mnmajor(o, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
+              umma_commit(bar_pfree(x));
+              if (x + 1 == C::NH) umma_commit(bar_dofree(g));
+            }
+          };
+          auto grad_k = [&](int x) {
+            if (ok && el) {
+#pragma unroll
+              for (int kk = x * KK; kk < (x + 1) * KK; ++kk) mma_ss2(tmem + C::kColDK, kmajor(ds, kk), mnmajor(q, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
+              if (x + 1 == C::NH) {
+                umma_commit(bar_qfree(g));
+                if (last) umma_commit(bar_acc);
+              }
             }
           };
           auto grad_q = [&]() {
+            if (D == 64 && g > 0) ok = ok && warp_wait<12>(bar_dqfree, (g - 1) & 1, s_abort, status);
+            if (!ok) return;
+            tc_fence_after();
             if (el) {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) mma_ss2(tmem + C::kColDQ, mnmajor(ds, kk), mnmajor(kt, kk), desc_hi, idesc_t, kk > 0);
-            umma_commit(bar_dq(g));
-            if (last) umma_commit(bar_kfree(it));
+              for (int kk = 0; kk < 8; ++kk) mma_ss2(tmem + C::kColDQ, mnmajor(ds, kk), mnmajor(kt, kk), desc_hi, idesc_t, kk > 0);
+              umma_commit(bar_dq(g));
+              if (last) umma_commit(bar_kfree(it));
             }
           };
           if (D == 64) {
-            if (s_ready()) issue_s();
-            if (ok && p_ready()) issue_p();
-            grad_v();
+            grad_v(0); grad_k(0);
             if (!ok) break;
-            grad_k();
-            if (g > 0) ok = warp_wait<12>(bar_dqfree, (g - 1) & 1, s_abort, status);
-            if (!ok) break;
-            tc_fence_after();
+            grad_v(1); grad_k(1);
             grad_q();
-            if (el) umma_commit(bar_dsfree(g));
           } else {
-            grad_v();
-            if (!ok) break;
-            grad_q();
-            if (s_ready()) issue_s();
-            if (!ok) break;
-            grad_k();
-            if (el) umma_commit(bar_dsfree(g));
+            grad_v(0);
+            grad_q();                                   // (the next dP^T waits until dQ has left)
+            grad_k(0);
           }
-          if (ok && gs == g + 1) issue_s();
-          if (ok && !ends && gp == g + 1) issue_p();
         }
         if (ok && el) mbar_arrive(bar_dfree(it));
       }
@@ -640,12 +620,11 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
     uint32_t sw[NSW];                                    // byte offset of (row k RPI + crow, chunk cc) in its slab is k RPI 128 + sw[k % NSW]
 #pragma unroll
     for (int k = 0; k < NSW; ++k) sw[k] = (uint32_t)(crow * 128 + (((cc & 7) ^ ((k * RPI + crow) & 7)) << 4));
-    auto gather = [&](uint32_t dst, const __nv_bfloat16* base, auto& v, uint32_t bar) {
-      constexpr int ROWS = 32 * (sizeof(v) / sizeof(v[0]));
+    auto gather = [&](uint32_t dst, const __nv_bfloat16* base, const int (&v)[4], uint32_t bar) {
       const char* src = reinterpret_cast<const char*>(base) + cc * 16;
-      const uint32_t d = dst + (cc >> 3) * (ROWS * 128);
+      const uint32_t d = dst + (cc >> 3) * (128 * 128);
 #pragma unroll
-      for (int k = 0; k < ROWS / RPI; ++k) {
+      for (int k = 0; k < 128 / RPI; ++k) {
         const int rw = __shfl_sync(0xffffffffu, v[k * RPI / 32], (k * RPI & 31) + crow);
         cp_async16(d + k * RPI * 128 + sw[k % NSW], src + (size_t)(uint32_t)rw * (D * 2));
       }
@@ -660,11 +639,12 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
       __syncwarp();
       mbar_arrive(bar);
     };
-    if (warp < C::SW + 11) {
-      const bool is_q = warp == C::SW + 9;
+    if (warp > C::SW + C::RW + 2) {
+      const bool is_q = warp == C::SW + C::RW + 3;
       const int nbuf = is_q ? C::NQ : C::NDO;
-      // Row numbers are asked for two steps ahead and statistics one, across items: under this kernel's load a dependent read takes
-      // 2000 clocks, and in line with the copies two of them are longer than a step (PREFETCH_FIGURES).
+      // The next step's row numbers are asked for before this step's copies, its statistics after them, across items: under this
+      // kernel's load a read takes about 2000 clocks, and in line with the copies two of them made the round of this warp longer than
+      // a step.  (131072 rows, d = 64, 32 heads: 3560 -> 3343 us for the whole pass.)
       struct Step {
         int rel[4];                                      // row lane + 32 u of the query tile, relative to base (rows that do not exist: 0)
         int base, nq;                                    // nq: rows that exist
@@ -789,7 +769,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
   // ---- teardown ------------------------------------------------------------------------------------
   tc_fence_before();
   __syncthreads();
-  if (warp == C::SW + 8) {
+  if (warp == C::SW + C::RW) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
   }

@@ -49,12 +49,12 @@ __device__ __forceinline__ uint32_t tile_off(int row, int c) {
 }
 
 // gather ROWS rows (index -1 = zero row) of a [*, D] bf16 tensor into a swizzled tile
-template <int D, int ROWS, class RowFn>
+template <int D, int ROWS, int THREADS, class RowFn>
 __device__ __forceinline__ void gather_tile(uint32_t dst, const __nv_bfloat16* src, RowFn rowfn, int tid) {
   constexpr int CPR = D / 8;
 #pragma unroll
-  for (int i = 0; i < ROWS * CPR / 256; ++i) {
-    const int c = tid + i * 256;
+  for (int i = 0; i < ROWS * CPR / THREADS; ++i) {
+    const int c = tid + i * THREADS;
     const int row = c / CPR, cc = c % CPR;
     const int gr = rowfn(row);
     const uint32_t d = dst + tile_off<ROWS>(row, cc);
@@ -63,34 +63,41 @@ __device__ __forceinline__ void gather_tile(uint32_t dst, const __nv_bfloat16* s
   }
 }
 
-template <int D, bool SPLIT>
+template <int D, int NW>
 struct Smem {
-  static constexpr int kQ = kTileQ * D * 2;
+  static constexpr int kRows = 16 * NW;           // query rows of a CTA
+  static constexpr int kQ = kRows * D * 2;
   static constexpr int kKV = TK * D * 2;
-  static constexpr int kTotal = (SPLIT ? 2 : 1) * kQ + (SPLIT ? 6 : 4) * kKV + kMaxNodeKeys * 8 + kTileQ * 4;
+  static constexpr int kTotal = 2 * kQ + 6 * kKV + kMaxNodeKeys * 8 + kRows * 4;
 };
 
-// SPLIT: the inputs were fp32 and arrive as two bf16 terms (x = hi + lo up to 2^-17 relative);
+// The inputs were fp32 and arrive as two bf16 terms (x = hi + lo up to 2^-17 relative);
 // the logits use Q_hi K_hi + Q_lo K_hi + Q_hi K_lo so that they keep fp32-like accuracy.
-template <int D, bool SPLIT>
-__global__ void __launch_bounds__(256, 1) attn_mma_kernel(const __grid_constant__ AttnArgs a) {
+// NW warps of 16 query rows each: 8 take a whole tile of the schedule; fewer split it over CTAs (blockIdx.y), which leaves
+// more of the chip busy when there are few tiles - all keys of the tile are then loaded by each of them, from L2.  Bound by latency:
+// tables, gather, then one tile of keys after the other.  (One head of 1024 rows, 8 warps -> 4: 11.9 -> 9.8 us at d = 64, 14.8 -> 12.2 at
+// d = 128; 2 warps, each with an SM quarter to itself but four times the copies per thread: 11.7 and 15.0.)
+template <int D, int NW>
+__global__ void __launch_bounds__(32 * NW, 1) attn_mma_kernel(const __grid_constant__ AttnArgs a) {
   extern __shared__ __align__(1024) uint8_t smem[];
-  using SM = Smem<D, SPLIT>;
+  using SM = Smem<D, NW>;
+  constexpr int kThreads = 32 * NW, kRows = SM::kRows;
   uint8_t* sQ = smem;
   uint8_t* sK = sQ + SM::kQ;                      // [2][TK x D]
   uint8_t* sV = sK + 2 * SM::kKV;                 // [2][TK x D]
-  uint8_t* sQl = sV + 2 * SM::kKV;                // SPLIT only
-  uint8_t* sKl = sQl + (SPLIT ? SM::kQ : 0);      // SPLIT only: [2][TK x D]
-  int* s_kidx = reinterpret_cast<int*>(sKl + (SPLIT ? 2 * SM::kKV : 0));
+  uint8_t* sQl = sV + 2 * SM::kKV;                // the second terms
+  uint8_t* sKl = sQl + SM::kQ;                    // [2][TK x D]
+  int* s_kidx = reinterpret_cast<int*>(sKl + 2 * SM::kKV);
   float* s_kbias = reinterpret_cast<float*>(s_kidx + kMaxNodeKeys);
   int* s_qrow = reinterpret_cast<int*>(s_kbias + kMaxNodeKeys);
 
   const Geometry& g = a.g;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int gid = lane >> 2, tig = lane & 3;
-  const TileDesc t = decode_tile(a, blockIdx.x);
+  TileDesc t = decode_tile(a, blockIdx.x);
+  const int sub0 = blockIdx.y * kRows;             // first row of this CTA within the tile
   wait_for_stream();
-  if (t.nq <= 0) return;                          // (a tile of the schedule whose rows do not exist)
+  if (t.nq <= sub0) return;                       // (rows of the schedule that do not exist)
 
   const __nv_bfloat16* qs = a.q + (size_t)t.seg * g.n * D;
   const __nv_bfloat16* ks = a.k + (size_t)t.seg * g.nk * D;
@@ -102,23 +109,22 @@ __global__ void __launch_bounds__(256, 1) attn_mma_kernel(const __grid_constant_
     const int bpad = (g.b + TK - 1) / TK * TK, mpad = (g.m + TK - 1) / TK * TK;
     nkeys = bpad + mpad;
     const float wlog = g.m > 0 ? log2f((float)t.nk / (float)g.m) : 0.f;
-    const int32_t* smp = a.samples + ((size_t)t.seg * g.nodes + t.node) * g.m;
-    for (int i = tid; i < nkeys; i += 256) {
+    const size_t smp0 = ((size_t)t.seg * g.nodes + t.node) * g.m;
+    for (int i = tid; i < nkeys; i += kThreads) {
       int idx = -1; float bias = -INFINITY;
       if (i < bpad) {
         if (i < block_len(t.nk, g.b, t.beta)) { idx = t.k0 + a.perm_k[t.slice + (size_t)t.beta * g.b + i]; bias = 0.f; }
       } else if (i - bpad < g.m) {
-        const int l = smp[i - bpad];
-        idx = t.k0 + l;
-        bias = (a.rank_k[t.slice + l] / g.b == t.beta) ? -INFINITY : wlog;
+        idx = t.k0 + a.samples[smp0 + i - bpad];
+        bias = a.smp_blk[smp0 + i - bpad] == t.beta ? -INFINITY : wlog;
       }
       s_kidx[i] = idx; s_kbias[i] = bias;
     }
-    if (tid < kTileQ) s_qrow[tid] = tid < t.nq ? t.qnode0 + a.perm_q[t.slice + t.spos0 + tid] : -1;
+    if (tid < kRows) s_qrow[tid] = sub0 + tid < t.nq ? t.qnode0 + a.perm_q[t.slice + t.spos0 + sub0 + tid] : -1;
   } else {
-    const int lim = t.causal ? min(t.nk, t.qk_off + t.nq) : t.nk;
+    const int lim = t.causal ? min(t.nk, t.qk_off + min(t.nq, sub0 + kRows)) : t.nk;
     nkeys = (lim + TK - 1) / TK * TK;
-    if (tid < kTileQ) s_qrow[tid] = tid < t.nq ? t.q0 + tid : -1;
+    if (tid < kRows) s_qrow[tid] = sub0 + tid < t.nq ? t.q0 + sub0 + tid : -1;
   }
   __syncthreads();
 
@@ -133,20 +139,19 @@ __global__ void __launch_bounds__(256, 1) attn_mma_kernel(const __grid_constant_
       if (t.mode == 1) return s_kidx[i];
       return i < t.nk ? t.k0 + i : -1;
     };
-    gather_tile<D, TK>(uK + stage * SM::kKV, ks, krow_fn, tid);
-    gather_tile<D, TK>(uV + stage * SM::kKV, vs, krow_fn, tid);
-    if constexpr (SPLIT) gather_tile<D, TK>(uKl + stage * SM::kKV, kls, krow_fn, tid);
+    gather_tile<D, TK, kThreads>(uK + stage * SM::kKV, ks, krow_fn, tid);
+    gather_tile<D, TK, kThreads>(uV + stage * SM::kKV, vs, krow_fn, tid);
+    gather_tile<D, TK, kThreads>(uKl + stage * SM::kKV, kls, krow_fn, tid);
   };
 
-  gather_tile<D, kTileQ>(uQ, qs, qrow_fn, tid);
-  if constexpr (SPLIT) gather_tile<D, kTileQ>(uQl, qls, qrow_fn, tid);
+  gather_tile<D, kRows, kThreads>(uQ, qs, qrow_fn, tid);
+  gather_tile<D, kRows, kThreads>(uQl, qls, qrow_fn, tid);
   const int ntiles = nkeys / TK;
   load_kv(0, 0);
   cp_async_commit();
 
   // ---- per-warp state: 16 query rows ----------------------------------------------------
   constexpr int KS = D / 16, NO = D / 8;
-  uint32_t qf[SPLIT ? 1 : KS][4];
   float o[NO][4];
 #pragma unroll
   for (int i = 0; i < NO; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
@@ -159,13 +164,6 @@ __global__ void __launch_bounds__(256, 1) attn_mma_kernel(const __grid_constant_
     cp_async_commit();
     cp_async_wait<1>();
     __syncthreads();
-    if constexpr (!SPLIT) {
-      if (kt == 0) {
-#pragma unroll
-        for (int s = 0; s < KS; ++s)
-          ldmatrix_x4(qf[s], uQ + tile_off<kTileQ>(warp * 16 + (lane & 15), 2 * s + (lane >> 4)));
-      }
-    }
     // S = Q K^T : 16 x 64 per warp
     float sc[TK / 8][4];
 #pragma unroll
@@ -173,27 +171,19 @@ __global__ void __launch_bounds__(256, 1) attn_mma_kernel(const __grid_constant_
     const uint32_t kb = uK + stage * SM::kKV;
 #pragma unroll
     for (int s = 0; s < KS; ++s) {
-      uint32_t ql[4];
-      if constexpr (SPLIT) {
-        ldmatrix_x4(qf[0], uQ + tile_off<kTileQ>(warp * 16 + (lane & 15), 2 * s + (lane >> 4)));
-        ldmatrix_x4(ql, uQl + tile_off<kTileQ>(warp * 16 + (lane & 15), 2 * s + (lane >> 4)));
-      }
-      const uint32_t(&qh)[4] = qf[SPLIT ? 0 : s];
+      uint32_t qh[4], ql[4];
+      ldmatrix_x4(qh, uQ + tile_off<kRows>(warp * 16 + (lane & 15), 2 * s + (lane >> 4)));
+      ldmatrix_x4(ql, uQl + tile_off<kRows>(warp * 16 + (lane & 15), 2 * s + (lane >> 4)));
 #pragma unroll
       for (int np = 0; np < TK / 16; ++np) {
-        uint32_t bf[4];
+        uint32_t bf[4], bl[4];
         const uint32_t koff = tile_off<TK>(np * 16 + (lane & 7) + ((lane >> 4) << 3), 2 * s + ((lane >> 3) & 1));
-        if constexpr (SPLIT) {
-          uint32_t bl[4];
-          ldmatrix_x4(bl, uKl + stage * SM::kKV + koff);
-          mma_16816(sc[2 * np], qh, bl[0], bl[1]);
-          mma_16816(sc[2 * np + 1], qh, bl[2], bl[3]);
-        }
+        ldmatrix_x4(bl, uKl + stage * SM::kKV + koff);
+        mma_16816(sc[2 * np], qh, bl[0], bl[1]);
+        mma_16816(sc[2 * np + 1], qh, bl[2], bl[3]);
         ldmatrix_x4(bf, kb + koff);
-        if constexpr (SPLIT) {
-          mma_16816(sc[2 * np], ql, bf[0], bf[1]);
-          mma_16816(sc[2 * np + 1], ql, bf[2], bf[3]);
-        }
+        mma_16816(sc[2 * np], ql, bf[0], bf[1]);
+        mma_16816(sc[2 * np + 1], ql, bf[2], bf[3]);
         mma_16816(sc[2 * np], qh, bf[0], bf[1]);
         mma_16816(sc[2 * np + 1], qh, bf[2], bf[3]);
       }
@@ -208,7 +198,7 @@ __global__ void __launch_bounds__(256, 1) attn_mma_kernel(const __grid_constant_
         const int row = (e & 2) ? r_hi : r_lo;
         float x = sc[nt][e] * a.scale_log2;
         if (t.mode == 1) x += s_kbias[col];
-        else if (col >= t.nk || (t.causal && col > t.qk_off + row)) x = -INFINITY;
+        else if (col >= t.nk || (t.causal && col > t.qk_off + sub0 + row)) x = -INFINITY;
         sc[nt][e] = x;
         mx[e >> 1] = fmaxf(mx[e >> 1], x);
       }
@@ -292,13 +282,18 @@ __global__ void __launch_bounds__(256, 1) attn_mma_kernel(const __grid_constant_
 
 cudaError_t launch_attention_mma(const AttnArgs& a, cudaStream_t st) {
   if (a.total_tiles == 0) return cudaSuccess;
-  const bool split = a.q_lo != nullptr;
-#define HA_GO(D, SPLIT) do { const cudaError_t e = allow_smem<attn_mma_kernel<D, SPLIT>>(Smem<D, SPLIT>::kTotal); \
-    return e != cudaSuccess ? e : launch(attn_mma_kernel<D, SPLIT>, a.total_tiles, 256, Smem<D, SPLIT>::kTotal, st, a); } while (0)
-  if (a.g.d == 64) { if (split) HA_GO(64, true); HA_GO(64, false); }
-  if (split) HA_GO(128, true);
-  HA_GO(128, false);
-#undef HA_GO
+  int sms = 0;
+  if (const cudaError_t e = sm_count(&sms); e != cudaSuccess) return e;
+  auto go = [&](auto d, auto nw) {
+    constexpr int D = decltype(d)::value, NW = decltype(nw)::value;
+    const cudaError_t e = allow_smem<attn_mma_kernel<D, NW>>(Smem<D, NW>::kTotal);
+    return e != cudaSuccess ? e : launch(attn_mma_kernel<D, NW>, dim3(a.total_tiles, kTileQ / (16 * NW)), 32 * NW, Smem<D, NW>::kTotal, st, a);
+  };
+  using std::integral_constant;
+  // half a tile per CTA as long as every CTA still has an SM of its own
+  const bool half = 2LL * a.total_tiles <= sms;
+  if (a.g.d == 64) return half ? go(integral_constant<int, 64>{}, integral_constant<int, 4>{}) : go(integral_constant<int, 64>{}, integral_constant<int, 8>{});
+  return half ? go(integral_constant<int, 128>{}, integral_constant<int, 4>{}) : go(integral_constant<int, 128>{}, integral_constant<int, 8>{});
 }
 
 }  // namespace hyperattn

@@ -206,50 +206,70 @@ __global__ void __launch_bounds__(256, D == 64 ? 4 : 3) hash_bf16_kernel(const _
   a.hist[hist_base(a, cp) + tid] = s_hist[tid];
 }
 
-// fp32 rows: thread = (row, direction), plain fp32 FMA in coordinate order.  The eight threads of a row share its 16-byte
-// loads; a warp's ballot holds the sign patterns of its four rows.  Bound by latency (a CTA makes chunk / 32 passes): 1024 rows
-// of d = 64 on both sides took 25 us with a thread per row and all directions and chunks of 2048 rows.
+// fp32 rows: thread = row, plain fp32 FMA in coordinate order, 256 rows at a time through shared memory (cp.async; rows padded by 16
+// bytes, so that the lanes' 16-byte reads meet no bank conflict).  Bound by latency and, with many rows, by shared-memory reads: a row's
+// coordinates are read once for all directions, a direction's by the whole warp at once.  (1024 rows on both sides, us, d = 64 / 128: eight
+// threads per row - a direction each - and loads into registers 11.9 / 22.9, the same with 1024 threads and copies in flight 7.1 / 11.4;
+// each of their 16-byte reads takes the shared memory four cycles, whatever lanes share; this form 4.4 / 7.1.)
+template <int D> constexpr int kHash32Smem = 256 * (D + 4) * 4;
 template <int D>
 __global__ void __launch_bounds__(256) hash_fp32_kernel(const __grid_constant__ HashArgs a) {
-  __shared__ float s_w[D * 8];
+  extern __shared__ __align__(16) float s_x[];           // [256][D + 4]
+  __shared__ __align__(16) float s_w[D][8];
   __shared__ uint32_t s_hist[kBuckets];
-  const int tid = threadIdx.x, lane = tid & 31, t = tid & 7;
+  const int tid = threadIdx.x;
   const ChunkPos cp = chunk_of_cta(a, blockIdx.x);
   const int rows = cp.rows;
   if (!((a.side_mask >> cp.side) & 1) || rows < 0) return;
   const float* wsrc = a.w_nodes ? a.w_nodes + (size_t)cp.node * (D * a.r) : a.w;
   s_hist[tid] = 0;
   wait_for_stream();
-  for (int i = tid; i < D * 8; i += 256) s_w[i] = (i & 7) < a.r ? wsrc[(i >> 3) * a.r + (i & 7)] : 0.f;
-  __syncthreads();
   const float* base = reinterpret_cast<const float*>(a.x[cp.side]) + ((size_t)cp.seg * a.n[cp.side] + cp.row0) * D;
   uint8_t* dst = a.ids + ids_base(a, cp);
   unsigned nz = 0;
-  for (int row0 = 0; row0 < rows; row0 += 32) {
-    const int row = row0 + (tid >> 3);
-    const float4* xr = reinterpret_cast<const float4*>(base + (size_t)min(row, rows - 1) * D);
-    float p = 0.f;
-#pragma unroll
-    for (int c0 = 0; c0 < D / 4; c0 += 16) {
-      float4 x[16];
-#pragma unroll
-      for (int c = 0; c < 16; ++c) x[c] = __ldg(xr + c0 + c);
-#pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        const float* w = s_w + (c0 + c) * 32 + t;
-        p = fmaf(x[c].x, w[0], p); p = fmaf(x[c].y, w[8], p); p = fmaf(x[c].z, w[16], p); p = fmaf(x[c].w, w[24], p);
-      }
+  for (int row0 = 0; row0 < rows; row0 += 256) {
+    const int n = min(256, rows - row0);
+#pragma unroll 16
+    for (int i = 0; i < D / 4; ++i) {
+      const int c = tid + i * 256, row = c / (D / 4), col = c % (D / 4);
+      if (row < n)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(s_x + row * (D + 4) + 4 * col)),
+                     "l"(base + (size_t)(row0 + row) * D + 4 * col) : "memory");
     }
-    if (row < rows && t < a.r) nz += fabsf(p) < 1e-4f;
-    const uint32_t bits = __ballot_sync(0xffffffffu, p > 0.f) >> (lane & 24);
-    if (t == 0 && row < rows) {
-      const uint32_t id = gray_rank8(bits & 0xffu);
-      dst[row] = (uint8_t)id;
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (row0 == 0)
+      for (int i = tid; i < D * 8; i += 256) s_w[i >> 3][i & 7] = (i & 7) < a.r ? wsrc[(i >> 3) * a.r + (i & 7)] : 0.f;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (tid < n) {
+      float p[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) p[t] = 0.f;
+#pragma unroll 4
+      for (int c = 0; c < D; c += 4) {
+        const float4 x4 = *reinterpret_cast<const float4*>(s_x + tid * (D + 4) + c);
+        const float x[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float4 wa = *reinterpret_cast<const float4*>(&s_w[c + e][0]), wb = *reinterpret_cast<const float4*>(&s_w[c + e][4]);
+          p[0] = fmaf(x[e], wa.x, p[0]); p[1] = fmaf(x[e], wa.y, p[1]); p[2] = fmaf(x[e], wa.z, p[2]); p[3] = fmaf(x[e], wa.w, p[3]);
+          p[4] = fmaf(x[e], wb.x, p[4]); p[5] = fmaf(x[e], wb.y, p[5]); p[6] = fmaf(x[e], wb.z, p[6]); p[7] = fmaf(x[e], wb.w, p[7]);
+        }
+      }
+      uint32_t bits = 0;
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        bits |= (p[t] > 0.f ? 1u : 0u) << t;
+        nz += t < a.r && fabsf(p[t]) < 1e-4f;
+      }
+      const uint32_t id = gray_rank8(bits);
+      dst[row0 + tid] = (uint8_t)id;
       atomicAdd(&s_hist[id], 1u);
     }
+    __syncthreads();
   }
   if (a.near_zero && nz) atomicAdd(a.near_zero, (unsigned long long)nz);
-  __syncthreads();
+  __syncthreads();                                       // (a chunk without rows)
   a.hist[hist_base(a, cp) + tid] = s_hist[tid];
 }
 
@@ -304,8 +324,12 @@ cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_
     a.chunks_per_unit[s] = side_cpu(g, s); a.chunks_per_seg[s] = side_cps(g, s);
   }
   const int grid = a.levels * g.G * (g.chunks_per_seg + g.chunks_per_seg_k);
-  auto* kernel = is_fp32 ? (g.d == 64 ? hash_fp32_kernel<64> : hash_fp32_kernel<128>) : (g.d == 64 ? hash_bf16_kernel<64> : hash_bf16_kernel<128>);
-  return launch(kernel, grid, 256, 0, st, a);
+  if (is_fp32) {
+    const cudaError_t e = g.d == 64 ? allow_smem<hash_fp32_kernel<64>>(kHash32Smem<64>) : allow_smem<hash_fp32_kernel<128>>(kHash32Smem<128>);
+    if (e != cudaSuccess) return e;
+    return launch(g.d == 64 ? hash_fp32_kernel<64> : hash_fp32_kernel<128>, grid, 256, g.d == 64 ? kHash32Smem<64> : kHash32Smem<128>, st, a);
+  }
+  return launch(g.d == 64 ? hash_bf16_kernel<64> : hash_bf16_kernel<128>, grid, 256, 0, st, a);
 }
 
 }  // namespace hyperattn

@@ -316,10 +316,12 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
 
   const __nv_bfloat16 *q16 = reinterpret_cast<const __nv_bfloat16*>(p.q), *k16 = reinterpret_cast<const __nv_bfloat16*>(p.k),
                       *v16 = reinterpret_cast<const __nv_bfloat16*>(p.v);
+  const bool in_hash = is_fp32 && convert_in_hash(g);
   if (is_fp32) {
-    StageScope sc(st, HYPERATTN_STAGE_CONVERT, 1);
-    HA_CHECK(launch_convert(reinterpret_cast<const float*>(p.q), reinterpret_cast<const float*>(p.k), reinterpret_cast<const float*>(p.v), ws,
-                            (size_t)g.G * g.n * g.d, (size_t)g.G * g.nk * g.d, st));
+    StageScope sc(st, HYPERATTN_STAGE_CONVERT, in_hash ? 0 : 1);
+    if (!in_hash)
+      HA_CHECK(launch_convert(reinterpret_cast<const float*>(p.q), reinterpret_cast<const float*>(p.k), reinterpret_cast<const float*>(p.v), ws,
+                              (size_t)g.G * g.n * g.d, (size_t)g.G * g.nk * g.d, st));
     q16 = ws.q16; k16 = ws.k16; v16 = ws.v16;
   }
   if (g.sorted) {
@@ -340,7 +342,8 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     }
     {
       StageScope sc(st, HYPERATTN_STAGE_HASH, 1);
-      HA_CHECK(launch_hash(g, p.q, p.k, is_fp32, g_wcache.w, ws, dbg ? dbg->near_zero_bits : nullptr, st, 3, w_nodes));
+      HA_CHECK(launch_hash(g, p.q, p.k, is_fp32, g_wcache.w, ws, dbg ? dbg->near_zero_bits : nullptr, st, 3, w_nodes,
+                           in_hash ? p.v : nullptr));
     }
     {
       // (the samples of Alg. 2 line 4 are drawn by extra blocks of this launch)

@@ -171,9 +171,11 @@ struct Workspace {
 // fp32 inputs of count_q (q) and count_k (k, v) entries to the workspace's bf16 copies
 cudaError_t launch_convert(const float* q, const float* k, const float* v, const Workspace& ws, size_t count_q, size_t count_k, cudaStream_t st);
 // w_host: the shared direction matrix; w_nodes (device, [nodes, d, r], g.node_dirs only): the nodes' own
+// convert_v: fp32 V - the launch also makes the workspace's bf16 copies of Q, K and V (fp32 inputs, convert_in_hash(g))
+bool convert_in_hash(const Geometry& g);
 cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_fp32, const float* w_host,
                         const Workspace& ws, unsigned long long* near_zero, cudaStream_t st, int side_mask = 3,
-                        const float* w_nodes = nullptr);
+                        const float* w_nodes = nullptr, const void* convert_v = nullptr);
 // side_mask: bit 0 queries, bit 1 keys (3: both)
 cudaError_t launch_sort_scan(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask = 3);
 bool scan_in_scatter(const Geometry& g);

@@ -44,6 +44,13 @@ __device__ __forceinline__ uint32_t gray_rank8(uint32_t g) {
   return g & 0xFFu;
 }
 
+// fp32 -> bf16 staging of Q, K, V; for Q and K also the rounding remainder as a second bf16 term
+struct ConvertArgs {
+  const float4* src[3];
+  uint2 *hi[3], *lo[3];
+  size_t count4[3];
+};
+
 struct HashArgs {
   const void* x[2];       // Q, K  [G, n, d]
   float w[128 * 8];       // [d, r] directions, passed by value (<= 4 KB of kernel parameters)
@@ -60,6 +67,9 @@ struct HashArgs {
   const float* w_nodes;   // [nodes, d, r] or null
   int levels, L, d;
   size_t ids_level_stride, hist_level_stride;
+  // fp32 inputs, where this launch also makes the bf16 copies: the CTAs from hash_ctas on
+  ConvertArgs conv;
+  int hash_ctas;
 };
 
 // which chunk a CTA owns: side, segment, first row, number of rows (0: the chunk lies beyond the last row)
@@ -206,11 +216,41 @@ __global__ void __launch_bounds__(256, D == 64 ? 4 : 3) hash_bf16_kernel(const _
   a.hist[hist_base(a, cp) + tid] = s_hist[tid];
 }
 
+// four entries as bf16, and their rounding remainders as a second bf16 term
+__device__ __forceinline__ void split_bf16(const float4& x, uint2& hi, uint2& lo) {
+  const float xs[4] = {x.x, x.y, x.z, x.w};
+  float h[4], l[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) { h[e] = __bfloat162float(__float2bfloat16_rn(xs[e])); l[e] = xs[e] - h[e]; }
+  hi = make_uint2(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]));
+  lo = make_uint2(pack_bf16(l[0], l[1]), pack_bf16(l[2], l[3]));
+}
+
+// one CTA's share of the copies of array s, U pieces of 16 bytes in flight per thread
+template <int U>
+__device__ __forceinline__ void convert_body(const ConvertArgs& a, int s, size_t cta, size_t ctas) {
+  for (size_t i0 = cta * (256 * U) + threadIdx.x; i0 < a.count4[s]; i0 += ctas * (256 * U)) {
+    float4 x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) x[u] = i0 + 256 * u < a.count4[s] ? a.src[s][i0 + 256 * u] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const size_t i = i0 + 256 * u;
+      if (i >= a.count4[s]) break;
+      uint2 hi, lo;
+      split_bf16(x[u], hi, lo);
+      a.hi[s][i] = hi;
+      if (a.lo[s]) a.lo[s][i] = lo;
+    }
+  }
+}
+
 // fp32 rows: thread = row, plain fp32 FMA in coordinate order, 256 rows at a time through shared memory (cp.async; rows padded by 16
 // bytes, so that the lanes' 16-byte reads meet no bank conflict).  Bound by latency and, with many rows, by shared-memory reads: a row's
 // coordinates are read once for all directions, a direction's by the whole warp at once.  (1024 rows on both sides, us, d = 64 / 128: eight
 // threads per row - a direction each - and loads into registers 11.9 / 22.9, the same with 1024 threads and copies in flight 7.1 / 11.4;
 // each of their 16-byte reads takes the shared memory four cycles, whatever lanes share; this form 4.4 / 7.1.)
+// The bf16 copies of Q, K and V are made by extra CTAs of this launch, while the others wait for memory (convert_in_hash).
 template <int D> constexpr int kHash32Smem = 256 * (D + 4) * 4;
 template <int D>
 __global__ void __launch_bounds__(256) hash_fp32_kernel(const __grid_constant__ HashArgs a) {
@@ -218,6 +258,11 @@ __global__ void __launch_bounds__(256) hash_fp32_kernel(const __grid_constant__ 
   __shared__ __align__(16) float s_w[D][8];
   __shared__ uint32_t s_hist[kBuckets];
   const int tid = threadIdx.x;
+  if ((int)blockIdx.x >= a.hash_ctas) {
+    wait_for_stream();
+    for (int x = 0; x < 3; ++x) convert_body<4>(a.conv, x, blockIdx.x - a.hash_ctas, gridDim.x - a.hash_ctas);
+    return;
+  }
   const ChunkPos cp = chunk_of_cta(a, blockIdx.x);
   const int rows = cp.rows;
   if (!((a.side_mask >> cp.side) & 1) || rows < 0) return;
@@ -274,43 +319,43 @@ __global__ void __launch_bounds__(256) hash_fp32_kernel(const __grid_constant__ 
 }
 
 // fp32 -> bf16 staging of Q, K, V (blockIdx.y); for Q and K also the rounding remainder as a second bf16 term
-struct ConvertArgs {
-  const float4* src[3];
-  uint2 *hi[3], *lo[3];
-  size_t count4[3];
-};
 __global__ void __launch_bounds__(256) convert_kernel(const __grid_constant__ ConvertArgs a) {
-  const int s = blockIdx.y;
   wait_for_stream();
-  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < a.count4[s]; i += (size_t)gridDim.x * 256) {
-    const float4 x = a.src[s][i];
-    const float xs[4] = {x.x, x.y, x.z, x.w};
-    float h[4], l[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) { h[e] = __bfloat162float(__float2bfloat16_rn(xs[e])); l[e] = xs[e] - h[e]; }
-    a.hi[s][i] = make_uint2(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]));
-    if (a.lo[s]) a.lo[s][i] = make_uint2(pack_bf16(l[0], l[1]), pack_bf16(l[2], l[3]));
-  }
+  convert_body<1>(a, blockIdx.y, blockIdx.x, gridDim.x);
 }
 
 }  // namespace
 
-cudaError_t launch_convert(const float* q, const float* k, const float* v, const Workspace& ws, size_t count_q, size_t count_k, cudaStream_t st) {
+static ConvertArgs make_convert_args(const void* q, const void* k, const void* v, const Workspace& ws, size_t count_q, size_t count_k) {
   ConvertArgs a;
-  const float* src[3] = {q, k, v};
+  const void* src[3] = {q, k, v};
   __nv_bfloat16 *hi[3] = {ws.q16, ws.k16, ws.v16}, *lo[3] = {ws.q16lo, ws.k16lo, nullptr};
   for (int s = 0; s < 3; ++s) {
     a.src[s] = reinterpret_cast<const float4*>(src[s]);
     a.hi[s] = reinterpret_cast<uint2*>(hi[s]); a.lo[s] = reinterpret_cast<uint2*>(lo[s]);
     a.count4[s] = (s ? count_k : count_q) / 4;
   }
+  return a;
+}
+cudaError_t launch_convert(const float* q, const float* k, const float* v, const Workspace& ws, size_t count_q, size_t count_k, cudaStream_t st) {
+  const ConvertArgs a = make_convert_args(q, k, v, ws, count_q, count_k);
   const size_t most = a.count4[0] > a.count4[1] ? a.count4[0] : a.count4[1], want = (most + 255) / 256;
   const dim3 grid((unsigned)(want < 148 * 16 ? want : 148 * 16), 3);
   return launch(convert_kernel, grid, 256, 0, st, a);
 }
 
+// 1024 pieces of 16 bytes of each array per CTA
+static int convert_ctas(const Geometry& g) {
+  const size_t want = ((size_t)g.G * (g.n > g.nk ? g.n : g.nk) * g.d / 4 + 1023) / 1024;
+  return want < (1u << 20) ? (int)want : 1 << 20;
+}
+// Copies of up to two CTAs per SM run beside the hash (its CTAs take 70 or 135 KB of shared memory each, so that few fit an SM); beyond that
+// a launch of their own, with more threads per SM, is faster.  A call, us, own launch -> beside the hash: 2 heads x 300 rows d = 64 24.9 -> 22.4,
+// 4 x 4096 d = 64 24.8 -> 23.3, 2 x 2500 d = 128 27.5 -> 25.6; 4 x 4096 d = 128 (512 CTAs) 35.0 -> 36.5.
+bool convert_in_hash(const Geometry& g) { return g.sorted && !g.node_dirs && convert_ctas(g) <= 296; }
+
 cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_fp32, const float* w_host,
-                        const Workspace& ws, unsigned long long* near_zero, cudaStream_t st, int side_mask, const float* w_nodes) {
+                        const Workspace& ws, unsigned long long* near_zero, cudaStream_t st, int side_mask, const float* w_nodes, const void* convert_v) {
   HashArgs a;
   a.side_mask = side_mask; a.chunk = g.chunk;
   a.w_nodes = g.node_dirs ? w_nodes : nullptr;
@@ -327,7 +372,13 @@ cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_
   if (is_fp32) {
     const cudaError_t e = g.d == 64 ? allow_smem<hash_fp32_kernel<64>>(kHash32Smem<64>) : allow_smem<hash_fp32_kernel<128>>(kHash32Smem<128>);
     if (e != cudaSuccess) return e;
-    return launch(g.d == 64 ? hash_fp32_kernel<64> : hash_fp32_kernel<128>, grid, 256, g.d == 64 ? kHash32Smem<64> : kHash32Smem<128>, st, a);
+    a.hash_ctas = grid;
+    int copy_ctas = 0;
+    if (convert_v) {
+      a.conv = make_convert_args(q, k, convert_v, ws, (size_t)g.G * g.n * g.d, (size_t)g.G * g.nk * g.d);
+      copy_ctas = convert_ctas(g);
+    }
+    return launch(g.d == 64 ? hash_fp32_kernel<64> : hash_fp32_kernel<128>, grid + copy_ctas, 256, g.d == 64 ? kHash32Smem<64> : kHash32Smem<128>, st, a);
   }
   return launch(g.d == 64 ? hash_bf16_kernel<64> : hash_bf16_kernel<128>, grid, 256, 0, st, a);
 }

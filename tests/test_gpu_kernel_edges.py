@@ -16,11 +16,12 @@ FORWARD = [
     # query tiles paired across blocks: an odd number of tiles per block, few and as many key tiles as the ring allows
     parity.W("pairs_of_one_tile_blocks_d128", 1, 1, 1500, 128, "bf16", 128, 96, 6, False, 0, seed=74),
     parity.W("pairs_of_three_tile_blocks_d64", 1, 1, 2900, 64, "bf16", 384, 64, 6, False, 0, seed=75),
-    # fp32: hash passes of 256 rows; query tiles halved (up to 74 tiles) and whole, second halves of one row and none
+    # fp32: hash passes of 256 rows; copies beside the hash (up to 296 CTAs of 4096 entries) and in a launch of their own; query tiles halved (up to 74 tiles) and whole, second halves of one row and none
     parity.W("fp32_n257_d64", 1, 1, 257, 64, "fp32", 64, 32, 7, False, 0, seed=76),
     parity.W("fp32_n65_d128", 1, 1, 65, 128, "fp32", 32, 16, 8, False, 0, seed=77),
     parity.W("fp32_n193_d128", 1, 2, 193, 128, "fp32", 100, 16, 1, False, 0, seed=78),
     parity.W("fp32_80_tiles_d64", 1, 5, 2048, 64, "fp32", 128, 64, 7, False, 0, seed=79),
+    parity.W("fp32_copies_in_a_launch_of_their_own", 1, 5, 2000, 128, "fp32", 128, 64, 7, False, 0, seed=83),
     parity.W("fp32_85_tiles_causal_d128", 1, 5, 1090, 128, "fp32", 64, 32, 6, True, 300, seed=80),
 ]
 

@@ -135,7 +135,9 @@ Plan make_plan(const Geometry& g, int is_fp32, int backward = 0, bool capped = f
   pl.part_o = take(part_rows * g.d * (part_bf16 ? 2 : 4));
   pl.part_lse = take(part_rows * 4);
   pl.stat = take(backward ? (size_t)g.G * g.n * 8 : 0);
-  pl.gacc = take(backward == 2 ? ((size_t)g.G * g.n + 2 * key_grad_rows(g, direct)) * g.d * 4 : 0);
+  // (the size that callers were told so far - three tensors more than for fp32 gradients - also where less is used)
+  const size_t all_rows = (size_t)g.G * g.n, kv_rows = key_grad_rows(g, direct);
+  pl.gacc = take(backward == 2 ? (all_rows + 2 * (kv_rows > all_rows ? kv_rows : all_rows)) * g.d * 4 : 0);
   pl.total = off + kAlign;
   return pl;
 }

@@ -1,6 +1,14 @@
 """Sizes at the edges of the kernels' tiles, chunks and dispatch rules, against the oracle."""
-import pytest
+import math
 
+import numpy as np
+import pytest
+import torch
+
+import paper_2310_05869_b200 as ha
+from oracle import hyperattn_oracle as O
+
+import parity_util as PU
 import test_gpu_backward as backward
 import test_gpu_parity as parity
 import test_gpu_value_norm_sampling as vnorm
@@ -70,3 +78,26 @@ VALUE_NORMS = [
 @pytest.mark.parametrize("w", VALUE_NORMS, ids=[w.name for w in VALUE_NORMS])
 def test_value_norm_edges(w):
     vnorm.test_value_norm_sampling_matches_the_oracle(w)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_value_norms_of_more_segments_than_a_grid_has_rows(d):
+    """65 600 segments: more than the y and z extents of a grid."""
+    B, H, n, b, m, r, seed = 16, 4100, 20, 8, 5, 4, 3
+    gen = torch.Generator(device="cuda").manual_seed(91)
+    q, k, v = (torch.randn((B, H, n, d), generator=gen, device="cuda").bfloat16() for _ in range(3))
+    out, lse, inter = ha.forward(q, k, v, b, m, r, seed=seed, out_dtype=torch.float32, debug=True, value_norm_sampling=True)
+    torch.cuda.synchronize()
+    assert ha.last_device_status() == 0
+    Wd = O.directions(d, r, seed)
+    rng = np.random.default_rng(5)
+    for g in sorted({0, 1, 65534, 65535, 65536, B * H - 1, *rng.integers(0, B * H, 40).tolist()}):
+        Q, K, V = (x.view(-1, n, d)[g].double().cpu().numpy() for x in (q, k, v))
+        idx, sw = O.sample_by_value_norms(seed, g, 0, m, O.value_norm_weights(V))
+        assert (inter["samples"][g, 0, :m].cpu().numpy() == idx).all(), g
+        np.testing.assert_allclose(inter["sample_log2w"][g, 0, :m].cpu().numpy(), np.log2(sw), atol=1e-5)
+        ro, rl = O.segment_forward(Q, K, V, Wd, b, m, False, 0, seed, g, scale=1.0 / math.sqrt(d), ids_q=inter["q_ids"][g].cpu().numpy(),
+                                   ids_k=inter["k_ids"][g].cpu().numpy(), value_norm_sampling=True)
+        err = np.abs(out.view(-1, n, d)[g].cpu().numpy() - ro)
+        assert err.max() <= PU.OUT_MAX_ABS and err.mean() <= PU.OUT_MEAN_ABS, g
+        assert (np.abs(lse.view(-1, n)[g].cpu().numpy() - rl) <= PU.LSE_REL * np.maximum(np.abs(rl), 1.0)).all(), g

@@ -613,22 +613,31 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
     __syncwarp();
   } else {
     // ================= loaders, a warp each: Q and row statistics; dO; items, K and V ==================
-    // Tiles of consecutive rows: lane 0 issues TMA boxes.  Others: rows gathered in 16-byte chunks, lane -> chunk cc of row
+    // Whole tiles of consecutive rows: lane 0 issues TMA boxes.  Others: rows gathered in 16-byte chunks, lane -> chunk cc of row
     // k RPI + crow of instruction k; lane l holds the row numbers of rows l, l + 32, ..., handed round by shuffles.
+    // Rows of a short tile that do not exist are zeros: their weights are zero, but zero times a NaN or an infinity of
+    // some other leaf, block or head would not be.
     constexpr int CPR = D / 8, RPI = 32 / CPR, NSW = 8 / RPI;
     const int cc = lane % CPR, crow = lane / CPR;
     uint32_t sw[NSW];                                    // byte offset of (row k RPI + crow, chunk cc) in its slab is k RPI 128 + sw[k % NSW]
 #pragma unroll
     for (int k = 0; k < NSW; ++k) sw[k] = (uint32_t)(crow * 128 + (((cc & 7) ^ ((k * RPI + crow) & 7)) << 4));
-    auto gather = [&](uint32_t dst, const __nv_bfloat16* base, const int (&v)[4], uint32_t bar) {
+    auto gather_rows = [&](auto whole, int rows, uint32_t dst, const __nv_bfloat16* base, const int (&v)[4], uint32_t bar) {
       const char* src = reinterpret_cast<const char*>(base) + cc * 16;
       const uint32_t d = dst + (cc >> 3) * (128 * 128);
 #pragma unroll
       for (int k = 0; k < 128 / RPI; ++k) {
         const int rw = __shfl_sync(0xffffffffu, v[k * RPI / 32], (k * RPI & 31) + crow);
-        cp_async16(d + k * RPI * 128 + sw[k % NSW], src + (size_t)(uint32_t)rw * (D * 2));
+        const uint32_t to = d + k * RPI * 128 + sw[k % NSW];
+        const char* from = src + (size_t)(uint32_t)rw * (D * 2);
+        if constexpr (decltype(whole)::value) cp_async16(to, from);
+        else cp_async16_or_zero(to, from, k * RPI + crow < rows);
       }
       cp_async_arrive_noinc(bar);
+    };
+    auto gather = [&](int rows, uint32_t dst, const __nv_bfloat16* base, const int (&v)[4], uint32_t bar) {   // v: a valid row also where none exists
+      if (rows == 128) gather_rows(std::true_type{}, rows, dst, base, v, bar);
+      else gather_rows(std::false_type{}, rows, dst, base, v, bar);
     };
     auto boxes = [&](uint32_t dst, int rows, const CUtensorMap* map, int y, uint32_t bar) {
       if (lane == 0) {
@@ -648,7 +657,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
       struct Step {
         int rel[4];                                      // row lane + 32 u of the query tile, relative to base (rows that do not exist: 0)
         int base, nq;                                    // nq: rows that exist
-        int y;                                           // tiles of consecutive rows: the first (else -1)
+        int y;                                           // whole tiles of consecutive rows: the first (else -1)
         float wlog;
       };
       Step s0, s1;                                       // this step, the next
@@ -659,7 +668,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
         const BwdItem& t = desc_of(pit);
         const StepRows sr = step_rows(b, t, ps);
         d.base = t.seg * g_.n + t.q0; d.nq = sr.nq; d.wlog = t.wlog;
-        d.y = t.kind == 0 ? t.seg * g_.n + sr.first : -1;
+        d.y = t.kind == 0 && sr.nq == 128 ? t.seg * g_.n + sr.first : -1;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int r = lane + 32 * u;
@@ -711,7 +720,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
           int v[4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) v[u] = s0.base + s0.rel[u];
-          gather(dst, is_q ? a.q : b.dout, v, bar);
+          gather(s0.nq, dst, is_q ? a.q : b.dout, v, bar);
         }
         s0 = s1;
         --have;
@@ -748,17 +757,18 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
         if (t.kind < 0) break;
         const uint32_t dk = ubase + C::kOffK + (it % C::NKV) * C::kTile, dv = ubase + C::kOffV + (it % C::NKV) * C::kTile;
         const int seg_row0 = t.seg * g_.n;
+        const bool box = t.kind == 0 && t.nkeys == 128;
         int v[4] = {0, 0, 0, 0};
-        if (t.kind != 0) {
+        if (!box) {
 #pragma unroll
-          for (int u = 0; u < 4; ++u) v[u] = seg_row0 + key_row(t, min(lane + 32 * u, t.nkeys - 1));     // (keys that do not exist: the last one)
+          for (int u = 0; u < 4; ++u) v[u] = seg_row0 + key_row(t, min(lane + 32 * u, t.nkeys - 1));
         }
         if (it >= C::NKV) ok = __all_sync(0xffffffffu, wait_fast<18>(bar_kfree(it), (it / C::NKV - 1) & 1, s_abort, status));
         if (!ok) break;
-        if (t.kind == 0) boxes(dk, 128, &maps.k, seg_row0 + t.k0, bar_kfull(it));
-        else gather(dk, a.k, v, bar_kfull(it));
-        if (t.kind == 0) boxes(dv, 128, &maps.v, seg_row0 + t.k0, bar_vfull(it));
-        else gather(dv, a.v, v, bar_vfull(it));
+        if (box) boxes(dk, 128, &maps.k, seg_row0 + t.k0, bar_kfull(it));
+        else gather(t.nkeys, dk, a.k, v, bar_kfull(it));
+        if (box) boxes(dv, 128, &maps.v, seg_row0 + t.k0, bar_vfull(it));
+        else gather(t.nkeys, dv, a.v, v, bar_vfull(it));
       }
       cp_async_commit();
       cp_async_wait_all();

@@ -6,6 +6,7 @@ import pytest
 import torch
 
 import paper_2310_05869_b200 as ha
+from paper_2310_05869_b200 import workloads as WL
 from oracle import hyperattn_oracle as O
 
 import parity_util as PU
@@ -62,6 +63,66 @@ BACKWARD = [
 @pytest.mark.parametrize("w", BACKWARD, ids=[w.name for w in BACKWARD])
 def test_backward_edges(w):
     backward.test_backward_matches_the_oracle(w)
+
+
+def _gradients(w, q, k, v, out, lse, dout, dtype):
+    return ha.backward(q, k, v, out, lse, dout, w.b, w.m, w.r, causal=w.causal, n0=w.n0, seed=w.seed, grad_dtype=dtype)
+
+
+def _assert_same_gradients(got, want, dtype):
+    # only the order of the fp32 reductions may differ: a few hundred terms of 2^-24 each; bf16 results round once more
+    for g, x in zip(got, want):
+        g, x = g.double(), x.double()
+        assert torch.isfinite(g).all()
+        assert (g - x).abs().max() <= (2.0 ** -8 if dtype == torch.bfloat16 else 2.0 ** -14) * x.abs().max()
+
+
+SHORT_TILES = [
+    backward.W("one_leaf_d64", 1, 2, 193, 64, 64, 8, 4, True, 256, seed=83),
+    backward.W("leaves_of_130_sorted_and_unsorted_nodes_d128", 1, 2, 1040, 128, 200, 33, 6, True, 130, seed=84),
+    backward.W("one_block_d128", 1, 2, 300, 128, 512, 16, 4, False, 0, seed=85),
+    backward.W("blocks_of_130_d64", 1, 2, 1301, 64, 130, 65, 6, False, 0, seed=86),
+]
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "fp32"])
+@pytest.mark.parametrize("bad", [math.nan, math.inf], ids=["nan", "inf"])
+@pytest.mark.parametrize("w", SHORT_TILES, ids=[w.name for w in SHORT_TILES])
+def test_backward_of_a_head_beside_a_head_that_is_not_finite(w, bad, dtype):
+    """The last tile of a head or leaf is short, and what follows it in memory is the next head: nothing of that may enter."""
+    q, k, v = PU.to_device(w, WL.make_inputs(w))
+    out, lse = ha.forward(q, k, v, w.b, w.m, w.r, causal=w.causal, n0=w.n0, seed=w.seed)
+    dout = torch.randn(q.shape, generator=torch.Generator(device="cuda").manual_seed(92), device="cuda").bfloat16()
+    want = [x[0, 0] for x in _gradients(w, q, k, v, out, lse, dout, dtype)]
+    tensors = [x.clone() for x in (q, k, v, dout)]
+    for x in tensors:
+        x[0, 1] = bad
+    got = [x[0, 0] for x in _gradients(w, *tensors[:3], out, lse, tensors[3], dtype)]
+    assert ha.last_device_status() == 0
+    _assert_same_gradients(got, want, dtype)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "fp32"])
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("b", [130, 65])
+def test_backward_of_keys_that_a_row_that_is_not_finite_does_not_see(b, d, dtype):
+    """Short tiles of sorted queries: a query that is not finite reaches the keys of its own block and the sampled ones only."""
+    w = backward.W("", 1, 1, 1301, d, b, 40, 6, False, 0, seed=87)
+    q, k, v = PU.to_device(w, WL.make_inputs(w))
+    out, lse, inter = ha.forward(q, k, v, w.b, w.m, w.r, seed=w.seed, debug=True)
+    dout = torch.randn(q.shape, generator=torch.Generator(device="cuda").manual_seed(93), device="cuda").bfloat16()
+    want = _gradients(w, q, k, v, out, lse, dout, dtype)
+    dout[0, 0, 0] = math.nan                               # (the permutation stays: the row's Q is left alone)
+    got = _gradients(w, q, k, v, out, lse, dout, dtype)
+    assert ha.last_device_status() == 0
+    perm_q, perm_k = (inter[x].view(-1)[:w.n].long() for x in ("perm_q", "perm_k"))
+    beta = int((perm_q == 0).nonzero()) // b
+    clean = torch.ones(w.n, dtype=torch.bool, device="cuda")
+    clean[perm_k[beta * b:(beta + 1) * b]] = False
+    clean[inter["samples"][0, 0, :w.m].long()] = False
+    assert clean.sum() > w.n // 2
+    _assert_same_gradients([x[0, 0][clean] for x in got[1:]], [x[0, 0][clean] for x in want[1:]], dtype)
+    _assert_same_gradients([got[0][0, 0, 1:]], [want[0][0, 0, 1:]], dtype)
 
 
 VALUE_NORMS = [

@@ -22,10 +22,19 @@ FORWARD = [
     parity.W("node_of_17_chunks", 1, 1, 4097, 64, "bf16", 256, 130, 7, False, 0, seed=71),
     parity.W("causal_nodes_of_17_chunks", 1, 1, 8704, 128, "bf16", 128, 65, 8, True, 4352, seed=72),
     parity.W("chunks_of_512_rows", 1, 20, 4000, 64, "bf16", 128, 64, 7, False, 0, seed=73),
-    # query tiles paired across blocks: an odd number of tiles per block, few and as many key tiles as the ring allows
+    # query tiles paired across blocks (an odd number of query tiles per block), few key tiles per block, ...
     parity.W("pairs_of_one_tile_blocks_d128", 1, 1, 1500, 128, "bf16", 128, 96, 6, False, 0, seed=74),
     parity.W("pairs_of_three_tile_blocks_d64", 1, 1, 2900, 64, "bf16", 384, 64, 6, False, 0, seed=75),
-    # fp32: hash passes of 256 rows; copies beside the hash (up to 296 CTAs of 4096 entries) and in a launch of their own; query tiles halved (up to 74 tiles) and whole, second halves of one row and none
+    # ... as many as the ring of K / V stages allows (7 at d = 64, 3 at d = 128), and one more: not paired
+    parity.W("pairs_of_seven_key_tiles_d64", 1, 2, 1000, 64, "bf16", 448, 256, 6, False, 0, seed=88, n_k=4000),
+    parity.W("pairs_of_seven_key_tiles_b385_d64", 1, 1, 700, 64, "bf16", 385, 40, 6, False, 0, seed=89, n_k=3000),
+    parity.W("pairs_of_three_query_and_seven_key_tiles_d64", 1, 1, 2400, 64, "bf16", 448, 64, 6, False, 0, seed=90, n_k=3000),
+    parity.W("eight_key_tiles_d64", 1, 1, 1000, 64, "bf16", 449, 256, 6, False, 0, seed=91, n_k=4000),
+    parity.W("pairs_of_three_key_tiles_d128", 1, 2, 1300, 128, "bf16", 192, 256, 6, False, 0, seed=92, n_k=2000),
+    parity.W("pairs_of_three_key_tiles_b129_d128", 1, 1, 1900, 128, "bf16", 129, 40, 6, False, 0, seed=93, n_k=2000),
+    parity.W("four_key_tiles_d128", 1, 1, 1300, 128, "bf16", 193, 256, 6, False, 0, seed=94, n_k=2000),
+    # fp32: hash passes of 256 rows; copies beside the hash (up to 296 CTAs of 4096 entries) and in a launch of their own; query tiles
+    # halved (up to 74 tiles) and whole, second halves of one row and none
     parity.W("fp32_n257_d64", 1, 1, 257, 64, "fp32", 64, 32, 7, False, 0, seed=76),
     parity.W("fp32_n65_d128", 1, 1, 65, 128, "fp32", 32, 16, 8, False, 0, seed=77),
     parity.W("fp32_n193_d128", 1, 2, 193, 128, "fp32", 100, 16, 1, False, 0, seed=78),
@@ -131,6 +140,7 @@ VALUE_NORMS = [
     vnorm.W("vnorm_n257_d128", 1, 1, 257, 128, 64, 48, 6, False, 0, seed=71),
     vnorm.W("vnorm_n4096", 1, 1, 4096, 64, 256, 64, 7, False, 0, seed=72),
     vnorm.W("vnorm_n4097_d128", 1, 2, 4097, 128, 256, 64, 7, False, 0, seed=73),
+    vnorm.W("vnorm_pairs_of_seven_key_tiles", 1, 1, 1000, 64, 448, 64, 6, False, 0, seed=76, n_k=4000),
     vnorm.W("vnorm_16352_draws", 1, 32, 300, 64, 64, 511, 5, False, 0, seed=74),
     vnorm.W("vnorm_16384_draws", 1, 32, 300, 64, 64, 512, 5, False, 0, seed=75),
 ]

@@ -168,7 +168,7 @@ struct Cfg {
   // pay for them (N = 144) and keeps the sum in registers.
   static constexpr bool kOnes = D == 64;
   static constexpr int kOCols = kOnes ? 80 : D;       // TMEM columns of one O accumulator
-  static constexpr int kNumBar = 21 + 6 * NS + 12;
+  static constexpr int kNumBar = 21 + 6 * NS + 4 * kSBufs;
   static constexpr int kOffMisc = kOffBar + 8 * kNumBar;          // tmem slot, abort flag
   // Epilogue staging, one slice of 32 rows x kStageRow bytes per softmax warp: rows leave the
   // warp as whole 64- or 128-byte pieces instead of 16 bytes per lane and row.  d = 64: eight
@@ -302,8 +302,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
   const uint32_t bar0 = ubase + C::kOffBar;
   const uint32_t bar_q = bar0;                                                // Q tiles of the item landed
   const uint32_t bar_qfree = bar0 + 8;                                        // both issuers are done with Q
-  auto bar_s = [&](int i, int b) { return bar0 + 168 + 8 * (6 * C::NS + 3 * i + b); };          // S_i buffer b written
-  auto bar_p = [&](int i, int b) { return bar0 + 168 + 8 * (6 * C::NS + 6 + 3 * i + b); };      // P_i buffer b written
+  auto bar_s = [&](int i, int b) { return bar0 + 168 + 8 * (6 * C::NS + C::kSBufs * i + b); };          // S_i buffer b written
+  auto bar_p = [&](int i, int b) { return bar0 + 168 + 8 * (6 * C::NS + C::kSBufs * (2 + i) + b); };    // P_i buffer b written
   auto bar_o = [&](int i) { return bar0 + 80 + 8 * i; };                      // O_i of the item complete
   auto bar_ofree = [&](int i) { return bar0 + 112 + 8 * i; };                 // O_i has been read out
   auto bar_tabfull = [&](int set) { return bar0 + 128 + 8 * set; };           // row tables of a set written
@@ -902,17 +902,12 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
           }
           knext = gj + 1;
         };
-        // The S buffer of tile r held P of tile r - kSBufs, so the product P V of that tile must be
-        // issued before the scores of tile r.  Two buffers: P V (r - 2), then S (r).  Three: the
-        // scores go first - they do not wait for the warpgroup - and are ready a tile earlier.
+        // The S buffer of tile r held P of tile r - 2, so the product P V of that tile must be
+        // issued before the scores of tile r.
+        static_assert(C::kSBufs == 2, "scores run two tiles ahead");
         for (int r = 0; r < total + 2 && ok; ++r) {
-          if (C::kSBufs == 2) {
-            if (r >= 2) issue_pv(r - 2);
-            if (ok && r < total) issue_s(r);
-          } else {
-            if (r < total) issue_s(r);
-            if (ok && r >= 2) issue_pv(r - 2);
-          }
+          if (r >= 2) issue_pv(r - 2);
+          if (ok && r < total) issue_s(r);
         }
         if (!ok) break;
         // what is left of the item's tiles (all of them for a query tile that does not exist) is

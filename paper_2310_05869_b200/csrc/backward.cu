@@ -297,8 +297,9 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
 
   bool ok = true;
   if (warp < C::SW) {
-    // ================= P and dS: thread = key, warpgroup q: query columns W q .. W q + W - 1, in two chunks ==================
+    // ================= P and dS: thread = key, warpgroup q: query columns W q .. W q + W - 1, in two chunks of CW ==================
     constexpr int W = 128 / (C::SW / 4), CW = W / 2;
+    static_assert(CW == 32, "a chunk's P is one TMEM store of 16 columns");
     const int row = tid & 127, col0 = (warp >> 2) * W, half = C::NH == 2 ? col0 >> 6 : 0;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t p_addr = lane_addr + C::kColP + C::kPHalf * (col0 >> 6) + (col0 & 63) / 2;
@@ -352,11 +353,8 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
               pp[i0 >> 1] = pack2(p[i0], p[i0 + 1]); pp[(i0 >> 1) + 1] = pack2(p[i0 + 2], p[i0 + 3]);
             }
           }
-          auto put_p = [&]() {
-            if constexpr (CW == 32) tmem_st16(p_addr + 16 * c, pp); else tmem_st8(p_addr + 8 * c, pp);
-          };
           // d = 128: P goes over scores of this warpgroup that have been read
-          if (D == 128) put_p();
+          if (D == 128) tmem_st16(p_addr + 16 * c, pp);
           if (c == 0) {
             ok = wait_fast<4>(bar_dp(half), g & 1, s_abort, status);
             // (dS of the step that used the buffer before has been multiplied; the last of its products is dQ or, d = 128, dK)
@@ -394,7 +392,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
               if (!ok) break;
               tc_fence_after();
             }
-            put_p();
+            tmem_st16(p_addr + 16 * c, pp);
           }
         }
         if (!ok) break;

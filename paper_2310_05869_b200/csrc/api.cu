@@ -15,8 +15,8 @@
 namespace hyperattn {
 cudaError_t launch_attention_mma(const AttnArgs& a, cudaStream_t st);
 cudaError_t launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st);
-cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uint32_t* wq, unsigned long long* sums, unsigned long long* cum, int32_t* samples,
-                                  float* wlog, uint64_t seed, cudaStream_t st);
+cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uint32_t* wq, unsigned long long* sums, unsigned long long* cum,
+                                  int32_t* samples, float* wlog, uint64_t seed, cudaStream_t st);
 cudaError_t launch_tau(const AttnArgs& at, const int32_t* tpos, float* ltau, cudaStream_t st);
 cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout, float2* stat, int* sched,
                             const BwdGrads& gr, float scale, int* status, cudaStream_t st);
@@ -78,10 +78,17 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
     const int bpad = (g.b + 127) / 128 * 128, mpad = (g.m + 127) / 128 * 128;
     if (2 * bpad + mpad > kMaxNodeKeys) return HYPERATTN_UNSUPPORTED_SHAPE;
   }
-  // Chunks of 2048 rows, halved (down to 256) while the hash has fewer than two CTAs for an SM: below that one chunk is the whole time
-  // (32 heads of 4096 rows: 14 us as 128 chunks, 9.5 us as 512; 12 heads 13 and 6 us; 356 chunks of 2048 are faster than 708 of 1024).
+  // Chunks of 2048 rows, halved (down to 256) while the hash has fewer than two CTAs for an SM: below that one chunk is the
+  // whole time, above it there are only more CTAs to start.  A call, us, with chunks of 2048 -> as the rule halves them, d = 64 and
+  // 128: 48 chunks 41.3 -> 35.8, 51.7 -> 44.0; 128 61.9 -> 59.5, 80.8 -> 79.2 (halved once only: 58.2, 76.2); 200 85.0 -> 80.5,
+  // 110.7 -> 105.0; 280 105.3 -> 103.3, but 143.8 -> 147.6: at d = 128 256 to 295 chunks would better stay.  Beyond the line, 2048 ->
+  // halved all the same: 400 136.8 -> 140.6, 203.3 -> 205.7; 392 of 4 x 100003 rows 140.4 -> 146.0, 201.1 -> 207.1.
+  auto hash_ctas = [&](int chunk) {
+    const long long units = g.npad / g.unit, cpu = (g.unit + chunk - 1) / chunk, cpu_k = (g.unit_k + chunk - 1) / chunk;
+    return g.G * units * cpu + g.G * (g.causal ? units : 1) * cpu_k;
+  };
   g.chunk = kSortChunk;
-  while (g.chunk > 256 && (long long)g.G * ((g.npad / g.unit) * ((g.unit + g.chunk - 1) / g.chunk) + (g.causal ? (g.npad / g.unit) : 1) * ((g.unit_k + g.chunk - 1) / g.chunk)) < 296) g.chunk /= 2;
+  while (g.chunk > 256 && hash_ctas(g.chunk) < 2 * kSms) g.chunk /= 2;
   g.chunks_per_unit = (g.unit + g.chunk - 1) / g.chunk;
   g.chunks_per_seg = (g.npad / g.unit) * g.chunks_per_unit;
   g.chunks_per_unit_k = (g.unit_k + g.chunk - 1) / g.chunk;
@@ -90,7 +97,8 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
 }
 
 struct Plan {
-  size_t q16, k16, v16, q16lo, k16lo, ids, hist, offs, perm_q, perm_k, rank_k, samples, tpos, ltau, vwq, vsum, vcum, swlog, wnodes, smp_blk, key_slot, sched, part_o, part_lse, total;
+  size_t q16, k16, v16, q16lo, k16lo, ids, hist, offs, perm_q, perm_k, rank_k, samples, tpos, ltau, vwq, vsum, vcum, swlog, wnodes;
+  size_t smp_blk, key_slot, sched, part_o, part_lse, total;
   size_t stat, gacc;    // backward only: (-lse, -<dO, O>) per row; fp32 gradient accumulators (bf16 gradients only)
 };
 
@@ -195,7 +203,8 @@ cudaEvent_t take_event() {
 
 struct StageScope {
   cudaStream_t st; int stage; int launches; bool on; cudaEvent_t beg = nullptr;
-  StageScope(cudaStream_t s, int stage_, int launches_) : st(s), stage(stage_), launches(launches_), on(g_profile && ((g_profile_mask >> stage_) & 1u)) {
+  StageScope(cudaStream_t s, int stage_, int launches_)
+      : st(s), stage(stage_), launches(launches_), on(g_profile && ((g_profile_mask >> stage_) & 1u)) {
     if (on) { beg = take_event(); cudaEventRecord(beg, st); }
   }
   ~StageScope() {
@@ -314,7 +323,8 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
   const hyperattn_debug* dbg = p.debug;
   if (g_profile) ++g_profile_calls;
   cudaError_t e = cudaSuccess;
-#define HA_CHECK(x) do { e = (x); if (e != cudaSuccess) { std::fprintf(stderr, "hyperattn: %s failed: %s\n", #x, cudaGetErrorString(e)); return HYPERATTN_CUDA_ERROR; } } while (0)
+#define HA_CHECK(x) do { e = (x); if (e != cudaSuccess) { \
+    std::fprintf(stderr, "hyperattn: %s failed: %s\n", #x, cudaGetErrorString(e)); return HYPERATTN_CUDA_ERROR; } } while (0)
 
   const __nv_bfloat16 *q16 = reinterpret_cast<const __nv_bfloat16*>(p.q), *k16 = reinterpret_cast<const __nv_bfloat16*>(p.k),
                       *v16 = reinterpret_cast<const __nv_bfloat16*>(p.v);
@@ -354,8 +364,9 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     }
     if (vnorm) {
       StageScope sc(st, HYPERATTN_STAGE_SAMPLE, 3);
-      HA_CHECK(launch_vnorm_sampling(g, v16, reinterpret_cast<uint32_t*>(base + pl.vwq), reinterpret_cast<unsigned long long*>(base + pl.vsum), reinterpret_cast<unsigned long long*>(base + pl.vcum),
-                                     ws.samples, reinterpret_cast<float*>(base + pl.swlog), p.seed, st));
+      HA_CHECK(launch_vnorm_sampling(g, v16, reinterpret_cast<uint32_t*>(base + pl.vwq), reinterpret_cast<unsigned long long*>(base + pl.vsum),
+                                     reinterpret_cast<unsigned long long*>(base + pl.vcum), ws.samples,
+                                     reinterpret_cast<float*>(base + pl.swlog), p.seed, st));
       if (dbg && dbg->sample_log2w)
         HA_CHECK(cudaMemcpyAsync(dbg->sample_log2w, base + pl.swlog, (size_t)g.G * g.nodes * g.m * 4, cudaMemcpyDeviceToDevice, st));
     }
@@ -369,8 +380,9 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
       const int sets = g.node_dirs ? g.levels : 1;
       for (int l = 0; l < sets; ++l) {
         const uint8_t* src = ws.ids + l * ids_level_stride(g);
-        if (dbg->q_ids) HA_CHECK(cudaMemcpyAsync(dbg->q_ids + (size_t)l * g.G * g.n, src, (size_t)g.G * g.n, cudaMemcpyDeviceToDevice, st));
-        if (dbg->k_ids) HA_CHECK(cudaMemcpyAsync(dbg->k_ids + (size_t)l * g.G * g.nk, src + (size_t)g.G * g.n, (size_t)g.G * g.nk, cudaMemcpyDeviceToDevice, st));
+        const size_t nq = (size_t)g.G * g.n, nkeys = (size_t)g.G * g.nk;
+        if (dbg->q_ids) HA_CHECK(cudaMemcpyAsync(dbg->q_ids + l * nq, src, nq, cudaMemcpyDeviceToDevice, st));
+        if (dbg->k_ids) HA_CHECK(cudaMemcpyAsync(dbg->k_ids + l * nkeys, src + nq, nkeys, cudaMemcpyDeviceToDevice, st));
       }
       if (dbg->perm_q) HA_CHECK(cudaMemcpyAsync(dbg->perm_q, ws.perm_q, lvl_bytes, cudaMemcpyDeviceToDevice, st));
       if (dbg->perm_k) HA_CHECK(cudaMemcpyAsync(dbg->perm_k, ws.perm_k, lvl_bytes, cudaMemcpyDeviceToDevice, st));

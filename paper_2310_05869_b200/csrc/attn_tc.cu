@@ -75,6 +75,12 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return d;
 }
 
+// adds the two bf16 numbers of a packed pair to two fp32 sums, as they are
+__device__ __forceinline__ void add_bf16_pair(float& lo, float& hi, uint32_t pair) {
+  asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}"
+      : "+f"(lo), "+f"(hi) : "r"(pair));
+}
+
 // Tiles with masked columns (a minority: the diagonal tiles of a causal leaf, padding, sampled
 // columns that fall into the query tile's own block): the masked scores are overwritten with
 // -inf in TMEM before the tile is read, so that the hot loop carries no mask code at all.
@@ -181,7 +187,8 @@ struct Cfg {
   static constexpr int kOffDesc = (kOffMisc + 16 + 15) / 16 * 16;   // ItemDesc [2], one per table set
   static constexpr int kOffStage = (kOffDesc + 2 * kDescBytes + 127) / 128 * 128;
   static constexpr int kOffOnes = (kOffStage + ((D == 64) ? 8 : 4) * kStageWarp + 1023) / 1024 * 1024;   // [TK keys x 128 B] of bf16 1.0
-  static constexpr int kOffBias = kOnes ? kOffOnes + TK * 128 : kOffStage + ((D == 64) ? 8 : 4) * kStageWarp;   // float [2][kMaxWeightedSamples]: log2 weight of every sampled column (weighted sampling only)
+  // float [2][kMaxWeightedSamples]: log2 weight of every sampled column (weighted sampling only)
+  static constexpr int kOffBias = kOnes ? kOffOnes + TK * 128 : kOffStage + ((D == 64) ? 8 : 4) * kStageWarp;
   static constexpr int kTotal = kOffBias + 2 * kMaxWeightedSamples * 4;
   static_assert(kTotal <= 232448, "shared memory");
   static_assert(D == 64 || 4 * kStageWarp <= kMaxNodeKeys * 4, "staging of query tile 0 must fit one key-row table");
@@ -319,7 +326,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
   HA_T0(t_cta);
 
   // A CTA of a launch in which some wait already timed out returns at once (nothing allocated
-  // yet), so a stuck launch drains quickly instead of timing out tile after tile.
+  // yet), so a stuck launch drains quickly instead of timing out tile after tile.  (Read before
+  // wait_for_stream(), on purpose: see there.)
   if (tid == 0) *s_abort = *reinterpret_cast<volatile int*>(status);
   __syncthreads();
   if (*s_abort) return;
@@ -344,7 +352,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if constexpr (C::kOnes) {
-    for (int k = tid; k < TK * 128 / 16; k += 384) *reinterpret_cast<uint4*>(smem + C::kOffOnes + 16 * k) = make_uint4(0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u);
+    constexpr uint32_t one2 = 0x3f803f80u;              // two bf16 ones
+    for (int k = tid; k < TK * 128 / 16; k += 384) *reinterpret_cast<uint4*>(smem + C::kOffOnes + 16 * k) = make_uint4(one2, one2, one2, one2);
     fence_async_smem();                                 // the tensor pipe reads the slab through the async proxy
   }
   if (warp == 8) {
@@ -408,7 +417,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       }
       return true;
     };
-    HA_LDECL(a_tab); HA_LDECL(a_ws); HA_LDECL(a_cmp); HA_LDECL(a_epi); HA_LDECL(a_gq); HA_LDECL(a_bo); HA_LDECL(a_tiles); HA_LDECL(a_ws0); HA_LDECL(a_c1); HA_LDECL(a_c2); HA_LDECL(a_c3); HA_LDECL(a_c4); HA_LDECL(a_e1); HA_LDECL(a_e2); HA_LDECL(a_e3);
+    HA_LDECL(a_tab); HA_LDECL(a_ws); HA_LDECL(a_cmp); HA_LDECL(a_epi); HA_LDECL(a_gq); HA_LDECL(a_bo); HA_LDECL(a_tiles); HA_LDECL(a_ws0);
+    HA_LDECL(a_c1); HA_LDECL(a_c2); HA_LDECL(a_c3); HA_LDECL(a_c4); HA_LDECL(a_e1); HA_LDECL(a_e2); HA_LDECL(a_e3);
     HA_T0(t_role);
     ok = __all_sync(0xffffffffu, gather_q(0));
     for (; ok; ++it) {
@@ -563,8 +573,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
               const float p0 = ex2(x0), p1 = ex2(x1);
               lt2 = fadd2(lt2, pack_f2(p0, p1));
               const uint32_t w = pack2(p0, p1);
-              if constexpr (!C::kOnes)
-                asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}" : "+f"(lrta), "+f"(lrtb) : "r"(w));
+              if constexpr (!C::kOnes) add_bf16_pair(lrta, lrtb, w);
               p[e >> 1] = w;
               if constexpr (PRECISE) {
                 // what the rounding to bf16 left over, as a second bf16 number (an infinite weight leaves NaN here, but it
@@ -572,8 +581,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
                 float r0, r1;
                 unpack_f2(fadd2(pack_f2(p0, p1), pack_f2(-__uint_as_float(w << 16), -__uint_as_float(w & 0xffff0000u))), r0, r1);
                 const uint32_t wl = pack2(r0, r1);
-                if constexpr (!C::kOnes)
-                  asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}" : "+f"(lrta), "+f"(lrtb) : "r"(wl));
+                if constexpr (!C::kOnes) add_bf16_pair(lrta, lrtb, wl);
                 plo[e >> 1] = wl;
               }
             }
@@ -611,8 +619,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
               const float p0 = ex2(x0), p1 = ex2(x1);
               lt2 = fadd2(lt2, pack_f2(p0, p1));
               const uint32_t w = pack2(p0, p1);
-              if constexpr (!C::kOnes)
-                asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}" : "+f"(lrta), "+f"(lrtb) : "r"(w));
+              if constexpr (!C::kOnes) add_bf16_pair(lrta, lrtb, w);
               p[e >> 1] = w;
             }
             tmem_st16(sbase + c * 16, p);
@@ -709,7 +716,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
           tmem_ld16_issue(lane_addr + colO, r);
           if constexpr (C::kOnes) {                     // the sum of the bf16 weights sits in column D of O
             uint32_t sumw;
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\ttcgen05.wait::ld.sync.aligned;\n" : "=r"(sumw) : "r"(lane_addr + colO + D) : "memory");
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\ttcgen05.wait::ld.sync.aligned;\n"
+                         : "=r"(sumw) : "r"(lane_addr + colO + D) : "memory");
             if (!capped_item) inv = 1.f / __uint_as_float(sumw);
           }
 #pragma unroll 1
@@ -769,18 +777,21 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
     if (row == 0 && i == 0) {
       HA_LFLUSH(9, a_tab); HA_LFLUSH(0, a_ws); HA_LFLUSH(2, a_cmp); HA_LFLUSH(15, a_epi); HA_LFLUSH(16, a_gq); HA_LFLUSH(17, a_bo);
       HA_LFLUSH(20, a_tiles); HA_TACC(18, t_role); HA_LFLUSH(19, it);
-      HA_LFLUSH(40, a_e1); HA_LFLUSH(41, a_e2); HA_LFLUSH(42, a_e3); HA_LFLUSH(24, a_ws0); HA_LFLUSH(22, a_c1); HA_LFLUSH(29, a_c2); HA_LFLUSH(30, a_c3); HA_LFLUSH(31, a_c4);
+      HA_LFLUSH(40, a_e1); HA_LFLUSH(41, a_e2); HA_LFLUSH(42, a_e3); HA_LFLUSH(24, a_ws0);
+      HA_LFLUSH(22, a_c1); HA_LFLUSH(29, a_c2); HA_LFLUSH(30, a_c3); HA_LFLUSH(31, a_c4);
     }
 #endif
   } else if (warp < 10) {
     // ================= MMA issue, a warp per query tile (warp 8: tile 0, warp 9: tile 1) ===========
     // Each issuer walks its own key tiles: scores run two tiles ahead of the PV products
-    // (S buffers alternate).  A tcgen05.mma occupies the issuing thread and the tensor pipe
-    // for about 55-65 cycles whatever its size, so the two chains are issued by two threads.
-    // The issuer shares its scheduler with two busy softmax warps and has no instruction-level
-    // parallelism of its own, so its loop is kept to a minimum of instructions: the whole warp walks it together with
-    // warp-uniform values and one elected lane issues, so that descriptors are made of uniform registers (a lone lane's have to be moved
-    // there one by one; d = 64 leaves 525 -> 497 us, node items 1207 -> 1141, d = 128 400 -> 378, split weights 2059 -> 1687); descriptors are two 32-bit words of which only the low one moves; waits are one probe in the common
+    // (S buffers alternate).  A tcgen05.mma occupies the issuer and the tensor pipe for about
+    // 45-65 cycles whatever its size, so the two chains are issued by two warps.  An issuer
+    // shares its scheduler with two busy softmax warps and has no instruction-level parallelism
+    // of its own, so its loop is kept to a minimum of instructions: the whole warp walks it
+    // with warp-uniform values and one elected lane issues, so that descriptors are made of
+    // uniform registers (a lone lane's have to be moved there one by one: 128 causal leaves of
+    // 4096 rows, d = 64, 525 -> 497 us; 32 heads x 32768 rows, d = 128, 400 -> 378); descriptors
+    // are two 32-bit words of which only the low one moves; waits are one probe in the common
     // case, everything unusual lives in out-of-line slow paths.
     const int i = warp - 8;
     {

@@ -11,11 +11,11 @@
 // softmax over everything a row sees, so every tile of every level uses the FINAL lse and delta.
 //
 // A work item is a tile of 128 KEYS and a run of query tiles (steps): the key tiles of a leaf against the query tiles from the
-// diagonal on, a key tile of a sorted block against the block's query tiles, a tile of a node's sampled keys against a chunk of the
-// node's query tiles.  dK and dV of the item stay in TMEM over its steps and leave once: by fp32 reductions, or, without recursion
-// and for keys that are not sampled, which no other item adds to, as bf16 results (32 heads x 32768 rows, d = 128: accumulators that need not
-// be cleared, added to and converted, 1934 -> 1416 us); dQ leaves after every step.  (The other way round - query tiles stay, dK and dV leave after every step - is twice the reductions and was what
-// the kernel's first version did, one phase after the other: 10 500 clocks per 128 x 128 tile at d = 64, 17 400 at d = 128.)
+// diagonal on, a key tile of a sorted block against the block's query tiles, a tile of a node's sampled keys against a chunk of
+// the node's query tiles.  dK and dV of the item stay in TMEM over its steps and leave once: by fp32 reductions, or, without
+// recursion and for keys that are not sampled, which no other item adds to, as bf16 results (32 heads x 32768 rows, d = 128:
+// accumulators that need not be cleared, added to and converted, 1936 -> 1409 us); dQ leaves after every step.  (The other way
+// round - query tiles stay, dK and dV leave after every step - is twice the reductions.)
 // Per step, all five products on the tcgen05 tensor cores, keys in the TMEM lanes of the first two:
 //     S^T  = K Q^T,  dP^T = V dO^T      operands in 128-byte-swizzled shared memory, K-major
 //     P^T  -> TMEM (bf16), dS^T -> shared memory (bf16, [key][query])          two warpgroups, 64 query columns each
@@ -28,9 +28,9 @@
 // which dQ comes before dK so that it leaves TMEM while dK and the next S^T are multiplied.
 // What bounds it: a step takes 4000 (causal leaves) to 5000 clocks (sorted blocks), of which no single unit is busy for half; the
 // load and store unit is the fullest (gathered copies, dS, results through shared memory, reductions at 25 bytes per clock), and
-// everything else in a chain waits behind it.  Time, us, of the whole pass, one chain -> two: 131072 rows, 32 heads 3335 -> 3025;
-// causal leaves of 4096 rows, 128 heads 1167 -> 1098; 12 heads x 4096 rows 59 -> 56 (d = 64; two chains at d = 128 are 10 % slower in the
-// leaves).  16 P warps instead of 8 force 64 registers a thread and are slower (3160).
+// everything else in a chain waits behind it.  One chain -> two, us of the whole pass: 131072 rows, 32 heads 3343 -> 3022; causal
+// leaves of 4096 rows, 128 heads 1167 -> 1105 (d = 64; two chains at d = 128 are 10 % slower in the leaves).  16 P warps instead
+// of 8 force 64 registers a thread and are slower (3160 us).
 //
 // Warp roles (672 threads): warps 0-7 P and dS; 8-15 dQ, dK and dV to global memory; 16 issue of S^T and dP^T (the warp also allocates
 // TMEM); 17 issue of the gradient products; 18 item descriptors, K and V; 19 Q and the row statistics; 20 dO.
@@ -195,7 +195,8 @@ struct Cfg {
 // The same threads clear the accumulators: 32 bytes of each.
 template <int D, bool OUT_FP32>
 __global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__ dout, const void* __restrict__ out, const float* __restrict__ lse,
-                                                       float2* __restrict__ stat, size_t rows, int* sched, float4* dq, float4* dk, float4* dv, size_t kv_rows) {
+                                                       float2* __restrict__ stat, size_t rows, int* sched, float4* dq, float4* dk, float4* dv,
+                                                       size_t kv_rows) {
   constexpr int LPR = D / 8;
   const size_t c = (size_t)blockIdx.x * 256 + threadIdx.x;
   wait_for_stream();
@@ -230,7 +231,8 @@ __global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__
 }
 
 template <int D>
-__global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_constant__ BwdArgs b, const __grid_constant__ BwdMaps maps, int* status) {
+__global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_constant__ BwdArgs b, const __grid_constant__ BwdMaps maps,
+                                                                  int* status) {
   using C = Cfg<D>;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
@@ -252,7 +254,8 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
   auto bar_kfull = [&](int it) { return bar0 + 8 * (18 + it % C::NKV); };         // K, V of an item landed
   auto bar_vfull = [&](int it) { return bar0 + 8 * (20 + it % C::NKV); };
   auto bar_kfree = [&](int it) { return bar0 + 8 * (22 + it % C::NKV); };         // dQ of the item multiplied: K and V are free
-  const uint32_t bar_dqfree = bar0 + 8 * 24, bar_acc = bar0 + 8 * 25, bar_accfree = bar0 + 8 * 26;   // dQ has left TMEM; dK, dV of the item complete; have left TMEM
+  // dQ has left TMEM; dK, dV of the item complete; dK, dV have left TMEM
+  const uint32_t bar_dqfree = bar0 + 8 * 24, bar_acc = bar0 + 8 * 25, bar_accfree = bar0 + 8 * 26;
   auto bar_dfull = [&](int it) { return bar0 + 8 * (27 + it % kDescs); };         // item descriptor written
   auto bar_dfree = [&](int it) { return bar0 + 8 * (27 + kDescs + it % kDescs); };
 
@@ -263,14 +266,18 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
 
   if (tid == 0) *s_abort = *reinterpret_cast<volatile int*>(status);
   __syncthreads();
-  if (*s_abort) return;                                 // (a launch in which some wait already timed out drains quickly)
+  if (*s_abort) return;         // (a launch in which some wait already timed out drains quickly; read early, see wait_for_stream())
   __syncthreads();
   if (tid == 0) {
     mbar_init(bar_dqfree, C::RW); mbar_init(bar_acc, 1); mbar_init(bar_accfree, C::RW);   // (one arrival per warp)
-    for (int x = 0; x < 2; ++x) { mbar_init(bar_s(x), 1); mbar_init(bar_dp(x), 1); mbar_init(bar_h(x), C::SW / C::NH); mbar_init(bar_pfree(x), 1); mbar_init(bar_dq(x), 1); mbar_init(bar_qfull(x), 64); mbar_init(bar_qfree(x), 1); mbar_init(bar_dofree(x), 1); }
+    for (int x = 0; x < 2; ++x) {
+      mbar_init(bar_s(x), 1); mbar_init(bar_dp(x), 1); mbar_init(bar_h(x), C::SW / C::NH); mbar_init(bar_pfree(x), 1); mbar_init(bar_dq(x), 1);
+      mbar_init(bar_qfull(x), 64); mbar_init(bar_qfree(x), 1); mbar_init(bar_dofree(x), 1);
+    }
     for (int x = 0; x < C::NDO; ++x) mbar_init(bar_dofull(x), 32);
     for (int x = 0; x < C::NKV; ++x) { mbar_init(bar_kfull(x), 32); mbar_init(bar_vfull(x), 32); mbar_init(bar_kfree(x), 1); }
-    for (int x = 0; x < kDescs; ++x) { mbar_init(bar_dfull(x), 1); mbar_init(bar_dfree(x), C::SW + C::RW + 4); }   // P and results warps, two issuers, loaders of Q and dO
+    // (P and results warps, two issuers, loaders of Q and dO)
+    for (int x = 0; x < kDescs; ++x) { mbar_init(bar_dfull(x), 1); mbar_init(bar_dfree(x), C::SW + C::RW + 4); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == C::SW + C::RW) {
@@ -448,7 +455,8 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
             const int gr = __shfl_sync(0xffffffffu, grow, 4 * (q0 + q) + (lane >> 3));
             if (gr >= 0) atomicAdd(reinterpret_cast<float4*>(base + (size_t)gr * D + NC * r_ + 32 * p + 4 * c), v[q]);
             else if (decltype(direct)::value && gr != kNoRow)
-              *reinterpret_cast<uint2*>(base16 + (size_t)~gr * D + NC * r_ + 32 * p + 4 * c) = make_uint2(pack2(v[q].x, v[q].y), pack2(v[q].z, v[q].w));
+              *reinterpret_cast<uint2*>(base16 + (size_t)~gr * D + NC * r_ + 32 * p + 4 * c) =
+                  make_uint2(pack2(v[q].x, v[q].y), pack2(v[q].z, v[q].w));
           }
         }
         __syncwarp();
@@ -517,13 +525,15 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
           const uint32_t q = C::kOffQ + (g & 1) * C::kTile, o = C::kOffDO + (g % C::NDO) * C::kTile;
           ok = warp_wait<10>(bar_qfull(g), (g >> 1) & 1, s_abort, status);
           auto scores = [&](int x) {
-            if (g > 0) ok = ok && warp_wait<14>(D == 64 ? bar_h(x) : bar_pfree(x), (g - 1) & 1, s_abort, status);   // (d = 128: P lies over the scores)
+            // (d = 128: P lies over the scores)
+            if (g > 0) ok = ok && warp_wait<14>(D == 64 ? bar_h(x) : bar_pfree(x), (g - 1) & 1, s_abort, status);
             if (!ok) return;
             if (x == 0) fence_async_smem();
             tc_fence_after();
             if (el) {
 #pragma unroll
-              for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColS + 64 * x, kmajor(k, ks), kmajor(q + x * 8192, ks), desc_hi, idesc_s, ks > 0);
+              for (int ks = 0; ks < D / 16; ++ks)
+                mma_ss2(tmem + C::kColS + 64 * x, kmajor(k, ks), kmajor(q + x * 8192, ks), desc_hi, idesc_s, ks > 0);
               umma_commit(bar_s(x));
             }
           };
@@ -538,7 +548,8 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
             if (!ok) return;
             if (el) {
 #pragma unroll
-              for (int ks = 0; ks < D / 16; ++ks) mma_ss2(tmem + C::kColDP + 64 * x, kmajor(v, ks), kmajor(o + x * 8192, ks), desc_hi, idesc_s, ks > 0);
+              for (int ks = 0; ks < D / 16; ++ks)
+                mma_ss2(tmem + C::kColDP + 64 * x, kmajor(v, ks), kmajor(o + x * 8192, ks), desc_hi, idesc_s, ks > 0);
               umma_commit(bar_dp(x));
             }
           };
@@ -568,7 +579,8 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
             if (el) {
 #pragma unroll
               for (int kk = x * KK; kk < (x + 1) * KK; ++kk)
-                mma_ts2(tmem + C::kColDV, tmem + C::kColP + (kk >> 2) * C::kPHalf + (kk & 3) * 8, mnmajor(o, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
+                mma_ts2(tmem + C::kColDV, tmem + C::kColP + (kk >> 2) * C::kPHalf + (kk & 3) * 8, mnmajor(o, kk), desc_hi, idesc_n,
+                        (s > 0 || kk > 0) ? 1u : 0u);
               umma_commit(bar_pfree(x));
               if (x + 1 == C::NH) umma_commit(bar_dofree(g));
             }
@@ -576,7 +588,8 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
           auto grad_k = [&](int x) {
             if (ok && el) {
 #pragma unroll
-              for (int kk = x * KK; kk < (x + 1) * KK; ++kk) mma_ss2(tmem + C::kColDK, kmajor(ds, kk), mnmajor(q, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
+              for (int kk = x * KK; kk < (x + 1) * KK; ++kk)
+                mma_ss2(tmem + C::kColDK, kmajor(ds, kk), mnmajor(q, kk), desc_hi, idesc_n, (s > 0 || kk > 0) ? 1u : 0u);
               if (x + 1 == C::NH) {
                 umma_commit(bar_qfree(g));
                 if (last) umma_commit(bar_acc);
@@ -633,7 +646,8 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
       }
       cp_async_arrive_noinc(bar);
     };
-    auto gather = [&](int rows, uint32_t dst, const __nv_bfloat16* base, const int (&v)[4], uint32_t bar) {   // v: a valid row also where none exists
+    // (v: a valid row also where none exists)
+    auto gather = [&](int rows, uint32_t dst, const __nv_bfloat16* base, const int (&v)[4], uint32_t bar) {
       if (rows == 128) gather_rows(std::true_type{}, rows, dst, base, v, bar);
       else gather_rows(std::false_type{}, rows, dst, base, v, bar);
     };
@@ -821,9 +835,10 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   {
     const unsigned grid = (unsigned)((rows * (g.d / 8) + 255) / 256);
     const uint4* d4 = reinterpret_cast<const uint4*>(dout);
-    auto* kernel = g.d == 64 ? (out_fp32 ? row_stat_kernel<64, true> : row_stat_kernel<64, false>) : (out_fp32 ? row_stat_kernel<128, true> : row_stat_kernel<128, false>);
-    const cudaError_t e = launch(kernel, grid, 256, 0, st, d4, out, lse, stat, rows, sched, reinterpret_cast<float4*>(gr.dq), reinterpret_cast<float4*>(gr.dk),
-                                 reinterpret_cast<float4*>(gr.dv), gr.kv_elems / g.d);
+    auto* kernel = g.d == 64 ? (out_fp32 ? row_stat_kernel<64, true> : row_stat_kernel<64, false>)
+                             : (out_fp32 ? row_stat_kernel<128, true> : row_stat_kernel<128, false>);
+    const cudaError_t e = launch(kernel, grid, 256, 0, st, d4, out, lse, stat, rows, sched, reinterpret_cast<float4*>(gr.dq),
+                                 reinterpret_cast<float4*>(gr.dk), reinterpret_cast<float4*>(gr.dv), gr.kv_elems / g.d);
     if (e != cudaSuccess) return e;
   }
   int sms = 0;
@@ -831,17 +846,21 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   BwdArgs b;
   b.a = a; b.dout = reinterpret_cast<const __nv_bfloat16*>(dout); b.stat = stat; b.scale = scale; b.sched = sched;
   b.dq = gr.dq; b.dk = gr.dk; b.dv = gr.dv;
-  b.dk16 = reinterpret_cast<__nv_bfloat16*>(gr.dk16); b.dv16 = reinterpret_cast<__nv_bfloat16*>(gr.dv16); b.key_slot = gr.key_slot; b.direct = gr.direct;
+  b.dk16 = reinterpret_cast<__nv_bfloat16*>(gr.dk16); b.dv16 = reinterpret_cast<__nv_bfloat16*>(gr.dv16);
+  b.key_slot = gr.key_slot; b.direct = gr.direct;
   b.leaf_ktiles = a.n_leaf_tiles ? (g.leaf + kTileK - 1) / kTileK : 0;
   b.block_ktiles = (g.b + kTileK - 1) / kTileK;
   b.smp_ktiles = (g.m + kTileK - 1) / kTileK;
-  // Sampled items take at most 16 query tiles (their dK and dV leave once per item) and fewer where that leaves less than
-  // about six items for an SM.
+  // Sampled items take at most 16 query tiles (their dK and dV leave once per item) and fewer, down to 2, where that leaves less
+  // than about six items for an SM.  The pass, us, with 2 / 4 / 8 / 16 / 32 tiles (* what the rule takes): 12 heads x 4096 rows
+  // 60* / 66 / 82 / 113 / 160, 32 x 32768 924 / 914 / 900 / 906* / 948 (d = 64); 32 x 4096 231 / 241* / 253 / 285 / 390, 32 x 32768
+  // 1736 / 1672 / 1641 / 1637* / 1708 (d = 128); 4 causal heads of 65536 rows 1006 / 1026 / 1040 / 1027-1058* / 1105 (d = 64).
   long long steps = 0;
   for (int l = 0; l < g.levels; ++l) {
     int s, q0, k0;
     node_rows(g, l, 0, s, q0, k0);
-    if (a.level_sorted[l]) steps += (long long)(g.causal ? (1 << l) : 1) * g.G * node_blocks(s, g.b) * a.tiles_per_block * (b.smp_ktiles + b.block_ktiles);
+    if (a.level_sorted[l])
+      steps += (long long)(g.causal ? (1 << l) : 1) * g.G * node_blocks(s, g.b) * a.tiles_per_block * (b.smp_ktiles + b.block_ktiles);
   }
   if (b.leaf_ktiles) steps += (long long)a.leaves_per_seg * g.G * b.leaf_ktiles * (a.dense_causal ? (b.leaf_ktiles + 1) / 2 : b.leaf_ktiles);
   const long long want = steps / (6LL * sms);
@@ -867,18 +886,22 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   if (!encode_rows_map(&maps.q, a.q, rows, g.d, 128) || !encode_rows_map(&maps.k, a.k, rows, g.d, 128) ||
       !encode_rows_map(&maps.v, a.v, rows, g.d, 128) || !encode_rows_map(&maps.dout, dout, rows, g.d, 128)) return cudaErrorInvalidValue;
   const unsigned grid = items < sms ? (unsigned)items : (unsigned)sms;      // persistent: one CTA per SM
-  cudaError_t e = g.d == 64 ? allow_smem<bwd_kernel<64>>(Cfg<64>::kTotal) : allow_smem<bwd_kernel<128>>(Cfg<128>::kTotal);
+  const int smem = g.d == 64 ? Cfg<64>::kTotal : Cfg<128>::kTotal;
+  cudaError_t e = g.d == 64 ? allow_smem<bwd_kernel<64>>(smem) : allow_smem<bwd_kernel<128>>(smem);
   if (e != cudaSuccess) return e;
-  e = launch(g.d == 64 ? bwd_kernel<64> : bwd_kernel<128>, grid, g.d == 64 ? Cfg<64>::kThreads : Cfg<128>::kThreads, g.d == 64 ? Cfg<64>::kTotal : Cfg<128>::kTotal, st, b, maps, status);
+  static_assert(Cfg<64>::kThreads == Cfg<128>::kThreads, "one block size");
+  e = launch(g.d == 64 ? bwd_kernel<64> : bwd_kernel<128>, grid, Cfg<64>::kThreads, smem, st, b, maps, status);
   if (e != cudaSuccess || !gr.dq16) return e;
   ToBf16Args c;
   const size_t elems[3] = {rows * g.d, gr.kv_elems, gr.kv_elems};
   const float* src[3] = {gr.dq, gr.dk, gr.dv};
   void* dst[3] = {gr.dq16, gr.dk16, gr.dv16};
-  for (int y = 0; y < 3; ++y) { c.src[y] = reinterpret_cast<const float4*>(src[y]); c.dst[y] = reinterpret_cast<uint4*>(dst[y]); c.count8[y] = elems[y] / 8; }
+  for (int y = 0; y < 3; ++y) {
+    c.src[y] = reinterpret_cast<const float4*>(src[y]); c.dst[y] = reinterpret_cast<uint4*>(dst[y]); c.count8[y] = elems[y] / 8;
+  }
   c.key_slot = gr.direct ? gr.key_slot : nullptr; c.samples = a.samples; c.n = g.n; c.m = g.m; c.lg_lpr = g.d == 64 ? 3 : 4;
   const size_t blocks = (c.count8[0] + 255) / 256;
-  return launch(to_bf16_kernel, dim3((unsigned)(blocks < 148 * 16 ? blocks : 148 * 16), gr.kv_elems ? 3 : 1), 256, 0, st, c);
+  return launch(to_bf16_kernel, dim3((unsigned)(blocks < 16 * (size_t)sms ? blocks : 16 * (size_t)sms), gr.kv_elems ? 3 : 1), 256, 0, st, c);
 }
 
 }  // namespace hyperattn

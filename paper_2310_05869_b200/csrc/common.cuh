@@ -13,6 +13,9 @@ constexpr int kSortChunk = 2048;      // most rows per histogram / scatter chunk
 constexpr int kBuckets = 256;         // 2^r with r <= 8
 constexpr int kTileQ = 128;           // query rows per attention tile
 constexpr int kMaxLevelsMerge = 24;   // deepest causal recursion supported
+// SMs of a B200, where a rule must not depend on the device in hand (workspace sizes are asked for without one) or a grid only has
+// to be large enough; the grids of the persistent kernels ask the device (sm_count)
+constexpr int kSms = 148;
 
 // ---- Philox4x32-10 (Salmon et al., SC'11); identical on host and device -------------
 struct Philox4 { uint32_t x[4]; };
@@ -74,7 +77,9 @@ struct Geometry {
 };
 // ids / histograms of a level start this many elements after those of level 0 (0: one set shared by all levels)
 __host__ __device__ inline size_t ids_level_stride(const Geometry& g) { return g.node_dirs ? (size_t)g.G * ((size_t)g.n + g.nk) : 0; }
-__host__ __device__ inline size_t hist_level_stride(const Geometry& g) { return g.node_dirs ? (size_t)g.G * (g.chunks_per_seg + g.chunks_per_seg_k) * kBuckets : 0; }
+__host__ __device__ inline size_t hist_level_stride(const Geometry& g) {
+  return g.node_dirs ? (size_t)g.G * (g.chunks_per_seg + g.chunks_per_seg_k) * kBuckets : 0;
+}
 
 // sorted blocks of a node of s rows: ceil(s / b) of them, the last one with the remaining rows
 // (Alg. 1 line 4: row i belongs to block floor(P(i) / b))
@@ -112,8 +117,11 @@ __host__ __device__ inline int side_cpl(const Geometry& g, int side) { return g.
 // Every kernel of a call is launched with programmatic stream serialisation: its launch is prepared while the kernel before
 // it on the stream runs, and its blocks wait in wait_for_stream() until that one has completed and its writes are visible.  So
 // nothing that an earlier kernel writes may be read - and nothing written - before it; since every kernel waits, all
-// earlier ones have completed by then, not only the last.  (Small calls gain 5-8 us; letting the next kernel's blocks in
-// early with griddepcontrol.launch_dependents costs large calls 3-7 %: they take slots from the kernel that still runs.)
+// earlier ones have completed by then, not only the last.  The one exception is the device status word, which the tcgen05
+// kernels look at first thing, before they allocate anything, so that the launches behind a wait that gave up drain quickly: a
+// value from before that moment costs no more than this, the follower's own waits being bounded too.
+// (Small calls gain 5-8 us; letting the next kernel's blocks in early with griddepcontrol.launch_dependents costs large calls
+// 3-7 %: they take slots from the kernel that still runs.)
 __device__ __forceinline__ void wait_for_stream() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <class... P, class... A>

@@ -101,7 +101,8 @@ __device__ __forceinline__ size_t ids_base(const HashArgs& a, const ChunkPos& c)
   return c.level * a.ids_level_stride + (c.side ? (size_t)a.G * a.n[0] : 0) + (size_t)c.seg * a.n[c.side] + c.row0;
 }
 __device__ __forceinline__ size_t hist_base(const HashArgs& a, const ChunkPos& c) {
-  return c.level * a.hist_level_stride + ((c.side ? (size_t)a.G * a.chunks_per_seg[0] : 0) + (size_t)c.seg * a.chunks_per_seg[c.side] + c.chunk) * kBuckets;
+  return c.level * a.hist_level_stride +
+         ((c.side ? (size_t)a.G * a.chunks_per_seg[0] : 0) + (size_t)c.seg * a.chunks_per_seg[c.side] + c.chunk) * kBuckets;
 }
 
 // One CTA = one chunk (<= a.chunk rows of one side of one segment).  Each warp walks over
@@ -340,7 +341,7 @@ static ConvertArgs make_convert_args(const void* q, const void* k, const void* v
 cudaError_t launch_convert(const float* q, const float* k, const float* v, const Workspace& ws, size_t count_q, size_t count_k, cudaStream_t st) {
   const ConvertArgs a = make_convert_args(q, k, v, ws, count_q, count_k);
   const size_t most = a.count4[0] > a.count4[1] ? a.count4[0] : a.count4[1], want = (most + 255) / 256;
-  const dim3 grid((unsigned)(want < 148 * 16 ? want : 148 * 16), 3);
+  const dim3 grid((unsigned)(want < 16 * kSms ? want : 16 * kSms), 3);
   return launch(convert_kernel, grid, 256, 0, st, a);
 }
 
@@ -349,13 +350,16 @@ static int convert_ctas(const Geometry& g) {
   const size_t want = ((size_t)g.G * (g.n > g.nk ? g.n : g.nk) * g.d / 4 + 1023) / 1024;
   return want < (1u << 20) ? (int)want : 1 << 20;
 }
-// Copies of up to two CTAs per SM run beside the hash (its CTAs take 70 or 135 KB of shared memory each, so that few fit an SM); beyond that
-// a launch of their own, with more threads per SM, is faster.  A call, us, own launch -> beside the hash: 2 heads x 300 rows d = 64 24.9 -> 22.4,
-// 4 x 4096 d = 64 24.8 -> 23.3, 2 x 2500 d = 128 27.5 -> 25.6; 4 x 4096 d = 128 (512 CTAs) 35.0 -> 36.5.
-bool convert_in_hash(const Geometry& g) { return g.sorted && !g.node_dirs && convert_ctas(g) <= 296; }
+// Copies of up to two CTAs per SM run beside the hash.  The hash's CTAs take 70 (d = 64) or 135 KB (d = 128) of shared memory each, so
+// that three or one fit an SM, and the copies' CTAs, being of the same launch, are as few; beyond the line a launch of their own has
+// more threads in flight.  A call, us, own launch -> beside the hash: d = 64, 16 copy CTAs 17.5 -> 16.5, 256 23.1 -> 22.7, 512
+// 39.2 -> 37.2 (three CTAs per SM are enough there: the line could lie higher); d = 128, 32 25.0 -> 23.8, 157 27.2 -> 25.2, 512
+// 35.2 -> 36.5, 1024 70.7 -> 77.8.
+bool convert_in_hash(const Geometry& g) { return g.sorted && !g.node_dirs && convert_ctas(g) <= 2 * kSms; }
 
 cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_fp32, const float* w_host,
-                        const Workspace& ws, unsigned long long* near_zero, cudaStream_t st, int side_mask, const float* w_nodes, const void* convert_v) {
+                        const Workspace& ws, unsigned long long* near_zero, cudaStream_t st, int side_mask,
+                        const float* w_nodes, const void* convert_v) {
   HashArgs a;
   a.side_mask = side_mask; a.chunk = g.chunk;
   a.w_nodes = g.node_dirs ? w_nodes : nullptr;
@@ -378,7 +382,8 @@ cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_
       a.conv = make_convert_args(q, k, convert_v, ws, (size_t)g.G * g.n * g.d, (size_t)g.G * g.nk * g.d);
       copy_ctas = convert_ctas(g);
     }
-    return launch(g.d == 64 ? hash_fp32_kernel<64> : hash_fp32_kernel<128>, grid + copy_ctas, 256, g.d == 64 ? kHash32Smem<64> : kHash32Smem<128>, st, a);
+    return launch(g.d == 64 ? hash_fp32_kernel<64> : hash_fp32_kernel<128>, grid + copy_ctas, 256,
+                  g.d == 64 ? kHash32Smem<64> : kHash32Smem<128>, st, a);
   }
   return launch(g.d == 64 ? hash_bf16_kernel<64> : hash_bf16_kernel<128>, grid, 256, 0, st, a);
 }

@@ -182,11 +182,18 @@ cudaError_t launch_merge(const Geometry& g, const Workspace& ws, void* out, floa
   auto pick = [&](auto dtag, auto pbtag) {
     constexpr int D = decltype(dtag)::value;
     constexpr bool PB = decltype(pbtag)::value;
-    if (g.L <= 3) go(merge_kernel<D, 3, PB>); else if (g.L <= 5) go(merge_kernel<D, 5, PB>); else if (g.L <= 8) go(merge_kernel<D, 8, PB>); else go(merge_kernel<D, kMaxLevelsMerge, PB>);
+    if (g.L <= 3) go(merge_kernel<D, 3, PB>);
+    else if (g.L <= 5) go(merge_kernel<D, 5, PB>);
+    else if (g.L <= 8) go(merge_kernel<D, 8, PB>);
+    else go(merge_kernel<D, kMaxLevelsMerge, PB>);
   };
   using std::integral_constant;
-  if (g.d == 64) { if (ws.part_bf16) pick(integral_constant<int, 64>{}, integral_constant<bool, true>{}); else pick(integral_constant<int, 64>{}, integral_constant<bool, false>{}); }
-  else { if (ws.part_bf16) pick(integral_constant<int, 128>{}, integral_constant<bool, true>{}); else pick(integral_constant<int, 128>{}, integral_constant<bool, false>{}); }
+  auto pick_d = [&](auto d) {
+    if (ws.part_bf16) pick(d, std::true_type{});
+    else pick(d, std::false_type{});
+  };
+  if (g.d == 64) pick_d(integral_constant<int, 64>{});
+  else pick_d(integral_constant<int, 128>{});
   return e;
 }
 

@@ -34,7 +34,9 @@ __device__ __forceinline__ int node_first_chunk(const Geometry& g, int level, in
   return ((side == 0 ? q0 : k0) / g.unit) * g.chunks_per_unit;
 }
 __device__ __forceinline__ size_t side_hist_base(const Geometry& g, int side) { return side ? (size_t)g.G * g.chunks_per_seg * kBuckets : 0; }
-__device__ __forceinline__ size_t side_offs_base(const Geometry& g, int side) { return side ? (size_t)g.levels * g.G * side_cpl(g, 0) * kBuckets : 0; }
+__device__ __forceinline__ size_t side_offs_base(const Geometry& g, int side) {
+  return side ? (size_t)g.levels * g.G * side_cpl(g, 0) * kBuckets : 0;
+}
 __device__ __forceinline__ size_t side_ids_base(const Geometry& g, int side) { return side ? (size_t)g.G * g.n : 0; }
 
 struct SampleArgs {
@@ -280,7 +282,11 @@ static SortArgs make_sort_args(const Geometry& g, const Workspace& ws, int side_
   return a;
 }
 
-// Nodes of at most kScanChunks chunks: the placement adds up the histograms itself (8 loads in flight, two rounds)
+// Nodes of at most kScanChunks chunks: the placement adds up the histograms itself (8 loads in flight, two rounds).  Every
+// CTA then reads its node's whole histogram, so that this grows with the square of the chunks while the launch that it saves
+// stays the same.  A call, us, scan launch -> in the placement: 1 head, 8 chunks 23.6 -> 21.9, 16 24.5 -> 22.7, 64 28.5 -> 25.2;
+// 32 heads, 8 chunks 171.9 -> 169.7, 16 322.3 -> 322.0, 24 486 -> 490, 64 1243 -> 1259; 4 causal heads, nodes of 32 chunks
+// 825 -> 830.  The line is where it stops paying with many heads; a few heads would gain 2-3 us beyond it as well.
 constexpr int kScanChunks = 16;
 bool scan_in_scatter(const Geometry& g) {
   const int most = g.causal ? (g.nl / g.unit) * g.chunks_per_unit : (g.chunks_per_seg > g.chunks_per_seg_k ? g.chunks_per_seg : g.chunks_per_seg_k);
@@ -289,12 +295,14 @@ bool scan_in_scatter(const Geometry& g) {
 
 static SampleArgs make_sample_args(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, int* blocks) {
   // (ws.tpos non-null: the probe rows of the capped row-sum estimate are drawn as well)
-  SampleArgs sa; sa.samples = ws.samples; sa.tpos = ws.tpos; sa.ltau = ws.ltau; sa.g = g; sa.k0 = (uint32_t)seed; sa.k1 = (uint32_t)(seed >> 32); sa.sched = ws.sched; sa.draw = with_samples;
+  SampleArgs sa;
+  sa.samples = ws.samples; sa.tpos = ws.tpos; sa.ltau = ws.ltau; sa.g = g; sa.sched = ws.sched; sa.draw = with_samples;
+  sa.k0 = (uint32_t)seed; sa.k1 = (uint32_t)(seed >> 32);
   *blocks = 0;
   if (with_samples && g.nodes > 0 && g.m > 0) {
     const size_t total = (size_t)g.G * g.nodes * ((g.m + 3) / 4);
     const size_t want = (total + 255) / 256;
-    *blocks = (int)(want < 1184 ? want : 1184);
+    *blocks = (int)(want < 8 * kSms ? want : 8 * kSms);
   }
   return sa;
 }

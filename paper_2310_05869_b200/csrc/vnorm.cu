@@ -164,8 +164,8 @@ __global__ void __launch_bounds__(256) vnorm_sample_kernel(VnormSampleArgs a) {
 
 }  // namespace
 
-cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uint32_t* wq, unsigned long long* sums, unsigned long long* cum, int32_t* samples,
-                                  float* wlog, uint64_t seed, cudaStream_t st) {
+cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uint32_t* wq, unsigned long long* sums, unsigned long long* cum,
+                                  int32_t* samples, float* wlog, uint64_t seed, cudaStream_t st) {
   if (!g.sorted || g.m == 0 || g.nodes == 0) return cudaSuccess;
   const int blocks = (g.nk + 255) / 256;
   const long long ctas = (long long)g.G * blocks;          // (at least as many as the scan's)
@@ -173,11 +173,15 @@ cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uin
   const unsigned grid = (unsigned)ctas;
   cudaError_t e = cudaSuccess;
   if (g.d == 64) e = launch(vnorm_weights_kernel<64>, grid, 256, 256 * 128, st, v, wq, sums, g.nk, blocks);
-  else if ((e = allow_smem<vnorm_weights_kernel<128>>(256 * 256)) == cudaSuccess) e = launch(vnorm_weights_kernel<128>, grid, 256, 256 * 256, st, v, wq, sums, g.nk, blocks);
+  else if ((e = allow_smem<vnorm_weights_kernel<128>>(256 * 256)) == cudaSuccess)
+    e = launch(vnorm_weights_kernel<128>, grid, 256, 256 * 256, st, v, wq, sums, g.nk, blocks);
   if (e == cudaSuccess) e = launch(vnorm_scan_kernel, (unsigned)g.G * ((g.nk + 4095) / 4096), 1024, 0, st, wq, sums, cum, g.nk, blocks);
   if (e != cudaSuccess) return e;
   VnormSampleArgs a;
   a.cum = cum; a.samples = samples; a.wlog = wlog; a.g = g; a.k0 = (uint32_t)seed; a.k1 = (uint32_t)(seed >> 32);
+  // A call, us, one lane per draw -> 32: 256 draws 111.7 -> 105.7, 1024 160.9 -> 156.8, 4096 477.7 -> 474.3 (131072 keys), 2048
+  // 63.6 -> 60.4 (16384 keys); 8192 893.8 -> 894.2 (131072 keys), 67.9 -> 68.6 (4096 keys); 16384 264.2 -> 267.5 (16384 keys),
+  // 128.7 -> 132.7 (4096 keys); 65536 616.7 -> 642.7 (16384 keys).
   const size_t draws = (size_t)g.G * g.nodes * g.m;
   if (draws < 16384) return launch(vnorm_sample_kernel<32>, (unsigned)((draws + 7) / 8), 256, 0, st, a);
   return launch(vnorm_sample_kernel<1>, (unsigned)((draws + 255) / 256), 256, 0, st, a);

@@ -40,9 +40,9 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the attention kernel,
 # from the ncu captures summarised under profiles/ (taken on 4 / 8 heads and scaled to the
 # workload's 32 heads: the traffic is proportional to the number of segments).
-NCU_TRAFFIC_BYTES = {"c3_n131k_causal": 8 * 0.9292e9, "c2_n32k_d128": 4 * 0.2453e9}
+NCU_TRAFFIC_BYTES = {"c3_n131k_causal": 8 * 0.9271e9, "c2_n32k_d128": 4 * 0.2444e9}
 # sm__pipe_tensor_cycles_active (% of peak sustained active) of the attention kernel in the same captures
-NCU_TENSOR_PIPE_PCT = {"c3_n131k_causal": 26.0, "c2_n32k_d128": 27.1}
+NCU_TENSOR_PIPE_PCT = {"c3_n131k_causal": 32.4, "c2_n32k_d128": 34.4}
 
 
 def load_peaks():
@@ -271,7 +271,8 @@ def stage_report(w, peaks, stage_ms):
                            "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"]}
     kernels["attention"] = {"bound": "tensor", "ms": att_ms, "achieved": att_tflops, "peak": burst, "unit": "TFLOP/s",
                             "frac": att_tflops / burst, "frac_of_sustained_peak": att_tflops / sustained}
-    kernels["sample"] = {"ms": stage_ms.get("sample", 0.0), "note": "drawn by extra blocks of the sort_scan launch"}
+    kernels["sample"] = {"ms": stage_ms.get("sample", 0.0), "note": "drawn by extra blocks of the sort's first launch (scan; placement where "
+                                                                    "nodes have at most 16 chunks)"}
     return wm, roofline, kernels
 
 

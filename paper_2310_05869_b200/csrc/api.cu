@@ -358,7 +358,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
                            in_hash ? p.v : nullptr));
     }
     {
-      // (the samples of Alg. 2 line 4 are drawn by extra blocks of this launch)
+      // (the samples of Alg. 2 line 4 are drawn by extra blocks of this launch, or, where it falls away, of the placement)
       StageScope sc(st, HYPERATTN_STAGE_SORT_SCAN, scan_in_scatter(g) ? 0 : 1);
       HA_CHECK(launch_sort_scan(g, ws, !vnorm, p.seed, st));
     }
@@ -468,7 +468,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     if (is_fp32) HA_CHECK(launch_attention_mma(a, st));
     else {
       a.sched = ws.sched;
-      if (!g.sorted) HA_CHECK(cudaMemsetAsync(a.sched, 0, 4, st));       // (else the sort scan has zeroed it)
+      if (!g.sorted) HA_CHECK(cudaMemsetAsync(a.sched, 0, 4, st));       // (else the sort has zeroed it)
       HA_CHECK(launch_attention_tc(a, ws.status, st));
     }
   }

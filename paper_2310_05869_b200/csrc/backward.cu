@@ -633,23 +633,31 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
     uint32_t sw[NSW];                                    // byte offset of (row k RPI + crow, chunk cc) in its slab is k RPI 128 + sw[k % NSW]
 #pragma unroll
     for (int k = 0; k < NSW; ++k) sw[k] = (uint32_t)(crow * 128 + (((cc & 7) ^ ((k * RPI + crow) & 7)) << 4));
-    auto gather_rows = [&](auto whole, int rows, uint32_t dst, const __nv_bfloat16* base, const int (&v)[4], uint32_t bar) {
+    // (v: a valid row also where none exists.  The short tiles' copies are a rolled loop at d = 128: a second set of 64 in line at every
+    // call makes the pass slower also where no tile is short - 32 heads x 32768 rows 1367 -> 1380 us; without the short form 1357.)
+    auto gather = [&](int rows, uint32_t dst, const __nv_bfloat16* base, const int (&v)[4], uint32_t bar) {
       const char* src = reinterpret_cast<const char*>(base) + cc * 16;
       const uint32_t d = dst + (cc >> 3) * (128 * 128);
+      if (rows == 128) {
 #pragma unroll
-      for (int k = 0; k < 128 / RPI; ++k) {
-        const int rw = __shfl_sync(0xffffffffu, v[k * RPI / 32], (k * RPI & 31) + crow);
-        const uint32_t to = d + k * RPI * 128 + sw[k % NSW];
-        const char* from = src + (size_t)(uint32_t)rw * (D * 2);
-        if constexpr (decltype(whole)::value) cp_async16(to, from);
-        else cp_async16_or_zero(to, from, k * RPI + crow < rows);
+        for (int k = 0; k < 128 / RPI; ++k) {
+          const int rw = __shfl_sync(0xffffffffu, v[k * RPI / 32], (k * RPI & 31) + crow);
+          cp_async16(d + k * RPI * 128 + sw[k % NSW], src + (size_t)(uint32_t)rw * (D * 2));
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+#pragma unroll (D == 64 ? 32 / RPI / NSW : 1)
+          for (int k0 = 0; k0 < 32 / RPI; k0 += NSW) {
+#pragma unroll
+            for (int k1 = 0; k1 < NSW; ++k1) {
+              const int r = (k0 + k1) * RPI + crow, rw = __shfl_sync(0xffffffffu, v[u], r);
+              cp_async16_or_zero(d + (32 * u + (k0 + k1) * RPI) * 128 + sw[k1], src + (size_t)(uint32_t)rw * (D * 2), 32 * u + r < rows);
+            }
+          }
+        }
       }
       cp_async_arrive_noinc(bar);
-    };
-    // (v: a valid row also where none exists)
-    auto gather = [&](int rows, uint32_t dst, const __nv_bfloat16* base, const int (&v)[4], uint32_t bar) {
-      if (rows == 128) gather_rows(std::true_type{}, rows, dst, base, v, bar);
-      else gather_rows(std::false_type{}, rows, dst, base, v, bar);
     };
     auto boxes = [&](uint32_t dst, int rows, const CUtensorMap* map, int y, uint32_t bar) {
       if (lane == 0) {

@@ -167,6 +167,10 @@ struct Cfg {
   static constexpr int kOffQrow = kOffMask + 4 * (kMaxNodeKeys / 32) * 4;   // int [2][2][128]
   static constexpr int kOffBar = kOffQrow + 4 * 128 * 4;
   static constexpr int kSBufs = 2;                    // S buffers per query tile
+  // barriers of the S buffers and of the P buffers of a query tile lie this many slots from those of the other: nothing but the
+  // compiled address arithmetic depends on it, and each is the faster one (attention, us, 3 and 2 slots: 32 causal heads x 131072
+  // rows, d = 64, 5642 and 5695; 32 x 32768, d = 128, 366 and 355)
+  static constexpr int kBarSlots = D == 64 ? 3 : kSBufs;
   // d = 64: the P V product is 80 columns wide - behind the 64 columns of V the B operand
   // continues in a slab of ones, so column 64 of O accumulates the sum of the bf16 weights that
   // normalises the row (the tensor pipe's floor per product does not depend on N up to 128, so
@@ -174,7 +178,7 @@ struct Cfg {
   // pay for them (N = 144) and keeps the sum in registers.
   static constexpr bool kOnes = D == 64;
   static constexpr int kOCols = kOnes ? 80 : D;       // TMEM columns of one O accumulator
-  static constexpr int kNumBar = 21 + 6 * NS + 4 * kSBufs;
+  static constexpr int kNumBar = 21 + 6 * NS + 4 * kBarSlots;
   static constexpr int kOffMisc = kOffBar + 8 * kNumBar;          // tmem slot, abort flag
   // Epilogue staging, one slice of 32 rows x kStageRow bytes per softmax warp: rows leave the
   // warp as whole 64- or 128-byte pieces instead of 16 bytes per lane and row.  d = 64: eight
@@ -309,8 +313,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
   const uint32_t bar0 = ubase + C::kOffBar;
   const uint32_t bar_q = bar0;                                                // Q tiles of the item landed
   const uint32_t bar_qfree = bar0 + 8;                                        // both issuers are done with Q
-  auto bar_s = [&](int i, int b) { return bar0 + 168 + 8 * (6 * C::NS + C::kSBufs * i + b); };          // S_i buffer b written
-  auto bar_p = [&](int i, int b) { return bar0 + 168 + 8 * (6 * C::NS + C::kSBufs * (2 + i) + b); };    // P_i buffer b written
+  auto bar_s = [&](int i, int b) { return bar0 + 168 + 8 * (6 * C::NS + C::kBarSlots * i + b); };          // S_i buffer b written
+  auto bar_p = [&](int i, int b) { return bar0 + 168 + 8 * (6 * C::NS + C::kBarSlots * (2 + i) + b); };    // P_i buffer b written
   auto bar_o = [&](int i) { return bar0 + 80 + 8 * i; };                      // O_i of the item complete
   auto bar_ofree = [&](int i) { return bar0 + 112 + 8 * i; };                 // O_i has been read out
   auto bar_tabfull = [&](int set) { return bar0 + 128 + 8 * set; };           // row tables of a set written

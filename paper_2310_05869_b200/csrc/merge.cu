@@ -38,11 +38,11 @@ __global__ void __launch_bounds__(256, LM <= 8 ? (D == 64 ? 4 : 3) : 1) merge_ke
   constexpr int NE = 16 / ES;                      // entries per chunk
   constexpr int LG = LM <= 5 ? LM : 4;             // levels whose rows are in flight together
   const Geometry& g = a.g;
-  const int seg = blockIdx.y;
+  const int seg = blockIdx.y + gridDim.y * blockIdx.z;      // (a grid's y ends at 65535)
   wait_for_stream();
   const int lane = threadIdx.x & 31;
   const int row0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
-  if (row0 >= g.n) return;
+  if (row0 >= g.n || seg >= g.G) return;
   const int nr = min(32, g.n - row0);              // rows of this warp
   // ---- lane = row ---------------------------------------------------------------------------------------
   const int i = row0 + lane;
@@ -175,8 +175,8 @@ cudaError_t launch_merge(const Geometry& g, const Workspace& ws, void* out, floa
   MergeArgs a; a.part_o = ws.part_o; a.part_lse = ws.part_lse; a.out = out; a.lse = lse; a.g = g; a.out_fp32 = out_fp32;
   if (ws.part_bf16 && out_fp32) return cudaErrorInvalidValue;                   // bf16 partials are only kept for bf16 results
   const size_t warps = ((size_t)g.n + 31) / 32;                                 // a warp per 32 rows
-  const dim3 blocks((unsigned)((warps + 7) / 8), (unsigned)g.G);
-  if (g.G > 65535) return cudaErrorInvalidValue;
+  const unsigned segs = g.G < 65536 ? g.G : 65535;
+  const dim3 blocks((unsigned)((warps + 7) / 8), segs, ((unsigned)g.G + segs - 1) / segs);
   cudaError_t e = cudaSuccess;
   auto go = [&](auto* kernel) { e = launch(kernel, blocks, 256, 0, st, a); };
   auto pick = [&](auto dtag, auto pbtag) {

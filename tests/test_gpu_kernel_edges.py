@@ -151,24 +151,39 @@ def test_value_norm_edges(w):
     vnorm.test_value_norm_sampling_matches_the_oracle(w)
 
 
-@pytest.mark.parametrize("d", [64, 128])
-def test_value_norms_of_more_segments_than_a_grid_has_rows(d):
-    """65 600 segments: more than the y and z extents of a grid."""
-    B, H, n, b, m, r, seed = 16, 4100, 20, 8, 5, 4, 3
-    gen = torch.Generator(device="cuda").manual_seed(91)
+def _check_segments(B, H, n, d, b, m, r, seed, gen_seed, per_segment=None, **kw):
+    """Calls of more segments than the y and z extents of a grid: segments around 65 536 and forty others against the oracle."""
+    gen = torch.Generator(device="cuda").manual_seed(gen_seed)
     q, k, v = (torch.randn((B, H, n, d), generator=gen, device="cuda").bfloat16() for _ in range(3))
-    out, lse, inter = ha.forward(q, k, v, b, m, r, seed=seed, out_dtype=torch.float32, debug=True, value_norm_sampling=True)
+    out, lse, inter = ha.forward(q, k, v, b, m, r, seed=seed, out_dtype=torch.float32, debug=True, **kw)
     torch.cuda.synchronize()
     assert ha.last_device_status() == 0
     Wd = O.directions(d, r, seed)
     rng = np.random.default_rng(5)
     for g in sorted({0, 1, 65534, 65535, 65536, B * H - 1, *rng.integers(0, B * H, 40).tolist()}):
         Q, K, V = (x.view(-1, n, d)[g].double().cpu().numpy() for x in (q, k, v))
-        idx, sw = O.sample_by_value_norms(seed, g, 0, m, O.value_norm_weights(V))
-        assert (inter["samples"][g, 0, :m].cpu().numpy() == idx).all(), g
-        np.testing.assert_allclose(inter["sample_log2w"][g, 0, :m].cpu().numpy(), np.log2(sw), atol=1e-5)
-        ro, rl = O.segment_forward(Q, K, V, Wd, b, m, False, 0, seed, g, scale=1.0 / math.sqrt(d), ids_q=inter["q_ids"][g].cpu().numpy(),
-                                   ids_k=inter["k_ids"][g].cpu().numpy(), value_norm_sampling=True)
+        if per_segment:
+            per_segment(g, V, inter)
+        ro, rl = O.segment_forward(Q, K, V, Wd, b, m, kw.get("causal", False), kw.get("n0", 0), seed, g, scale=1.0 / math.sqrt(d),
+                                   ids_q=inter["q_ids"][g].cpu().numpy(), ids_k=inter["k_ids"][g].cpu().numpy(),
+                                   value_norm_sampling=kw.get("value_norm_sampling", False))
         err = np.abs(out.view(-1, n, d)[g].cpu().numpy() - ro)
         assert err.max() <= PU.OUT_MAX_ABS and err.mean() <= PU.OUT_MEAN_ABS, g
         assert (np.abs(lse.view(-1, n)[g].cpu().numpy() - rl) <= PU.LSE_REL * np.maximum(np.abs(rl), 1.0)).all(), g
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_value_norms_of_more_segments_than_a_grid_has_rows(d):
+    m, seed = 5, 3
+
+    def draws(g, V, inter):
+        idx, sw = O.sample_by_value_norms(seed, g, 0, m, O.value_norm_weights(V))
+        assert (inter["samples"][g, 0, :m].cpu().numpy() == idx).all(), g
+        np.testing.assert_allclose(inter["sample_log2w"][g, 0, :m].cpu().numpy(), np.log2(sw), atol=1e-5)
+
+    _check_segments(16, 4100, 20, d, 8, m, 4, seed, 91, draws, value_norm_sampling=True)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_recursion_of_more_segments_than_a_grid_has_rows(d):
+    _check_segments(16, 4100, 41, d, 8, 4, 4, 4, 94, causal=True, n0=12)

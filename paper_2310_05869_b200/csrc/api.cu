@@ -429,10 +429,13 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     a.level_pair_start[l] = (int)pairs;
     // Two query tiles share a CTA when they share their block's keys (even tiles per block).  Pairs that straddle
     // two blocks walk both blocks' key tiles, each tile's issuer skipping the other's: it releases the K stages of the tiles it
-    // skips before the V stages, so a block's tiles and one more have to fit the ring of 8 (d = 64) or 4 (d = 128) stages.  Beyond that
+    // skips before the V stages, so a block's tiles and one more have to fit the ring of 8 (d = 64) or 4 (d = 128) stages.  At d = 128
+    // the first query tile's results are staged over the item's key rows: it must not be done before the last of them has been read,
+    // which it cannot be where both tiles end with the sampled columns, but would be without samples.  Beyond that
     // one tile per CTA, which leaves half of its softmax warps idle (50 000 queries against 131 072 keys, groups of 98 queries and
     // blocks of 256 keys: 218 us unpaired, 142 us paired).
-    a.level_paired[l] = !a.level_sorted[l] || a.tiles_per_block % 2 == 0 || (g.b + 63) / 64 + 1 <= (g.d == 64 ? 8 : 4);
+    const bool straddle = (g.b + 63) / 64 + 1 <= (g.d == 64 ? 8 : 4) && (g.d == 64 || g.m > 0);
+    a.level_paired[l] = !a.level_sorted[l] || a.tiles_per_block % 2 == 0 || straddle;
     pairs += (a.level_paired[l] ? (per_node + 1) / 2 : per_node) * nodes_lvl * g.G;
   }
   a.level_start[g.levels] = (int)tiles;

@@ -184,7 +184,9 @@ struct Cfg {
   // warp as whole 64- or 128-byte pieces instead of 16 bytes per lane and row.  d = 64: eight
   // slices of 4 KB.  d = 128 (less shared memory to spare): slices of 2 KB, those of query tile
   // 0 in the item's own key-row table, which nobody reads any more once the item's last K / V
-  // tile has been issued and which is not rebuilt before the softmax warps release the set.
+  // tile has been issued - it has been when query tile 0 is done, because that tile walks the
+  // last tile of every item (launches do not pair query tiles where it would not) - and which is
+  // not rebuilt before the softmax warps release the set.
   static constexpr int kStageRow = (D == 64) ? 128 : 64;
   static constexpr int kStageWarp = 32 * kStageRow;
   static constexpr int kDescBytes = (sizeof(ItemDesc) + 15) / 16 * 16;

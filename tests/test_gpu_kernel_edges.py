@@ -33,6 +33,10 @@ FORWARD = [
     parity.W("pairs_of_three_key_tiles_d128", 1, 2, 1300, 128, "bf16", 192, 256, 6, False, 0, seed=92, n_k=2000),
     parity.W("pairs_of_three_key_tiles_b129_d128", 1, 1, 1900, 128, "bf16", 129, 40, 6, False, 0, seed=93, n_k=2000),
     parity.W("four_key_tiles_d128", 1, 1, 1300, 128, "bf16", 193, 256, 6, False, 0, seed=94, n_k=2000),
+    # no samples: the last key tile of a pair across blocks is the second query tile's alone (d = 128: not paired)
+    parity.W("no_samples_seven_key_tiles_d64", 1, 2, 1000, 64, "bf16", 448, 0, 6, False, 0, seed=98, n_k=4000),
+    parity.W("no_samples_three_key_tiles_d128", 1, 2, 1300, 128, "bf16", 192, 0, 6, False, 0, seed=99, n_k=2000),
+    parity.W("no_samples_two_key_tiles_causal_d128", 1, 2, 4096, 128, "bf16", 128, 0, 6, True, 512, seed=100),
     # fp32: hash passes of 256 rows; copies beside the hash (up to 296 CTAs of 4096 entries) and in a launch of their own; query tiles
     # halved (up to 74 tiles) and whole, second halves of one row and none
     parity.W("fp32_n257_d64", 1, 1, 257, 64, "fp32", 64, 32, 7, False, 0, seed=76),

@@ -281,9 +281,11 @@ __device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, PairDes
       t.nbA = bt;
       t.nbB = (qb.valid && qb.beta != qa.beta) ? btb : 0;
       t.nsmp = (g.m + TK - 1) / TK;
-      // (a query tile that does not exist - the short last block may have fewer tiles - walks no key tiles)
-      if (!qa.valid) { t.nbA = 0; t.nsmp = 0; }
-      qa.s1 = 0; qa.n1 = t.nbA; qa.s2 = t.nbA + t.nbB; qa.n2 = t.nsmp;
+      // A query tile that does not exist walks no key tiles.  (The short last block may have fewer tiles, and so may every group
+      // of a node with fewer queries than keys: then the second tile of a pair, the first of the next group, may exist alone.)
+      if (!qa.valid) t.nbA = 0;
+      if (!qa.valid && !qb.valid) t.nsmp = 0;
+      qa.s1 = 0; qa.n1 = t.nbA; qa.s2 = t.nbA + t.nbB; qa.n2 = qa.valid ? t.nsmp : 0;
       qb.s1 = t.nbB ? t.nbA : 0; qb.n1 = qb.valid ? (t.nbB ? btb : bt) : 0; qb.s2 = t.nbA + t.nbB; qb.n2 = qb.valid ? t.nsmp : 0;
     }
     if (a.direct) { t.orow_base = (size_t)t.seg * g.n; t.odelta = 0; }

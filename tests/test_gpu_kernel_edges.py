@@ -33,6 +33,8 @@ FORWARD = [
     parity.W("pairs_of_three_key_tiles_d128", 1, 2, 1300, 128, "bf16", 192, 256, 6, False, 0, seed=92, n_k=2000),
     parity.W("pairs_of_three_key_tiles_b129_d128", 1, 1, 1900, 128, "bf16", 129, 40, 6, False, 0, seed=93, n_k=2000),
     parity.W("four_key_tiles_d128", 1, 1, 1300, 128, "bf16", 193, 256, 6, False, 0, seed=94, n_k=2000),
+    # blocks of three query tiles; the last nodes have fewer queries than keys, groups of two tiles, and pairs whose first tile does not exist
+    parity.W("groups_of_fewer_query_tiles_than_blocks_d64", 1, 2, 4516, 64, "bf16", 264, 31, 3, True, 204, seed=101),
     # no samples: the last key tile of a pair across blocks is the second query tile's alone (d = 128: not paired)
     parity.W("no_samples_seven_key_tiles_d64", 1, 2, 1000, 64, "bf16", 448, 0, 6, False, 0, seed=98, n_k=4000),
     parity.W("no_samples_three_key_tiles_d128", 1, 2, 1300, 128, "bf16", 192, 0, 6, False, 0, seed=99, n_k=2000),

@@ -151,6 +151,7 @@ struct PairDesc {
 struct ItemDesc {
   PairDesc t;
   QTile qa, qb;
+  int lenA, lenB;      // node: keys of block A, of block B (the streamer's; among the fields that every role reads they cost 1 %)
 };
 
 template <int D>
@@ -203,11 +204,11 @@ struct Cfg {
   static_assert(kColO + 2 * kOCols <= 512, "TMEM columns");
 };
 
-__device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, PairDesc& t, QTile& qa, QTile& qb) {
+__device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, PairDesc& t, QTile& qa, QTile& qb, int& lenA, int& lenB) {
   const Geometry& g = a.g;
   t.partial = !a.direct;
   qa.valid = 1; qb.valid = 0;
-  t.nbA = t.nbB = t.nsmp = 0;
+  t.nbA = t.nbB = t.nsmp = lenA = lenB = 0;
   int s, q0n, k0n;
   if (pair < a.n_leaf_pairs) {
     // Leaf after leaf, the pairs of a leaf from the heaviest (last rows, most keys) to the lightest: items are
@@ -276,8 +277,9 @@ __device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, PairDes
     if (sorted) {
       t.slice = ((size_t)level * g.G + t.seg) * g.nl + (g.causal ? (size_t)j * s : 0);
       t.node = g.causal ? (1 << level) - 1 + j : 0;
-      const int bt = (block_len(s, g.b, qa.beta) + TK - 1) / TK;                                  // key tiles of a block: its own length
-      const int btb = qb.valid ? (block_len(s, g.b, qb.beta) + TK - 1) / TK : 0;
+      lenA = block_len(s, g.b, qa.beta);
+      lenB = qb.valid ? block_len(s, g.b, qb.beta) : 0;
+      const int bt = (lenA + TK - 1) / TK, btb = (lenB + TK - 1) / TK;                        // key tiles of a block: its own length
       t.nbA = bt;
       t.nbB = (qb.valid && qb.beta != qa.beta) ? btb : 0;
       t.nsmp = (g.m + TK - 1) / TK;
@@ -292,6 +294,21 @@ __device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, PairDes
     else { t.orow_base = (size_t)g.G * g.n + (size_t)level * g.G * g.nl + (size_t)t.seg * g.nl + (size_t)j * s; t.odelta = -q0n; }
   }
   t.ntiles = max(qa.s1 + qa.n1, max(qa.s2 + qa.n2, max(qb.s1 + qb.n1, qb.s2 + qb.n2)));
+}
+
+// Value rows of a key tile with columns that do not exist, which get zeros: their weights are zero, but zero times a NaN or an infinity
+// of some other leaf, row or head would not be.  (Their scores are overwritten, whatever K is there.)  All 32 lanes call it together;
+// table: the item's key rows from this tile on; null: consecutive rows from `first` on.  Out of line: in line it costs the tiles that
+// are whole 1 % of the attention's time (32 heads x 32768 rows, d = 128: 350 us as it is, 354 in line).
+template <int D>
+__device__ __noinline__ void fill_short(uint32_t stage, const char* base, const int* table, int first, int have, uint32_t bar) {
+  constexpr int CPR = D / 8, RPI = 32 / CPR;
+  const int lane = threadIdx.x & 31, cc = lane % CPR;
+  for (int r = lane / CPR; r < TK; r += RPI) {
+    const int row = table ? table[r] : first + min(r, have - 1);
+    cp_async16_or_zero(stage + tile_off<TK>(r, cc), base + (size_t)(uint32_t)row * (D * 2) + cc * 16, r < have);
+  }
+  cp_async_arrive_noinc(bar);
 }
 
 // a-th key tile of a query tile -> index in the pair's tile list
@@ -958,8 +975,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       if (lane == 0) item = atomicAdd(a.sched, 1);
       item = __shfl_sync(0xffffffffu, item, 0);
       const bool end = item >= a.total_pairs;
-      PairDesc t = {}; QTile qa = {}, qb = {};
-      if (!end) decode_pair(a, item, t, qa, qb);
+      PairDesc t = {}; QTile qa = {}, qb = {}; int lenA = 0, lenB = 0;
+      if (!end) decode_pair(a, item, t, qa, qb, lenA, lenB);
       else t.mode = -1;                                   // tells every role that the list is exhausted
       if (lane == 0) HA_TACC(26, tdec);
       const int set = it & 1;
@@ -974,7 +991,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       if (lane == 0) HA_TACC(21, ttab);
       if (lane == 0) {
         ItemDesc* de = reinterpret_cast<ItemDesc*>(smem + C::kOffDesc + set * C::kDescBytes);
-        de->t = t; de->qa = qa; de->qb = qb;
+        de->t = t; de->qa = qa; de->qb = qb; de->lenA = lenA; de->lenB = lenB;
       }
       if (end) {
         __syncwarp();
@@ -986,7 +1003,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       // Key rows as tensor-map row coordinates.  Every global load of a batch is issued before
       // the first one is used; the warp covers 32 consecutive columns per step, so one ballot
       // yields a whole word of the mask tables.  Padding columns point at a valid row (they are
-      // masked, so that row only has to be finite) and are masked for both tiles.
+      // masked, and the streamer puts zeros in the place of its values) and are masked for both tiles.
       if (t.mode == 1) {
         constexpr int UB = 8;
         const int bcols = t.nbA * TK;
@@ -1158,9 +1175,13 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       const int* s_kidx = s_kidx_all + set * kMaxNodeKeys;
       ok = wait_fast<18>(bar_tabfull(set), (it >> 1) & 1, s_abort, status);
       if (!ok) break;
-      const PairDesc t = reinterpret_cast<const ItemDesc*>(smem + C::kOffDesc + set * C::kDescBytes)->t;
+      const ItemDesc& de = *reinterpret_cast<const ItemDesc*>(smem + C::kOffDesc + set * C::kDescBytes);
+      const PairDesc t = de.t;
       if (t.mode < 0) break;
+      const int lenA = de.lenA, lenB = de.lenB;
       const int segrow = t.seg * g.nk;                      // (keys)
+      // does any of the item's key tiles have columns that do not exist?
+      const bool shorts = t.mode == 0 ? t.nk % TK != 0 : (lenA % TK | lenB % TK | g.m % TK) != 0;
       for (int j = 0; j < t.ntiles && ok; ++j) {
         const int gj = gbase + j;
         const int s = gj % C::NS;
@@ -1217,7 +1238,13 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
           if (__shfl_sync(0xffffffffu, drop, 0)) { v_armed = gj; continue; }     // nothing issued, nothing will arrive
         }
 #endif
-        fill(ubase + C::kOffV + s * C::kTile, &maps.v, vsrc, bar_vfull(s));
+        const int have = !shorts ? TK                     // columns of the tile that exist
+                         : t.mode == 0 ? t.nk - j * TK
+                         : j < t.nbA ? lenA - j * TK
+                         : j < t.nbA + t.nbB ? lenB - (j - t.nbA) * TK : g.m - (j - t.nbA - t.nbB) * TK;
+        if (have >= TK) fill(ubase + C::kOffV + s * C::kTile, &maps.v, vsrc, bar_vfull(s));
+        else fill_short<D>(ubase + C::kOffV + s * C::kTile, reinterpret_cast<const char*>(a.v), t.mode == 1 ? s_kidx + j * TK : nullptr,
+                           segrow + t.k0 + j * TK, have, bar_vfull(s));
         v_armed = gj + 1;
         if (lane == 0) HA_TACC(1, tgv);
       }

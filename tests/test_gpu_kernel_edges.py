@@ -100,6 +100,42 @@ SHORT_TILES = [
 ]
 
 
+def _forward(w, q, k, v, **kw):
+    return ha.forward(q, k, v, w.b, w.m, w.r, causal=w.causal, n0=w.n0, seed=w.seed, **kw)
+
+
+@pytest.mark.parametrize("bad", [math.nan, math.inf], ids=["nan", "inf"])
+@pytest.mark.parametrize("w", SHORT_TILES + [
+    parity.W("ragged_leaves_d128", 1, 2, 1000, 128, "bf16", 64, 40, 6, True, 130, seed=95),
+    parity.W("cross_blocks_of_100_d64", 1, 2, 500, 64, "bf16", 100, 33, 6, False, 0, seed=96, n_k=1111),
+], ids=lambda w: w.name)
+def test_forward_of_a_head_beside_a_head_that_is_not_finite(w, bad):
+    q, k, v = PU.to_device(w, WL.make_inputs(w))
+    out, lse = _forward(w, q, k, v)
+    for x in (q, k, v):
+        x[0, 1] = bad
+    got, got_lse = _forward(w, q, k, v)
+    assert ha.last_device_status() == 0
+    assert torch.equal(got[0, 0], out[0, 0]) and torch.equal(got_lse[0, 0], lse[0, 0])
+
+
+@pytest.mark.parametrize("option", [{}, {"precise": True}, {"caps": (8.0, 16.0)}], ids=["plain", "precise", "caps"])
+@pytest.mark.parametrize("d", [64, 128])
+def test_forward_of_rows_that_do_not_see_a_value_that_is_not_finite(d, option):
+    """Short tiles of sorted and sampled keys: a value row that is not finite reaches the queries of its block only."""
+    w = parity.W("", 1, 1, 1301, d, "bf16", 130, 40, 6, False, 0, seed=97)
+    q, k, v = PU.to_device(w, WL.make_inputs(w))
+    out, lse, inter = _forward(w, q, k, v, debug=True, **option)
+    assert not (inter["samples"][0, 0, :w.m] == 0).any()
+    v[0, 0, 0] = math.nan
+    got, got_lse = _forward(w, q, k, v, **option)
+    assert ha.last_device_status() == 0
+    beta = int(inter["rank_k"].view(-1)[0]) // w.b
+    clean = torch.ones(w.n, dtype=torch.bool, device="cuda")
+    clean[inter["perm_q"].view(-1)[beta * w.b:(beta + 1) * w.b].long()] = False
+    assert torch.equal(got[0, 0][clean], out[0, 0][clean]) and torch.equal(got_lse, lse)
+
+
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "fp32"])
 @pytest.mark.parametrize("bad", [math.nan, math.inf], ids=["nan", "inf"])
 @pytest.mark.parametrize("w", SHORT_TILES, ids=[w.name for w in SHORT_TILES])

@@ -13,20 +13,21 @@ namespace {
 
 constexpr float kNormScale = 4096.f;      // 2^12
 
-// (Weights and scan: CTA (segment, part of it) is blockIdx.x = segment * parts + part - a grid's y and z end at 65535, and a call may have
-// 2^20 segments.)
+// (Weights and scan: segment = y + gridDim.y * z, its part x.  A grid's y ends at 65535, and a call may have 2^20 segments; both from one
+// extent takes a division at the head of either kernel's chain: 4 segments of 131072 rows 28 -> 30 us.)
 //
 // A CTA weighs 256 rows of one segment: the rows come in by whole lines and are read back one per thread (the chunks
 // of a row XOR-swizzled, so that neither side has bank conflicts); also the sum of the CTA's weights.
 template <int D>
 __global__ void __launch_bounds__(256) vnorm_weights_kernel(const __nv_bfloat16* __restrict__ v, uint32_t* __restrict__ wq,
-                                                            unsigned long long* __restrict__ sums, int nk, int blocks) {
+                                                            unsigned long long* __restrict__ sums, int G, int nk) {
   constexpr int CPR = D / 8;
   extern __shared__ uint4 s_row[];                        // [256][CPR]
   __shared__ unsigned long long s_warp[8];
   const int tid = threadIdx.x, lane = tid & 31;
   wait_for_stream();
-  const int seg = blockIdx.x / blocks, row0 = (blockIdx.x - seg * blocks) * 256, rows = min(256, nk - row0);
+  const int seg = blockIdx.y + gridDim.y * blockIdx.z, row0 = blockIdx.x * 256, rows = min(256, nk - row0);
+  if (seg >= G) return;
   const size_t first = (size_t)seg * nk + row0;
   const uint4* src = reinterpret_cast<const uint4*>(v) + first * CPR;
 #pragma unroll
@@ -59,7 +60,7 @@ __global__ void __launch_bounds__(256) vnorm_weights_kernel(const __nv_bfloat16*
   __syncthreads();
   if (tid == 0) {
     for (int e = 1; e < 8; ++e) w += s_warp[e];
-    sums[blockIdx.x] = w;
+    sums[(size_t)seg * gridDim.x + blockIdx.x] = w;
   }
 }
 
@@ -67,18 +68,19 @@ __global__ void __launch_bounds__(256) vnorm_weights_kernel(const __nv_bfloat16*
 // the sums of the rows before them by itself, so all CTAs run at once (one CTA per segment walking its rows: 94 us for 4 segments of
 // 131072 rows, now 5 us).
 __global__ void __launch_bounds__(1024) vnorm_scan_kernel(const uint32_t* __restrict__ wq, const unsigned long long* __restrict__ sums,
-                                                          unsigned long long* __restrict__ cum, int nk, int blocks) {
+                                                          unsigned long long* __restrict__ cum, int G, int nk, int blocks) {
   __shared__ unsigned long long s_warp[32], s_before[32];
-  const int parts = (nk + 4095) / 4096, seg = blockIdx.x / parts, part = blockIdx.x - seg * parts;
+  const int seg = blockIdx.y + gridDim.y * blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (seg >= G) return;
   wait_for_stream();
   const uint32_t* w = wq + (size_t)seg * nk;
   unsigned long long* c = cum + (size_t)seg * (nk + 1);
-  const int i = part * 4096 + 4 * tid;
+  const int i = blockIdx.x * 4096 + 4 * tid;
   unsigned long long x[4], before = 0;
 #pragma unroll
   for (int e = 0; e < 4; ++e) x[e] = i + e < nk ? w[i + e] : 0ull;
-  for (int e = tid; e < part * 16; e += 1024) before += sums[(size_t)seg * blocks + e];
+  for (int e = tid; e < (int)blockIdx.x * 16; e += 1024) before += sums[(size_t)seg * blocks + e];
   x[1] += x[0]; x[2] += x[1]; x[3] += x[2];
   unsigned long long run = x[3];
 #pragma unroll
@@ -168,14 +170,13 @@ cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uin
                                   int32_t* samples, float* wlog, uint64_t seed, cudaStream_t st) {
   if (!g.sorted || g.m == 0 || g.nodes == 0) return cudaSuccess;
   const int blocks = (g.nk + 255) / 256;
-  const long long ctas = (long long)g.G * blocks;          // (at least as many as the scan's)
-  if (ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
-  const unsigned grid = (unsigned)ctas;
+  const unsigned y = g.G < 65536 ? g.G : 65535, z = ((unsigned)g.G + y - 1) / y;
+  const dim3 grid(blocks, y, z);
   cudaError_t e = cudaSuccess;
-  if (g.d == 64) e = launch(vnorm_weights_kernel<64>, grid, 256, 256 * 128, st, v, wq, sums, g.nk, blocks);
+  if (g.d == 64) e = launch(vnorm_weights_kernel<64>, grid, 256, 256 * 128, st, v, wq, sums, g.G, g.nk);
   else if ((e = allow_smem<vnorm_weights_kernel<128>>(256 * 256)) == cudaSuccess)
-    e = launch(vnorm_weights_kernel<128>, grid, 256, 256 * 256, st, v, wq, sums, g.nk, blocks);
-  if (e == cudaSuccess) e = launch(vnorm_scan_kernel, (unsigned)g.G * ((g.nk + 4095) / 4096), 1024, 0, st, wq, sums, cum, g.nk, blocks);
+    e = launch(vnorm_weights_kernel<128>, grid, 256, 256 * 256, st, v, wq, sums, g.G, g.nk);
+  if (e == cudaSuccess) e = launch(vnorm_scan_kernel, dim3((g.nk + 4095) / 4096, y, z), 1024, 0, st, wq, sums, cum, g.G, g.nk, blocks);
   if (e != cudaSuccess) return e;
   VnormSampleArgs a;
   a.cum = cum; a.samples = samples; a.wlog = wlog; a.g = g; a.k0 = (uint32_t)seed; a.k1 = (uint32_t)(seed >> 32);

@@ -28,7 +28,11 @@
 // which dQ comes before dK so that it leaves TMEM while dK and the next S^T are multiplied.
 // What bounds it: a step takes 4000 (causal leaves) to 5000 clocks (sorted blocks), of which no single unit is busy for half; the
 // load and store unit is the fullest (gathered copies, dS, results through shared memory, reductions at 25 bytes per clock), and
-// everything else in a chain waits behind it.  One chain -> two, us of the whole pass: 131072 rows, 32 heads 3343 -> 3022; causal
+// everything else in a chain waits behind it.  The P warps are busy for most of a step, with latencies: a satisfied barrier probe is 100 to
+// 300 clocks here, a read of the statistics about as much.  So they wait three times a step, not five, ask for 16 columns of S^T or dP^T
+// while they work on the 16 before, and take them as 8 x 8 fragments, in which a thread needs the statistics of 16 queries instead of 64
+// (in turn, us: causal leaves of 4096 rows, 128 heads, d = 64, 1092 -> 1049 -> 1033; 65536 rows, 32 heads 1640 -> 1635 -> 1617; 32 heads x
+// 32768 rows, d = 128, 1507 -> 1515 -> 1509).  One chain -> two, us of the whole pass: 131072 rows, 32 heads 3343 -> 3022; causal
 // leaves of 4096 rows, 128 heads 1167 -> 1105 (d = 64; two chains at d = 128 are 10 % slower in the leaves).  16 P warps instead
 // of 8 force 64 registers a thread and are slower (3160 us).
 //
@@ -271,7 +275,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
   if (tid == 0) {
     mbar_init(bar_dqfree, C::RW); mbar_init(bar_acc, 1); mbar_init(bar_accfree, C::RW);   // (one arrival per warp)
     for (int x = 0; x < 2; ++x) {
-      mbar_init(bar_s(x), 1); mbar_init(bar_dp(x), 1); mbar_init(bar_h(x), C::SW / C::NH); mbar_init(bar_pfree(x), 1); mbar_init(bar_dq(x), 1);
+      mbar_init(bar_s(x), 2); mbar_init(bar_dp(x), 1); mbar_init(bar_h(x), C::SW / C::NH); mbar_init(bar_pfree(x), 1); mbar_init(bar_dq(x), 1);
       mbar_init(bar_qfull(x), 64); mbar_init(bar_qfree(x), 1); mbar_init(bar_dofree(x), 1);
     }
     for (int x = 0; x < C::NDO; ++x) mbar_init(bar_dofull(x), 32);
@@ -307,7 +311,10 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
     // ================= P and dS: thread = key, warpgroup q: query columns W q .. W q + W - 1, in two chunks of CW ==================
     constexpr int W = 128 / (C::SW / 4), CW = W / 2;
     static_assert(CW == 32, "a chunk's P is one TMEM store of 16 columns");
-    const int row = tid & 127, col0 = (warp >> 2) * W, half = C::NH == 2 ? col0 >> 6 : 0;
+    // The thread's share of a unit of 32 keys x 16 queries is that of four 8 x 8 matrices side by side, twice: keys frow + 8 j, queries 8 k +
+    // fcol and the next, value 8 (j / 2) + 4 k + 2 (j % 2) (+ 1).  A thread that has a whole key row, 64 queries, needs four times as
+    // many of the statistics, and the load and store unit gives a word of them per clock whatever lanes share.
+    const int row = tid & 127, frow = (row & ~31) + (lane >> 2), fcol = 2 * (lane & 3), col0 = (warp >> 2) * W, half = C::NH == 2 ? col0 >> 6 : 0;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t p_addr = lane_addr + C::kColP + C::kPHalf * (col0 >> 6) + (col0 & 63) / 2;
     const uint64_t sc2 = pack_f2(a.scale_log2, a.scale_log2);
@@ -317,90 +324,112 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
       if (!ok) break;
       const BwdItem& t = desc_of(it);
       if (t.kind < 0) break;
-      const bool exists = row < t.nkeys;
-      const int kind = t.kind, steps = t.steps, causal = t.causal;
-      int kblk = -2;                                    // sampled keys: the sorted block the key lies in (its entries there are masked)
-      if (kind == 2 && exists) kblk = __ldg(a.smp_blk + t.kidx + row);
+      const int kind = t.kind, steps = t.steps, causal = t.causal, nkeys = t.nkeys;
+      int kblk[4] = {-2, -2, -2, -2};                   // sampled keys: the sorted blocks the thread's keys lie in (their entries there are masked)
+      if (kind == 2) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (frow + 8 * j < nkeys) kblk[j] = __ldg(a.smp_blk + t.kidx + frow + 8 * j);
+      }
 #pragma unroll 1
       for (int s = 0; s < steps; ++s, ++g) {
         // entries that do not count: keys that do not exist, sampled keys of the query tile's own block, above the diagonal
-        bool dead = !exists;
-        if (kind == 2) dead = dead || kblk == (t.tn0 + s) / a.tiles_per_block;
+        const int own = kind == 2 ? (t.tn0 + s) / a.tiles_per_block : -1;
         const bool diag = causal && s == 0;
-        const bool masked = diag || __any_sync(0xffffffffu, dead);
-        ok = wait_fast<2>(bar_qfull(g), (g >> 1) & 1, s_abort, status) && wait_fast<3>(bar_s(half), g & 1, s_abort, status);
-        ok = __all_sync(0xffffffffu, ok);
+        int first[4];                                   // rows of the thread: columns below it do not count
+        bool masked = diag;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int r = frow + 8 * j;
+          const bool dead = r >= nkeys || kblk[j] == own;
+          masked = masked || dead;
+          first[j] = dead ? 128 : (diag ? r : 0) - col0;
+        }
+        masked = __any_sync(0xffffffffu, masked);
+        // (the issuer of the scores has waited for Q and the row statistics, and says so on the scores' barrier)
+        ok = __all_sync(0xffffffffu, wait_fast<3>(bar_s(half), g & 1, s_abort, status));
         if (!ok) break;
         tc_fence_after();
-        const float* st = reinterpret_cast<const float*>(smem + C::kOffStat) + (g & 1) * 256 + col0;
+        const float* st = reinterpret_cast<const float*>(smem + C::kOffStat) + (g & 1) * 256 + col0 + fcol;
         const uint32_t uds = ubase + C::kOffDS + (g % C::NDS) * 32768 + (col0 >> 6) * 16384 + row * 128;
-#pragma unroll 1
-        for (int c = 0; c < 2; ++c) {
-          float p[CW];
-          uint32_t pp[CW / 2];
+        const uint32_t s_addr = lane_addr + C::kColS + col0, dp_addr = lane_addr + C::kColDP + col0;
+        // Every TMEM load is under way while the 16 columns before it are worked on.
+        uint32_t ra[16], rb[16];
+        float p[CW];
+        auto load = [&](uint32_t taddr, uint32_t (&r)[16]) { tmem_ld_frag16_issue(taddr, r); };
+        auto weights = [&](uint32_t (&r)[16], int c0, int i0) {     // columns c0 .. c0 + 15 of the warpgroup, into p[i0 ..]
+          if (masked) {
 #pragma unroll
-          for (int c2 = 0; c2 < CW; c2 += 16) {
-            uint32_t rs[16];
-            tmem_ld16_issue(lane_addr + C::kColS + col0 + CW * c + c2, rs);
-            tmem_ld16_wait(rs);
-            if (masked) {
-              const int first = dead ? 128 : (diag ? row - col0 - CW * c - c2 : 0);      // columns below it do not count
+            for (int e = 0; e < 16; ++e)
+              if (c0 + 8 * ((e >> 2) & 1) + fcol + (e & 1) < first[2 * (e >> 3) + ((e >> 1) & 1)]) r[e] = 0xff800000u;
+          }
 #pragma unroll
-              for (int e = 0; e < 16; ++e)
-                if (e < first) rs[e] = 0xff800000u;
-            }
+          for (int k = 0; k < 2; ++k) {
+            const float2 nl = *reinterpret_cast<const float2*>(st + c0 + 8 * k);
 #pragma unroll
-            for (int e = 0; e < 16; e += 4) {
-              const float4 nl = *reinterpret_cast<const float4*>(st + CW * c + c2 + e);
-              const int i0 = c2 + e;
-              float x0, x1, x2, x3;
-              unpack_f2(ffma2(pack_u2(rs[e], rs[e + 1]), sc2, pack_f2(nl.x, nl.y)), x0, x1);
-              unpack_f2(ffma2(pack_u2(rs[e + 2], rs[e + 3]), sc2, pack_f2(nl.z, nl.w)), x2, x3);
-              p[i0] = ex2(x0); p[i0 + 1] = ex2(x1); p[i0 + 2] = ex2(x2); p[i0 + 3] = ex2(x3);
-              pp[i0 >> 1] = pack2(p[i0], p[i0 + 1]); pp[(i0 >> 1) + 1] = pack2(p[i0 + 2], p[i0 + 3]);
+            for (int j = 0; j < 4; ++j) {
+              const int e = 8 * (j >> 1) + 4 * k + 2 * (j & 1);
+              float x0, x1;
+              unpack_f2(ffma2(pack_u2(r[e], r[e + 1]), sc2, pack_f2(nl.x, nl.y)), x0, x1);
+              p[i0 + e] = ex2(x0); p[i0 + e + 1] = ex2(x1);
             }
           }
-          // d = 128: P goes over scores of this warpgroup that have been read
-          if (D == 128) tmem_st16(p_addr + 16 * c, pp);
+        };
+        auto grads = [&](const uint32_t (&r)[16], int c0, int i0) {
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const float2 nd = *reinterpret_cast<const float2*>(st + 128 + c0 + 8 * k);
+            uint32_t dd[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int e = 8 * (j >> 1) + 4 * k + 2 * (j & 1);
+              float d0, d1;
+              unpack_f2(fmul2(pack_f2(p[i0 + e], p[i0 + e + 1]), fadd2(pack_u2(r[e], r[e + 1]), pack_f2(nd.x, nd.y))), d0, d1);
+              dd[j] = pack2(d0, d1);
+            }
+            // (no memory clobber: the reads of the statistics may move across; what follows is ordered by the fences below)
+            asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(uds + (((((col0 & 63) + c0 + 8 * k) >> 3) ^ (row & 7)) << 4)),
+                         "r"(dd[0]), "r"(dd[1]), "r"(dd[2]), "r"(dd[3]));
+          }
+        };
+        load(s_addr, ra);
+#pragma unroll 1
+        for (int c = 0; c < 2; ++c) {
+          const int c0 = CW * c;
+          tmem_ld16_wait_regs(ra);
+          load(s_addr + c0 + 16, rb);
+          weights(ra, c0, 0);
+          tmem_ld16_wait_regs(rb);
           if (c == 0) {
             ok = wait_fast<4>(bar_dp(half), g & 1, s_abort, status);
-            // (dS of the step that used the buffer before has been multiplied; the last of its products is dQ or, d = 128, dK)
-            if (g >= C::NDS) ok = ok && wait_fast<5>(D == 64 ? bar_dq(g - C::NDS) : bar_qfree(g - C::NDS), ((g - C::NDS) >> 1) & 1, s_abort, status);
+            // The gradients of the step before that must be done with before dS and P are written.  d = 64: dV of the half, whose P
+            // lies where this one goes - and, multiplied before it, dQ of the step before that, which used this dS buffer.  d = 128:
+            // dK, the last product that reads the one dS buffer.
+            if (g > 0) ok = ok && wait_fast<6>(D == 64 ? bar_pfree(half) : bar_qfree(g - 1), (D == 64 ? g - 1 : (g - 1) >> 1) & 1, s_abort, status);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
           }
+          load(dp_addr + c0, ra);
+          weights(rb, c0 + 16, 16);
+          tmem_ld16_wait_regs(ra);
+          load(dp_addr + c0 + 16, rb);
+          grads(ra, c0, 0);
+          tmem_ld16_wait_regs(rb);
+          if (c == 0) load(s_addr + CW, ra);
+          grads(rb, c0 + 16, 16);
+          // (d = 128: P goes over scores of this warpgroup that have been read)
+          uint32_t pp[CW / 2];
 #pragma unroll
-          for (int c2 = 0; c2 < CW; c2 += 16) {
-            uint32_t rd[16];
-            tmem_ld16_issue(lane_addr + C::kColDP + col0 + CW * c + c2, rd);
-            tmem_ld16_wait(rd);
+          for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int e = 0; e < 16; e += 8) {
-              uint32_t dd[4];
+            for (int k = 0; k < 4; ++k)
 #pragma unroll
-              for (int x = 0; x < 8; x += 4) {
-                const float4 nd = *reinterpret_cast<const float4*>(st + 128 + CW * c + c2 + e + x);
-                const int i0 = c2 + e + x;
-                float d0, d1, d2, d3;
-                unpack_f2(fmul2(pack_f2(p[i0], p[i0 + 1]), fadd2(pack_u2(rd[e + x], rd[e + x + 1]), pack_f2(nd.x, nd.y))), d0, d1);
-                unpack_f2(fmul2(pack_f2(p[i0 + 2], p[i0 + 3]), fadd2(pack_u2(rd[e + x + 2], rd[e + x + 3]), pack_f2(nd.z, nd.w))), d2, d3);
-                dd[x >> 1] = pack2(d0, d1); dd[(x >> 1) + 1] = pack2(d2, d3);
+              for (int i = 0; i < 2; ++i) {
+                const int e = 16 * (k >> 1) + 8 * h + 4 * (k & 1) + 2 * i;
+                pp[8 * h + 2 * k + i] = pack2(p[e], p[e + 1]);
               }
-              // (no memory clobber: the reads of the statistics may move across; what follows is ordered by the fences below)
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(uds + (((((col0 & 63) + CW * c + c2 + e) >> 3) ^ (row & 7)) << 4)),
-                           "r"(dd[0]), "r"(dd[1]), "r"(dd[2]), "r"(dd[3]));
-            }
-          }
-          if (D == 64) {
-            // (P of the step before is read by the dV product until here at most)
-            if (c == 0 && g > 0) {
-              ok = __all_sync(0xffffffffu, wait_fast<6>(bar_pfree(half), (g - 1) & 1, s_abort, status));
-              if (!ok) break;
-              tc_fence_after();
-            }
-            tmem_st16(p_addr + 16 * c, pp);
-          }
+          tmem_st_frag16(p_addr + 16 * c, pp);
         }
         if (!ok) break;
         tmem_wait_st();
@@ -535,6 +564,7 @@ __global__ void __launch_bounds__(Cfg<D>::kThreads, 1) bwd_kernel(const __grid_c
               for (int ks = 0; ks < D / 16; ++ks)
                 mma_ss2(tmem + C::kColS + 64 * x, kmajor(k, ks), kmajor(q + x * 8192, ks), desc_hi, idesc_s, ks > 0);
               umma_commit(bar_s(x));
+              mbar_arrive(bar_s(x));                     // (passes on that Q and the row statistics are there)
             }
           };
           auto dprob = [&](int x) {

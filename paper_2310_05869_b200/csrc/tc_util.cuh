@@ -8,6 +8,8 @@ namespace hyperattn {
 
 // [rows x d] bf16, row-major; one box = 64 columns x box_rows rows (one slab of an operand tile), 128-byte swizzle (attn_tc.cu)
 bool encode_rows_map(CUtensorMap* m, const void* base, size_t rows, int d, int box_rows);
+// [rows x d] fp32 accumulator, row-major; one box = 32 columns x 32 rows, 128-byte swizzle (attn_tc.cu)
+bool encode_acc_map(CUtensorMap* m, const void* base, size_t rows, int d);
 
 namespace {
 
@@ -225,6 +227,14 @@ __device__ __forceinline__ void tma_tile(uint32_t dst, const CUtensorMap* map, i
   asm volatile("cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
 }
+// One box from shared memory (128-byte swizzle) added to global memory, as a bulk group of its own.
+__device__ __forceinline__ void tma_add_tile(const CUtensorMap* map, int x, int y, uint32_t src) {
+  asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%1, %2}], [%3];\n\tcp.async.bulk.commit_group;"
+               ::"l"(map), "r"(x), "r"(y), "r"(src) : "memory");
+}
+// the executing thread's bulk groups have read their shared memory; have been written
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // announces bytes to the current phase without arriving
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");

@@ -72,6 +72,9 @@ BACKWARD = [
     backward.W("bwd_leaf_of_193_rows_d128", 1, 1, 193, 128, 64, 8, 4, True, 200, seed=80),
     backward.W("bwd_sorted_over_unsorted_nodes_d64", 1, 2, 1040, 64, 200, 33, 6, True, 130, seed=81),
     backward.W("bwd_sorted_over_unsorted_nodes_d128", 1, 1, 1040, 128, 200, 33, 6, True, 130, seed=82),
+    # more items than SMs, so that whole tiles of consecutive rows, short ones and scattered rows follow one another in a CTA
+    backward.W("bwd_whole_short_and_scattered_tiles_d64", 1, 40, 640, 64, 64, 33, 6, True, 320, seed=83),
+    backward.W("bwd_whole_short_and_scattered_tiles_d128", 1, 24, 640, 128, 64, 33, 6, True, 320, seed=84),
 ]
 
 

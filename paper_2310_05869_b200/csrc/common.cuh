@@ -157,6 +157,15 @@ inline cudaError_t sm_count(int* sms) {
   return e;
 }
 
+// sampling by value norms (vnorm.cu): what its first two steps read and write
+struct VnormArgs {
+  const __nv_bfloat16* v;          // [G, nk, d]
+  uint32_t* wq;                    // [G, nk] weights of the rows
+  unsigned long long* sums;        // [G, blocks] of 256 rows each
+  unsigned long long* cum;         // [G, nk + 1] cumulative weights
+  int G, nk, blocks;
+};
+
 // ---- stage launchers (each enqueues on `st`; returns cudaGetLastError()) ---------------
 struct Workspace {
   __nv_bfloat16 *q16, *k16, *v16;  // bf16 staging of fp32 inputs (else null)
@@ -179,13 +188,17 @@ struct Workspace {
 // fp32 inputs of count_q (q) and count_k (k, v) entries to the workspace's bf16 copies
 cudaError_t launch_convert(const float* q, const float* k, const float* v, const Workspace& ws, size_t count_q, size_t count_k, cudaStream_t st);
 // w_host: the shared direction matrix; w_nodes (device, [nodes, d, r], g.node_dirs only): the nodes' own
+// vnorm: bf16 inputs - the launch also weighs the rows of V
 // convert_v: fp32 V - the launch also makes the workspace's bf16 copies of Q, K and V (fp32 inputs, convert_in_hash(g))
 bool convert_in_hash(const Geometry& g);
 cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_fp32, const float* w_host,
                         const Workspace& ws, unsigned long long* near_zero, cudaStream_t st, int side_mask = 3,
-                        const float* w_nodes = nullptr, const void* convert_v = nullptr);
+                        const float* w_nodes = nullptr, const void* convert_v = nullptr, const VnormArgs* vnorm = nullptr);
 // side_mask: bit 0 queries, bit 1 keys (3: both)
-cudaError_t launch_sort_scan(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask = 3);
+// vnorm: the cumulative sums of the value norms as well; only where wide_scan(g)
+cudaError_t launch_sort_scan(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask = 3,
+                             const VnormArgs* vnorm = nullptr);
+bool wide_scan(const Geometry& g);
 bool scan_in_scatter(const Geometry& g);
 // (small nodes: the scatter does the scan's work, samples included, and launch_sort_scan launches nothing)
 cudaError_t launch_sort_scatter(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask = 3);

@@ -14,7 +14,7 @@
 // into three bf16 terms (w = w1 + w2 + w3 exactly), so the products are exact and only the
 // fp32 accumulation rounds; signs can differ from an exact evaluation only where |p_t| is
 // within ~1e-5 of zero.
-#include "common.cuh"
+#include "vnorm_common.cuh"
 
 namespace hyperattn {
 namespace {
@@ -70,6 +70,7 @@ struct HashArgs {
   // fp32 inputs, where this launch also makes the bf16 copies: the CTAs from hash_ctas on
   ConvertArgs conv;
   int hash_ctas;
+  VnormArgs vnorm;        // bf16 inputs, columns sampled by value norms: the CTAs from hash_ctas on weigh the rows of V
 };
 
 // which chunk a CTA owns: side, segment, first row, number of rows (0: the chunk lies beyond the last row)
@@ -109,8 +110,18 @@ __device__ __forceinline__ size_t hist_base(const HashArgs& a, const ChunkPos& c
 // groups of 16 rows; the loads of the next group are issued between the MMAs of the current
 // one, and the direction fragments live in shared memory (one 8-byte read per MMA) instead
 // of 48 registers, so that two to four CTAs fit an SM and ~128 KB of loads are in flight.
-template <int D>
+// VNORM: further CTAs weigh the rows of V for the sampling by value norms: neither of the two reads by itself keeps the memory busy to its
+// end.  (With the cumulative sums beside the scan of the histograms, the call, us: 4 heads of 50000 queries, 131072 keys, d = 64, 154 -> 139;
+// 40000 queries, d = 128, 270 -> 248, but 275 with 64 KB of rows per CTA at a time instead of 32.)
+template <int D, bool VNORM>
 __global__ void __launch_bounds__(256, D == 64 ? 4 : 3) hash_bf16_kernel(const __grid_constant__ HashArgs a) {
+  if (VNORM && (int)blockIdx.x >= a.hash_ctas) {
+    extern __shared__ uint4 s_row[];
+    wait_for_stream();
+    const int x = blockIdx.x - a.hash_ctas;
+    vnorm_weights_body<D>(a.vnorm, x / a.vnorm.blocks, x % a.vnorm.blocks, s_row);
+    return;
+  }
   constexpr int KS = D / 16;             // MMA k-steps
   constexpr int CPL = D / 32;            // 16-byte chunks per lane per row
   __shared__ __align__(16) uint8_t s_ids[kSortChunk];
@@ -359,7 +370,7 @@ bool convert_in_hash(const Geometry& g) { return g.sorted && !g.node_dirs && con
 
 cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_fp32, const float* w_host,
                         const Workspace& ws, unsigned long long* near_zero, cudaStream_t st, int side_mask,
-                        const float* w_nodes, const void* convert_v) {
+                        const float* w_nodes, const void* convert_v, const VnormArgs* vnorm) {
   HashArgs a;
   a.side_mask = side_mask; a.chunk = g.chunk;
   a.w_nodes = g.node_dirs ? w_nodes : nullptr;
@@ -385,7 +396,13 @@ cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_
     return launch(g.d == 64 ? hash_fp32_kernel<64> : hash_fp32_kernel<128>, grid + copy_ctas, 256,
                   g.d == 64 ? kHash32Smem<64> : kHash32Smem<128>, st, a);
   }
-  return launch(g.d == 64 ? hash_bf16_kernel<64> : hash_bf16_kernel<128>, grid, 256, 0, st, a);
+  if (vnorm) {
+    a.hash_ctas = grid;
+    a.vnorm = *vnorm;
+    const unsigned ctas = (unsigned)grid + (unsigned)vnorm->G * (unsigned)vnorm->blocks;
+    return launch(g.d == 64 ? hash_bf16_kernel<64, true> : hash_bf16_kernel<128, true>, ctas, 256, kVnormSmem, st, a);
+  }
+  return launch(g.d == 64 ? hash_bf16_kernel<64, false> : hash_bf16_kernel<128, false>, grid, 256, 0, st, a);
 }
 
 }  // namespace hyperattn

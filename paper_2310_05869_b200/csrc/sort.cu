@@ -8,7 +8,7 @@
 // permutation unique.
 #include <type_traits>
 
-#include "common.cuh"
+#include "vnorm_common.cuh"
 
 namespace hyperattn {
 namespace {
@@ -50,12 +50,12 @@ struct SampleArgs {
 };
 
 // Alg. 2 line 4: m i.i.d. uniform key indices per (segment, node); word w of Philox call c is
-// sample 4c + w, mapped to [0, N) by a 64-bit multiply-high.  `block` of `nblocks` blocks of 256 threads.
+// sample 4c + w, mapped to [0, N) by a 64-bit multiply-high.  `block` of `nblocks` blocks.
 __device__ __forceinline__ void samples_body(const SampleArgs& a, int block, int nblocks) {
   const Geometry& g = a.g;
   const int calls = (g.m + 3) / 4;
   const size_t total = (size_t)g.G * g.nodes * calls;
-  for (size_t i = (size_t)block * 256 + threadIdx.x; i < total; i += (size_t)nblocks * 256) {
+  for (size_t i = (size_t)block * blockDim.x + threadIdx.x; i < total; i += (size_t)nblocks * blockDim.x) {
     const int c = (int)(i % calls);
     const int nd = (int)((i / calls) % g.nodes);
     const int seg = (int)(i / ((size_t)calls * g.nodes));
@@ -82,15 +82,25 @@ __device__ __forceinline__ void samples_body(const SampleArgs& a, int block, int
   }
 }
 
-// One CTA per (side, level, segment, node): thread v owns bucket v.  The launch carries the
-// sampling as extra blocks (both are tiny and independent of each other).
-__global__ void __launch_bounds__(256) sort_scan_kernel(SortArgs a, SampleArgs sa, int scan_blocks) {
-  __shared__ uint32_t s_tot[kBuckets];
+// One CTA per (side, level, segment, node): thread v of each of NG groups owns bucket v of its share of the node's chunks.  All
+// latency: one group reads the chunks in batches one after the other, four groups a quarter each.  The launch carries the sampling as extra
+// blocks, or the cumulative sums of the value norms (NG = 4; all are tiny and independent of each other).
+template <int NG>
+__global__ void __launch_bounds__(256 * NG) sort_scan_kernel(SortArgs a, SampleArgs sa, VnormArgs va, int scan_blocks, int sample_blocks) {
+  __shared__ uint32_t s_tot[NG][kBuckets], s_warp[NG][8];
   wait_for_stream();
   if (sa.sched && blockIdx.x == 0 && threadIdx.x == 0) *sa.sched = 0;
-  if ((int)blockIdx.x >= scan_blocks) { samples_body(sa, blockIdx.x - scan_blocks, gridDim.x - scan_blocks); return; }
+  if ((int)blockIdx.x >= scan_blocks) {
+    const int x = blockIdx.x - scan_blocks;
+    if (x < sample_blocks) samples_body(sa, x, sample_blocks);
+    else if (NG == 4) {
+      const int parts = (va.nk + 4095) / 4096;
+      vnorm_scan_body(va, (x - sample_blocks) / parts, (x - sample_blocks) % parts);
+    }
+    return;
+  }
   const Geometry& g = a.g;
-  const int v = threadIdx.x;
+  const int v = threadIdx.x & (kBuckets - 1), grp = threadIdx.x / kBuckets, lane = threadIdx.x & 31;
   int cta = blockIdx.x;
   // nodes of all levels are enumerated heap-style: per (side, seg): sum over levels of 2^level
   const int nodes_per = g.causal ? g.nodes : 1;
@@ -105,33 +115,42 @@ __global__ void __launch_bounds__(256) sort_scan_kernel(SortArgs a, SampleArgs s
   const uint32_t* h = a.hist + level * hist_level_stride(g) + side_hist_base(g, side) + ((size_t)seg * side_cps(g, side) + first) * kBuckets;
   const int lvl_chunk0 = g.causal ? j * nchunks : 0;
   uint32_t* o = a.offs + side_offs_base(g, side) + (((size_t)level * g.G + seg) * side_cpl(g, side) + lvl_chunk0) * kBuckets;
-  // pass 1: bucket totals of the node (eight loads in flight: the kernel is all latency)
-  uint32_t tot = 0;
-  for (int c0 = 0; c0 < nchunks; c0 += 8) {
-    uint32_t t[8];
+  constexpr int UB = NG == 1 ? 8 : 16;                   // loads in flight
+  const int share = (nchunks + NG - 1) / NG, begin = grp * share, end = min(nchunks, begin + share);
+  uint32_t t[UB];
+  auto load = [&](int c0) {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) t[u] = c0 + u < nchunks ? h[(size_t)(c0 + u) * kBuckets + v] : 0u;
+    for (int u = 0; u < UB; ++u) t[u] = c0 + u < end ? h[(size_t)(c0 + u) * kBuckets + v] : 0u;
+  };
+  // pass 1: bucket totals of the share
+  uint32_t mine = 0;
+  for (int c0 = begin; c0 < end; c0 += UB) {
+    load(c0);
 #pragma unroll
-    for (int u = 0; u < 8; ++u) tot += t[u];
+    for (int u = 0; u < UB; ++u) mine += t[u];
   }
-  // exclusive scan of the bucket totals over v
-  s_tot[v] = tot;
+  s_tot[grp][v] = mine;
   __syncthreads();
-  for (int off = 1; off < kBuckets; off <<= 1) {
-    const uint32_t add = v >= off ? s_tot[v - off] : 0u;
-    __syncthreads();
-    s_tot[v] += add;
-    __syncthreads();
+  // exclusive scan over v of the node's bucket totals, in every group; run: also what the bucket has in the shares before this one
+  uint32_t tot = 0, run = 0;
+#pragma unroll
+  for (int e = 0; e < NG; ++e) { const uint32_t x = s_tot[e][v]; tot += x; if (e < grp) run += x; }
+  uint32_t incl = tot;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const uint32_t x = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += x;
   }
+  if (lane == 31) s_warp[grp][v >> 5] = incl;
+  __syncthreads();
+  run += incl - tot;
+  for (int e = 0; e < (v >> 5); ++e) run += s_warp[grp][e];
   // pass 2: first position of bucket v in every chunk = buckets before v + the same bucket in earlier chunks
-  uint32_t run = s_tot[v] - tot;
-  for (int c0 = 0; c0 < nchunks; c0 += 8) {
-    uint32_t t[8];
+  for (int c0 = begin; c0 < end; c0 += UB) {
+    if (share > UB) load(c0);                            // (else they are still there)
 #pragma unroll
-    for (int u = 0; u < 8; ++u) t[u] = c0 + u < nchunks ? h[(size_t)(c0 + u) * kBuckets + v] : 0u;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      if (c0 + u < nchunks) o[(size_t)(c0 + u) * kBuckets + v] = run;
+    for (int u = 0; u < UB; ++u) {
+      if (c0 + u < end) o[(size_t)(c0 + u) * kBuckets + v] = run;
       run += t[u];
     }
   }
@@ -293,6 +312,11 @@ bool scan_in_scatter(const Geometry& g) {
   return most <= kScanChunks;
 }
 
+// Four groups of threads per node while every node has an SM of its own.  (A call, us, one group -> four: 4 heads of 40000 rows, 8 nodes of 20
+// chunks, 74.0 -> 73.2; 4 causal heads of 100003 rows, 248 nodes, 592 -> 597.)
+static int scan_ctas(const Geometry& g) { return 2 * g.G * (g.causal ? g.nodes : 1); }
+bool wide_scan(const Geometry& g) { return !scan_in_scatter(g) && scan_ctas(g) <= kSms; }
+
 static SampleArgs make_sample_args(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, int* blocks) {
   // (ws.tpos non-null: the probe rows of the capped row-sum estimate are drawn as well)
   SampleArgs sa;
@@ -308,13 +332,18 @@ static SampleArgs make_sample_args(const Geometry& g, const Workspace& ws, bool 
 }
 
 // scan of the chunk histograms; with_samples: the same launch also draws the samples (Alg. 2 line 4)
-cudaError_t launch_sort_scan(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask) {
+cudaError_t launch_sort_scan(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask,
+                             const VnormArgs* vnorm) {
   if (!g.sorted || scan_in_scatter(g)) return cudaSuccess;
   const SortArgs a = make_sort_args(g, ws, side_mask);
-  const int scan_blocks = 2 * g.G * (g.causal ? g.nodes : 1);
+  const int scan_blocks = scan_ctas(g);
   int sample_blocks;
   const SampleArgs sa = make_sample_args(g, ws, with_samples, seed, &sample_blocks);
-  return launch(sort_scan_kernel, scan_blocks + sample_blocks, 256, 0, st, a, sa, scan_blocks);
+  if (!wide_scan(g)) return launch(sort_scan_kernel<1>, scan_blocks + sample_blocks, 256, 0, st, a, sa, VnormArgs{}, scan_blocks, sample_blocks);
+  sample_blocks = (sample_blocks + 3) / 4;
+  const int vnorm_blocks = vnorm ? g.G * ((g.nk + 4095) / 4096) : 0;
+  return launch(sort_scan_kernel<4>, scan_blocks + sample_blocks + vnorm_blocks, 1024, 0, st, a, sa, vnorm ? *vnorm : VnormArgs{}, scan_blocks,
+                sample_blocks);
 }
 
 cudaError_t launch_sort_scatter(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask) {

@@ -5,102 +5,27 @@
 // of a row is accumulated in fp32 in coordinate order (bf16 squares are exact in fp32) and cut to a
 // multiple of 2^-12; cumulative sums are 64-bit integers; a draw is the first key whose cumulative
 // weight exceeds floor(x * total / 2^32), x the Philox word the uniform sampler would have used.
-// Three small kernels: weights (streams V once), per-segment cumulative sums, draws.
-#include "common.cuh"
+// Three small steps: weights (streams V once), per-segment cumulative sums, draws.  The first two have launches of their own here
+// where the hash (fp32 inputs) or the scan of the histograms (few chunks, or many nodes) does not carry them.
+#include "vnorm_common.cuh"
 
 namespace hyperattn {
 namespace {
 
-constexpr float kNormScale = 4096.f;      // 2^12
-
 // (Weights and scan: segment = y + gridDim.y * z, its part x.  A grid's y ends at 65535, and a call may have 2^20 segments; both from one
 // extent takes a division at the head of either kernel's chain: 4 segments of 131072 rows 28 -> 30 us.)
-//
-// A CTA weighs 256 rows of one segment: the rows come in by whole lines and are read back one per thread (the chunks
-// of a row XOR-swizzled, so that neither side has bank conflicts); also the sum of the CTA's weights.
 template <int D>
-__global__ void __launch_bounds__(256) vnorm_weights_kernel(const __nv_bfloat16* __restrict__ v, uint32_t* __restrict__ wq,
-                                                            unsigned long long* __restrict__ sums, int G, int nk) {
-  constexpr int CPR = D / 8;
-  extern __shared__ uint4 s_row[];                        // [256][CPR]
-  __shared__ unsigned long long s_warp[8];
-  const int tid = threadIdx.x, lane = tid & 31;
+__global__ void __launch_bounds__(256) vnorm_weights_kernel(VnormArgs a) {
+  extern __shared__ uint4 s_row[];
   wait_for_stream();
-  const int seg = blockIdx.y + gridDim.y * blockIdx.z, row0 = blockIdx.x * 256, rows = min(256, nk - row0);
-  if (seg >= G) return;
-  const size_t first = (size_t)seg * nk + row0;
-  const uint4* src = reinterpret_cast<const uint4*>(v) + first * CPR;
-#pragma unroll
-  for (int e = 0; e < CPR; ++e) {
-    const int c = tid + 256 * e, r = c / CPR, cc = c % CPR;
-    if (r < rows) s_row[r * CPR + (cc ^ (r & 7))] = __ldg(src + c);
-  }
-  __syncthreads();
-  unsigned long long w = 0;
-  if (tid < rows) {
-    float acc = 0.f;
-#pragma unroll
-    for (int c = 0; c < CPR; ++c) {
-      const uint4 x = s_row[tid * CPR + (c ^ (tid & 7))];
-      const uint32_t words[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float lo = __uint_as_float(words[e] << 16), hi = __uint_as_float(words[e] & 0xffff0000u);
-        acc = __fadd_rn(acc, __fmul_rn(lo, lo));          // (coordinate order, no fused multiply-add: the stated arithmetic)
-        acc = __fadd_rn(acc, __fmul_rn(hi, hi));
-      }
-    }
-    const uint32_t q = (uint32_t)(acc * kNormScale);      // exact scaling, truncation = floor (acc >= 0)
-    wq[first + tid] = q;
-    w = q;
-  }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-  if (lane == 0) s_warp[tid >> 5] = w;
-  __syncthreads();
-  if (tid == 0) {
-    for (int e = 1; e < 8; ++e) w += s_warp[e];
-    sums[(size_t)seg * gridDim.x + blockIdx.x] = w;
-  }
+  const int seg = blockIdx.y + gridDim.y * blockIdx.z;
+  if (seg < a.G) vnorm_weights_body<D>(a, seg, blockIdx.x, s_row);
 }
 
-// cum[seg][0] = 0, cum[seg][i + 1] = wq[seg][0] + ... + wq[seg][i] (64-bit).  A CTA does 4096 rows of one segment and adds up
-// the sums of the rows before them by itself, so all CTAs run at once (one CTA per segment walking its rows: 94 us for 4 segments of
-// 131072 rows, now 5 us).
-__global__ void __launch_bounds__(1024) vnorm_scan_kernel(const uint32_t* __restrict__ wq, const unsigned long long* __restrict__ sums,
-                                                          unsigned long long* __restrict__ cum, int G, int nk, int blocks) {
-  __shared__ unsigned long long s_warp[32], s_before[32];
-  const int seg = blockIdx.y + gridDim.y * blockIdx.z;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (seg >= G) return;
+__global__ void __launch_bounds__(1024) vnorm_scan_kernel(VnormArgs a) {
   wait_for_stream();
-  const uint32_t* w = wq + (size_t)seg * nk;
-  unsigned long long* c = cum + (size_t)seg * (nk + 1);
-  const int i = blockIdx.x * 4096 + 4 * tid;
-  unsigned long long x[4], before = 0;
-#pragma unroll
-  for (int e = 0; e < 4; ++e) x[e] = i + e < nk ? w[i + e] : 0ull;
-  for (int e = tid; e < (int)blockIdx.x * 16; e += 1024) before += sums[(size_t)seg * blocks + e];
-  x[1] += x[0]; x[2] += x[1]; x[3] += x[2];
-  unsigned long long run = x[3];
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long t = __shfl_up_sync(0xffffffffu, run, o);
-    if (lane >= o) run += t;
-  }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
-  if (lane == 31) { s_warp[warp] = run; s_before[warp] = before; }
-  __syncthreads();
-  // sums of the warps before this one, and of everything before the CTA
-  unsigned long long t = s_before[lane] + (lane < warp ? s_warp[lane] : 0ull);
-#pragma unroll
-  for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  t += run - x[3];
-#pragma unroll
-  for (int e = 0; e < 4; ++e)
-    if (i + e < nk) c[i + e + 1] = t + x[e];
-  if (i == 0) c[0] = 0;
+  const int seg = blockIdx.y + gridDim.y * blockIdx.z;
+  if (seg < a.G) vnorm_scan_body(a, seg, blockIdx.x);
 }
 
 struct VnormSampleArgs {
@@ -166,20 +91,20 @@ __global__ void __launch_bounds__(256) vnorm_sample_kernel(VnormSampleArgs a) {
 
 }  // namespace
 
-cudaError_t launch_vnorm_sampling(const Geometry& g, const __nv_bfloat16* v, uint32_t* wq, unsigned long long* sums, unsigned long long* cum,
-                                  int32_t* samples, float* wlog, uint64_t seed, cudaStream_t st) {
+// weights_done, scan_done: launches before this one have made them
+cudaError_t launch_vnorm_sampling(const Geometry& g, const VnormArgs& v, bool weights_done, bool scan_done, int32_t* samples, float* wlog,
+                                  uint64_t seed, cudaStream_t st) {
   if (!g.sorted || g.m == 0 || g.nodes == 0) return cudaSuccess;
-  const int blocks = (g.nk + 255) / 256;
   const unsigned y = g.G < 65536 ? g.G : 65535, z = ((unsigned)g.G + y - 1) / y;
-  const dim3 grid(blocks, y, z);
   cudaError_t e = cudaSuccess;
-  if (g.d == 64) e = launch(vnorm_weights_kernel<64>, grid, 256, 256 * 128, st, v, wq, sums, g.G, g.nk);
-  else if ((e = allow_smem<vnorm_weights_kernel<128>>(256 * 256)) == cudaSuccess)
-    e = launch(vnorm_weights_kernel<128>, grid, 256, 256 * 256, st, v, wq, sums, g.G, g.nk);
-  if (e == cudaSuccess) e = launch(vnorm_scan_kernel, dim3((g.nk + 4095) / 4096, y, z), 1024, 0, st, wq, sums, cum, g.G, g.nk, blocks);
+  if (!weights_done) {
+    const dim3 grid(v.blocks, y, z);
+    e = launch(g.d == 64 ? vnorm_weights_kernel<64> : vnorm_weights_kernel<128>, grid, 256, kVnormSmem, st, v);
+  }
+  if (e == cudaSuccess && !scan_done) e = launch(vnorm_scan_kernel, dim3((g.nk + 4095) / 4096, y, z), 1024, 0, st, v);
   if (e != cudaSuccess) return e;
   VnormSampleArgs a;
-  a.cum = cum; a.samples = samples; a.wlog = wlog; a.g = g; a.k0 = (uint32_t)seed; a.k1 = (uint32_t)(seed >> 32);
+  a.cum = v.cum; a.samples = samples; a.wlog = wlog; a.g = g; a.k0 = (uint32_t)seed; a.k1 = (uint32_t)(seed >> 32);
   // A call, us, one lane per draw -> 32: 256 draws 111.7 -> 105.7, 1024 160.9 -> 156.8, 4096 477.7 -> 474.3 (131072 keys), 2048
   // 63.6 -> 60.4 (16384 keys); 8192 893.8 -> 894.2 (131072 keys), 67.9 -> 68.6 (4096 keys); 16384 264.2 -> 267.5 (16384 keys),
   // 128.7 -> 132.7 (4096 keys); 65536 616.7 -> 642.7 (16384 keys).

@@ -196,6 +196,26 @@ def test_value_norm_edges(w):
     vnorm.test_value_norm_sampling_matches_the_oracle(w)
 
 
+@pytest.mark.parametrize("n,causal,value_norms", [(4097, False, True), (16385, False, False), (70001, False, True), (300000, False, False),
+                                                  (300000, False, True), (65536, True, False), (65536, True, True), (40000, True, True)])
+def test_sort_of_many_chunks(n, causal, value_norms):
+    """Nodes of 17 to 293 chunks: the scan by one group of threads (many nodes) or by four, and what else its launch carries."""
+    w = parity.W("", 1, 2 if causal else 1, n, 64, "bf16", 256, 64, 7, causal, 1024 if n == 65536 else 10000, seed=98)
+    gen = torch.Generator(device="cuda").manual_seed(98)
+    q, k, v = (torch.randn((w.B, w.H, n, w.d), generator=gen, device="cuda").bfloat16() for _ in range(3))
+    _, _, inter = _forward(w, q, k, v, debug=True, value_norm_sampling=value_norms)
+    assert ha.last_device_status() == 0
+    s = n // 2 if causal else n                            # (the first level's node: the lengths are even)
+    for ids, perm, first in ((inter["q_ids"], inter["perm_q"], n - s), (inter["k_ids"], inter["perm_k"], 0)):
+        for g in range(w.G):
+            want = torch.sort(ids[g, first:first + s].int(), stable=True).indices
+            assert torch.equal(perm[0, g, :s].long(), want)
+    if value_norms:
+        V = v[0, 0].double().cpu().numpy()
+        idx, _ = O.sample_by_value_norms(w.seed, 0, 0, w.m, O.value_norm_weights(V)[:s])
+        assert (inter["samples"].cpu().numpy()[0, 0, :w.m] == idx).all()
+
+
 def _check_segments(B, H, n, d, b, m, r, seed, gen_seed, per_segment=None, **kw):
     """Calls of more segments than the y and z extents of a grid: segments around 65 536 and forty others against the oracle."""
     gen = torch.Generator(device="cuda").manual_seed(gen_seed)

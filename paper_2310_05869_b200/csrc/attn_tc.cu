@@ -3,7 +3,7 @@
 // One CTA owns a PAIR of query tiles (2 x 128 rows) that are neighbours in the tile order of
 // their leaf / recursion node, and walks once over the key tiles (64 keys each) that either
 // of them needs:
-//     S_i = Q_i K^T      tcgen05.mma, operands in 128B-swizzled shared memory, S_i in TMEM
+//     S_i = Q_i K^T      tcgen05.mma, operands in 128B-swizzled shared memory (d = 64: Q_i from TMEM), S_i in TMEM
 //     P_i = exp2(S_i*c + bias - m)   softmax warpgroup i: one thread per query row (TMEM
 //                                    lane); P_i is written back over S_i as bf16
 //     O_i += P_i V       tcgen05.mma with P_i read from TMEM, V MN-major in shared memory
@@ -25,7 +25,7 @@
 //
 // Warp roles (384 threads): warps 0-3 and 4-7 softmax + epilogue of query tile 0 and 1,
 // warps 8 and 9 MMA issue for query tile 0 and 1 (warp 8 also allocates TMEM, all 512
-// columns: per query tile two S buffers of 64, then O0, O1), warp 10 prepares work items (row tables of the
+// columns: per query tile two S buffers of 64, then O0, O1 and, d = 64, Q0, Q1), warp 10 prepares work items (row tables of the
 // NEXT item while this one computes, TMA boxes of Q), warp 11 streams K / V tiles through
 // the stage ring, across item boundaries.  Gathered Q tiles are fetched by the 256 softmax
 // threads, for the next item, right before they write the current item's results.
@@ -201,7 +201,13 @@ struct Cfg {
   static_assert(D == 64 || 4 * kStageWarp <= kMaxNodeKeys * 4, "staging of query tile 0 must fit one key-row table");
   static constexpr int kTmemCols = 512;
   static constexpr int kColO = 64 * 2 * kSBufs;       // S buffer b of tile i at 64 (kSBufs i + b); O_i at kColO + kOCols i
-  static_assert(kColO + 2 * kOCols <= 512, "TMEM columns");
+  // d = 64 has columns to spare for Q: copied from shared memory once per item, it is the A operand of the scores from there.  Read from
+  // shared memory with every key tile (16 KB, beside 8 of K and 10 of V) it keeps the tensor pipe waiting and costs power, which
+  // is what bounds the clock here.  (Attention, us, shared memory -> TMEM: 128 causal leaves of 4096 rows 454 -> 440; 32 heads x 65536
+  // rows 614 -> 604; 16 causal heads x 32768 673 -> 658.)
+  static constexpr bool kQTmem = D == 64;
+  static constexpr int kColQ = kColO + 2 * kOCols;    // Q_i at kColQ + i D / 2 (pairs of bf16)
+  static_assert(kColQ + (kQTmem ? D : 0) <= 512, "TMEM columns");
 };
 
 __device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, PairDesc& t, QTile& qa, QTile& qb, int& lenA, int& lenB) {
@@ -836,6 +842,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       constexpr uint32_t dv_step = (uint32_t)(C::kTile >> 4) - (C::kOnes ? ((uint32_t)(C::kTile >> 4) << 16) : 0u);   // per stage
       const uint32_t ocol = tmem + C::kColO + C::kOCols * i;
       const uint32_t scol = tmem + 64 * C::kSBufs * i;
+      const uint32_t qcol = tmem + C::kColQ + (D / 2) * i;
       bool ok = true;
       int gbase = 0;                        // global index (all items) of the item's first key tile
       int knext = 0, vnext = 0;             // next global tile whose K / V stage this issuer has to observe and release
@@ -880,6 +887,15 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
         if (!ok) break;
         HA_LACC(b_q, tq);
         fence_async_smem();
+        if constexpr (C::kQTmem) {
+          // (the scores of the item before have been multiplied: this item's Q was not asked for until then.  Copies and the products
+          // issued after them by the same thread run in order.)
+          tc_fence_after();
+          if (el && total > 0) {
+#pragma unroll
+            for (int ks = 0; ks < D / 16; ++ks) tmem_cp_128x256b(qcol + ks * 8, dq_lo + ks * (32 >> 4), desc_hi);
+          }
+        }
         if (total == 0 && el) mbar_arrive(bar_qfree);
         auto issue_pv = [&](int a2) {
           // ---- O += P V of key tile a2 ----------------------------------------------------------
@@ -929,9 +945,11 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
           const uint32_t dk_lo = dk_lo0 + (uint32_t)s * (C::kTile >> 4);
           if (el) {
 #pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks)
-              mma_ss2(dcol, dq_lo + (((ks >> 2) * (128 * 128) + (ks & 3) * 32) >> 4),
-                      dk_lo + (((ks >> 2) * (TK * 128) + (ks & 3) * 32) >> 4), desc_hi, idesc_s, ks > 0);
+            for (int ks = 0; ks < D / 16; ++ks) {
+              const uint32_t dk = dk_lo + (((ks >> 2) * (TK * 128) + (ks & 3) * 32) >> 4);
+              if constexpr (C::kQTmem) mma_ts2(dcol, qcol + ks * 8, dk, desc_hi, idesc_s, ks > 0);
+              else mma_ss2(dcol, dq_lo + (((ks >> 2) * (128 * 128) + (ks & 3) * 32) >> 4), dk, desc_hi, idesc_s, ks > 0);
+            }
             umma_commit(bar_s(i, gw % C::kSBufs));
             umma_commit(bar_kempty(i, s));
             if (r == total - 1) umma_commit(bar_qfree);     // nothing of this item reads Q any more

@@ -62,8 +62,25 @@ struct AttnArgs {
   int level_pair_start[kMaxLevels + 1];
   int level_paired[kMaxLevels];      // 1: CTAs of this level own two query tiles, 0: one
   int total_pairs;
+  int tail_leaves;                   // last leaves that are handed out rank by rank (tail_leaves(), set by the launchers)
   int* sched;                        // work counter of the launch (global memory, zero at launch): next item to hand out
 };
+
+// Items of leaves are handed out leaf by leaf, the heaviest first; where nothing follows them, one leaf at a time the last heavy item
+// would start when little is left beside it.  So the last leaves - two rounds of all SMs - go rank by rank: the heaviest items of all
+// of them first.
+inline int tail_leaves(int leaves, int items_per_leaf, int sms) {
+  const int two_rounds = (2 * sms + items_per_leaf - 1) / items_per_leaf;
+  return leaves < two_rounds ? leaves : two_rounds;
+}
+// item of a leaf list -> leaf and rank (0: the heaviest item of the leaf)
+__device__ __forceinline__ void leaf_of_item(int item, int items, int per_leaf, int tail_leaves, int& leaf, int& rank) {
+  const int tail = item - (items - tail_leaves * per_leaf);
+  if (tail_leaves > 0 && tail >= 0) {
+    rank = tail / tail_leaves;
+    leaf = items / per_leaf - tail_leaves + tail % tail_leaves;
+  } else { rank = item % per_leaf; leaf = item / per_leaf; }
+}
 
 struct TileDesc {
   int mode;            // 0 dense, 1 node

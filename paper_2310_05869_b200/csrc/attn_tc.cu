@@ -220,8 +220,11 @@ __device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, PairDes
     // Leaf after leaf, the pairs of a leaf from the heaviest (last rows, most keys) to the lightest: items are
     // handed out in this order, so the CTAs that run at the same time work on a handful of neighbouring leaves
     // and find each other's K / V tiles in L2, and the list still ends with light items.
-    const int uu = a.pairs_per_leaf - 1 - pair % a.pairs_per_leaf;
-    const int rem = pair / a.pairs_per_leaf;
+    // (The last leaves of a call without node items: all heavy pairs first, see tail_leaves().  128 leaves of 4096 rows, d = 64, 440 -> 408
+    // us; 64 leaves, d = 128, 300 -> 271.)
+    int rem, rank;
+    leaf_of_item(pair, a.n_leaf_pairs, a.pairs_per_leaf, a.tail_leaves, rem, rank);
+    const int uu = a.pairs_per_leaf - 1 - rank;
     t.seg = rem / a.leaves_per_seg;
     const int leaf = rem % a.leaves_per_seg;
     t.mode = 0; t.causal = a.dense_causal;
@@ -1360,10 +1363,12 @@ cudaError_t launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st)
   if (e != cudaSuccess) return e;
   const int grid = a.total_pairs < sms ? a.total_pairs : sms;     // persistent: one CTA per SM walks the item list
   const bool variant = a.capped || a.sample_wlog;
+  AttnArgs b = a;
+  b.tail_leaves = a.dense_causal && a.total_pairs == a.n_leaf_pairs ? tail_leaves(a.n_leaf_pairs / a.pairs_per_leaf, a.pairs_per_leaf, sms) : 0;
   if (variant && (a.precise || (a.capped && a.sample_wlog))) return cudaErrorInvalidValue;
   const bool late = a.g.d == 128 && !a.direct && !a.part_bf16;
 #define HA_GO(D, LATE, PRECISE, CAPPED) do { e = allow_smem<attn_tc_kernel<D, LATE, PRECISE, CAPPED>>(Cfg<D>::kTotal); \
-    return e != cudaSuccess ? e : launch(attn_tc_kernel<D, LATE, PRECISE, CAPPED>, grid, 384, Cfg<D>::kTotal, st, a, maps, status); } while (0)
+    return e != cudaSuccess ? e : launch(attn_tc_kernel<D, LATE, PRECISE, CAPPED>, grid, 384, Cfg<D>::kTotal, st, b, maps, status); } while (0)
   if (a.g.d == 64) {
     if (variant) HA_GO(64, false, false, true);
     if (a.precise) HA_GO(64, false, true, false);

@@ -39,6 +39,8 @@ FORWARD = [
     parity.W("no_samples_seven_key_tiles_d64", 1, 2, 1000, 64, "bf16", 448, 0, 6, False, 0, seed=98, n_k=4000),
     parity.W("no_samples_three_key_tiles_d128", 1, 2, 1300, 128, "bf16", 192, 0, 6, False, 0, seed=99, n_k=2000),
     parity.W("no_samples_two_key_tiles_causal_d128", 1, 2, 4096, 128, "bf16", 128, 0, 6, True, 512, seed=100),
+    # leaves alone: the last 148 go rank by rank, the ones before leaf by leaf
+    parity.W("leaves_for_more_than_two_rounds", 1, 160, 300, 64, "bf16", 64, 8, 4, True, 512, seed=102),
     # fp32: hash passes of 256 rows; copies beside the hash (up to 296 CTAs of 4096 entries) and in a launch of their own; query tiles
     # halved (up to 74 tiles) and whole, second halves of one row and none
     parity.W("fp32_n257_d64", 1, 1, 257, 64, "fp32", 64, 32, 7, False, 0, seed=76),
@@ -72,6 +74,7 @@ BACKWARD = [
     backward.W("bwd_leaf_of_193_rows_d128", 1, 1, 193, 128, 64, 8, 4, True, 200, seed=80),
     backward.W("bwd_sorted_over_unsorted_nodes_d64", 1, 2, 1040, 64, 200, 33, 6, True, 130, seed=81),
     backward.W("bwd_sorted_over_unsorted_nodes_d128", 1, 1, 1040, 128, 200, 33, 6, True, 130, seed=82),
+    backward.W("bwd_leaves_for_more_than_two_rounds_d64", 1, 110, 300, 64, 64, 8, 4, True, 512, seed=85),
     # more items than SMs, so that whole tiles of consecutive rows, short ones and scattered rows follow one another in a CTA
     backward.W("bwd_whole_short_and_scattered_tiles_d64", 1, 40, 640, 64, 64, 33, 6, True, 320, seed=83),
     backward.W("bwd_whole_short_and_scattered_tiles_d128", 1, 24, 640, 128, 64, 33, 6, True, 320, seed=84),

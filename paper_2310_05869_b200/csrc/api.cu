@@ -15,8 +15,8 @@
 namespace hyperattn {
 cudaError_t launch_attention_mma(const AttnArgs& a, cudaStream_t st);
 cudaError_t launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st);
-cudaError_t launch_vnorm_sampling(const Geometry& g, const VnormArgs& v, bool weights_done, bool scan_done, int32_t* samples, float* wlog,
-                                  uint64_t seed, cudaStream_t st);
+cudaError_t launch_vnorm_sampling(const Geometry& g, const VnormArgs& v, bool scan_done, int32_t* samples, float* wlog, uint64_t seed,
+                                  cudaStream_t st);
 cudaError_t launch_tau(const AttnArgs& at, const int32_t* tpos, float* ltau, cudaStream_t st);
 cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout, float2* stat, int* sched,
                             const BwdGrads& gr, float scale, int* status, cudaStream_t st);
@@ -352,15 +352,15 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
       HA_CHECK(cudaMemcpyAsync(base + pl.wnodes, g_wnodes.w.data(), per * g.nodes * 4, cudaMemcpyHostToDevice, st));
       w_nodes = reinterpret_cast<const float*>(base + pl.wnodes);
     }
-    // (sampling by value norms: the rows of V are weighed beside the hash - fp32 values are still on their way to bf16 then - and the
-    // weights added up beside the scan of the histograms)
+    // (sampling by value norms, bf16 inputs only: the rows of V are weighed beside the hash, and the weights added up beside the scan of the
+    // histograms where that is wide enough)
     const VnormArgs va = {v16, reinterpret_cast<uint32_t*>(base + pl.vwq), reinterpret_cast<unsigned long long*>(base + pl.vsum),
                           reinterpret_cast<unsigned long long*>(base + pl.vcum), g.G, g.nk, (g.nk + 255) / 256};
-    const bool weights_in_hash = vnorm && !is_fp32, sums_in_scan = weights_in_hash && wide_scan(g);
+    const bool sums_in_scan = vnorm && wide_scan(g);
     {
       StageScope sc(st, HYPERATTN_STAGE_HASH, 1);
       HA_CHECK(launch_hash(g, p.q, p.k, is_fp32, g_wcache.w, ws, dbg ? dbg->near_zero_bits : nullptr, st, 3, w_nodes,
-                           in_hash ? p.v : nullptr, weights_in_hash ? &va : nullptr));
+                           in_hash ? p.v : nullptr, vnorm ? &va : nullptr));
     }
     {
       // (the samples of Alg. 2 line 4 are drawn by extra blocks of this launch, or, where it falls away, of the placement)
@@ -368,8 +368,8 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
       HA_CHECK(launch_sort_scan(g, ws, !vnorm, p.seed, st, 3, sums_in_scan ? &va : nullptr));
     }
     if (vnorm) {
-      StageScope sc(st, HYPERATTN_STAGE_SAMPLE, 3 - weights_in_hash - sums_in_scan);
-      HA_CHECK(launch_vnorm_sampling(g, va, weights_in_hash, sums_in_scan, ws.samples, reinterpret_cast<float*>(base + pl.swlog), p.seed, st));
+      StageScope sc(st, HYPERATTN_STAGE_SAMPLE, sums_in_scan ? 1 : 2);
+      HA_CHECK(launch_vnorm_sampling(g, va, sums_in_scan, ws.samples, reinterpret_cast<float*>(base + pl.swlog), p.seed, st));
       if (dbg && dbg->sample_log2w)
         HA_CHECK(cudaMemcpyAsync(dbg->sample_log2w, base + pl.swlog, (size_t)g.G * g.nodes * g.m * 4, cudaMemcpyDeviceToDevice, st));
     }

@@ -5,23 +5,14 @@
 // of a row is accumulated in fp32 in coordinate order (bf16 squares are exact in fp32) and cut to a
 // multiple of 2^-12; cumulative sums are 64-bit integers; a draw is the first key whose cumulative
 // weight exceeds floor(x * total / 2^32), x the Philox word the uniform sampler would have used.
-// Three small steps: weights (streams V once), per-segment cumulative sums, draws.  The first two have launches of their own here
-// where the hash (fp32 inputs) or the scan of the histograms (few chunks, or many nodes) does not carry them.
+// Three small steps: weights (streams V once; further blocks of the hash launch), per-segment cumulative sums (further blocks of the
+// scan of the histograms, or, with few chunks or many nodes, a launch of their own here), draws.
 #include "vnorm_common.cuh"
 
 namespace hyperattn {
 namespace {
 
-// (Weights and scan: segment = y + gridDim.y * z, its part x.  A grid's y ends at 65535, and a call may have 2^20 segments; both from one
-// extent takes a division at the head of either kernel's chain: 4 segments of 131072 rows 28 -> 30 us.)
-template <int D>
-__global__ void __launch_bounds__(256) vnorm_weights_kernel(VnormArgs a) {
-  extern __shared__ uint4 s_row[];
-  wait_for_stream();
-  const int seg = blockIdx.y + gridDim.y * blockIdx.z;
-  if (seg < a.G) vnorm_weights_body<D>(a, seg, blockIdx.x, s_row);
-}
-
+// (Segment = y + gridDim.y * z, its part x: a grid's y ends at 65535, and a call may have 2^20 segments.)
 __global__ void __launch_bounds__(1024) vnorm_scan_kernel(VnormArgs a) {
   wait_for_stream();
   const int seg = blockIdx.y + gridDim.y * blockIdx.z;
@@ -91,17 +82,13 @@ __global__ void __launch_bounds__(256) vnorm_sample_kernel(VnormSampleArgs a) {
 
 }  // namespace
 
-// weights_done, scan_done: launches before this one have made them
-cudaError_t launch_vnorm_sampling(const Geometry& g, const VnormArgs& v, bool weights_done, bool scan_done, int32_t* samples, float* wlog,
-                                  uint64_t seed, cudaStream_t st) {
+// (the weights are there: the hash launch has made them)  scan_done: so are their cumulative sums
+cudaError_t launch_vnorm_sampling(const Geometry& g, const VnormArgs& v, bool scan_done, int32_t* samples, float* wlog, uint64_t seed,
+                                  cudaStream_t st) {
   if (!g.sorted || g.m == 0 || g.nodes == 0) return cudaSuccess;
   const unsigned y = g.G < 65536 ? g.G : 65535, z = ((unsigned)g.G + y - 1) / y;
   cudaError_t e = cudaSuccess;
-  if (!weights_done) {
-    const dim3 grid(v.blocks, y, z);
-    e = launch(g.d == 64 ? vnorm_weights_kernel<64> : vnorm_weights_kernel<128>, grid, 256, kVnormSmem, st, v);
-  }
-  if (e == cudaSuccess && !scan_done) e = launch(vnorm_scan_kernel, dim3((g.nk + 4095) / 4096, y, z), 1024, 0, st, v);
+  if (!scan_done) e = launch(vnorm_scan_kernel, dim3((g.nk + 4095) / 4096, y, z), 1024, 0, st, v);
   if (e != cudaSuccess) return e;
   VnormSampleArgs a;
   a.cum = v.cum; a.samples = samples; a.wlog = wlog; a.g = g; a.k0 = (uint32_t)seed; a.k1 = (uint32_t)(seed >> 32);

@@ -1,5 +1,5 @@
-// Device bodies of the value-norm sampling (vnorm.cu) that also run as extra blocks of other launches: the weights beside the hash
-// (hash.cu), the cumulative sums beside the scan of the histograms (sort.cu).
+// Device bodies of the value-norm sampling (vnorm.cu) that run as extra blocks of other launches: the weights beside the hash (hash.cu), the
+// cumulative sums beside the scan of the histograms (sort.cu; else in a launch of their own).
 #pragma once
 #include "common.cuh"
 

@@ -503,6 +503,17 @@ int hyperattn_backward(const hyperattn_params* p, const hyperattn_grads* grads) 
   return forward_impl(*p, 0, grads);
 }
 
+// (for the tests, not part of the interface) which build of the backward kernel a call takes
+int hyperattn_internal_backward_build(const hyperattn_params* p, int* boxes, int* results_warps) {
+  if (!p || !boxes || !results_warps) return HYPERATTN_INVALID_ARGUMENT;
+  Geometry g;
+  const int rc = build_geometry(*p, g);
+  if (rc) return rc;
+  const BwdBuild build = backward_build(g);
+  *boxes = build.boxes; *results_warps = build.results_warps;
+  return HYPERATTN_OK;
+}
+
 int hyperattn_backward_workspace_bytes(const hyperattn_params* p, int grad_dtype, size_t* bytes) {
   if (!p || !bytes) return HYPERATTN_INVALID_ARGUMENT;
   Geometry g;

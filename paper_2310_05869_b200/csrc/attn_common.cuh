@@ -29,6 +29,13 @@ struct BwdGrads {
   int direct;                  // every key has one tile only besides the samples: its bf16 dK and dV leave from there
 };
 
+// which build of the backward kernel a call takes (backward.cu)
+struct BwdBuild {
+  bool boxes;                  // whole tiles of consecutive rows leave as boxes
+  int results_warps;
+};
+BwdBuild backward_build(const Geometry& g);
+
 struct AttnArgs {
   const __nv_bfloat16 *q, *k, *v;    // [G, n, D]
   const __nv_bfloat16 *q_lo, *k_lo;  // second bf16 term of fp32 inputs (else null)

@@ -37,6 +37,41 @@ __global__ void __launch_bounds__(256) to_bf16_kernel(const __grid_constant__ To
 
 }  // namespace
 
+// What pays is whole tiles of 128 consecutive rows (leaves, nodes that are not sorted): their dQ leaves as a box at every step, with a few
+// instructions.  What costs: the boxes' code in the results warps at every short tile and at every tile of sorted rows, and, with half of the
+// warps, those tiles themselves and the dK and dV of every key tile, behind which the next item waits.  So the rules weigh steps on whole
+// tiles against key tiles of consecutive rows (`items`) and all other steps.  The pass, us, without boxes / with boxes / four results
+// warps (* what the rules take).  d = 64, causal leaves alone: 1024 leaves of 127 rows 57.5* / 59.1 / 63.6, 781 of 256 85.5* / 86.5 / 98.5, 390 of 512
+// 106 / 104* / 115, 195 of 1024 150 / 148 / 150*, 130 of 1536 195 / 192 / 185*, 128 of 4096 999 / 931 / 869*; exact, 2048 heads of 127
+// rows 108* / 111 / 119, 781 of 256 93.6 / 92.1* / 100, 32 of 4096 452 / 423 / 386*; 32768 rows, 16 heads, in leaves of 512 (blocks of 64) 1764* / 1793 / 1923,
+// 1024 1336 / 1327* / 1352, 2048 1385 / 1356 / 1335*, 4096 1667 / 1602 / 1539*; 64 heads of 1600 rows in leaves of 100 under nodes that are not
+// sorted 179* / 179 / 189; no recursion, 32 heads of 4096 rows 131* / 134 / 142.  d = 128, without and with boxes: 1024 leaves of 100 rows 87.8* / 88.3,
+// 781 of 256 162* / 161, 390 of 512 197 / 191*, 64 of 4096 945 / 827*; 32 heads of 32768 rows without recursion 1494* / 1514.
+BwdBuild backward_build(const Geometry& g) {
+  long long whole = 0, other = 0, items = 0;            // per segment
+  if (g.causal || !g.sorted) {
+    const long long leaves = g.npad / g.leaf, kts = (g.leaf + kTileK - 1) / kTileK, full = g.leaf / kTileQ;
+    const long long on_full = g.causal ? full * (full + 1) / 2 : kts * full, all = g.causal ? kts * (kts + 1) / 2 : kts * kts;
+    whole += leaves * on_full; other += leaves * (all - on_full); items += leaves * kts;
+  }
+  for (int l = 0; l < g.levels; ++l) {
+    int s, q0, k0;
+    node_rows(g, l, 0, s, q0, k0);
+    const long long nodes = g.causal ? 1 << l : 1;
+    if (g.b < s) {
+      const long long key_tiles = (g.b + kTileK - 1) / kTileK + (g.m + kTileK - 1) / kTileK;
+      other += nodes * node_blocks(s, g.b) * ((g.b + kTileQ - 1) / kTileQ) * key_tiles;
+    } else {
+      const long long kts = (s + kTileK - 1) / kTileK, full = s / kTileQ;
+      whole += nodes * kts * full; other += nodes * kts * (kts - full); items += nodes * kts;
+    }
+  }
+  BwdBuild r;
+  r.boxes = whole > 0 && 4 * whole >= 7 * items + other;
+  r.results_warps = g.d == 64 && whole > 0 && 2 * whole >= 9 * items + other ? 4 : 8;
+  return r;
+}
+
 // a: the forward schedule (permutations, samples, tile geometry); the accumulators of gr are cleared here
 cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout, float2* stat, int* sched,
                             const BwdGrads& gr, float scale, int* status, cudaStream_t st) {
@@ -73,8 +108,7 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
     if (a.level_sorted[l])
       steps += (long long)(g.causal ? (1 << l) : 1) * g.G * node_blocks(s, g.b) * a.tiles_per_block * (b.smp_ktiles + b.block_ktiles);
   }
-  const long long leaf_steps = b.leaf_ktiles ? (long long)a.leaves_per_seg * g.G * b.leaf_ktiles * (a.dense_causal ? (b.leaf_ktiles + 1) / 2 : b.leaf_ktiles) : 0;
-  steps += leaf_steps;
+  if (b.leaf_ktiles) steps += (long long)a.leaves_per_seg * g.G * b.leaf_ktiles * (a.dense_causal ? (b.leaf_ktiles + 1) / 2 : b.leaf_ktiles);
   const long long want = steps / (6LL * sms);
   b.chunk = (int)(want < 2 ? 2 : (want > 16 ? 16 : want));
   long long items = b.leaf_ktiles ? (long long)g.G * a.leaves_per_seg * b.leaf_ktiles : 0;
@@ -102,8 +136,7 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   maps.dk = maps.dv = maps.dq;
   if (!gr.direct && (!encode_acc_map(&maps.dk, gr.dk, rows, g.d) || !encode_acc_map(&maps.dv, gr.dv, rows, g.d))) return cudaErrorInvalidValue;
   const unsigned grid = items < sms ? (unsigned)items : (unsigned)sms;      // persistent: one CTA per SM
-  bool boxes = b.leaf_ktiles > 0;                       // are there tiles of consecutive rows?
-  for (int l = 0; l < g.levels; ++l) boxes = boxes || !a.level_sorted[l];
+  const BwdBuild build = backward_build(g);
   cudaError_t e;
   auto go = [&](auto dim, auto with_boxes, auto results_warps) {
     constexpr int D = decltype(dim)::value, RW = decltype(results_warps)::value;
@@ -117,10 +150,9 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   using d64 = integral_constant<int, 64>;
   using d128 = integral_constant<int, 128>;
   using eight = integral_constant<int, 8>;
-  // Four results warps where leaves are at least a third of the steps (they gain 6 to 7 % there and lose 3 % in the sorted nodes).
-  if (g.d == 64 && boxes && 3 * leaf_steps >= steps) e = launch_bwd_leaves_d64(b, maps, grid, status, st);
-  else if (g.d == 64) e = boxes ? go(d64{}, bool_constant<true>{}, eight{}) : go(d64{}, bool_constant<false>{}, eight{});
-  else e = boxes ? go(d128{}, bool_constant<true>{}, eight{}) : go(d128{}, bool_constant<false>{}, eight{});
+  if (build.results_warps == 4) e = launch_bwd_leaves_d64(b, maps, grid, status, st);
+  else if (g.d == 64) e = build.boxes ? go(d64{}, bool_constant<true>{}, eight{}) : go(d64{}, bool_constant<false>{}, eight{});
+  else e = build.boxes ? go(d128{}, bool_constant<true>{}, eight{}) : go(d128{}, bool_constant<false>{}, eight{});
   if (e != cudaSuccess || !gr.dq16) return e;
   ToBf16Args c;
   const size_t elems[3] = {rows * g.d, gr.kv_elems, gr.kv_elems};

@@ -130,3 +130,23 @@ def test_node_projections_match_the_oracle():
         w = ha.get_projections(64, 7, 5, node=node)
         assert np.array_equal(w, O.directions(64, 7, 5, node=node))
     assert not np.array_equal(ha.get_projections(64, 7, 5, node=1), ha.get_projections(64, 7, 5))
+
+
+# (boxes, results warps) by what a call's steps are: whole tiles of 128 consecutive rows, which leave as boxes; short tiles of consecutive
+# rows and tiles of sorted rows, which leave row by row and want eight warps; and how often dK and dV leave (once per key tile)
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("kw,boxes,warps", [
+    (dict(n=64, causal=1, n0=64), 0, 8), (dict(n=127, causal=1, n0=128), 0, 8), (dict(n=128, causal=1, n0=128), 0, 8),
+    (dict(n=300, causal=1, n0=512), 0, 8), (dict(n=127, block=128), 0, 8), (dict(n=200, block=256), 0, 8),
+    (dict(n=512, causal=1, n0=512), 1, 8), (dict(n=768, causal=1, n0=768), 1, 8), (dict(n=300, block=512), 1, 8),
+    (dict(n=1536, causal=1, n0=1536), 1, 4), (dict(n=4096, causal=1, n0=4096), 1, 4), (dict(n=4096, block=4096), 1, 4),
+    (dict(n=6400, block=64, causal=1, n0=100), 0, 8), (dict(n=1600, block=800, causal=1, n0=100), 0, 8),
+    (dict(n=32768, block=64, causal=1, n0=512), 0, 8), (dict(n=32768, block=256, samples=256, causal=1, n0=1024), 1, 8),
+    (dict(n=32768, block=256, samples=256, causal=1, n0=2048), 1, 4), (dict(n=131072, block=256, samples=256, causal=1, n0=4096), 1, 4),
+    (dict(n=8192, block=4096, causal=1, n0=512), 1, 4),
+    (dict(n=4096, block=256, samples=256), 0, 8), (dict(n=32768, block=64), 0, 8),
+], ids=lambda x: "_".join(f"{k}{v}" for k, v in x.items()) if isinstance(x, dict) else str(x))
+def test_build_of_the_backward_kernel(d, kw, boxes, warps):
+    got = C.c_int(-1), C.c_int(-1)
+    assert ha.lib().hyperattn_internal_backward_build(C.byref(_params(d=d, **kw)), C.byref(got[0]), C.byref(got[1])) == 0
+    assert (got[0].value, got[1].value) == (boxes, warps if d == 64 else 8)

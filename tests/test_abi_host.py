@@ -145,6 +145,9 @@ def test_node_projections_match_the_oracle():
     (dict(n=32768, block=256, samples=256, causal=1, n0=2048), 1, 4), (dict(n=131072, block=256, samples=256, causal=1, n0=4096), 1, 4),
     (dict(n=8192, block=4096, causal=1, n0=512), 1, 4),
     (dict(n=4096, block=256, samples=256), 0, 8), (dict(n=32768, block=64), 0, 8),
+    # the shapes of test_gpu_kernel_edges.py whose items are more than the SMs: every build of the kernel is run there
+    (dict(H=40, n=640, block=64, samples=33, causal=1, n0=320), 0, 8), (dict(H=110, n=300, block=64, samples=8, causal=1, n0=512), 0, 8),
+    (dict(H=16, n=1400, block=64, samples=33, causal=1, n0=700), 1, 8), (dict(H=4, n=3400, block=64, samples=33, causal=1, n0=1700), 1, 4),
 ], ids=lambda x: "_".join(f"{k}{v}" for k, v in x.items()) if isinstance(x, dict) else str(x))
 def test_build_of_the_backward_kernel(d, kw, boxes, warps):
     got = C.c_int(-1), C.c_int(-1)

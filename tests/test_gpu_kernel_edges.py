@@ -75,9 +75,15 @@ BACKWARD = [
     backward.W("bwd_sorted_over_unsorted_nodes_d64", 1, 2, 1040, 64, 200, 33, 6, True, 130, seed=81),
     backward.W("bwd_sorted_over_unsorted_nodes_d128", 1, 1, 1040, 128, 200, 33, 6, True, 130, seed=82),
     backward.W("bwd_leaves_for_more_than_two_rounds_d64", 1, 110, 300, 64, 64, 8, 4, True, 512, seed=85),
-    # more items than SMs, so that whole tiles of consecutive rows, short ones and scattered rows follow one another in a CTA
+    # more items than SMs, so that whole tiles of consecutive rows, short ones and scattered rows follow one another in a CTA, in every build
+    # of the kernel (test_abi_host.py holds these shapes to the builds): without boxes ...
     backward.W("bwd_whole_short_and_scattered_tiles_d64", 1, 40, 640, 64, 64, 33, 6, True, 320, seed=83),
     backward.W("bwd_whole_short_and_scattered_tiles_d128", 1, 24, 640, 128, 64, 33, 6, True, 320, seed=84),
+    # ... with boxes and eight results warps ...
+    backward.W("bwd_boxes_short_and_scattered_tiles_d64", 1, 16, 1400, 64, 64, 33, 6, True, 700, seed=86),
+    backward.W("bwd_boxes_short_and_scattered_tiles_d128", 1, 12, 1400, 128, 64, 33, 6, True, 700, seed=87),
+    # ... and with four (d = 64)
+    backward.W("bwd_four_results_warps_short_and_scattered_tiles_d64", 1, 4, 3400, 64, 64, 33, 6, True, 1700, seed=88),
 ]
 
 

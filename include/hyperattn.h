@@ -256,10 +256,11 @@ int hyperattn_last_device_status(void* stream, int* status);
  * for every stage, the summed device milliseconds and launch count since the last
  * hyperattn_profile_reset().  Stage indices: */
 enum {
-  HYPERATTN_STAGE_CONVERT = 0, /* fp32 -> bf16 staging copy (fp32 inputs only) */
-  HYPERATTN_STAGE_HASH = 1,    /* Def. 1 hash of Q and K rows + chunk histograms */
-  HYPERATTN_STAGE_SAMPLE = 2,  /* Alg. 2 line 4: drawn inside the SORT_SCAN launch, so always 0 here */
-  HYPERATTN_STAGE_SORT_SCAN = 3,
+  HYPERATTN_STAGE_CONVERT = 0, /* fp32 -> bf16 staging copy (fp32 inputs only; 0 launches where it runs inside the HASH launch) */
+  HYPERATTN_STAGE_HASH = 1,    /* Def. 1 hash of Q and K rows + chunk histograms; value-norm sampling: reads and weighs V too */
+  HYPERATTN_STAGE_SAMPLE = 2,  /* Alg. 2 line 4.  Uniform sampling: drawn inside the SORT_SCAN (or SORT_SCATTER) launch, 0 here;
+                                  value-norm sampling: the draws, and the cumulative weights unless SORT_SCAN makes them */
+  HYPERATTN_STAGE_SORT_SCAN = 3,    /* (0 launches where the scatter does it) value-norm sampling, few nodes: cumulative weights too */
   HYPERATTN_STAGE_SORT_SCATTER = 4, /* Alg. 1 line 3 */
   HYPERATTN_STAGE_ATTENTION = 5,    /* block + sampled + causal-leaf contractions */
   HYPERATTN_STAGE_MERGE = 6,        /* Alg. 4 line 5 carried to outputs */

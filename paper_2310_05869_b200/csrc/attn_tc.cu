@@ -220,8 +220,7 @@ __device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, PairDes
     // Leaf after leaf, the pairs of a leaf from the heaviest (last rows, most keys) to the lightest: items are
     // handed out in this order, so the CTAs that run at the same time work on a handful of neighbouring leaves
     // and find each other's K / V tiles in L2, and the list still ends with light items.
-    // (The last leaves of a call without node items: all heavy pairs first, see tail_leaves().  128 leaves of 4096 rows, d = 64, 440 -> 408
-    // us; 64 leaves, d = 128, 300 -> 271.)
+    // (The last leaves of a call without node items: all heavy pairs first, see tail_leaves().)
     int rem, rank;
     leaf_of_item(pair, a.n_leaf_pairs, a.pairs_per_leaf, a.tail_leaves, rem, rank);
     const int uu = a.pairs_per_leaf - 1 - rank;

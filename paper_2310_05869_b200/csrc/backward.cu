@@ -38,15 +38,15 @@ __global__ void __launch_bounds__(256) to_bf16_kernel(const __grid_constant__ To
 }  // namespace
 
 // What pays is whole tiles of 128 consecutive rows (leaves, nodes that are not sorted): their dQ leaves as a box at every step, with a few
-// instructions.  What costs: the boxes' code in the results warps at every short tile and at every tile of sorted rows, and, with half of the
-// warps, those tiles themselves and the dK and dV of every key tile, behind which the next item waits.  So the rules weigh steps on whole
-// tiles against key tiles of consecutive rows (`items`) and all other steps.  The pass, us, without boxes / with boxes / four results
-// warps (* what the rules take).  d = 64, causal leaves alone: 1024 leaves of 127 rows 57.5* / 59.1 / 63.6, 781 of 256 85.5* / 86.5 / 98.5, 390 of 512
-// 106 / 104* / 115, 195 of 1024 150 / 148 / 150*, 130 of 1536 195 / 192 / 185*, 128 of 4096 999 / 931 / 869*; exact, 2048 heads of 127
-// rows 108* / 111 / 119, 781 of 256 93.6 / 92.1* / 100, 32 of 4096 452 / 423 / 386*; 32768 rows, 16 heads, in leaves of 512 (blocks of 64) 1764* / 1793 / 1923,
-// 1024 1336 / 1327* / 1352, 2048 1385 / 1356 / 1335*, 4096 1667 / 1602 / 1539*; 64 heads of 1600 rows in leaves of 100 under nodes that are not
-// sorted 179* / 179 / 189; no recursion, 32 heads of 4096 rows 131* / 134 / 142.  d = 128, without and with boxes: 1024 leaves of 100 rows 87.8* / 88.3,
-// 781 of 256 162* / 161, 390 of 512 197 / 191*, 64 of 4096 945 / 827*; 32 heads of 32768 rows without recursion 1494* / 1514.
+// instructions.  What costs: the boxes' code in the results warps at every short tile and at every tile of sorted rows, and, with half of the warps,
+// those tiles themselves and the dK and dV of every key tile, behind which the next item waits.  So the rules weigh steps on whole tiles against key
+// tiles of consecutive rows (`items`) and all other steps.  The pass, us, without boxes / with boxes / four results warps (* what the rules take).
+// d = 64, causal leaves alone: 1024 leaves of 127 rows 57.5* / 59.1 / 63.6, 781 of 256 85.5* / 86.5 / 98.5, 390 of 512 106 / 104* / 115, 195 of 1024
+// 150 / 148 / 150*, 130 of 1536 195 / 192 / 185*, 128 of 4096 999 / 931 / 869*; exact, 2048 heads of 127 rows 108* / 111 / 119, 781 of 256 93.6 /
+// 92.1* / 100, 32 of 4096 452 / 423 / 386*; 32768 rows, 16 heads, in leaves of 512 (blocks of 64) 1764* / 1793 / 1923, 1024 1336 / 1327* / 1352,
+// 2048 1385 / 1356 / 1335*, 4096 1667 / 1602 / 1539*; 64 heads of 1600 rows in leaves of 100 under nodes that are not sorted 179* / 179 / 189; no
+// recursion, 32 heads of 4096 rows 131* / 134 / 142.  d = 128, without and with boxes: 1024 leaves of 100 rows 87.8* / 88.3, 781 of 256 162* / 161,
+// 390 of 512 197 / 191*, 64 of 4096 945 / 827*; 32 heads of 32768 rows without recursion 1494* / 1514.
 BwdBuild backward_build(const Geometry& g) {
   long long whole = 0, other = 0, items = 0;            // per segment
   if (g.causal || !g.sorted) {

@@ -26,15 +26,17 @@
 // through independently, half a step apart, with S^T, dP^T, P^T, dV, dK and dQ side by side in TMEM; the tensor pipe needs about 2000
 // clocks per step, the exponentials 1024.  d = 128 has not the TMEM columns (P^T goes over S^T, dQ over dP^T): one chain, in
 // which dQ comes before dK so that it leaves TMEM while dK and the next S^T are multiplied.
-// What bounds it: a step takes 4000 (causal leaves) to 5000 clocks (sorted blocks), of which no single unit is busy for half; the
-// load and store unit is the fullest (gathered copies, dS, results through shared memory, reductions at 25 bytes per clock), and
-// everything else in a chain waits behind it.  The P warps are busy for most of a step, with latencies: a satisfied barrier probe is 100 to
-// 300 clocks here, a read of the statistics about as much.  So they wait three times a step, not five, ask for 16 columns of S^T or dP^T
-// while they work on the 16 before, and take them as 8 x 8 fragments, in which a thread needs the statistics of 16 queries instead of 64
-// (in turn, us: causal leaves of 4096 rows, 128 heads, d = 64, 1092 -> 1049 -> 1033; 65536 rows, 32 heads 1640 -> 1635 -> 1617; 32 heads x
-// 32768 rows, d = 128, 1507 -> 1515 -> 1509).  One chain -> two, us of the whole pass: 131072 rows, 32 heads 3343 -> 3022; causal
-// leaves of 4096 rows, 128 heads 1167 -> 1105 (d = 64; two chains at d = 128 are 10 % slower in the leaves).  16 P warps instead
-// of 8 force 64 registers a thread and are slower (3160 us).
+// What bounds it, sorted blocks (about 5000 clocks a step): the load and store unit, whose data pipe is busy for 58 % (d = 64) or 52 % (d = 128) of
+// the time beside 26 and 29 % of the tensor pipe - gathered copies, dS, statistics, results through shared memory, reductions at 25 bytes per clock
+// - and everything else in a chain waits behind it.  Causal leaves (less than 4000 clocks): no unit by itself; the results leave through the TMA
+// unit, load and store unit and tensor pipe are level at 44 and 43 %, the exponential unit at 34, and the rest is hand-overs of a chain.  The P
+// warps are busy for most of a step, with latencies: a satisfied barrier probe is 100 to 300 clocks here, a read of the statistics about as much.
+// So they wait three times a step, not five, ask for 16 columns of S^T or dP^T while they work on the 16 before, and take them as 8 x 8 fragments,
+// in which a thread needs the statistics of 16 queries instead of 64 (in turn, us: causal leaves of 4096 rows, 128 heads, d = 64, 1092 -> 1049 ->
+// 1033; 65536 rows, 32 heads 1640 -> 1635 -> 1617; 32 heads x 32768 rows, d = 128, 1507 -> 1515 -> 1509; items of one or two steps on tiles that are
+// not whole lose 1 to 3 %: 2048 heads of 127 rows, exact, 105.7 -> 108.1).  One chain -> two, us of the whole pass: 131072 rows, 32 heads 3343 ->
+// 3022; causal leaves of 4096 rows, 128 heads 1167 -> 1105 (d = 64; two chains at d = 128 are 10 % slower in the leaves).  16 P warps instead of 8
+// force 64 registers a thread and are slower (3160 us).
 //
 // Warp roles (672 threads; with four results warps 544): warps 0-7 P and dS; 8-15 (8-11) dQ, dK and dV to global memory; then a warp each: issue
 // of S^T and dP^T (it also allocates TMEM); issue of the gradient products; item descriptors, K and V; Q and the row statistics; dO.
@@ -99,8 +101,7 @@ __device__ __forceinline__ bool decode_item(const BwdArgs& b, int item, BwdItem&
   if (item < b.n_leaf_items) {
     // leaf after leaf, heaviest key tile (the first: every query tile sees it) first; the CTAs that run at the same time work on
     // a few neighbouring leaves and find each other's rows - and dQ accumulators - in L2
-    // (the last leaves of a call without node items: all heavy tiles first, see tail_leaves(); the pass, us: 128 leaves of 4096
-    // rows, d = 64, 992 -> 958; 64 leaves, d = 128, 872 -> 817)
+    // (the last leaves of a call without node items: all heavy tiles first, see tail_leaves())
     int kt, rem;
     leaf_of_item(item, b.n_leaf_items, b.leaf_ktiles, a.tail_leaves, rem, kt);
     t.seg = rem / a.leaves_per_seg;
@@ -242,11 +243,11 @@ __global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__
   if (row < rows && c % LPR == 0) stat[row] = make_float2(-lse[row] * 1.4426950408889634f, -acc);
 }
 
-// BOXES: the call has items of consecutive rows (leaves of the recursion, nodes that are not sorted)
-// RW: results warps.  With eight the block has 21 warps, six of them on one quarter of the SM, which leaves 80 registers a thread; with four it has
-// 17 and 96.  Whole tiles of consecutive rows need no more than four - a box goes out with a few instructions - and the P warps gain from
-// the registers; scattered rows keep eight busy.  (d = 64, the pass, us, 8 -> 4: 128 causal leaves of 4096 rows 956 -> 894, 16 causal heads x 32768
-// 1677 -> 1585; 32 heads x 65536 rows without leaves 1633 -> 1689; d = 128, 64 leaves 838 -> 998.)
+// BOXES: whole tiles of consecutive rows (leaves of the recursion, nodes that are not sorted) leave as boxes; without, all rows by reductions
+// RW: results warps.  With eight the block has 21 warps, six of them on one quarter of the SM, which leaves 80 registers a thread; with four it has 17
+// and 96.  Whole tiles of consecutive rows need no more than four while they follow one another - a box goes out with a few instructions - and the P
+// warps gain from the registers; scattered rows, and dK and dV of items of few steps, keep eight busy.  (Which build a call takes: backward_build()
+// in backward.cu, with figures.  d = 128 always has eight: 64 leaves of 4096 rows 838 us, with four 998.)
 template <int D, bool BOXES, int RW>
 __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __grid_constant__ BwdArgs b, const __grid_constant__ BwdMaps maps,
                                                                   int* status) {
@@ -321,7 +322,8 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
 
   bool ok = true;
   if (warp < C::SW) {
-    // ================= P and dS: thread = key, warpgroup q: query columns W q .. W q + W - 1, in two chunks of CW ==================
+    // ================= P and dS: warp = 32 keys, warpgroup q: query columns W q .. W q + W - 1, in two chunks of CW; a thread has a fragment's
+    // share, two queries of every eight for four keys ===================
     constexpr int W = 128 / (C::SW / 4), CW = W / 2;
     static_assert(CW == 32, "a chunk's P is one TMEM store of 16 columns");
     // The thread's share of a unit of 32 keys x 16 queries is that of four 8 x 8 matrices side by side, twice: keys frow + 8 j, queries 8 k +
@@ -457,7 +459,7 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
     }
   } else if (warp < C::SW + C::RW) {
     // ================= results, fp32 reductions into the accumulators: dQ after every step, dK and dV after every item; warpgroup
-    // r takes half of the columns ==================
+    // r of RW / 4 takes NC columns ===================
     const int r_ = (warp - C::SW) >> 2, row = tid & 127;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     constexpr int NC = D * 4 / C::RW;                // columns of a result that this warpgroup takes
@@ -504,8 +506,8 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
         __syncwarp();
       }
     };
-    // Whole tiles of consecutive rows: a box per 32 columns, added by the TMA unit (causal leaves, 128 heads x 4096 rows, d = 64, the pass:
-    // 1037 -> 1007 us).  In code of its own: one routine for both slows the scattered rows by 8 %.
+    // Whole tiles of consecutive rows: a box per 32 columns, added by the TMA unit (causal leaves, 128 heads x 4096 rows, d = 64, the pass, eight
+    // results warps: 999 -> 931 us).  In code of its own: one routine for both slows the scattered rows by 8 %.
     auto staged_read = [&]() {                          // the boxes before have been read out of the staging buffer
       if (lane == 0) bulk_wait_read();
       __syncwarp();

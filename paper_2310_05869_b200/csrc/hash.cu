@@ -110,9 +110,11 @@ __device__ __forceinline__ size_t hist_base(const HashArgs& a, const ChunkPos& c
 // groups of 16 rows; the loads of the next group are issued between the MMAs of the current
 // one, and the direction fragments live in shared memory (one 8-byte read per MMA) instead
 // of 48 registers, so that two to four CTAs fit an SM and ~128 KB of loads are in flight.
-// VNORM: further CTAs weigh the rows of V for the sampling by value norms: neither of the two reads by itself keeps the memory busy to its
-// end.  (With the cumulative sums beside the scan of the histograms, the call, us: 4 heads of 50000 queries, 131072 keys, d = 64, 154 -> 139;
-// 40000 queries, d = 128, 270 -> 248, but 275 with 64 KB of rows per CTA at a time instead of 32.)
+// VNORM: further CTAs weigh the rows of V for the sampling by value norms: neither of the two reads by itself keeps the memory busy to its end.
+// (With the cumulative sums beside the scan of the histograms, the call, us: 4 heads of 50000 queries, 131072 keys, d = 64, 154 -> 139; 40000
+// queries, d = 128, 270 -> 248, but 275 with 64 KB of rows per CTA at a time instead of 32.  The 32 KB are asked for by every CTA of the launch; it
+// pays also where the hash alone fills the chip: 32 heads of 131072 rows 1510 -> 1481, of 32768 414 -> 398, 128 of 4096 226 -> 215, 512 of 1024 192
+// -> 187, d = 128, 32 of 32768 601 -> 575, 32 of 4096 108 -> 103, 32 causal ones of 16384 1034 -> 982.)
 template <int D, bool VNORM>
 __global__ void __launch_bounds__(256, D == 64 ? 4 : 3) hash_bf16_kernel(const __grid_constant__ HashArgs a) {
   if (VNORM && (int)blockIdx.x >= a.hash_ctas) {

@@ -210,7 +210,8 @@ struct Cfg {
   static_assert(kColQ + (kQTmem ? D : 0) <= 512, "TMEM columns");
 };
 
-__device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, PairDesc& t, QTile& qa, QTile& qb, int& lenA, int& lenB) {
+// only: the pair's query tile that the item consists of, -1: both
+__device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, int only, PairDesc& t, QTile& qa, QTile& qb, int& lenA, int& lenB) {
   const Geometry& g = a.g;
   t.partial = !a.direct;
   qa.valid = 1; qb.valid = 0;
@@ -264,9 +265,9 @@ __device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, PairDes
     QTile* qs[2] = {&qa, &qb};
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const int tn = paired ? 2 * pn + i : pn;
+      const int tn = paired ? 2 * pn + (only < 0 ? i : only) : pn;
       QTile& q = *qs[i];
-      q.valid = tn < tiles_node && (paired || i == 0);
+      q.valid = tn < tiles_node && (i == 0 || (paired && only < 0));
       q.row0 = 0;
       if (sorted) {
         q.beta = tn / a.tiles_per_block;
@@ -994,9 +995,10 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       int item = 0;
       if (lane == 0) item = atomicAdd(a.sched, 1);
       item = __shfl_sync(0xffffffffu, item, 0);
-      const bool end = item >= a.total_pairs;
+      const bool end = item >= a.total_pairs + a.split_pairs;
       PairDesc t = {}; QTile qa = {}, qb = {}; int lenA = 0, lenB = 0;
-      if (!end) decode_pair(a, item, t, qa, qb, lenA, lenB);
+      const int tail = item - (a.total_pairs - a.split_pairs);     // the last pairs: each query tile an item
+      if (!end) decode_pair(a, tail < 0 ? item : item - ((tail + 1) >> 1), tail < 0 ? -1 : tail & 1, t, qa, qb, lenA, lenB);
       else t.mode = -1;                                   // tells every role that the list is exhausted
       if (lane == 0) HA_TACC(26, tdec);
       const int set = it & 1;
@@ -1360,9 +1362,11 @@ cudaError_t launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st)
   int sms = 0;
   cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
-  const int grid = a.total_pairs < sms ? a.total_pairs : sms;     // persistent: one CTA per SM walks the item list
   const bool variant = a.capped || a.sample_wlog;
   AttnArgs b = a;
+  b.split_pairs = split_pairs(a, sms);
+  const int items = a.total_pairs + b.split_pairs;
+  const int grid = items < sms ? items : sms;                     // persistent: one CTA per SM walks the item list
   b.tail_leaves = a.dense_causal && a.total_pairs == a.n_leaf_pairs ? tail_leaves(a.n_leaf_pairs / a.pairs_per_leaf, a.pairs_per_leaf, sms) : 0;
   if (variant && (a.precise || (a.capped && a.sample_wlog))) return cudaErrorInvalidValue;
   const bool late = a.g.d == 128 && !a.direct && !a.part_bf16;

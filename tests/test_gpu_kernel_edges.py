@@ -57,6 +57,27 @@ def test_forward_edges(w):
     parity.test_small_configs_every_stage(w)
 
 
+# heads of a call whose pairs of query tiles are split (at most 74 of 148 SMs have one left), and of one whose pairs are not
+SPLIT = [(64, 1000, 1000, 256, 64, 18, 20),              # two tiles of a block; a short last block
+         (128, 1100, 1100, 256, 130, 14, 16),            # ... whose second tile does not exist
+         (64, 1100, 1100, 100, 33, 12, 13),              # pairs across blocks, an odd number of tiles
+         (128, 600, 1500, 128, 64, 9, 13),               # ... fewer queries than keys
+         (64, 20000, 20000, 256, 256, 2, 3)]             # behind a round of whole pairs
+
+
+@pytest.mark.parametrize("d,n,n_k,b,m,split,whole", SPLIT)
+def test_split_pairs_give_the_same_results(d, n, n_k, b, m, split, whole):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(7)
+    q, k, v = (torch.randn(1, whole, rows, d, generator=gen, device="cuda").bfloat16() for rows in (n, n_k, n_k))
+    want = ha.forward(q, k, v, b, m, 6, seed=3, out_dtype=torch.float32)
+    got = ha.forward(q[:, :split], k[:, :split], v[:, :split], b, m, 6, seed=3, out_dtype=torch.float32)
+    # the same bits, but for the order of the sampled columns where a pair has tiles of two blocks: fp32 sums of b + m weighted values
+    assert float((got[0] - want[0][:, :split]).abs().max()) <= (b + m) * 2.0 ** -24 * float(v.abs().max())
+    assert float((got[1] - want[1][:, :split]).abs().max()) <= (b + m) * 2.0 ** -24
+    assert ha.last_device_status() == 0
+
+
 BACKWARD = [
     # key tiles and query halves of 1, 2, 63 .. 66, 127 and 128 rows; chunks of query tiles that do not divide the node
     backward.W("bwd_blocks_of_64_d64", 1, 1, 1090, 64, 64, 129, 6, False, 0, seed=70),

@@ -457,7 +457,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     gr.kv_elems = kv_elems;
     gr.dq16 = g32 ? nullptr : bw->dq; gr.dk16 = g32 ? nullptr : bw->dk; gr.dv16 = g32 ? nullptr : bw->dv;
     gr.direct = direct; gr.key_slot = ws.key_slot;
-    StageScope sc(st, HYPERATTN_STAGE_BACKWARD, 2 + (g32 ? 0 : 1));
+    StageScope sc(st, HYPERATTN_STAGE_BACKWARD, 2 + (g32 ? 0 : 1) + (backward_split(g, kv_elems) ? 1 : 0));
     HA_CHECK(launch_backward(a, p.out, out_fp32, p.lse, bw->dout, reinterpret_cast<float2*>(base + pl.stat), ws.sched, gr, scale, ws.status, st));
     return HYPERATTN_OK;
   }

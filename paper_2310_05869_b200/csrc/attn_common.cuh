@@ -34,7 +34,9 @@ struct BwdBuild {
   bool boxes;                  // whole tiles of consecutive rows leave as boxes
   int results_warps;
 };
-BwdBuild backward_build(const Geometry& g);
+BwdBuild backward_build(const Geometry& g, bool leaves = true, bool nodes = true);
+// leaves and nodes in launches of their own (kv_elems: entries of the fp32 dK)
+bool backward_split(const Geometry& g, size_t kv_elems);
 
 struct AttnArgs {
   const __nv_bfloat16 *q, *k, *v;    // [G, n, D]

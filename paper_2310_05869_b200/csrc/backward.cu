@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(256) to_bf16_kernel(const __grid_constant__ To
 
 }  // namespace
 
-// What pays is whole tiles of 128 consecutive rows (leaves, nodes that are not sorted): their dQ leaves as a box at every step, with a few
+// (with_leaves, with_nodes: what the launch has of the call's items.)  What pays is whole tiles of 128 consecutive rows (leaves, nodes that are not sorted): their dQ leaves as a box at every step, with a few
 // instructions.  What costs: the boxes' code in the results warps at every short tile and at every tile of sorted rows, and, with half of the warps,
 // those tiles themselves and the dK and dV of every key tile, behind which the next item waits.  So the rules weigh steps on whole tiles against key
 // tiles of consecutive rows (`items`) and all other steps.  The pass, us, without boxes / with boxes / four results warps (* what the rules take).
@@ -47,14 +47,14 @@ __global__ void __launch_bounds__(256) to_bf16_kernel(const __grid_constant__ To
 // 2048 1385 / 1356 / 1335*, 4096 1667 / 1602 / 1539*; 64 heads of 1600 rows in leaves of 100 under nodes that are not sorted 179* / 179 / 189; no
 // recursion, 32 heads of 4096 rows 131* / 134 / 142.  d = 128, without and with boxes: 1024 leaves of 100 rows 87.8* / 88.3, 781 of 256 162* / 161,
 // 390 of 512 197 / 191*, 64 of 4096 945 / 827*; 32 heads of 32768 rows without recursion 1494* / 1514.
-BwdBuild backward_build(const Geometry& g) {
+BwdBuild backward_build(const Geometry& g, bool with_leaves, bool with_nodes) {
   long long whole = 0, other = 0, items = 0;            // per segment
-  if (g.causal || !g.sorted) {
+  if (with_leaves && (g.causal || !g.sorted)) {
     const long long leaves = g.npad / g.leaf, kts = (g.leaf + kTileK - 1) / kTileK, full = g.leaf / kTileQ;
     const long long on_full = g.causal ? full * (full + 1) / 2 : kts * full, all = g.causal ? kts * (kts + 1) / 2 : kts * kts;
     whole += leaves * on_full; other += leaves * (all - on_full); items += leaves * kts;
   }
-  for (int l = 0; l < g.levels; ++l) {
+  for (int l = 0; l < g.levels && with_nodes; ++l) {
     int s, q0, k0;
     node_rows(g, l, 0, s, q0, k0);
     const long long nodes = g.causal ? 1 << l : 1;
@@ -72,19 +72,28 @@ BwdBuild backward_build(const Geometry& g) {
   return r;
 }
 
+// With recursion every row of dK and dV gets one contribution from its leaf and more from the nodes above it.  The leaves in a launch of their own, first, write
+// theirs, so that the accumulators need not be cleared, and leaves and nodes take the build that is best for each.  Against that stand a launch and
+// the end of the first one, where SMs run out of items: it pays from 192 MiB of accumulators on, where leaves leave as boxes.  (The pass, us, one launch ->
+// two: 32 heads of 131072 rows, d = 64, 16322 -> 16046 and, another time, 16239 -> 15962, 16 of 32768 (256 MiB) 1715 -> 1708 and 1719 -> 1700, 8 of
+// 32768, d = 128, (256 MiB) 1680 -> 1609 and 1669 -> 1614; 4 of 65536, d = 64, (128 MiB) 972 -> 984.)
+constexpr size_t kSplitBytes = 192u << 20;
+bool backward_split(const Geometry& g, size_t kv_elems) { return g.L > 0 && kv_elems * 8 >= kSplitBytes && backward_build(g, true, false).boxes; }
+
 // a: the forward schedule (permutations, samples, tile geometry); the accumulators of gr are cleared here
 cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout, float2* stat, int* sched,
                             const BwdGrads& gr, float scale, int* status, cudaStream_t st) {
   const Geometry& g = a.g;
   const size_t rows = (size_t)g.G * g.n;
   if (rows > 0x7fffffffull) return cudaErrorInvalidValue;            // TMA row coordinates are 32-bit
+  const bool split = backward_split(g, gr.kv_elems);
   {
     const unsigned grid = (unsigned)((rows * (g.d / 8) + 255) / 256);
     const uint4* d4 = reinterpret_cast<const uint4*>(dout);
     auto* kernel = g.d == 64 ? (out_fp32 ? row_stat_kernel<64, true> : row_stat_kernel<64, false>)
                              : (out_fp32 ? row_stat_kernel<128, true> : row_stat_kernel<128, false>);
     const cudaError_t e = launch(kernel, grid, 256, 0, st, d4, out, lse, stat, rows, sched, reinterpret_cast<float4*>(gr.dq),
-                                 reinterpret_cast<float4*>(gr.dk), reinterpret_cast<float4*>(gr.dv), gr.kv_elems / g.d);
+                                 reinterpret_cast<float4*>(gr.dk), reinterpret_cast<float4*>(gr.dv), split ? 0 : gr.kv_elems / g.d);
     if (e != cudaSuccess) return e;
   }
   int sms = 0;
@@ -93,7 +102,7 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   b.a = a; b.dout = reinterpret_cast<const __nv_bfloat16*>(dout); b.stat = stat; b.scale = scale; b.sched = sched;
   b.dq = gr.dq; b.dk = gr.dk; b.dv = gr.dv;
   b.dk16 = reinterpret_cast<__nv_bfloat16*>(gr.dk16); b.dv16 = reinterpret_cast<__nv_bfloat16*>(gr.dv16);
-  b.key_slot = gr.key_slot; b.direct = gr.direct;
+  b.key_slot = gr.key_slot; b.direct = gr.direct; b.kv_first = 0;
   b.leaf_ktiles = a.n_leaf_tiles ? (g.leaf + kTileK - 1) / kTileK : 0;
   b.block_ktiles = (g.b + kTileK - 1) / kTileK;
   b.smp_ktiles = (g.m + kTileK - 1) / kTileK;
@@ -128,17 +137,14 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   b.level_item_start[g.levels] = (int)items;
   b.total_items = (int)items;
   if (items == 0) return cudaSuccess;
-  b.a.tail_leaves = a.dense_causal && items == b.n_leaf_items ? tail_leaves(b.n_leaf_items / b.leaf_ktiles, b.leaf_ktiles, sms) : 0;
+  b.a.tail_leaves = a.dense_causal && (split || items == b.n_leaf_items) ? tail_leaves(b.n_leaf_items / b.leaf_ktiles, b.leaf_ktiles, sms) : 0;
   BwdMaps maps;
   if (!encode_rows_map(&maps.q, a.q, rows, g.d, 128) || !encode_rows_map(&maps.k, a.k, rows, g.d, 128) ||
       !encode_rows_map(&maps.v, a.v, rows, g.d, 128) || !encode_rows_map(&maps.dout, dout, rows, g.d, 128) ||
       !encode_acc_map(&maps.dq, gr.dq, rows, g.d)) return cudaErrorInvalidValue;
   maps.dk = maps.dv = maps.dq;
   if (!gr.direct && (!encode_acc_map(&maps.dk, gr.dk, rows, g.d) || !encode_acc_map(&maps.dv, gr.dv, rows, g.d))) return cudaErrorInvalidValue;
-  const unsigned grid = items < sms ? (unsigned)items : (unsigned)sms;      // persistent: one CTA per SM
-  const BwdBuild build = backward_build(g);
-  cudaError_t e;
-  auto go = [&](auto dim, auto with_boxes, auto results_warps) {
+  auto go = [&](auto dim, auto with_boxes, auto results_warps, unsigned grid) {
     constexpr int D = decltype(dim)::value, RW = decltype(results_warps)::value;
     constexpr bool BOXES = decltype(with_boxes)::value;
     using C = Cfg<D, RW>;
@@ -150,9 +156,22 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   using d64 = integral_constant<int, 64>;
   using d128 = integral_constant<int, 128>;
   using eight = integral_constant<int, 8>;
-  if (build.results_warps == 4) e = launch_bwd_leaves_d64(b, maps, grid, status, st);
-  else if (g.d == 64) e = build.boxes ? go(d64{}, bool_constant<true>{}, eight{}) : go(d64{}, bool_constant<false>{}, eight{});
-  else e = build.boxes ? go(d128{}, bool_constant<true>{}, eight{}) : go(d128{}, bool_constant<false>{}, eight{});
+  auto run = [&](BwdBuild build) {
+    const unsigned grid = b.total_items < sms ? (unsigned)b.total_items : (unsigned)sms;     // persistent: one CTA per SM
+    if (build.results_warps == 4) return launch_bwd_leaves_d64(b, maps, grid, status, st);
+    if (g.d == 64) return build.boxes ? go(d64{}, bool_constant<true>{}, eight{}, grid) : go(d64{}, bool_constant<false>{}, eight{}, grid);
+    return build.boxes ? go(d128{}, bool_constant<true>{}, eight{}, grid) : go(d128{}, bool_constant<false>{}, eight{}, grid);
+  };
+  cudaError_t e;
+  if (split) {
+    b.total_items = b.n_leaf_items; b.kv_first = 1;
+    e = run(backward_build(g, true, false));
+    if (e != cudaSuccess) return e;
+    b.total_items = (int)items - b.n_leaf_items; b.kv_first = 0; b.sched = sched + 1; b.a.tail_leaves = 0;
+    for (int l = g.levels; l >= 0; --l) b.level_item_start[l] -= b.n_leaf_items;
+    b.n_leaf_items = 0;
+    e = run(backward_build(g, false, true));
+  } else e = run(backward_build(g));
   if (e != cudaSuccess || !gr.dq16) return e;
   ToBf16Args c;
   const size_t elems[3] = {rows * g.d, gr.kv_elems, gr.kv_elems};

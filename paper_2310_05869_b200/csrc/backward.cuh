@@ -62,6 +62,7 @@ struct BwdArgs {
   __nv_bfloat16 *dk16, *dv16;  // direct: dK and dV of the keys without samples
   const int32_t* key_slot;     // direct: [G, n] the sample that stands for a key, -1: none (null: none for any)
   int direct;
+  int kv_first;                // (kBoxes) nothing has been added to dK and dV yet and every row is written once: the accumulators need not be cleared
   float scale;
   int* sched;                  // work counter of the launch, zero at launch
   // items: the key tiles of the leaves, then level by level those of the nodes
@@ -205,7 +206,7 @@ struct Cfg {
 };
 
 // (-lse log2 e, -<dO, O>) of every row: D / 8 lanes per row, 16 bytes of dO and O each (HBM-bound).
-// The same threads clear the accumulators: 32 bytes of each.
+// The same threads clear the accumulators, 32 bytes of each (kv_rows rows of dK and dV), and the work counters of two launches.
 template <int D, bool OUT_FP32>
 __global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__ dout, const void* __restrict__ out, const float* __restrict__ lse,
                                                        float2* __restrict__ stat, size_t rows, int* sched, float4* dq, float4* dk, float4* dv,
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__
   constexpr int LPR = D / 8;
   const size_t c = (size_t)blockIdx.x * 256 + threadIdx.x;
   wait_for_stream();
-  if (c == 0) *sched = 0;
+  if (c == 0) sched[0] = sched[1] = 0;
   const size_t row = c / LPR;
   float acc = 0.f;
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -497,7 +498,9 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const int gr = __shfl_sync(0xffffffffu, grow, 4 * (q0 + q) + (lane >> 3));
-            if (gr >= 0) atomicAdd(reinterpret_cast<float4*>(base + (size_t)gr * D + NC * r_ + 32 * p + 4 * c), v[q]);
+            float4* dst = reinterpret_cast<float4*>(base + (size_t)gr * D + NC * r_ + 32 * p + 4 * c);
+            if (BOXES && decltype(direct)::value && gr >= 0 && b.kv_first) *dst = v[q];
+            else if (gr >= 0) atomicAdd(dst, v[q]);
             else if (decltype(direct)::value && gr != kNoRow)
               *reinterpret_cast<uint2*>(base16 + (size_t)~gr * D + NC * r_ + 32 * p + 4 * c) =
                   make_uint2(pack2(v[q].x, v[q].y), pack2(v[q].z, v[q].w));
@@ -512,7 +515,7 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
       if (lane == 0) bulk_wait_read();
       __syncwarp();
     };
-    auto out_boxes = [&](uint32_t taddr, float f, const CUtensorMap* map, int y, uint32_t bar_done) {
+    auto out_boxes = [&](auto first, uint32_t taddr, float f, const CUtensorMap* map, int y, uint32_t bar_done) {
 #pragma unroll
       for (int p = 0; p < NC / 32; ++p) {
         uint32_t r[32];
@@ -531,7 +534,10 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
                        "f"(__uint_as_float(r[4 * x + 2]) * f), "f"(__uint_as_float(r[4 * x + 3]) * f) : "memory");
         fence_async_smem();
         __syncwarp();
-        if (lane == 0) tma_add_tile(map, NC * r_ + 32 * p, y, stage);
+        if (lane == 0) {
+          if (decltype(first)::value && b.kv_first) tma_put_tile(map, NC * r_ + 32 * p, y, stage);
+          else tma_add_tile(map, NC * r_ + 32 * p, y, stage);
+        }
       }
     };
     uint32_t g = 0;
@@ -560,7 +566,7 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
         if (!ok) break;
         tc_fence_after();
         if (box) {
-          out_boxes(lane_addr + C::kColDQ, b.scale, &maps.dq, seg_row0 + sr.first + (row & ~31), bar_dqfree);
+          out_boxes(std::false_type{}, lane_addr + C::kColDQ, b.scale, &maps.dq, seg_row0 + sr.first + (row & ~31), bar_dqfree);
           continue;
         }
         if (BOXES && t.kind == 0) staged_read();
@@ -572,8 +578,8 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
       tc_fence_after();
       if (BOXES && t.kind == 0 && t.nkeys == kTileK && !b.direct) {
         const int y = seg_row0 + t.k0 + (row & ~31);
-        out_boxes(lane_addr + C::kColDV, 1.f, &maps.dv, y, 0);
-        out_boxes(lane_addr + C::kColDK, b.scale, &maps.dk, y, bar_accfree);
+        out_boxes(std::true_type{}, lane_addr + C::kColDV, 1.f, &maps.dv, y, 0);
+        out_boxes(std::true_type{}, lane_addr + C::kColDK, b.scale, &maps.dk, y, bar_accfree);
       } else {
         if (BOXES && t.kind == 0) staged_read();
         out_rows(std::true_type{}, lane_addr + C::kColDV, 1.f, b.dv, b.dv16, kr, 0);

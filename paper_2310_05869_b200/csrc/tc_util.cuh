@@ -236,6 +236,11 @@ __device__ __forceinline__ void tma_add_tile(const CUtensorMap* map, int x, int 
   asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%1, %2}], [%3];\n\tcp.async.bulk.commit_group;"
                ::"l"(map), "r"(x), "r"(y), "r"(src) : "memory");
 }
+// the same, written instead of added
+__device__ __forceinline__ void tma_put_tile(const CUtensorMap* map, int x, int y, uint32_t src) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];\n\tcp.async.bulk.commit_group;"
+               ::"l"(map), "r"(x), "r"(y), "r"(src) : "memory");
+}
 // the executing thread's bulk groups have read their shared memory; have been written
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }

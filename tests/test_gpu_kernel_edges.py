@@ -78,6 +78,35 @@ def test_split_pairs_give_the_same_results(d, n, n_k, b, m, split, whole):
     assert ha.last_device_status() == 0
 
 
+# calls whose leaves go first and write dK and dV (from 192 MiB of fp32 accumulators on), against calls of few heads, which add everything
+SPLIT_BACKWARD = [(64, 26, 16384, 4096), (64, 26, 16800, 2100), (64, 40, 10240, 700), (128, 13, 16384, 4096)]
+
+
+@pytest.mark.parametrize("d,H,n,n0", SPLIT_BACKWARD)
+@pytest.mark.parametrize("grad_dtype", [torch.float32, torch.bfloat16])
+def test_backward_with_leaves_in_a_launch_of_their_own(d, H, n, n0, grad_dtype):
+    assert 8 * H * n * d >= 192 << 20
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(13)
+    q, k, v, dout = (torch.randn(1, H, n, d, generator=gen, device="cuda").bfloat16() for _ in range(4))
+    args, kw = (256, 128, 6), dict(causal=True, n0=n0, seed=4)
+    out, lse = ha.forward(q, k, v, *args, **kw)
+    stale = [torch.full((1, H, n, d), float("nan"), dtype=grad_dtype, device="cuda") for _ in range(3)]
+    del stale                                              # (the gradients' memory holds NaN)
+    got = ha.backward(q, k, v, out, lse, dout, *args, grad_dtype=grad_dtype, **kw)
+    few = 2
+    part = [x[:, :few].contiguous() for x in (q, k, v, out, lse, dout)]
+    want = ha.backward(*part, *args, grad_dtype=grad_dtype, **kw)
+    for x, y in zip(got, want):
+        # the same terms in another order: at most 200 partial sums of fp32 (2 x 200 x 2^-24 of the terms' absolute values, which add up to a few
+        # times the largest entry), and bf16 results may be a step apart (2^(e - 7) for 2^e <= |y|)
+        x, y = x[:, :few].float(), y.float()
+        assert torch.isfinite(x).all()
+        limit = 1e-4 * float(y.abs().max()) + (2.0 ** -7 * y.abs() if grad_dtype == torch.bfloat16 else 0.0)
+        assert bool(((x - y).abs() <= limit).all())
+    assert ha.last_device_status() == 0
+
+
 BACKWARD = [
     # key tiles and query halves of 1, 2, 63 .. 66, 127 and 128 rows; chunks of query tiles that do not divide the node
     backward.W("bwd_blocks_of_64_d64", 1, 1, 1090, 64, 64, 129, 6, False, 0, seed=70),

@@ -6,8 +6,6 @@
 // node, so the histogram of a chunk is the same at every level of the causal recursion and
 // only the scan differs per level.  Ties keep the original row order, which makes the
 // permutation unique.
-#include <type_traits>
-
 #include "vnorm_common.cuh"
 
 namespace hyperattn {
@@ -159,10 +157,15 @@ __global__ void __launch_bounds__(256 * NG) sort_scan_kernel(SortArgs a, SampleA
 // One CTA per (side, level, segment, chunk of the level): stable placement of <= g.chunk rows.  SCAN: the launch takes over
 // the scan's work where nodes have few chunks - every CTA adds up the histograms of its node's chunks by itself and extra blocks draw the
 // samples - which saves a small call one launch of three.
-template <int R, bool SCAN>
-__global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a, SampleArgs sa, int place_blocks) {
-  __shared__ __align__(16) uint32_t s_cnt[8][kBuckets];   // per-warp running positions
-  __shared__ uint8_t s_id[kSortChunk];
+// Bound by instruction issue.  A row's place among the rows of its warp's range comes from a word per bucket into which the lanes of a group put a bit
+// each, and is kept in a register until the ranges before it are counted, so that every row is looked up once.  (Before: a histogram of the ranges,
+// then a ballot per id bit and group.  Kernel, us, ballots -> words: 32 heads x 131072 rows 47.9 -> 42.6, 32 causal ones 129 -> 110, 4 causal x 100003
+// 19.5 -> 17.1; with the scan's work in it 32 x 32768, d = 128, 17.5 -> 17.4 - five CTAs an SM; four 18.9, six, with spills, 17.4 to 18.3 -, 32 x 4096 5.7 -> 5.5.
+// Rows that are all in one bucket set their bits one after another, as the histogram counted them before.)
+template <bool SCAN>
+__global__ void __launch_bounds__(256, SCAN ? 5 : 6) sort_scatter_kernel(SortArgs a, SampleArgs sa, int place_blocks) {
+  // per warp and bucket: lanes of the row group at hand that are in the bucket; rows of the warp's range counted so far, then its first position
+  __shared__ __align__(16) uint2 s_bkt[8][kBuckets];
   const Geometry& g = a.g;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (SCAN && (int)blockIdx.x >= place_blocks) {
@@ -212,13 +215,37 @@ __global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a, SampleArg
       for (int e = 0; e < 8; ++e) { tot += x[e]; if (c0 + e < cn) before += x[e]; }
     }
   }
-  for (int i = tid; i < rows; i += 256) s_id[i] = ids[i];
-  for (int i = tid; i < 8 * kBuckets / 4; i += 256) reinterpret_cast<uint4*>(&s_cnt[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
-  __syncthreads();
-  // per-warp histograms of consecutive sub-ranges of an eighth of the chunk
+  // A warp has an eighth of the chunk, in groups of 32 consecutive rows.
+  constexpr int GROUPS = kSortChunk / 8 / 32;
   const int wbeg = warp * (g.chunk / 8);
   const int wend = min(rows, wbeg + g.chunk / 8);
-  for (int i = wbeg + lane; i < wend; i += 32) atomicAdd(&s_cnt[warp][s_id[i]], 1u);
+  uint32_t row_id[GROUPS];
+#pragma unroll
+  for (int k = 0; k < GROUPS; ++k) {
+    const int i = wbeg + 32 * k + lane;
+    row_id[k] = i < wend ? ids[i] : 0u;
+  }
+#pragma unroll
+  for (int k = 0; k < 8 * kBuckets / 2 / 256; ++k) reinterpret_cast<uint4*>(&s_bkt[0][0])[tid + 256 * k] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  uint2* bkt = s_bkt[warp];
+  // A row's place among the rows of the range with its id: those of earlier groups, and the lanes before it in the bucket's word, into which every
+  // lane has put its bit.
+#pragma unroll
+  for (int k = 0; k < GROUPS; ++k) {
+    if (wbeg + 32 * k < wend) {                          // (the same for the whole warp)
+      const bool act = wbeg + 32 * k + lane < wend;
+      const uint32_t id = row_id[k];
+      if (act) atomicOr(&bkt[id].x, 1u << lane);
+      __syncwarp();
+      const uint2 b = bkt[id];
+      const int before = __popc(b.x & ((1u << lane) - 1u));
+      __syncwarp();
+      if (act && before == 0) bkt[id] = make_uint2(0u, b.y + __popc(b.x));
+      __syncwarp();
+      row_id[k] = id | (b.y + before) << 8;
+    }
+  }
   __syncthreads();
   uint32_t run;
   if (SCAN) {
@@ -240,30 +267,16 @@ __global__ void __launch_bounds__(256) sort_scatter_kernel(SortArgs a, SampleArg
     run = o[tid];
   }
 #pragma unroll
-  for (int w = 0; w < 8; ++w) { const uint32_t t = s_cnt[w][tid]; s_cnt[w][tid] = run; run += t; }
+  for (int w = 0; w < 8; ++w) { const uint32_t t = s_bkt[w][tid].y; s_bkt[w][tid].y = run; run += t; }
   __syncthreads();
   const size_t slice = ((size_t)level * g.G + seg) * g.nl + (g.causal ? (size_t)j * s : 0);
   int32_t* perm = (side == 0 ? a.perm_q : a.perm_k) + slice;
   int32_t* rank = side == 1 ? a.rank_k + slice : nullptr;
-  for (int i0 = wbeg; i0 < wend; i0 += 32) {
-    const int i = i0 + lane;
-    const bool act = i < wend;
-    const uint32_t id = act ? s_id[i] : 0u;
-    // lanes with the same bucket id: one ballot per id bit (ids have at most 8 bits; a generic
-    // match.any costs several times more)
-    uint32_t peers = __ballot_sync(0xffffffffu, act);
 #pragma unroll
-    for (int bit = 0; bit < R; ++bit) {                 // (ids have R bits)
-      const uint32_t bal = __ballot_sync(0xffffffffu, (id >> bit) & 1u);
-      peers &= ((id >> bit) & 1u) ? bal : ~bal;
-    }
-    const int before = __popc(peers & ((1u << lane) - 1u));
-    uint32_t pos = 0;
-    if (act) pos = s_cnt[warp][id] + before;
-    __syncwarp();
-    if (act && before == 0) s_cnt[warp][id] += __popc(peers);
-    __syncwarp();
-    if (act) {
+  for (int k = 0; k < GROUPS; ++k) {
+    const int i = wbeg + 32 * k + lane;
+    if (i < wend) {
+      const uint32_t pos = bkt[row_id[k] & 255u].y + (row_id[k] >> 8);
       perm[pos] = local0 + i;
       if (rank) rank[local0 + i] = (int32_t)pos;
       if (side == 1 && a.key_slot) a.key_slot[(size_t)seg * g.nk + local0 + i] = -1;
@@ -352,22 +365,8 @@ cudaError_t launch_sort_scatter(const Geometry& g, const Workspace& ws, bool wit
   const int grid = g.levels * g.G * (((side_mask & 1) ? side_cpl(g, 0) : 0) + ((side_mask & 2) ? side_cpl(g, 1) : 0));
   int sample_blocks;
   const SampleArgs sa = make_sample_args(g, ws, with_samples, seed, &sample_blocks);
-  auto go = [&](auto r) {                                // the hash width is a template parameter of the ballot loop
-    constexpr int R = decltype(r)::value;
-    if (scan_in_scatter(g)) return launch(sort_scatter_kernel<R, true>, grid + sample_blocks, 256, 0, st, a, sa, grid);
-    return launch(sort_scatter_kernel<R, false>, grid, 256, 0, st, a, sa, grid);
-  };
-  using std::integral_constant;
-  switch (g.r) {
-    case 1: return go(integral_constant<int, 1>{});
-    case 2: return go(integral_constant<int, 2>{});
-    case 3: return go(integral_constant<int, 3>{});
-    case 4: return go(integral_constant<int, 4>{});
-    case 5: return go(integral_constant<int, 5>{});
-    case 6: return go(integral_constant<int, 6>{});
-    case 7: return go(integral_constant<int, 7>{});
-    default: return go(integral_constant<int, 8>{});
-  }
+  if (scan_in_scatter(g)) return launch(sort_scatter_kernel<true>, grid + sample_blocks, 256, 0, st, a, sa, grid);
+  return launch(sort_scatter_kernel<false>, grid, 256, 0, st, a, sa, grid);
 }
 
 }  // namespace hyperattn

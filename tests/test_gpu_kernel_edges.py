@@ -78,6 +78,41 @@ def test_split_pairs_give_the_same_results(d, n, n_k, b, m, split, whole):
     assert ha.last_device_status() == 0
 
 
+# the permutations are stable sorts of the bucket ids: chunks of 256, 512, 1024, 1280, 1792 and 2048 rows, whole and short ranges of a
+# warp, hash widths of 1 and 8 bits, and rows that are all equal
+SORTED = [("random", 1, 1000, 1000, 64, 7, False, 0), ("random", 20, 3999, 3999, 64, 8, False, 0), ("random", 32, 4096, 1030, 64, 1, False, 0),
+          ("random", 16, 9000, 9000, 64, 7, True, 4096), ("random", 4, 100003, 100003, 64, 7, True, 4096), ("random", 40, 16384, 16384, 64, 8, False, 0),
+          ("equal", 2, 5000, 5000, 128, 7, False, 0), ("equal", 40, 9000, 9000, 64, 7, True, 2500)]
+
+
+@pytest.mark.parametrize("kind,H,n,n_k,d,r,causal,n0", SORTED)
+def test_permutations_are_stable_sorts_of_the_ids(kind, H, n, n_k, d, r, causal, n0):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(11)
+    q, k, v = (torch.randn(1, H, rows, d, generator=gen, device="cuda").bfloat16() for rows in (n, n_k, n_k))
+    if kind == "equal":
+        q, k = (x[:, :, :1].expand_as(x) for x in (q, k))
+    inter = ha.forward(q, k, v, 128, 32, r, causal=causal, n0=n0, seed=5, debug=True)[2]
+    ids = {"q": inter["q_ids"].int(), "k": inter["k_ids"].int()}
+    L = 0
+    while causal and -(-n >> L) > n0:
+        L += 1
+    npad = -(-n >> L) << L
+    for level in range(max(L, 1)):
+        s = npad >> (level + 1)
+        for j in range(1 << level if causal else 1):
+            for side, first, end in (("q", (2 * j + 1) * s, (2 * j + 2) * s), ("k", 2 * j * s, (2 * j + 1) * s)) if causal else (("q", 0, n), ("k", 0, n_k)):
+                rows = min(end, n if side == "q" else n_k) - first
+                if rows <= 0:
+                    continue
+                want = torch.sort(ids[side][:, first:first + rows], dim=1, stable=True).indices.int()
+                at = j * s if causal else 0
+                assert torch.equal(inter["perm_" + side][level, :, at:at + rows], want)
+                if side == "k":
+                    assert torch.equal(torch.gather(inter["rank_k"][level, :, at:at + rows], 1, want.long()),
+                                       torch.arange(rows, dtype=torch.int32, device="cuda").expand(H, rows))
+
+
 # calls whose leaves go first and write dK and dV (from 192 MiB of fp32 accumulators on), against calls of few heads, which add everything
 SPLIT_BACKWARD = [(64, 26, 16384, 4096), (64, 26, 16800, 2100), (64, 40, 10240, 700), (128, 13, 16384, 4096)]
 

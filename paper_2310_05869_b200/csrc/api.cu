@@ -78,17 +78,31 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
     const int bpad = (g.b + 127) / 128 * 128, mpad = (g.m + 127) / 128 * 128;
     if (2 * bpad + mpad > kMaxNodeKeys) return HYPERATTN_UNSUPPORTED_SHAPE;
   }
-  // Chunks of 2048 rows, halved (down to 256) while the hash has fewer than two CTAs for an SM: below that one chunk is the
-  // whole time, above it there are only more CTAs to start.  A call, us, with chunks of 2048 -> as the rule halves them, d = 64 and
-  // 128: 48 chunks 41.3 -> 35.8, 51.7 -> 44.0; 128 61.9 -> 59.5, 80.8 -> 79.2 (halved once only: 58.2, 76.2); 200 85.0 -> 80.5,
-  // 110.7 -> 105.0; 280 105.3 -> 103.3, but 143.8 -> 147.6: at d = 128 256 to 295 chunks would better stay.  Beyond the line, 2048 ->
-  // halved all the same: 400 136.8 -> 140.6, 203.3 -> 205.7; 392 of 4 x 100003 rows 140.4 -> 146.0, 201.1 -> 207.1.
+  // Rows per chunk: 2048, halved (down to 256) while the hash has fewer than two CTAs for an SM and the share of the busiest SM gets cheaper - a CTA
+  // costs as much as 256 rows beside its own, and one alone on an SM as much as two - and evened out over the unit: 2250 rows are two chunks of at
+  // most 1280, not one of 2048 and one of 202.  A call, us, halved below 296 CTAs whatever the share and not evened -> this rule: 32 heads x 4096 rows
+  // (256 CTAs instead of 512) 56.5 -> 55.4, 13 x 9333 58.8 -> 54.7, 21 x 6001 56.6 -> 55.9, 16 causal x 9000 139.1 -> 138.5; d = 128, 32 x 4096 78.9 ->
+  // 74.3, 17 x 8192 82.9 -> 78.4, 35 x 8192 (280 instead of 560) 155.5 -> 150.3, but at d = 64 101.3 -> 102.2; hash of 4 causal x 100003 25.6 -> 22.9.
+  // Beyond two CTAs for an SM: 38 x 8192 112.0 -> 111.4 halved, but 50000 queries x 131072 keys 138.7 -> 141.5 (twice the chunks to scan).
+  auto even = [&](int chunk) {
+    auto side = [&](int unit) { const int k = (unit + chunk - 1) / chunk; return ((unit + k - 1) / k + 255) / 256 * 256; };
+    return side(g.unit) > side(g.unit_k) ? side(g.unit) : side(g.unit_k);
+  };
   auto hash_ctas = [&](int chunk) {
     const long long units = g.npad / g.unit, cpu = (g.unit + chunk - 1) / chunk, cpu_k = (g.unit_k + chunk - 1) / chunk;
     return g.G * units * cpu + g.G * (g.causal ? units : 1) * cpu_k;
   };
-  g.chunk = kSortChunk;
-  while (g.chunk > 256 && hash_ctas(g.chunk) < 2 * kSms) g.chunk /= 2;
+  auto share = [&](int chunk) {
+    const long long per_sm = (hash_ctas(chunk) + kSms - 1) / kSms;
+    return (chunk + 256) * (per_sm < 2 ? 2 : per_sm);
+  };
+  g.chunk = even(kSortChunk);
+  for (int half = kSortChunk / 2; half >= 256 && hash_ctas(g.chunk) < 2 * kSms; half /= 2) {
+    const int chunk = even(half);
+    if (chunk == g.chunk) continue;
+    if (share(chunk) >= share(g.chunk)) break;
+    g.chunk = chunk;
+  }
   g.chunks_per_unit = (g.unit + g.chunk - 1) / g.chunk;
   g.chunks_per_seg = (g.npad / g.unit) * g.chunks_per_unit;
   g.chunks_per_unit_k = (g.unit_k + g.chunk - 1) / g.chunk;

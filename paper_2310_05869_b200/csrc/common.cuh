@@ -62,7 +62,7 @@ struct Geometry {
   int causal;          // 1: causal with L >= 1 levels or a single causal leaf
   int L;               // number of recursion levels with off-diagonal nodes (0: none)
   int leaf;            // rows per exact leaf (n if L == 0)
-  int chunk;           // rows per chunk: kSortChunk, or less where the problem is small (a multiple of 256)
+  int chunk;           // rows per chunk: at most kSortChunk, a multiple of 256
   int unit;            // rows per unit (query side; both sides of a causal call)
   int chunks_per_unit;
   int chunks_per_seg;  // (npad / unit) * chunks_per_unit

@@ -327,10 +327,15 @@ __device__ __forceinline__ int tile_of(const QTile& q, int a) { return a < q.n1 
 // PRECISE: every softmax weight enters the P V product as a pair of bf16 numbers hi + lo (relative error
 // 2^-17 instead of 2^-9): lo is written into the second half of the S buffer and multiplied by V with a
 // second set of products.
-// CAPPED: the sampled part of a sorted node's row sum carries the caps of Alg. 2 (lines 6, 7 and 9).
-template <int D, bool GATHER_LATE, bool PRECISE, bool CAPPED>
+// RULE, of the sampled columns of sorted nodes: kCapped: their part of the row sum carries the caps of Alg. 2 (lines 6, 7 and 9); kWeighted: every
+// column has a weight of its own (columns drawn by value norms).  (One build for
+// both, calls, us, -> two: 4 heads of 50000 queries, 131072 keys, by value norms 138.3 -> 129.0, 16 of 32768, d = 128, 306 -> 295, capped, 8 of 16384
+// 159.8 -> 149.9.)
+enum SampleRule { kUniform, kCapped, kWeighted };
+template <int D, bool GATHER_LATE, bool PRECISE, SampleRule RULE>
 __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ TmaMaps maps, int* status) {
   using C = Cfg<D>;
+  constexpr bool CAPPED = RULE == kCapped, WEIGHTED = RULE == kWeighted;
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr int MW = kMaxNodeKeys / 32;
   int* s_kidx_all = reinterpret_cast<int*>(smem + C::kOffIdx);              // [2][kMaxNodeKeys]
@@ -479,12 +484,12 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       // Alg. 2 with caps (sorted nodes only): the masked row sum (block part) is complete when the first
       // sampled tile starts; from then on every sampled weight enters the row sum as min(weight, (N/m) C_i),
       // C_i = cap_scale m / (N ln N) (masked_i + tau / kappa), while the numerator keeps the weight itself.
-      const bool capped_item = CAPPED && t.mode == 1 && g.m > 0 && a.capped;
+      const bool capped_item = CAPPED && t.mode == 1 && g.m > 0;
       float lblk = 0.f;             // masked row sum in units of 2^m_ref
       bool in_samples = false;
       float capfac = 0.f, lfloor = -INFINITY;     // (N/m) cap_scale m / (N ln N); log2(tau / kappa)
       // weighted sampling (columns drawn by value norms): every sampled column carries its own log2 weight
-      const bool weighted_item = CAPPED && t.mode == 1 && a.sample_wlog != nullptr;
+      const bool weighted_item = WEIGHTED && t.mode == 1;
       const float* s_bias = reinterpret_cast<const float*>(smem + C::kOffBias) + set * kMaxWeightedSamples;
       if (capped_item) {
         capfac = a.cap_scale / (logf((float)t.nk));
@@ -660,11 +665,11 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
           };
           HA_T0(tc2);
           if constexpr (PRECISE) tmem_ld32_wait(rb);     // the lo halves overwrite the second half of the scores
-          if (CAPPED && capped_tile) chunk_exp_capped(ra, 0); else if (CAPPED && weighted_tile) chunk_exp_weighted(ra, 0); else chunk_exp(ra, 0);
+          if (CAPPED && capped_tile) chunk_exp_capped(ra, 0); else if (WEIGHTED && weighted_tile) chunk_exp_weighted(ra, 0); else chunk_exp(ra, 0);
           HA_LACC(a_c2, tc2);
           HA_T0(tc3);
           tmem_ld32_wait(rb);
-          if (CAPPED && capped_tile) chunk_exp_capped(rb, 1); else if (CAPPED && weighted_tile) chunk_exp_weighted(rb, 1); else chunk_exp(rb, 1);
+          if (CAPPED && capped_tile) chunk_exp_capped(rb, 1); else if (WEIGHTED && weighted_tile) chunk_exp_weighted(rb, 1); else chunk_exp(rb, 1);
           HA_LACC(a_c3, tc3);
           float lt0, lt1;
           unpack_f2((CAPPED && capped_tile) ? ltu2 : lt2, lt0, lt1);
@@ -1065,7 +1070,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
           __syncwarp();
           int nfront = 0, nback = 0;                      // unmasked samples placed from the front, masked ones from the back
           float* s_bias = reinterpret_cast<float*>(smem + C::kOffBias) + set * kMaxWeightedSamples;
-          const float* swl = a.sample_wlog ? a.sample_wlog + ((size_t)t.seg * g.nodes + t.node) * g.m : nullptr;
+          const float* swl = WEIGHTED ? a.sample_wlog + ((size_t)t.seg * g.nodes + t.node) * g.m : nullptr;
           float bmax = -INFINITY;
           const unsigned lt_mask = (1u << lane) - 1u;
           for (int c00 = lane; c00 < ncols - nblk; c00 += 32 * UB) {
@@ -1091,7 +1096,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
                 else pos = nblk + g.m - 1 - (nback + __popc(bb & lt_mask));
                 nfront += __popc(bf); nback += __popc(bb);
                 s_kidx[pos] = segrow_k + (valid ? t.k0 + l[u] : 0);
-                if (CAPPED && swl) {                      // weighted sampling: the column's own log2 weight travels with it
+                if (WEIGHTED) {                      // weighted sampling: the column's own log2 weight travels with it
                   const float wl = valid ? swl[c] : 0.f;
                   s_bias[pos - nblk] = wl;
                   if (valid) bmax = fmaxf(bmax, wl);
@@ -1101,7 +1106,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
               }
             }
           }
-          if (CAPPED && swl) {
+          if (WEIGHTED) {
 #pragma unroll
             for (int o = 16; o; o >>= 1) bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
             if (lane == 0) reinterpret_cast<ItemDesc*>(smem + C::kOffDesc + set * C::kDescBytes)->t.bias_max = bmax;
@@ -1362,25 +1367,26 @@ cudaError_t launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st)
   int sms = 0;
   cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
-  const bool variant = a.capped || a.sample_wlog;
   AttnArgs b = a;
   b.split_pairs = split_pairs(a, sms);
   const int items = a.total_pairs + b.split_pairs;
   const int grid = items < sms ? items : sms;                     // persistent: one CTA per SM walks the item list
   b.tail_leaves = a.dense_causal && a.total_pairs == a.n_leaf_pairs ? tail_leaves(a.n_leaf_pairs / a.pairs_per_leaf, a.pairs_per_leaf, sms) : 0;
-  if (variant && (a.precise || (a.capped && a.sample_wlog))) return cudaErrorInvalidValue;
+  if ((a.capped != 0) + (a.sample_wlog != nullptr) + (a.precise != 0) > 1) return cudaErrorInvalidValue;
   const bool late = a.g.d == 128 && !a.direct && !a.part_bf16;
-#define HA_GO(D, LATE, PRECISE, CAPPED) do { e = allow_smem<attn_tc_kernel<D, LATE, PRECISE, CAPPED>>(Cfg<D>::kTotal); \
-    return e != cudaSuccess ? e : launch(attn_tc_kernel<D, LATE, PRECISE, CAPPED>, grid, 384, Cfg<D>::kTotal, st, b, maps, status); } while (0)
+#define HA_GO(D, LATE, PRECISE, RULE) do { e = allow_smem<attn_tc_kernel<D, LATE, PRECISE, RULE>>(Cfg<D>::kTotal); \
+    return e != cudaSuccess ? e : launch(attn_tc_kernel<D, LATE, PRECISE, RULE>, grid, 384, Cfg<D>::kTotal, st, b, maps, status); } while (0)
   if (a.g.d == 64) {
-    if (variant) HA_GO(64, false, false, true);
-    if (a.precise) HA_GO(64, false, true, false);
-    HA_GO(64, false, false, false);
+    if (a.capped) HA_GO(64, false, false, kCapped);
+    if (a.sample_wlog) HA_GO(64, false, false, kWeighted);
+    if (a.precise) HA_GO(64, false, true, kUniform);
+    HA_GO(64, false, false, kUniform);
   }
-  if (variant) { if (late) HA_GO(128, true, false, true); HA_GO(128, false, false, true); }
-  if (a.precise) { if (late) HA_GO(128, true, true, false); HA_GO(128, false, true, false); }
-  if (late) HA_GO(128, true, false, false);
-  HA_GO(128, false, false, false);
+  if (a.capped) { if (late) HA_GO(128, true, false, kCapped); HA_GO(128, false, false, kCapped); }
+  if (a.sample_wlog) { if (late) HA_GO(128, true, false, kWeighted); HA_GO(128, false, false, kWeighted); }
+  if (a.precise) { if (late) HA_GO(128, true, true, kUniform); HA_GO(128, false, true, kUniform); }
+  if (late) HA_GO(128, true, false, kUniform);
+  HA_GO(128, false, false, kUniform);
 #undef HA_GO
 }
 

@@ -5,6 +5,8 @@ namespace hyperattn {
 
 // backward_leaves.cu
 cudaError_t launch_bwd_leaves_d64(const BwdArgs& b, const BwdMaps& maps, unsigned grid, int* status, cudaStream_t st);
+// backward_first.cu
+cudaError_t launch_bwd_first(const BwdArgs& b, const BwdMaps& maps, int results_warps, unsigned grid, int* status, cudaStream_t st);
 
 namespace {
 
@@ -102,7 +104,7 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   b.a = a; b.dout = reinterpret_cast<const __nv_bfloat16*>(dout); b.stat = stat; b.scale = scale; b.sched = sched;
   b.dq = gr.dq; b.dk = gr.dk; b.dv = gr.dv;
   b.dk16 = reinterpret_cast<__nv_bfloat16*>(gr.dk16); b.dv16 = reinterpret_cast<__nv_bfloat16*>(gr.dv16);
-  b.key_slot = gr.key_slot; b.direct = gr.direct; b.kv_first = 0;
+  b.key_slot = gr.key_slot; b.direct = gr.direct;
   b.leaf_ktiles = a.n_leaf_tiles ? (g.leaf + kTileK - 1) / kTileK : 0;
   b.block_ktiles = (g.b + kTileK - 1) / kTileK;
   b.smp_ktiles = (g.m + kTileK - 1) / kTileK;
@@ -146,10 +148,10 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   if (!gr.direct && (!encode_acc_map(&maps.dk, gr.dk, rows, g.d) || !encode_acc_map(&maps.dv, gr.dv, rows, g.d))) return cudaErrorInvalidValue;
   auto go = [&](auto dim, auto with_boxes, auto results_warps, unsigned grid) {
     constexpr int D = decltype(dim)::value, RW = decltype(results_warps)::value;
-    constexpr bool BOXES = decltype(with_boxes)::value;
+    constexpr BwdOut OUT = decltype(with_boxes)::value ? kBoxes : kRows;
     using C = Cfg<D, RW>;
-    const cudaError_t allowed = allow_smem<bwd_kernel<D, BOXES, RW>>(C::kTotal);
-    return allowed != cudaSuccess ? allowed : launch(bwd_kernel<D, BOXES, RW>, grid, C::kThreads, C::kTotal, st, b, maps, status);
+    const cudaError_t allowed = allow_smem<bwd_kernel<D, OUT, RW>>(C::kTotal);
+    return allowed != cudaSuccess ? allowed : launch(bwd_kernel<D, OUT, RW>, grid, C::kThreads, C::kTotal, st, b, maps, status);
   };
   using std::integral_constant;
   using std::bool_constant;
@@ -164,10 +166,10 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   };
   cudaError_t e;
   if (split) {
-    b.total_items = b.n_leaf_items; b.kv_first = 1;
-    e = run(backward_build(g, true, false));
+    b.total_items = b.n_leaf_items;
+    e = launch_bwd_first(b, maps, backward_build(g, true, false).results_warps, b.total_items < sms ? b.total_items : sms, status, st);
     if (e != cudaSuccess) return e;
-    b.total_items = (int)items - b.n_leaf_items; b.kv_first = 0; b.sched = sched + 1; b.a.tail_leaves = 0;
+    b.total_items = (int)items - b.n_leaf_items; b.sched = sched + 1; b.a.tail_leaves = 0;
     for (int l = g.levels; l >= 0; --l) b.level_item_start[l] -= b.n_leaf_items;
     b.n_leaf_items = 0;
     e = run(backward_build(g, false, true));

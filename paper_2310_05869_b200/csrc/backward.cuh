@@ -62,7 +62,6 @@ struct BwdArgs {
   __nv_bfloat16 *dk16, *dv16;  // direct: dK and dV of the keys without samples
   const int32_t* key_slot;     // direct: [G, n] the sample that stands for a key, -1: none (null: none for any)
   int direct;
-  int kv_first;                // (kBoxes) nothing has been added to dK and dV yet and every row is written once: the accumulators need not be cleared
   float scale;
   int* sched;                  // work counter of the launch, zero at launch
   // items: the key tiles of the leaves, then level by level those of the nodes
@@ -244,15 +243,19 @@ __global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__
   if (row < rows && c % LPR == 0) stat[row] = make_float2(-lse[row] * 1.4426950408889634f, -acc);
 }
 
-// BOXES: whole tiles of consecutive rows (leaves of the recursion, nodes that are not sorted) leave as boxes; without, all rows by reductions
+// How results leave.  kRows: every row by reductions.  kBoxes: whole tiles of consecutive rows (leaves of the recursion, nodes that are not sorted) as boxes.
+// kFirst: as kBoxes, but dK and dV are written, not added: every key row has one item and nothing has been added to it yet.  (A build of its own: as a switch
+// in kBoxes it made calls that do not use it 1 to 2 % slower, 11 causal heads of 5512 rows 149.2 -> 152.0 us, 128 leaves 1014 -> 1027.)
+enum BwdOut { kRows, kBoxes, kFirst };
 // RW: results warps.  With eight the block has 21 warps, six of them on one quarter of the SM, which leaves 80 registers a thread; with four it has 17
 // and 96.  Whole tiles of consecutive rows need no more than four while they follow one another - a box goes out with a few instructions - and the P
 // warps gain from the registers; scattered rows, and dK and dV of items of few steps, keep eight busy.  (Which build a call takes: backward_build()
 // in backward.cu, with figures.  d = 128 always has eight: 64 leaves of 4096 rows 838 us, with four 998.)
-template <int D, bool BOXES, int RW>
+template <int D, BwdOut OUT, int RW>
 __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __grid_constant__ BwdArgs b, const __grid_constant__ BwdMaps maps,
                                                                   int* status) {
   using C = Cfg<D, RW>;
+  constexpr bool BOXES = OUT != kRows;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
@@ -499,7 +502,7 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
           for (int q = 0; q < 4; ++q) {
             const int gr = __shfl_sync(0xffffffffu, grow, 4 * (q0 + q) + (lane >> 3));
             float4* dst = reinterpret_cast<float4*>(base + (size_t)gr * D + NC * r_ + 32 * p + 4 * c);
-            if (BOXES && decltype(direct)::value && gr >= 0 && b.kv_first) *dst = v[q];
+            if (OUT == kFirst && decltype(direct)::value) { if (gr >= 0) *dst = v[q]; }
             else if (gr >= 0) atomicAdd(dst, v[q]);
             else if (decltype(direct)::value && gr != kNoRow)
               *reinterpret_cast<uint2*>(base16 + (size_t)~gr * D + NC * r_ + 32 * p + 4 * c) =
@@ -535,7 +538,7 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
         fence_async_smem();
         __syncwarp();
         if (lane == 0) {
-          if (decltype(first)::value && b.kv_first) tma_put_tile(map, NC * r_ + 32 * p, y, stage);
+          if (OUT == kFirst && decltype(first)::value) tma_put_tile(map, NC * r_ + 32 * p, y, stage);
           else tma_add_tile(map, NC * r_ + 32 * p, y, stage);
         }
       }

@@ -8,8 +8,8 @@ namespace hyperattn {
 
 cudaError_t launch_bwd_leaves_d64(const BwdArgs& b, const BwdMaps& maps, unsigned grid, int* status, cudaStream_t st) {
   using C = Cfg<64, 4>;
-  const cudaError_t e = allow_smem<bwd_kernel<64, true, 4>>(C::kTotal);
-  return e != cudaSuccess ? e : launch(bwd_kernel<64, true, 4>, grid, C::kThreads, C::kTotal, st, b, maps, status);
+  const cudaError_t e = allow_smem<bwd_kernel<64, kBoxes, 4>>(C::kTotal);
+  return e != cudaSuccess ? e : launch(bwd_kernel<64, kBoxes, 4>, grid, C::kThreads, C::kTotal, st, b, maps, status);
 }
 
 }  // namespace hyperattn

@@ -331,8 +331,11 @@ __device__ __forceinline__ int tile_of(const QTile& q, int a) { return a < q.n1 
 // column has a weight of its own (columns drawn by value norms).  (One build for
 // both, calls, us, -> two: 4 heads of 50000 queries, 131072 keys, by value norms 138.3 -> 129.0, 16 of 32768, d = 128, 306 -> 295, capped, 8 of 16384
 // 159.8 -> 149.9.)
+// NODE: a call without recursion: all items are tiles of one sorted node and their results final.  What a build does not need is not in the way of
+// the softmax warps: calls, us, in a build for everything -> this one: 32 heads of 4096 rows 55.2 -> 52.9, 12 of 4096 33.6 -> 31.9, 32 of 16384 173.7 ->
+// 167.5, 32 of 131072 1289 -> 1229-1253; d = 128, 32 of 32768 516 -> 497-503; by value norms, 50000 queries and 131072 keys, 4 heads 129.2 -> 121.8.
 enum SampleRule { kUniform, kCapped, kWeighted };
-template <int D, bool GATHER_LATE, bool PRECISE, SampleRule RULE>
+template <int D, bool GATHER_LATE, bool PRECISE, SampleRule RULE, bool NODE>
 __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ TmaMaps maps, int* status) {
   using C = Cfg<D>;
   constexpr bool CAPPED = RULE == kCapped, WEIGHTED = RULE == kWeighted;
@@ -434,7 +437,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       if (nit >= 1) good = wait_fast<20>(bar_qfree, (nit - 1) & 1, s_abort, status);
       if (!good) return false;
       const QTile &qa = de.qa, &qb = de.qb;
-      if (t.mode == 1) {
+      if (NODE || t.mode == 1) {
         constexpr int CPR = D / 8;
         constexpr int RS = 256 / CPR;                       // rows covered by the 256 threads per step
         const int cq = tid % CPR, rq0 = tid / CPR;
@@ -474,22 +477,22 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       if (t.mode < 0) break;                              // the work list is exhausted
       const QTile q = i ? de.qb : de.qa;
       const int total = q.n1 + q.n2;
-      const float wlog = (t.mode == 1 && g.m > 0) ? log2f((float)t.nk / (float)g.m) : 0.f;   // log2(N/m): weight of a sampled column
+      const float wlog = ((NODE || t.mode == 1) && g.m > 0) ? log2f((float)t.nk / (float)g.m) : 0.f;   // log2(N/m): weight of a sampled column
       // key tiles of this item with masked columns for this query tile, one bit per tile (an item has at most 32)
       unsigned tile_masked = 0;
-      if (t.mode == 1) tile_masked = __ballot_sync(0xffffffffu, lane < t.ntiles && (s_mask[2 * lane] | s_mask[2 * lane + 1]) != 0);
+      if (NODE || t.mode == 1) tile_masked = __ballot_sync(0xffffffffu, lane < t.ntiles && (s_mask[2 * lane] | s_mask[2 * lane + 1]) != 0);
       float m_ref = -INFINITY;
       uint64_t l01 = 0;             // l: unrounded row sum (two partial sums, packed)
       float lra = 0.f, lrb = 0.f;   // lr: sum of the bf16 weights (two partial sums; the mixed-precision add takes the bf16 halves as they are)
       // Alg. 2 with caps (sorted nodes only): the masked row sum (block part) is complete when the first
       // sampled tile starts; from then on every sampled weight enters the row sum as min(weight, (N/m) C_i),
       // C_i = cap_scale m / (N ln N) (masked_i + tau / kappa), while the numerator keeps the weight itself.
-      const bool capped_item = CAPPED && t.mode == 1 && g.m > 0;
+      const bool capped_item = CAPPED && (NODE || t.mode == 1) && g.m > 0;
       float lblk = 0.f;             // masked row sum in units of 2^m_ref
       bool in_samples = false;
       float capfac = 0.f, lfloor = -INFINITY;     // (N/m) cap_scale m / (N ln N); log2(tau / kappa)
       // weighted sampling (columns drawn by value norms): every sampled column carries its own log2 weight
-      const bool weighted_item = WEIGHTED && t.mode == 1;
+      const bool weighted_item = WEIGHTED && (NODE || t.mode == 1);
       const float* s_bias = reinterpret_cast<const float*>(smem + C::kOffBias) + set * kMaxWeightedSamples;
       if (capped_item) {
         capfac = a.cap_scale / (logf((float)t.nk));
@@ -512,8 +515,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
         const bool table = (tile_masked >> j) & 1u;
         // (weighted sampling: the tile's columns have weights of their own; the largest one stands in where one number is needed)
         const bool weighted_tile = weighted_item && j >= t.nbA + t.nbB;
-        const float ubias = (t.mode == 1 && j >= t.nbA + t.nbB) ? (weighted_tile ? t.bias_max : wlog) : 0.f;
-        const bool dense_mask = t.mode != 1 && ((j * TK + TK > t.nk) || (t.causal && j * TK + TK - 1 > q.row0));
+        const float ubias = ((NODE || t.mode == 1) && j >= t.nbA + t.nbB) ? (weighted_tile ? t.bias_max : wlog) : 0.f;
+        const bool dense_mask = !(NODE || t.mode == 1) && ((j * TK + TK > t.nk) || (t.causal && j * TK + TK - 1 > q.row0));
         // The 64 scores of this row are read from TMEM once; then (1) the row maximum, (2)
         // exponentials, row sums and the bf16 P written over the first half of the S buffer.
         // The reference maximum only moves when the tile exceeds it by more than 2^32, and then
@@ -731,8 +734,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
           constexpr int RB = C::kStageRow;
           constexpr int LPR = RB / 16, RPI = 32 / LPR, NI = 32 / RPI;
           constexpr int NP = D / 16;
-          const bool f32o = t.partial ? !a.part_bf16 : a.out_fp32;
-          char* obase = reinterpret_cast<char*>(t.partial ? a.part_o : a.out);
+          const bool f32o = (!NODE && t.partial) ? !a.part_bf16 : a.out_fp32;
+          char* obase = reinterpret_cast<char*>((!NODE && t.partial) ? a.part_o : a.out);
           const long long myoff = qr >= 0 ? (long long)(orow * (size_t)(D * (f32o ? 4 : 2))) : -1;
           long long roff[NI];
 #pragma unroll
@@ -743,7 +746,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
           const int crow = lane / LPR, cc = lane % LPR;
           const int lg_pps = f32o ? (RB == 128 ? 1 : 0) : (RB == 128 ? 2 : 1);   // log2(pieces per staging step)
           if (qr >= 0) {
-            if (t.partial) a.part_lse[orow] = lse;
+            if (!NODE && t.partial) a.part_lse[orow] = lse;
             else a.lse[orow] = lse;
           }
           uint32_t r[16];
@@ -1031,7 +1034,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       // the first one is used; the warp covers 32 consecutive columns per step, so one ballot
       // yields a whole word of the mask tables.  Padding columns point at a valid row (they are
       // masked, and the streamer puts zeros in the place of its values) and are masked for both tiles.
-      if (t.mode == 1) {
+      if (NODE || t.mode == 1) {
         constexpr int UB = 8;
         const int bcols = t.nbA * TK;
         const int nblk = (t.nbA + t.nbB) * TK;            // columns of the block part (multiple of 64)
@@ -1123,7 +1126,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
         for (int k = 0; k < 4; ++k) {
           const int r = 4 * lane + k;
           qr[i][k] = -1;
-          if (q.valid && r < q.nq) qr[i][k] = t.mode == 1 ? t.qnode0 + a.perm_q[t.slice + q.spos0 + r] : q.q0 + r;
+          if (q.valid && r < q.nq) qr[i][k] = (NODE || t.mode == 1) ? t.qnode0 + a.perm_q[t.slice + q.spos0 + r] : q.q0 + r;
         }
       }
 #pragma unroll
@@ -1134,7 +1137,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       if (lane == 0) HA_TACC(10, ttab);
       // Sorted query rows are read once in the whole forward pass, so they come from HBM: ask for
       // them now (the softmax threads gather them a whole item later) so that they are found in L2.
-      if (t.mode == 1) {
+      if (NODE || t.mode == 1) {
         const char* qbase = reinterpret_cast<const char*>(a.q) + (size_t)segrow * (D * 2);
 #pragma unroll
         for (int i = 0; i < 2; ++i)
@@ -1154,7 +1157,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       }
       if (lane == 0) HA_TACC(27, tqf);
       HA_T0(tqi);
-      if (t.mode == 0) {
+      if (!NODE && t.mode == 0) {
         // consecutive rows: one box per 64 columns and tile (rows past the tile's end are other
         // rows of the tensor or zeros: their results are never stored)
         if (lane == 0) {
@@ -1208,18 +1211,18 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       const int lenA = de.lenA, lenB = de.lenB;
       const int segrow = t.seg * g.nk;                      // (keys)
       // does any of the item's key tiles have columns that do not exist?
-      const bool shorts = t.mode == 0 ? t.nk % TK != 0 : (lenA % TK | lenB % TK | g.m % TK) != 0;
+      const bool shorts = (!NODE && t.mode == 0) ? t.nk % TK != 0 : (lenA % TK | lenB % TK | g.m % TK) != 0;
       for (int j = 0; j < t.ntiles && ok; ++j) {
         const int gj = gbase + j;
         const int s = gj % C::NS;
         const int use = gj / C::NS;
         int4 rows[QUADS];
-        if (t.mode == 1) {
+        if (NODE || t.mode == 1) {
 #pragma unroll
           for (int k = 0; k < QUADS; ++k) rows[k] = *reinterpret_cast<const int4*>(s_kidx + j * TK + 4 * (rq + k * R));
         }
         auto fill = [&](uint32_t stage, const CUtensorMap* map, const char* src, uint32_t bar) {
-          if (t.mode == 0) {
+          if (!NODE && t.mode == 0) {
             // (rows past the end of the key range are masked by the softmax warps)
             if (lane == 0) {
               mbar_expect_tx(bar, C::kTile);
@@ -1266,11 +1269,11 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
         }
 #endif
         const int have = !shorts ? TK                     // columns of the tile that exist
-                         : t.mode == 0 ? t.nk - j * TK
+                         : (!NODE && t.mode == 0) ? t.nk - j * TK
                          : j < t.nbA ? lenA - j * TK
                          : j < t.nbA + t.nbB ? lenB - (j - t.nbA) * TK : g.m - (j - t.nbA - t.nbB) * TK;
         if (have >= TK) fill(ubase + C::kOffV + s * C::kTile, &maps.v, vsrc, bar_vfull(s));
-        else fill_short<D>(ubase + C::kOffV + s * C::kTile, reinterpret_cast<const char*>(a.v), t.mode == 1 ? s_kidx + j * TK : nullptr,
+        else fill_short<D>(ubase + C::kOffV + s * C::kTile, reinterpret_cast<const char*>(a.v), (NODE || t.mode == 1) ? s_kidx + j * TK : nullptr,
                            segrow + t.k0 + j * TK, have, bar_vfull(s));
         v_armed = gj + 1;
         if (lane == 0) HA_TACC(1, tgv);
@@ -1373,9 +1376,11 @@ cudaError_t launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st)
   const int grid = items < sms ? items : sms;                     // persistent: one CTA per SM walks the item list
   b.tail_leaves = a.dense_causal && a.total_pairs == a.n_leaf_pairs ? tail_leaves(a.n_leaf_pairs / a.pairs_per_leaf, a.pairs_per_leaf, sms) : 0;
   if ((a.capped != 0) + (a.sample_wlog != nullptr) + (a.precise != 0) > 1) return cudaErrorInvalidValue;
+  const bool node = a.n_leaf_pairs == 0 && a.g.levels == 1 && a.level_sorted[0] && a.direct;
   const bool late = a.g.d == 128 && !a.direct && !a.part_bf16;
-#define HA_GO(D, LATE, PRECISE, RULE) do { e = allow_smem<attn_tc_kernel<D, LATE, PRECISE, RULE>>(Cfg<D>::kTotal); \
-    return e != cudaSuccess ? e : launch(attn_tc_kernel<D, LATE, PRECISE, RULE>, grid, 384, Cfg<D>::kTotal, st, b, maps, status); } while (0)
+#define HA_RUN(D, LATE, PRECISE, RULE, NODE) do { e = allow_smem<attn_tc_kernel<D, LATE, PRECISE, RULE, NODE>>(Cfg<D>::kTotal); \
+    return e != cudaSuccess ? e : launch(attn_tc_kernel<D, LATE, PRECISE, RULE, NODE>, grid, 384, Cfg<D>::kTotal, st, b, maps, status); } while (0)
+#define HA_GO(D, LATE, PRECISE, RULE) do { if (!LATE && node) HA_RUN(D, false, PRECISE, RULE, true); HA_RUN(D, LATE, PRECISE, RULE, false); } while (0)
   if (a.g.d == 64) {
     if (a.capped) HA_GO(64, false, false, kCapped);
     if (a.sample_wlog) HA_GO(64, false, false, kWeighted);
@@ -1388,6 +1393,7 @@ cudaError_t launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st)
   if (late) HA_GO(128, true, false, kUniform);
   HA_GO(128, false, false, kUniform);
 #undef HA_GO
+#undef HA_RUN
 }
 
 }  // namespace hyperattn

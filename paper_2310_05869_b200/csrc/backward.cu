@@ -5,6 +5,8 @@ namespace hyperattn {
 
 // backward_leaves.cu
 cudaError_t launch_bwd_leaves_d64(const BwdArgs& b, const BwdMaps& maps, unsigned grid, int* status, cudaStream_t st);
+// backward_nodes.cu
+cudaError_t launch_bwd_nodes(const BwdArgs& b, const BwdMaps& maps, unsigned grid, int* status, cudaStream_t st);
 // backward_first.cu
 cudaError_t launch_bwd_first(const BwdArgs& b, const BwdMaps& maps, int results_warps, unsigned grid, int* status, cudaStream_t st);
 
@@ -158,8 +160,11 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
   using d64 = integral_constant<int, 64>;
   using d128 = integral_constant<int, 128>;
   using eight = integral_constant<int, 8>;
+  bool nodes_alone = (split || b.n_leaf_items == 0) && g.levels > 0;
+  for (int l = 0; l < g.levels; ++l) nodes_alone = nodes_alone && a.level_sorted[l];
   auto run = [&](BwdBuild build) {
     const unsigned grid = b.total_items < sms ? (unsigned)b.total_items : (unsigned)sms;     // persistent: one CTA per SM
+    if (nodes_alone) return launch_bwd_nodes(b, maps, grid, status, st);
     if (build.results_warps == 4) return launch_bwd_leaves_d64(b, maps, grid, status, st);
     if (g.d == 64) return build.boxes ? go(d64{}, bool_constant<true>{}, eight{}, grid) : go(d64{}, bool_constant<false>{}, eight{}, grid);
     return build.boxes ? go(d128{}, bool_constant<true>{}, eight{}, grid) : go(d128{}, bool_constant<false>{}, eight{}, grid);

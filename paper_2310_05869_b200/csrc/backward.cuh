@@ -246,7 +246,10 @@ __global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__
 // How results leave.  kRows: every row by reductions.  kBoxes: whole tiles of consecutive rows (leaves of the recursion, nodes that are not sorted) as boxes.
 // kFirst: as kBoxes, but dK and dV are written, not added: every key row has one item and nothing has been added to it yet.  (A build of its own: as a switch
 // in kBoxes it made calls that do not use it 1 to 2 % slower, 11 causal heads of 5512 rows 149.2 -> 152.0 us, 128 leaves 1014 -> 1027.)
-enum BwdOut { kRows, kBoxes, kFirst };
+// kNodes: as kRows, where all items are tiles of sorted nodes.  (The pass, us, kRows -> kNodes, in the case of recursion also kFirst knowing that it has
+// leaves alone: 12 heads of 4096 rows 59.7 -> 58.6, 10 of 20000 194.5 -> 190.4, 32 of 65536 1797 -> 1766, 32 causal of 131072 16199 -> 15871; d =
+// 128, 32 of 32768 1665 -> 1657, 8 causal of 32768 1620 -> 1584.)
+enum BwdOut { kRows, kBoxes, kFirst, kNodes };
 // RW: results warps.  With eight the block has 21 warps, six of them on one quarter of the SM, which leaves 80 registers a thread; with four it has 17
 // and 96.  Whole tiles of consecutive rows need no more than four while they follow one another - a box goes out with a few instructions - and the P
 // warps gain from the registers; scattered rows, and dK and dV of items of few steps, keep eight busy.  (Which build a call takes: backward_build()
@@ -255,7 +258,9 @@ template <int D, BwdOut OUT, int RW>
 __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __grid_constant__ BwdArgs b, const __grid_constant__ BwdMaps maps,
                                                                   int* status) {
   using C = Cfg<D, RW>;
-  constexpr bool BOXES = OUT != kRows;
+  constexpr bool BOXES = OUT == kBoxes || OUT == kFirst;
+  // (kFirst: leaves alone)
+  auto consecutive = [](const BwdItem& t) { return OUT == kFirst || (OUT != kNodes && t.kind == 0); };
   extern __shared__ __align__(1024) uint8_t smem[];
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
@@ -315,13 +320,13 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
   auto wait_desc = [&](int it) { return wait_fast<1>(bar_dfull(it), (it / kDescs) & 1, s_abort, status); };
   // key row (segment-relative) of key r of an item's tile, r < nkeys
   auto key_row = [&](const BwdItem& t, int r) -> int {
-    if (t.kind == 0) return t.k0 + r;
+    if (consecutive(t)) return t.k0 + r;
     return t.k0 + __ldg((t.kind == 1 ? a.perm_k : a.samples) + t.kidx + r);
   };
   // query row (segment-relative) of row r of a step, -1: does not exist
   auto query_row = [&](const BwdItem& t, const StepRows& sr, int r) -> int {
     if (r >= sr.nq) return -1;
-    return t.kind == 0 ? sr.first + r : t.q0 + __ldg(a.perm_q + t.slice + sr.first + r);
+    return consecutive(t) ? sr.first + r : t.q0 + __ldg(a.perm_q + t.slice + sr.first + r);
   };
 
   bool ok = true;
@@ -345,7 +350,7 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
       if (t.kind < 0) break;
       const int kind = t.kind, steps = t.steps, causal = t.causal, nkeys = t.nkeys;
       int kblk[4] = {-2, -2, -2, -2};                   // sampled keys: the sorted blocks the thread's keys lie in (their entries there are masked)
-      if (kind == 2) {
+      if (OUT != kFirst && kind == 2) {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
           if (frow + 8 * j < nkeys) kblk[j] = __ldg(a.smp_blk + t.kidx + frow + 8 * j);
@@ -353,8 +358,8 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
 #pragma unroll 1
       for (int s = 0; s < steps; ++s, ++g) {
         // entries that do not count: keys that do not exist, sampled keys of the query tile's own block, above the diagonal
-        const int own = kind == 2 ? (t.tn0 + s) / a.tiles_per_block : -1;
-        const bool diag = causal && s == 0;
+        const int own = OUT != kFirst && kind == 2 ? (t.tn0 + s) / a.tiles_per_block : -1;
+        const bool diag = OUT != kNodes && causal && s == 0;
         int first[4];                                   // rows of the thread: columns below it do not count
         bool masked = diag;
 #pragma unroll
@@ -555,7 +560,7 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
       if (row < t.nkeys) {
         kr = seg_row0 + key_row(t, row);
         if (b.direct) {                                 // the key's tile has all of its gradient, or the sample's row collects it
-          const int slot = t.kind != 0 && b.key_slot ? __ldg(b.key_slot + kr) : -1;
+          const int slot = !consecutive(t) && b.key_slot ? __ldg(b.key_slot + kr) : -1;
           kr = slot >= 0 ? t.seg * g_.m + slot : ~kr;
         }
       }
@@ -563,7 +568,7 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
 #pragma unroll 1
       for (int s = 0; s < steps; ++s, ++g) {
         const StepRows sr = step_rows(b, t, s);
-        const bool box = BOXES && t.kind == 0 && sr.nq == kTileQ;
+        const bool box = BOXES && consecutive(t) && sr.nq == kTileQ;
         const int qr = query_row(t, sr, row);
         ok = __all_sync(0xffffffffu, wait_fast<7>(bar_dq(g), (g >> 1) & 1, s_abort, status));
         if (!ok) break;
@@ -572,19 +577,19 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
           out_boxes(std::false_type{}, lane_addr + C::kColDQ, b.scale, &maps.dq, seg_row0 + sr.first + (row & ~31), bar_dqfree);
           continue;
         }
-        if (BOXES && t.kind == 0) staged_read();
+        if (BOXES && consecutive(t)) staged_read();
         out_rows(std::false_type{}, lane_addr + C::kColDQ, b.scale, b.dq, nullptr, qr >= 0 ? seg_row0 + qr : kNoRow, bar_dqfree);
       }
       if (!ok) break;
       ok = __all_sync(0xffffffffu, wait_fast<8>(bar_acc, it & 1, s_abort, status));
       if (!ok) break;
       tc_fence_after();
-      if (BOXES && t.kind == 0 && t.nkeys == kTileK && !b.direct) {
+      if (BOXES && consecutive(t) && t.nkeys == kTileK && !b.direct) {
         const int y = seg_row0 + t.k0 + (row & ~31);
         out_boxes(std::true_type{}, lane_addr + C::kColDV, 1.f, &maps.dv, y, 0);
         out_boxes(std::true_type{}, lane_addr + C::kColDK, b.scale, &maps.dk, y, bar_accfree);
       } else {
-        if (BOXES && t.kind == 0) staged_read();
+        if (BOXES && consecutive(t)) staged_read();
         out_rows(std::true_type{}, lane_addr + C::kColDV, 1.f, b.dv, b.dv16, kr, 0);
         out_rows(std::true_type{}, lane_addr + C::kColDK, b.scale, b.dk, b.dk16, kr, bar_accfree);
       }
@@ -786,11 +791,11 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
         const BwdItem& t = desc_of(pit);
         const StepRows sr = step_rows(b, t, ps);
         d.base = t.seg * g_.n + t.q0; d.nq = sr.nq; d.wlog = t.wlog;
-        d.y = t.kind == 0 && sr.nq == 128 ? t.seg * g_.n + sr.first : -1;
+        d.y = consecutive(t) && sr.nq == 128 ? t.seg * g_.n + sr.first : -1;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int r = lane + 32 * u;
-          d.rel[u] = r < sr.nq ? (t.kind == 0 ? sr.first - t.q0 + r : __ldg(a.perm_q + t.slice + sr.first + r)) : 0;
+          d.rel[u] = r < sr.nq ? (consecutive(t) ? sr.first - t.q0 + r : __ldg(a.perm_q + t.slice + sr.first + r)) : 0;
         }
         ++have;
         if (++ps == t.steps) {
@@ -833,7 +838,7 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
           for (int u = 0; u < 4; ++u) { st[lane + 32 * u] = n0[u].x + s0.wlog; st[128 + lane + 32 * u] = n0[u].y; }
           mbar_arrive(bar);
         }
-        if (s0.y >= 0) boxes(dst, 128, is_q ? &maps.q : &maps.dout, s0.y, bar);
+        if (OUT != kNodes && s0.y >= 0) boxes(dst, 128, is_q ? &maps.q : &maps.dout, s0.y, bar);
         else {
           int v[4];
 #pragma unroll
@@ -875,7 +880,7 @@ __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __gr
         if (t.kind < 0) break;
         const uint32_t dk = ubase + C::kOffK + (it % C::NKV) * C::kTile, dv = ubase + C::kOffV + (it % C::NKV) * C::kTile;
         const int seg_row0 = t.seg * g_.n;
-        const bool box = t.kind == 0 && t.nkeys == 128;
+        const bool box = consecutive(t) && t.nkeys == 128;
         int v[4] = {0, 0, 0, 0};
         if (!box) {
 #pragma unroll

@@ -409,7 +409,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     }
   }
 
-  // ---- attention tiles: one launch over leaves and all recursion levels -------------------
+  // ---- attention tiles: leaves and all recursion levels, one launch or two -------------------
   AttnArgs a;
   std::memset(&a, 0, sizeof(a));
   a.q = q16; a.k = k16; a.v = v16; a.g = g;
@@ -483,12 +483,12 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     if (dbg && dbg->log2_tau) HA_CHECK(cudaMemcpyAsync(dbg->log2_tau, ws.ltau, (size_t)g.G * g.nodes * 4, cudaMemcpyDeviceToDevice, st));
   }
   {
-    StageScope sc(st, HYPERATTN_STAGE_ATTENTION, 1);
+    StageScope sc(st, HYPERATTN_STAGE_ATTENTION, is_fp32 || !attention_in_two(a) ? 1 : 2);
     // bf16 inputs: tcgen05 path; fp32 inputs: split-bf16 logits on the warp-level MMA path
     if (is_fp32) HA_CHECK(launch_attention_mma(a, st));
     else {
       a.sched = ws.sched;
-      if (!g.sorted) HA_CHECK(cudaMemsetAsync(a.sched, 0, 4, st));       // (else the sort has zeroed it)
+      if (!g.sorted) HA_CHECK(cudaMemsetAsync(a.sched, 0, 8, st));       // (else the sort has zeroed it)
       HA_CHECK(launch_attention_tc(a, ws.status, st));
     }
   }

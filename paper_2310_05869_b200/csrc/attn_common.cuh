@@ -10,7 +10,7 @@
 //          as an additive log2(N/m) on the logit, or minus infinity when the sampled key
 //          lies in block beta itself (the factor 1 - M^H).
 // All tiles of all recursion levels and all leaves of one forward call form one flat list
-// so that a single launch covers them; heavy (leaf) tiles come first.
+// so that one launch covers them, or two a part of it each; heavy (leaf) tiles come first.
 #pragma once
 #include "common.cuh"
 
@@ -72,8 +72,9 @@ struct AttnArgs {
   int level_paired[kMaxLevels];      // 1: CTAs of this level own two query tiles, 0: one
   int total_pairs;
   int tail_leaves;                   // last leaves that are handed out rank by rank (tail_leaves(), set by the launchers)
+  int skip_at, skip;                 // a launch of a part of the list: the pairs from skip_at on are those skip further on (set by the launcher)
   int split_pairs;                   // last pairs of the list whose query tiles are items of their own (split_pairs(), set by the launcher)
-  int* sched;                        // work counter of the launch (global memory, zero at launch): next item to hand out
+  int* sched;                        // work counters of up to two launches (global memory, zero at launch): next item to hand out
 };
 
 // Items of leaves are handed out leaf by leaf, the heaviest first; where nothing follows them, one leaf at a time the last heavy item would start
@@ -106,6 +107,9 @@ inline int split_pairs(const AttnArgs& a, int sms) {
   const int rest = a.total_pairs % sms;
   return 2 * rest <= sms ? rest : 0;
 }
+
+// sorted nodes, and leaves with nodes that are not sorted, in launches of their own (attn_tc.cu)
+bool attention_in_two(const AttnArgs& a);
 
 struct TileDesc {
   int mode;            // 0 dense, 1 node

@@ -331,14 +331,18 @@ __device__ __forceinline__ int tile_of(const QTile& q, int a) { return a < q.n1 
 // column has a weight of its own (columns drawn by value norms).  (One build for
 // both, calls, us, -> two: 4 heads of 50000 queries, 131072 keys, by value norms 138.3 -> 129.0, 16 of 32768, d = 128, 306 -> 295, capped, 8 of 16384
 // 159.8 -> 149.9.)
-// NODE: a call without recursion: all items are tiles of one sorted node and their results final.  What a build does not need is not in the way of
-// the softmax warps: calls, us, in a build for everything -> this one: 32 heads of 4096 rows 55.2 -> 52.9, 12 of 4096 33.6 -> 31.9, 32 of 16384 173.7 ->
-// 167.5, 32 of 131072 1289 -> 1229-1253; d = 128, 32 of 32768 516 -> 497-503; by value norms, 50000 queries and 131072 keys, 4 heads 129.2 -> 121.8.
+// KIND, what the items of the launch are: kFinalNodes: tiles of one sorted node, a call without recursion; kPartialNodes: of sorted nodes of a recursion;
+// kDenseItems: leaves, and nodes that are not sorted; kAnyItems: all of these.  What a build does not need is not in the way of the softmax warps: calls,
+// us, in a build for everything -> in its own: 32 heads of 4096 rows 55.2 -> 52.9, 12 of 4096 33.6 -> 31.9, 32 of 16384 173.7 -> 167.5, 32 of 131072
+// 1289 -> 1229-1253; d = 128, 32 of 32768 516 -> 497-503; by value norms, 50000 queries and 131072 keys, 4 heads 129.2 -> 121.8; leaves alone, 128 of
+// 4096 422 -> 413, d = 128, 64 of 4096 313 -> 302.
 enum SampleRule { kUniform, kCapped, kWeighted };
-template <int D, bool GATHER_LATE, bool PRECISE, SampleRule RULE, bool NODE>
+enum ItemKind { kAnyItems, kFinalNodes, kPartialNodes, kDenseItems };
+template <int D, bool GATHER_LATE, bool PRECISE, SampleRule RULE, ItemKind KIND>
 __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ TmaMaps maps, int* status) {
   using C = Cfg<D>;
   constexpr bool CAPPED = RULE == kCapped, WEIGHTED = RULE == kWeighted;
+  constexpr bool NODE = KIND == kFinalNodes || KIND == kPartialNodes, DENSE = KIND == kDenseItems;
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr int MW = kMaxNodeKeys / 32;
   int* s_kidx_all = reinterpret_cast<int*>(smem + C::kOffIdx);              // [2][kMaxNodeKeys]
@@ -362,6 +366,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
   auto bar_kempty = [&](int i, int s) { return bar0 + 168 + 8 * ((2 + i) * C::NS + s); };     // released by issuer i
   auto bar_vempty = [&](int i, int s) { return bar0 + 168 + 8 * ((4 + i) * C::NS + s); };
 
+  auto is_node = [](const PairDesc& t) { return NODE || (!DENSE && t.mode == 1); };
+  auto is_partial = [](const PairDesc& t) { return KIND == kPartialNodes || (KIND != kFinalNodes && t.partial); };
   const Geometry& g = a.g;
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);       // (known to be the same for the whole warp)
@@ -437,7 +443,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       if (nit >= 1) good = wait_fast<20>(bar_qfree, (nit - 1) & 1, s_abort, status);
       if (!good) return false;
       const QTile &qa = de.qa, &qb = de.qb;
-      if (NODE || t.mode == 1) {
+      if (is_node(t)) {
         constexpr int CPR = D / 8;
         constexpr int RS = 256 / CPR;                       // rows covered by the 256 threads per step
         const int cq = tid % CPR, rq0 = tid / CPR;
@@ -477,22 +483,22 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       if (t.mode < 0) break;                              // the work list is exhausted
       const QTile q = i ? de.qb : de.qa;
       const int total = q.n1 + q.n2;
-      const float wlog = ((NODE || t.mode == 1) && g.m > 0) ? log2f((float)t.nk / (float)g.m) : 0.f;   // log2(N/m): weight of a sampled column
+      const float wlog = (is_node(t) && g.m > 0) ? log2f((float)t.nk / (float)g.m) : 0.f;   // log2(N/m): weight of a sampled column
       // key tiles of this item with masked columns for this query tile, one bit per tile (an item has at most 32)
       unsigned tile_masked = 0;
-      if (NODE || t.mode == 1) tile_masked = __ballot_sync(0xffffffffu, lane < t.ntiles && (s_mask[2 * lane] | s_mask[2 * lane + 1]) != 0);
+      if (is_node(t)) tile_masked = __ballot_sync(0xffffffffu, lane < t.ntiles && (s_mask[2 * lane] | s_mask[2 * lane + 1]) != 0);
       float m_ref = -INFINITY;
       uint64_t l01 = 0;             // l: unrounded row sum (two partial sums, packed)
       float lra = 0.f, lrb = 0.f;   // lr: sum of the bf16 weights (two partial sums; the mixed-precision add takes the bf16 halves as they are)
       // Alg. 2 with caps (sorted nodes only): the masked row sum (block part) is complete when the first
       // sampled tile starts; from then on every sampled weight enters the row sum as min(weight, (N/m) C_i),
       // C_i = cap_scale m / (N ln N) (masked_i + tau / kappa), while the numerator keeps the weight itself.
-      const bool capped_item = CAPPED && (NODE || t.mode == 1) && g.m > 0;
+      const bool capped_item = CAPPED && is_node(t) && g.m > 0;
       float lblk = 0.f;             // masked row sum in units of 2^m_ref
       bool in_samples = false;
       float capfac = 0.f, lfloor = -INFINITY;     // (N/m) cap_scale m / (N ln N); log2(tau / kappa)
       // weighted sampling (columns drawn by value norms): every sampled column carries its own log2 weight
-      const bool weighted_item = WEIGHTED && (NODE || t.mode == 1);
+      const bool weighted_item = WEIGHTED && is_node(t);
       const float* s_bias = reinterpret_cast<const float*>(smem + C::kOffBias) + set * kMaxWeightedSamples;
       if (capped_item) {
         capfac = a.cap_scale / (logf((float)t.nk));
@@ -515,8 +521,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
         const bool table = (tile_masked >> j) & 1u;
         // (weighted sampling: the tile's columns have weights of their own; the largest one stands in where one number is needed)
         const bool weighted_tile = weighted_item && j >= t.nbA + t.nbB;
-        const float ubias = ((NODE || t.mode == 1) && j >= t.nbA + t.nbB) ? (weighted_tile ? t.bias_max : wlog) : 0.f;
-        const bool dense_mask = !(NODE || t.mode == 1) && ((j * TK + TK > t.nk) || (t.causal && j * TK + TK - 1 > q.row0));
+        const float ubias = (is_node(t) && j >= t.nbA + t.nbB) ? (weighted_tile ? t.bias_max : wlog) : 0.f;
+        const bool dense_mask = !is_node(t) && ((j * TK + TK > t.nk) || (t.causal && j * TK + TK - 1 > q.row0));
         // The 64 scores of this row are read from TMEM once; then (1) the row maximum, (2)
         // exponentials, row sums and the bf16 P written over the first half of the S buffer.
         // The reference maximum only moves when the tile exceeds it by more than 2^32, and then
@@ -734,8 +740,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
           constexpr int RB = C::kStageRow;
           constexpr int LPR = RB / 16, RPI = 32 / LPR, NI = 32 / RPI;
           constexpr int NP = D / 16;
-          const bool f32o = (!NODE && t.partial) ? !a.part_bf16 : a.out_fp32;
-          char* obase = reinterpret_cast<char*>((!NODE && t.partial) ? a.part_o : a.out);
+          const bool f32o = is_partial(t) ? !a.part_bf16 : a.out_fp32;
+          char* obase = reinterpret_cast<char*>(is_partial(t) ? a.part_o : a.out);
           const long long myoff = qr >= 0 ? (long long)(orow * (size_t)(D * (f32o ? 4 : 2))) : -1;
           long long roff[NI];
 #pragma unroll
@@ -746,7 +752,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
           const int crow = lane / LPR, cc = lane % LPR;
           const int lg_pps = f32o ? (RB == 128 ? 1 : 0) : (RB == 128 ? 2 : 1);   // log2(pieces per staging step)
           if (qr >= 0) {
-            if (!NODE && t.partial) a.part_lse[orow] = lse;
+            if (is_partial(t)) a.part_lse[orow] = lse;
             else a.lse[orow] = lse;
           }
           uint32_t r[16];
@@ -1006,7 +1012,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       const bool end = item >= a.total_pairs + a.split_pairs;
       PairDesc t = {}; QTile qa = {}, qb = {}; int lenA = 0, lenB = 0;
       const int tail = item - (a.total_pairs - a.split_pairs);     // the last pairs: each query tile an item
-      if (!end) decode_pair(a, tail < 0 ? item : item - ((tail + 1) >> 1), tail < 0 ? -1 : tail & 1, t, qa, qb, lenA, lenB);
+      const int pair = tail < 0 ? item : item - ((tail + 1) >> 1);
+      if (!end) decode_pair(a, pair + (pair >= a.skip_at ? a.skip : 0), tail < 0 ? -1 : tail & 1, t, qa, qb, lenA, lenB);
       else t.mode = -1;                                   // tells every role that the list is exhausted
       if (lane == 0) HA_TACC(26, tdec);
       const int set = it & 1;
@@ -1034,7 +1041,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       // the first one is used; the warp covers 32 consecutive columns per step, so one ballot
       // yields a whole word of the mask tables.  Padding columns point at a valid row (they are
       // masked, and the streamer puts zeros in the place of its values) and are masked for both tiles.
-      if (NODE || t.mode == 1) {
+      if (is_node(t)) {
         constexpr int UB = 8;
         const int bcols = t.nbA * TK;
         const int nblk = (t.nbA + t.nbB) * TK;            // columns of the block part (multiple of 64)
@@ -1126,7 +1133,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
         for (int k = 0; k < 4; ++k) {
           const int r = 4 * lane + k;
           qr[i][k] = -1;
-          if (q.valid && r < q.nq) qr[i][k] = (NODE || t.mode == 1) ? t.qnode0 + a.perm_q[t.slice + q.spos0 + r] : q.q0 + r;
+          if (q.valid && r < q.nq) qr[i][k] = is_node(t) ? t.qnode0 + a.perm_q[t.slice + q.spos0 + r] : q.q0 + r;
         }
       }
 #pragma unroll
@@ -1137,7 +1144,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       if (lane == 0) HA_TACC(10, ttab);
       // Sorted query rows are read once in the whole forward pass, so they come from HBM: ask for
       // them now (the softmax threads gather them a whole item later) so that they are found in L2.
-      if (NODE || t.mode == 1) {
+      if (is_node(t)) {
         const char* qbase = reinterpret_cast<const char*>(a.q) + (size_t)segrow * (D * 2);
 #pragma unroll
         for (int i = 0; i < 2; ++i)
@@ -1157,7 +1164,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       }
       if (lane == 0) HA_TACC(27, tqf);
       HA_T0(tqi);
-      if (!NODE && t.mode == 0) {
+      if (!is_node(t)) {
         // consecutive rows: one box per 64 columns and tile (rows past the tile's end are other
         // rows of the tensor or zeros: their results are never stored)
         if (lane == 0) {
@@ -1211,18 +1218,18 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
       const int lenA = de.lenA, lenB = de.lenB;
       const int segrow = t.seg * g.nk;                      // (keys)
       // does any of the item's key tiles have columns that do not exist?
-      const bool shorts = (!NODE && t.mode == 0) ? t.nk % TK != 0 : (lenA % TK | lenB % TK | g.m % TK) != 0;
+      const bool shorts = !is_node(t) ? t.nk % TK != 0 : (lenA % TK | lenB % TK | g.m % TK) != 0;
       for (int j = 0; j < t.ntiles && ok; ++j) {
         const int gj = gbase + j;
         const int s = gj % C::NS;
         const int use = gj / C::NS;
         int4 rows[QUADS];
-        if (NODE || t.mode == 1) {
+        if (is_node(t)) {
 #pragma unroll
           for (int k = 0; k < QUADS; ++k) rows[k] = *reinterpret_cast<const int4*>(s_kidx + j * TK + 4 * (rq + k * R));
         }
         auto fill = [&](uint32_t stage, const CUtensorMap* map, const char* src, uint32_t bar) {
-          if (!NODE && t.mode == 0) {
+          if (!is_node(t)) {
             // (rows past the end of the key range are masked by the softmax warps)
             if (lane == 0) {
               mbar_expect_tx(bar, C::kTile);
@@ -1269,11 +1276,11 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
         }
 #endif
         const int have = !shorts ? TK                     // columns of the tile that exist
-                         : (!NODE && t.mode == 0) ? t.nk - j * TK
+                         : !is_node(t) ? t.nk - j * TK
                          : j < t.nbA ? lenA - j * TK
                          : j < t.nbA + t.nbB ? lenB - (j - t.nbA) * TK : g.m - (j - t.nbA - t.nbB) * TK;
         if (have >= TK) fill(ubase + C::kOffV + s * C::kTile, &maps.v, vsrc, bar_vfull(s));
-        else fill_short<D>(ubase + C::kOffV + s * C::kTile, reinterpret_cast<const char*>(a.v), (NODE || t.mode == 1) ? s_kidx + j * TK : nullptr,
+        else fill_short<D>(ubase + C::kOffV + s * C::kTile, reinterpret_cast<const char*>(a.v), is_node(t) ? s_kidx + j * TK : nullptr,
                            segrow + t.k0 + j * TK, have, bar_vfull(s));
         v_armed = gj + 1;
         if (lane == 0) HA_TACC(1, tgv);
@@ -1360,40 +1367,83 @@ bool encode_acc_map(CUtensorMap* m, const void* base, size_t rows, int d) {
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+namespace {
+
+template <int D, bool LATE, bool PRECISE, SampleRule RULE, ItemKind KIND>
+cudaError_t run_build(const AttnArgs& b, const TmaMaps& maps, int grid, int* status, cudaStream_t st) {
+  const cudaError_t e = allow_smem<attn_tc_kernel<D, LATE, PRECISE, RULE, KIND>>(Cfg<D>::kTotal);
+  return e != cudaSuccess ? e : launch(attn_tc_kernel<D, LATE, PRECISE, RULE, KIND>, grid, 384, Cfg<D>::kTotal, st, b, maps, status);
+}
+
+// the launch of a part of the list: b.total_pairs pairs, those from b.skip_at on b.skip further on
+template <int D, ItemKind KIND>
+cudaError_t run_items(const AttnArgs& b, const TmaMaps& maps, int sms, int* status, cudaStream_t st) {
+  const int items = b.total_pairs + b.split_pairs, grid = items < sms ? items : sms;     // persistent: one CTA per SM walks the item list
+  // (fp32 partial results of d = 128: see the epilogue)
+  constexpr bool CAN_BE_LATE = D == 128 && KIND != kFinalNodes;
+  const bool late = CAN_BE_LATE && !b.direct && !b.part_bf16;
+  if constexpr (KIND != kDenseItems) {
+    if (b.capped) return late ? run_build<D, CAN_BE_LATE, false, kCapped, KIND>(b, maps, grid, status, st) : run_build<D, false, false, kCapped, KIND>(b, maps, grid, status, st);
+    if (b.sample_wlog) return late ? run_build<D, CAN_BE_LATE, false, kWeighted, KIND>(b, maps, grid, status, st) : run_build<D, false, false, kWeighted, KIND>(b, maps, grid, status, st);
+  }
+  if (b.precise) return late ? run_build<D, CAN_BE_LATE, true, kUniform, KIND>(b, maps, grid, status, st) : run_build<D, false, true, kUniform, KIND>(b, maps, grid, status, st);
+  return late ? run_build<D, CAN_BE_LATE, false, kUniform, KIND>(b, maps, grid, status, st) : run_build<D, false, false, kUniform, KIND>(b, maps, grid, status, st);
+}
+
+// pairs of the sorted nodes (the first levels: nodes get smaller from level to level)
+void sorted_pairs(const AttnArgs& a, int& first, int& end) {
+  int l = 0;
+  while (l < a.g.levels && a.level_sorted[l]) ++l;
+  first = a.n_leaf_pairs; end = l > 0 ? a.level_pair_start[l] : a.n_leaf_pairs;
+}
+
+}  // namespace
+
+// A call with recursion gains by two launches what their own builds are faster by, about 2 %, and loses the end of the first launch and the heavy items at
+// the end of the second, 10 to 15 us: from 64 pairs of query tiles for an SM on.  (Calls, us, one launch -> two: 32 heads of 131072 rows, 387 pairs
+// for an SM, 6636 -> 6476, d = 128, split weights, 64 of 16384, 69 pairs, 1976 -> 1944; 4 of 100003, 38 pairs, 592 -> 593, 8 of 50000, 32 pairs, 537 -> 542,
+// d = 128, 8 of 32768, 17 pairs, 514 -> 530, 16 of 9000, 8 pairs, 138 -> 149.)
+constexpr int kTwoLaunches = 64;
+bool attention_in_two(const AttnArgs& a) {
+  int first, end, sms = 0;
+  sorted_pairs(a, first, end);
+  return end > first && end - first < a.total_pairs && sm_count(&sms) == cudaSuccess && a.total_pairs >= (long long)kTwoLaunches * sms;
+}
+
 cudaError_t launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st) {
   if (a.total_pairs == 0) return cudaSuccess;
   const size_t rows = (size_t)a.g.G * a.g.n, rows_k = (size_t)a.g.G * a.g.nk;
   if (rows > 0x7fffffffull || rows_k > 0x7fffffffull) return cudaErrorInvalidValue;        // row coordinates are 32-bit
+  if ((a.capped != 0) + (a.sample_wlog != nullptr) + (a.precise != 0) > 1) return cudaErrorInvalidValue;
   TmaMaps maps;
   if (!encode_rows_map(&maps.q, a.q, rows, a.g.d, 128) || !encode_rows_map(&maps.k, a.k, rows_k, a.g.d, TK) ||
       !encode_rows_map(&maps.v, a.v, rows_k, a.g.d, TK)) return cudaErrorInvalidValue;
   int sms = 0;
   cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
+  auto run = [&](const AttnArgs& b, auto kind) {
+    constexpr ItemKind KIND = decltype(kind)::value;
+    return a.g.d == 64 ? run_items<64, KIND>(b, maps, sms, status, st) : run_items<128, KIND>(b, maps, sms, status, st);
+  };
+  using any = std::integral_constant<ItemKind, kAnyItems>;
+  using final_nodes = std::integral_constant<ItemKind, kFinalNodes>;
+  using partial_nodes = std::integral_constant<ItemKind, kPartialNodes>;
+  using dense = std::integral_constant<ItemKind, kDenseItems>;
   AttnArgs b = a;
   b.split_pairs = split_pairs(a, sms);
-  const int items = a.total_pairs + b.split_pairs;
-  const int grid = items < sms ? items : sms;                     // persistent: one CTA per SM walks the item list
-  b.tail_leaves = a.dense_causal && a.total_pairs == a.n_leaf_pairs ? tail_leaves(a.n_leaf_pairs / a.pairs_per_leaf, a.pairs_per_leaf, sms) : 0;
-  if ((a.capped != 0) + (a.sample_wlog != nullptr) + (a.precise != 0) > 1) return cudaErrorInvalidValue;
-  const bool node = a.n_leaf_pairs == 0 && a.g.levels == 1 && a.level_sorted[0] && a.direct;
-  const bool late = a.g.d == 128 && !a.direct && !a.part_bf16;
-#define HA_RUN(D, LATE, PRECISE, RULE, NODE) do { e = allow_smem<attn_tc_kernel<D, LATE, PRECISE, RULE, NODE>>(Cfg<D>::kTotal); \
-    return e != cudaSuccess ? e : launch(attn_tc_kernel<D, LATE, PRECISE, RULE, NODE>, grid, 384, Cfg<D>::kTotal, st, b, maps, status); } while (0)
-#define HA_GO(D, LATE, PRECISE, RULE) do { if (!LATE && node) HA_RUN(D, false, PRECISE, RULE, true); HA_RUN(D, LATE, PRECISE, RULE, false); } while (0)
-  if (a.g.d == 64) {
-    if (a.capped) HA_GO(64, false, false, kCapped);
-    if (a.sample_wlog) HA_GO(64, false, false, kWeighted);
-    if (a.precise) HA_GO(64, false, true, kUniform);
-    HA_GO(64, false, false, kUniform);
+  b.skip_at = b.skip = b.tail_leaves = 0;
+  int first, end;
+  sorted_pairs(a, first, end);
+  if (end == a.total_pairs && first == 0) return run(b, final_nodes{});
+  const bool two = attention_in_two(a), no_nodes = first == end;
+  if (two) {                                              // the nodes first: their items are light and equal
+    b.total_pairs = end - first; b.skip = first;
+    e = run(b, partial_nodes{});
+    if (e != cudaSuccess) return e;
+    b.total_pairs = a.total_pairs - (end - first); b.skip_at = first; b.skip = end - first; b.sched = a.sched + 1;
   }
-  if (a.capped) { if (late) HA_GO(128, true, false, kCapped); HA_GO(128, false, false, kCapped); }
-  if (a.sample_wlog) { if (late) HA_GO(128, true, false, kWeighted); HA_GO(128, false, false, kWeighted); }
-  if (a.precise) { if (late) HA_GO(128, true, true, kUniform); HA_GO(128, false, true, kUniform); }
-  if (late) HA_GO(128, true, false, kUniform);
-  HA_GO(128, false, false, kUniform);
-#undef HA_GO
-#undef HA_RUN
+  if (a.dense_causal && b.total_pairs == a.n_leaf_pairs) b.tail_leaves = tail_leaves(a.n_leaf_pairs / a.pairs_per_leaf, a.pairs_per_leaf, sms);
+  return two || no_nodes ? run(b, dense{}) : run(b, any{});
 }
 
 }  // namespace hyperattn

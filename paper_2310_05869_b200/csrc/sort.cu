@@ -87,7 +87,7 @@ template <int NG>
 __global__ void __launch_bounds__(256 * NG) sort_scan_kernel(SortArgs a, SampleArgs sa, VnormArgs va, int scan_blocks, int sample_blocks) {
   __shared__ uint32_t s_tot[NG][kBuckets], s_warp[NG][8];
   wait_for_stream();
-  if (sa.sched && blockIdx.x == 0 && threadIdx.x == 0) *sa.sched = 0;
+  if (sa.sched && blockIdx.x == 0 && threadIdx.x == 0) sa.sched[0] = sa.sched[1] = 0;
   if ((int)blockIdx.x >= scan_blocks) {
     const int x = blockIdx.x - scan_blocks;
     if (x < sample_blocks) samples_body(sa, x, sample_blocks);
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(256, SCAN ? 5 : 6) sort_scatter_kernel(SortArg
   if (rows <= 0) return;
 
   wait_for_stream();
-  if (SCAN && sa.sched && blockIdx.x == 0 && tid == 0) *sa.sched = 0;
+  if (SCAN && sa.sched && blockIdx.x == 0 && tid == 0) sa.sched[0] = sa.sched[1] = 0;
   const uint8_t* ids = a.ids + level * ids_level_stride(g) + side_ids_base(g, side) + (size_t)seg * side_rows(g, side) + row0;
   // SCAN: bucket tid's total over the node, and over the node's chunks before this one
   uint32_t tot = 0, before = 0;

@@ -113,6 +113,32 @@ def test_permutations_are_stable_sorts_of_the_ids(kind, H, n, n_k, d, r, causal,
                                        torch.arange(rows, dtype=torch.int32, device="cuda").expand(H, rows))
 
 
+# calls large enough for sorted nodes and everything else in launches of their own, against calls of few heads in one launch: the same bits
+TWO_LAUNCHES = [(64, 64, 2048, 256, torch.bfloat16, {}), (64, 40, 128, 256, torch.bfloat16, {}), (64, 64, 2048, 256, torch.float32, dict(precise=True)),
+                (128, 64, 2048, 256, torch.bfloat16, {}), (128, 64, 2048, 250, torch.float32, {}), (128, 64, 2048, 256, torch.float32, dict(precise=True)),
+                (64, 64, 2048, 256, torch.bfloat16, dict(caps=(8.0, 16.0))), (128, 64, 2048, 256, torch.float32, dict(value_norm_sampling=True))]
+
+
+@pytest.mark.parametrize("d,H,n0,b,out_dtype,option", TWO_LAUNCHES)
+def test_nodes_and_leaves_in_launches_of_their_own(d, H, n0, b, out_dtype, option):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(17)
+    q, k, v = (torch.randn(1, H, 16384, d, generator=gen, device="cuda").bfloat16() for _ in range(3))
+    kw = dict(causal=True, n0=n0, seed=2, out_dtype=out_dtype, **option)
+    few, launches, results = 3, [], []
+    for heads in (H, few):
+        ha.profile_reset()
+        ha.profile_enable(True)
+        results.append(ha.forward(q[:, :heads], k[:, :heads], v[:, :heads], b, 128, 6, **kw))
+        torch.cuda.synchronize()
+        ha.profile_enable(False)
+        launches.append(ha.profile_read()["launches"]["attention"])
+    assert launches[0] == launches[1] + 1
+    for x, y in zip(*results):
+        assert torch.equal(x[:, :few], y)
+    assert ha.last_device_status() == 0
+
+
 # calls whose leaves go first and write dK and dV (from 192 MiB of fp32 accumulators on), against calls of few heads, which add everything
 SPLIT_BACKWARD = [(64, 26, 16384, 4096), (64, 26, 16800, 2100), (64, 40, 10240, 700), (128, 13, 16384, 4096)]
 

@@ -78,16 +78,15 @@ struct AttnArgs {
 };
 
 // Items of leaves are handed out leaf by leaf, the heaviest first; where nothing follows them, one leaf at a time the last heavy item would start
-// when little is left beside it.  So the last leaves - two rounds of all SMs - go rank by rank: the heaviest items of all of them first.  (Forward,
+// when little is left beside it.  So the last leaves - four rounds of all SMs - go rank by rank: the heaviest items of all of them first.  (Forward,
 // d = 64, us, leaf by leaf -> two rounds: 64 leaves of 1024 rows 36.9 -> 30.7, 20 of 4096 113.7 -> 89.9, 128 of 4096 453 -> 407, 16 of 8192 291 ->
-// 223, 4 of 32768 993 -> 826, 300 of 512 39.9 -> 36.9, 8 of 4096 61.5 -> 59.7; d = 128, 20 of 4096 130 -> 106.  In another run, one round / two /
-// four / all leaves: 64 leaves of 1024 rows 33.3 / 30.7 / 30.7 / 30.7, 20 of 4096 109 / 90.8 / 88.5 / 88.7, 128 of 4096 421 / 408 / 398 / 398, 16 of
-// 8192 250 / 224 / 201 / 201, 300 of 512 36.9 / 37.0 / 37.7 / 37.7, 8 of 4096 60.4 / 60.7 / 61.2 / 61.2; backward, 64 of 2048 153 / 146 / 138 / 136,
-// 128 of 4096 903 / 896 / 863 / 1077, d = 128, 64 of 4096 869 / 825 / 812 / 887.  One round is too few, all leaves lose the L2; where leaves are
-// few, two or four make no difference, else four would be better.)
+// 223, 4 of 32768 993 -> 826, 300 of 512 39.9 -> 36.9, 8 of 4096 61.5 -> 59.7; d = 128, 20 of 4096 130 -> 106.  Two rounds -> four, another build: 128 of
+// 4096 413 -> 407, 32 of 3000 78.0 -> 72.8, 20 of 4096 88.8 -> 87.4, 16 of 8192 222 -> 199, but 300 of 512 36.1 -> 36.8; d = 128, 64 of 4096 302 ->
+// 290; backward, 128 of 4096 1003 -> 989, 32 of 3000 162 -> 151, 20 of 4096 174 -> 159, 16 of 8192 487 -> 452, 64 of 2048 158 -> 151, 300 of 512 85.8 ->
+// 83.2, d = 128, 64 of 4096 946 -> 925.  One round is too few, all leaves lose the L2 (backward, 128 of 4096 863 with four rounds, 1077 with all).)
 inline int tail_leaves(int leaves, int items_per_leaf, int sms) {
-  const int two_rounds = (2 * sms + items_per_leaf - 1) / items_per_leaf;
-  return leaves < two_rounds ? leaves : two_rounds;
+  const int rounds = (4 * sms + items_per_leaf - 1) / items_per_leaf;
+  return leaves < rounds ? leaves : rounds;
 }
 // item of a leaf list -> leaf and rank (0: the heaviest item of the leaf)
 __device__ __forceinline__ void leaf_of_item(int item, int items, int per_leaf, int tail_leaves, int& leaf, int& rank) {

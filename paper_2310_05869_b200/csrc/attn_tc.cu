@@ -127,7 +127,7 @@ struct QTile {
   int nq;        // valid rows
   int q0;        // dense: first query row (segment-relative)
   int row0;      // dense causal: local index of the tile's first row (relative to the first key)
-  int beta;      // node: block
+  int beta;      // node: block (of a second tile that does not exist: -1)
   int spos0;     // node: first sorted position
   int s1, n1, s2, n2;
 };
@@ -265,9 +265,9 @@ __device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, int onl
     QTile* qs[2] = {&qa, &qb};
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const int tn = paired ? 2 * pn + (only < 0 ? i : only) : pn;
+      const int tn = paired ? 2 * pn + (only == 1 ? 1 - i : i) : pn;
       QTile& q = *qs[i];
-      q.valid = tn < tiles_node && (i == 0 || (paired && only < 0));
+      q.valid = tn < tiles_node && (i == 0 || paired);
       q.row0 = 0;
       if (sorted) {
         q.beta = tn / a.tiles_per_block;
@@ -275,6 +275,9 @@ __device__ __forceinline__ void decode_pair(const AttnArgs& a, int pair, int onl
         q.spos0 = q.beta * t.bq + sub * kTileQ;
         q.nq = t.bq > 0 ? min(kTileQ, block_len(t.nq_node, t.bq, q.beta) - sub * kTileQ) : 0;
         if (q.nq <= 0) q.valid = 0;                       // the group (a short last one, or one past the node's queries) has no such tile
+        // (qb's block stays where the pair is split: the order of the sampled columns is that of the pair)
+        if (i == 1 && !q.valid) q.beta = -1;
+        if (i == 1 && only >= 0) q.valid = 0;
         q.q0 = 0;
       } else {
         q.q0 = q0n + tn * kTileQ;
@@ -1075,6 +1078,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
         // (1 - M^H) of Alg. 2 line 7).  The samples are an unordered multiset, so the masked ones
         // (for either query tile) are moved to the end of the sample part: only its last tile(s)
         // then carry mask bits, every other sampled tile takes the softmax warps' fast path.
+        // (For a split pair too, so that the columns are added in the same order: whether a call
+        // splits its pairs depends on how many heads it has, and a head's result must not.)
         if (nblk < ncols) {
           for (int wd = (nblk >> 5) + lane; wd < (ncols >> 5); wd += 32) { s_mask[wd] = 0; s_mask[MW + wd] = 0; }
           __syncwarp();
@@ -1097,7 +1102,7 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
               if (c - lane < ncols - nblk) {              // warp-uniform
                 const bool valid = l[u] >= 0;
                 const bool m0 = !valid || blk[u] == qa.beta;
-                const bool m1 = !valid || (qb.valid && blk[u] == qb.beta);
+                const bool m1 = !valid || blk[u] == qb.beta;
                 const unsigned bf = __ballot_sync(0xffffffffu, valid && !(m0 || m1));
                 const unsigned bb = __ballot_sync(0xffffffffu, valid && (m0 || m1));
                 int pos;

@@ -58,23 +58,46 @@ def test_forward_edges(w):
 
 
 # heads of a call whose pairs of query tiles are split (at most 74 of 148 SMs have one left), and of one whose pairs are not
-SPLIT = [(64, 1000, 1000, 256, 64, 18, 20),              # two tiles of a block; a short last block
-         (128, 1100, 1100, 256, 130, 14, 16),            # ... whose second tile does not exist
-         (64, 1100, 1100, 100, 33, 12, 13),              # pairs across blocks, an odd number of tiles
-         (128, 600, 1500, 128, 64, 9, 13),               # ... fewer queries than keys
-         (64, 20000, 20000, 256, 256, 2, 3)]             # behind a round of whole pairs
+SPLIT = [(64, 1000, 1000, 256, 64, 18, 20, {}),          # two tiles of a block; a short last block
+         (128, 1100, 1100, 256, 130, 14, 16, {}),        # ... whose second tile does not exist
+         (64, 1100, 1100, 100, 33, 12, 13, {}),          # pairs across blocks, an odd number of tiles
+         (64, 1100, 1100, 100, 33, 12, 13, dict(precise=True)),
+         (64, 1100, 1100, 100, 130, 12, 13, dict(caps=(8.0, 16.0))),
+         (64, 1100, 1100, 100, 130, 12, 13, dict(value_norm_sampling=True)),
+         (64, 2900, 2900, 384, 200, 6, 7, {}),           # ... of three tiles each, the last of which do not exist
+         (128, 600, 1500, 128, 64, 9, 13, {}),           # ... fewer queries than keys
+         (128, 600, 1500, 128, 200, 9, 13, dict(value_norm_sampling=True)),
+         (64, 20000, 20000, 256, 256, 2, 3, {})]         # behind a round of whole pairs
 
 
-@pytest.mark.parametrize("d,n,n_k,b,m,split,whole", SPLIT)
-def test_split_pairs_give_the_same_results(d, n, n_k, b, m, split, whole):
+@pytest.mark.parametrize("d,n,n_k,b,m,split,whole,option", SPLIT)
+def test_split_pairs_give_the_same_results(d, n, n_k, b, m, split, whole, option):
     gen = torch.Generator(device="cuda")
     gen.manual_seed(7)
     q, k, v = (torch.randn(1, whole, rows, d, generator=gen, device="cuda").bfloat16() for rows in (n, n_k, n_k))
-    want = ha.forward(q, k, v, b, m, 6, seed=3, out_dtype=torch.float32)
-    got = ha.forward(q[:, :split], k[:, :split], v[:, :split], b, m, 6, seed=3, out_dtype=torch.float32)
-    # the same bits, but for the order of the sampled columns where a pair has tiles of two blocks: fp32 sums of b + m weighted values
-    assert float((got[0] - want[0][:, :split]).abs().max()) <= (b + m) * 2.0 ** -24 * float(v.abs().max())
-    assert float((got[1] - want[1][:, :split]).abs().max()) <= (b + m) * 2.0 ** -24
+    want = ha.forward(q, k, v, b, m, 6, seed=3, out_dtype=torch.float32, **option)
+    got = ha.forward(q[:, :split], k[:, :split], v[:, :split], b, m, 6, seed=3, out_dtype=torch.float32, **option)
+    for x, y in zip(got, want):
+        assert torch.equal(x, y[:, :split])
+    assert ha.last_device_status() == 0
+
+
+# host buffers go through in up to sixteen groups, calls of their own: the same bits as one call of all heads, where only one of the two splits
+# its pairs, and whatever else goes by the number of heads
+@pytest.mark.parametrize("H,n,n_k,d,b,m,dtype,kw", [
+    (32, 4096, 4096, 64, 128, 256, torch.bfloat16, {}), (16, 1100, 1100, 64, 100, 33, torch.bfloat16, {}), (16, 600, 1500, 128, 128, 64, torch.bfloat16, {}),
+    (32, 4096, 4096, 64, 256, 256, torch.bfloat16, {}), (40, 1500, 1500, 64, 100, 33, torch.bfloat16, dict(causal=True, n0=400)),
+    (32, 1100, 1100, 64, 100, 33, torch.float32, {}), (20, 1500, 1500, 128, 100, 33, torch.float32, dict(causal=True, n0=400))])
+def test_host_buffers_in_groups_give_the_same_bits(H, n, n_k, d, b, m, dtype, kw):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(19)
+    q, k, v = (torch.randn(1, H, rows, d, generator=gen, device="cuda").to(dtype) for rows in (n, n_k, n_k))
+    want = ha.forward(q, k, v, b, m, 6, seed=3, **kw)
+    got = [torch.empty(x.shape, dtype=x.dtype).pin_memory() for x in want]
+    ha.forward_host(*(x.cpu().pin_memory() for x in (q, k, v)), *got, b, m, 6, seed=3, **kw)
+    torch.cuda.synchronize()
+    for x, y in zip(got, want):
+        assert torch.equal(x, y.cpu())
     assert ha.last_device_status() == 0
 
 

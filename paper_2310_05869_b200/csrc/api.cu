@@ -463,6 +463,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     const size_t elems = (size_t)g.G * g.n * g.d;
     const bool g32 = bw->grad_dtype == HYPERATTN_FP32;
     const size_t kv_elems = key_grad_rows(g, direct) * g.d;
+    BwdLaunch launches[2];
     BwdGrads gr;
     float* acc = reinterpret_cast<float*>(base + pl.gacc);
     gr.dq = g32 ? reinterpret_cast<float*>(bw->dq) : acc;
@@ -471,7 +472,7 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     gr.kv_elems = kv_elems;
     gr.dq16 = g32 ? nullptr : bw->dq; gr.dk16 = g32 ? nullptr : bw->dk; gr.dv16 = g32 ? nullptr : bw->dv;
     gr.direct = direct; gr.key_slot = ws.key_slot;
-    StageScope sc(st, HYPERATTN_STAGE_BACKWARD, 2 + (g32 ? 0 : 1) + (backward_split(g, kv_elems) ? 1 : 0));
+    StageScope sc(st, HYPERATTN_STAGE_BACKWARD, 1 + backward_launches(g, launches) + (g32 ? 0 : 1));
     HA_CHECK(launch_backward(a, p.out, out_fp32, p.lse, bw->dout, reinterpret_cast<float2*>(base + pl.stat), ws.sched, gr, scale, ws.status, st));
     return HYPERATTN_OK;
   }
@@ -517,14 +518,20 @@ int hyperattn_backward(const hyperattn_params* p, const hyperattn_grads* grads) 
   return forward_impl(*p, 0, grads);
 }
 
-// (for the tests, not part of the interface) which build of the backward kernel a call takes
-int hyperattn_internal_backward_build(const hyperattn_params* p, int* boxes, int* results_warps) {
-  if (!p || !boxes || !results_warps) return HYPERATTN_INVALID_ARGUMENT;
+// (for the tests, not part of the interface) the launches of the backward kernel that a call makes: how many (out[0]), and of each which items
+// it has (1 leaves, 2 nodes, 3 all), how its results leave (BwdOut) and its results warps
+int hyperattn_internal_backward_launches(const hyperattn_params* p, int out[7]) {
+  if (!p || !out) return HYPERATTN_INVALID_ARGUMENT;
   Geometry g;
   const int rc = build_geometry(*p, g);
   if (rc) return rc;
-  const BwdBuild build = backward_build(g);
-  *boxes = build.boxes; *results_warps = build.results_warps;
+  BwdLaunch launches[2] = {};
+  out[0] = backward_launches(g, launches);
+  for (int i = 0; i < 2; ++i) {
+    out[1 + 3 * i] = launches[i].leaves + 2 * launches[i].nodes;
+    out[2 + 3 * i] = launches[i].out;
+    out[3 + 3 * i] = launches[i].results_warps;
+  }
   return HYPERATTN_OK;
 }
 

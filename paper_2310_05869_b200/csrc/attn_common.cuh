@@ -29,14 +29,15 @@ struct BwdGrads {
   int direct;                  // every key has one tile only besides the samples: its bf16 dK and dV leave from there
 };
 
-// which build of the backward kernel a call takes (backward.cu)
-struct BwdBuild {
-  bool boxes;                  // whole tiles of consecutive rows leave as boxes
+// The launches of the backward kernel that a call makes - one for all items, or one for the leaves and one for the nodes behind it -
+// and the build that each takes (backward.cu)
+enum BwdOut { kRows, kBoxes, kFirst, kNodes };     // how results leave (backward.cuh)
+struct BwdLaunch {
+  bool leaves, nodes;          // what it has of the call's items
+  BwdOut out;
   int results_warps;
 };
-BwdBuild backward_build(const Geometry& g, bool leaves = true, bool nodes = true);
-// leaves and nodes in launches of their own (kv_elems: entries of the fp32 dK)
-bool backward_split(const Geometry& g, size_t kv_elems);
+int backward_launches(const Geometry& g, BwdLaunch launches[2]);
 
 struct AttnArgs {
   const __nv_bfloat16 *q, *k, *v;    // [G, n, D]

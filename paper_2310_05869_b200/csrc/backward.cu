@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(256) to_bf16_kernel(const __grid_constant__ To
 
 }  // namespace
 
-// (with_leaves, with_nodes: what the launch has of the call's items.)  What pays is whole tiles of 128 consecutive rows (leaves, nodes that are not sorted): their dQ leaves as a box at every step, with a few
+// What pays is whole tiles of 128 consecutive rows (leaves, nodes that are not sorted): their dQ leaves as a box at every step, with a few
 // instructions.  What costs: the boxes' code in the results warps at every short tile and at every tile of sorted rows, and, with half of the warps,
 // those tiles themselves and the dK and dV of every key tile, behind which the next item waits.  So the rules weigh steps on whole tiles against key
 // tiles of consecutive rows (`items`) and all other steps.  The pass, us, without boxes / with boxes / four results warps (* what the rules take).
@@ -51,14 +51,16 @@ __global__ void __launch_bounds__(256) to_bf16_kernel(const __grid_constant__ To
 // 2048 1385 / 1356 / 1335*, 4096 1667 / 1602 / 1539*; 64 heads of 1600 rows in leaves of 100 under nodes that are not sorted 179* / 179 / 189; no
 // recursion, 32 heads of 4096 rows 131* / 134 / 142.  d = 128, without and with boxes: 1024 leaves of 100 rows 87.8* / 88.3, 781 of 256 162* / 161,
 // 390 of 512 197 / 191*, 64 of 4096 945 / 827*; 32 heads of 32768 rows without recursion 1494* / 1514.
-BwdBuild backward_build(const Geometry& g, bool with_leaves, bool with_nodes) {
+static BwdLaunch launch_of(const Geometry& g, bool with_leaves, bool with_nodes) {
+  BwdLaunch r = {with_leaves && (g.causal || !g.sorted), with_nodes && g.levels > 0, kRows, 8};
+  bool sorted = !r.leaves;                              // all items are tiles of sorted nodes
   long long whole = 0, other = 0, items = 0;            // per segment
-  if (with_leaves && (g.causal || !g.sorted)) {
+  if (r.leaves) {
     const long long leaves = g.npad / g.leaf, kts = (g.leaf + kTileK - 1) / kTileK, full = g.leaf / kTileQ;
     const long long on_full = g.causal ? full * (full + 1) / 2 : kts * full, all = g.causal ? kts * (kts + 1) / 2 : kts * kts;
     whole += leaves * on_full; other += leaves * (all - on_full); items += leaves * kts;
   }
-  for (int l = 0; l < g.levels && with_nodes; ++l) {
+  for (int l = 0; l < g.levels && r.nodes; ++l) {
     int s, q0, k0;
     node_rows(g, l, 0, s, q0, k0);
     const long long nodes = g.causal ? 1 << l : 1;
@@ -67,30 +69,41 @@ BwdBuild backward_build(const Geometry& g, bool with_leaves, bool with_nodes) {
       other += nodes * node_blocks(s, g.b) * ((g.b + kTileQ - 1) / kTileQ) * key_tiles;
     } else {
       const long long kts = (s + kTileK - 1) / kTileK, full = s / kTileQ;
+      sorted = false;
       whole += nodes * kts * full; other += nodes * kts * (kts - full); items += nodes * kts;
     }
   }
-  BwdBuild r;
-  r.boxes = whole > 0 && 4 * whole >= 7 * items + other;
-  r.results_warps = g.d == 64 && whole > 0 && 2 * whole >= 9 * items + other ? 4 : 8;
+  if (whole > 0 && 4 * whole >= 7 * items + other) r.out = kBoxes;
+  if (g.d == 64 && whole > 0 && 2 * whole >= 9 * items + other) r.results_warps = 4;     // (kBoxes all the more)
+  if (sorted) r.out = kNodes;
   return r;
 }
 
-// With recursion every row of dK and dV gets one contribution from its leaf and more from the nodes above it.  The leaves in a launch of their own, first, write
-// theirs, so that the accumulators need not be cleared, and leaves and nodes take the build that is best for each.  Against that stand a launch and
-// the end of the first one, where SMs run out of items: it pays from 192 MiB of accumulators on, where leaves leave as boxes.  (The pass, us, one launch ->
-// two: 32 heads of 131072 rows, d = 64, 16322 -> 16046 and, another time, 16239 -> 15962, 16 of 32768 (256 MiB) 1715 -> 1708 and 1719 -> 1700, 8 of
-// 32768, d = 128, (256 MiB) 1680 -> 1609 and 1669 -> 1614; 4 of 65536, d = 64, (128 MiB) 972 -> 984.)
+// With recursion every row of dK and dV gets one contribution from its leaf and more from the nodes above it.  The leaves in a launch of their own,
+// first, write theirs, so that the accumulators need not be cleared, and leaves and nodes take the build that is best for each.  Against that stand a
+// launch and the end of the first one, where SMs run out of items: it pays from 192 MiB of accumulators on, where leaves leave as boxes.  (The pass,
+// us, one launch -> two: 32 heads of 131072 rows, d = 64, 16322 -> 16046 and, another time, 16239 -> 15962, 16 of 32768 (256 MiB) 1715 -> 1708 and
+// 1719 -> 1700, 8 of 32768, d = 128, (256 MiB) 1680 -> 1609 and 1669 -> 1614; 4 of 65536, d = 64, (128 MiB) 972 -> 984.)
 constexpr size_t kSplitBytes = 192u << 20;
-bool backward_split(const Geometry& g, size_t kv_elems) { return g.L > 0 && kv_elems * 8 >= kSplitBytes && backward_build(g, true, false).boxes; }
+int backward_launches(const Geometry& g, BwdLaunch launches[2]) {
+  launches[0] = launch_of(g, true, false);
+  if (g.L > 0 && (size_t)g.G * g.n * g.d * 8 >= kSplitBytes && launches[0].out == kBoxes) {
+    launches[0].out = kFirst;
+    launches[1] = launch_of(g, false, true);
+    return 2;
+  }
+  launches[0] = launch_of(g, true, true);
+  return 1;
+}
 
-// a: the forward schedule (permutations, samples, tile geometry); the accumulators of gr are cleared here
+// a: the forward schedule (permutations, samples, tile geometry); the accumulators of gr are cleared here, but for what the first launch writes
 cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, const float* lse, const void* dout, float2* stat, int* sched,
                             const BwdGrads& gr, float scale, int* status, cudaStream_t st) {
   const Geometry& g = a.g;
   const size_t rows = (size_t)g.G * g.n;
   if (rows > 0x7fffffffull) return cudaErrorInvalidValue;            // TMA row coordinates are 32-bit
-  const bool split = backward_split(g, gr.kv_elems);
+  BwdLaunch launches[2];
+  const bool split = backward_launches(g, launches) == 2;
   {
     const unsigned grid = (unsigned)((rows * (g.d / 8) + 255) / 256);
     const uint4* d4 = reinterpret_cast<const uint4*>(dout);
@@ -148,37 +161,33 @@ cudaError_t launch_backward(const AttnArgs& a, const void* out, int out_fp32, co
       !encode_acc_map(&maps.dq, gr.dq, rows, g.d)) return cudaErrorInvalidValue;
   maps.dk = maps.dv = maps.dq;
   if (!gr.direct && (!encode_acc_map(&maps.dk, gr.dk, rows, g.d) || !encode_acc_map(&maps.dv, gr.dv, rows, g.d))) return cudaErrorInvalidValue;
-  auto go = [&](auto dim, auto with_boxes, auto results_warps, unsigned grid) {
-    constexpr int D = decltype(dim)::value, RW = decltype(results_warps)::value;
-    constexpr BwdOut OUT = decltype(with_boxes)::value ? kBoxes : kRows;
-    using C = Cfg<D, RW>;
-    const cudaError_t allowed = allow_smem<bwd_kernel<D, OUT, RW>>(C::kTotal);
-    return allowed != cudaSuccess ? allowed : launch(bwd_kernel<D, OUT, RW>, grid, C::kThreads, C::kTotal, st, b, maps, status);
+  auto go = [&](auto dim, auto how, unsigned grid) {
+    constexpr int D = decltype(dim)::value;
+    constexpr BwdOut OUT = decltype(how)::value;
+    using C = Cfg<D, 8>;
+    const cudaError_t allowed = allow_smem<bwd_kernel<D, OUT, 8>>(C::kTotal);
+    return allowed != cudaSuccess ? allowed : launch(bwd_kernel<D, OUT, 8>, grid, C::kThreads, C::kTotal, st, b, maps, status);
   };
-  using std::integral_constant;
-  using std::bool_constant;
-  using d64 = integral_constant<int, 64>;
-  using d128 = integral_constant<int, 128>;
-  using eight = integral_constant<int, 8>;
-  bool nodes_alone = (split || b.n_leaf_items == 0) && g.levels > 0;
-  for (int l = 0; l < g.levels; ++l) nodes_alone = nodes_alone && a.level_sorted[l];
-  auto run = [&](BwdBuild build) {
-    const unsigned grid = b.total_items < sms ? (unsigned)b.total_items : (unsigned)sms;     // persistent: one CTA per SM
-    if (nodes_alone) return launch_bwd_nodes(b, maps, grid, status, st);
-    if (build.results_warps == 4) return launch_bwd_leaves_d64(b, maps, grid, status, st);
-    if (g.d == 64) return build.boxes ? go(d64{}, bool_constant<true>{}, eight{}, grid) : go(d64{}, bool_constant<false>{}, eight{}, grid);
-    return build.boxes ? go(d128{}, bool_constant<true>{}, eight{}, grid) : go(d128{}, bool_constant<false>{}, eight{}, grid);
+  using d64 = std::integral_constant<int, 64>;
+  using d128 = std::integral_constant<int, 128>;
+  using rows_out = std::integral_constant<BwdOut, kRows>;
+  using boxes_out = std::integral_constant<BwdOut, kBoxes>;
+  auto run = [&](const BwdLaunch& l) {
+    const unsigned grid = b.total_items < sms ? b.total_items : sms;      // persistent: one CTA per SM
+    if (l.out == kNodes) return launch_bwd_nodes(b, maps, grid, status, st);
+    if (l.out == kFirst) return launch_bwd_first(b, maps, l.results_warps, grid, status, st);
+    if (l.results_warps == 4) return launch_bwd_leaves_d64(b, maps, grid, status, st);
+    if (g.d == 64) return l.out == kBoxes ? go(d64{}, boxes_out{}, grid) : go(d64{}, rows_out{}, grid);
+    return l.out == kBoxes ? go(d128{}, boxes_out{}, grid) : go(d128{}, rows_out{}, grid);
   };
-  cudaError_t e;
-  if (split) {
-    b.total_items = b.n_leaf_items;
-    e = launch_bwd_first(b, maps, backward_build(g, true, false).results_warps, b.total_items < sms ? b.total_items : sms, status, st);
-    if (e != cudaSuccess) return e;
+  if (split) b.total_items = b.n_leaf_items;
+  cudaError_t e = run(launches[0]);
+  if (e == cudaSuccess && split) {
     b.total_items = (int)items - b.n_leaf_items; b.sched = sched + 1; b.a.tail_leaves = 0;
     for (int l = g.levels; l >= 0; --l) b.level_item_start[l] -= b.n_leaf_items;
     b.n_leaf_items = 0;
-    e = run(backward_build(g, false, true));
-  } else e = run(backward_build(g));
+    e = run(launches[1]);
+  }
   if (e != cudaSuccess || !gr.dq16) return e;
   ToBf16Args c;
   const size_t elems[3] = {rows * g.d, gr.kv_elems, gr.kv_elems};

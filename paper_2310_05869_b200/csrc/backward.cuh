@@ -249,10 +249,9 @@ __global__ void __launch_bounds__(256) row_stat_kernel(const uint4* __restrict__
 // kNodes: as kRows, where all items are tiles of sorted nodes.  (The pass, us, kRows -> kNodes, in the case of recursion also kFirst knowing that it has
 // leaves alone: 12 heads of 4096 rows 59.7 -> 58.6, 10 of 20000 194.5 -> 190.4, 32 of 65536 1797 -> 1766, 32 causal of 131072 16199 -> 15871; d =
 // 128, 32 of 32768 1665 -> 1657, 8 causal of 32768 1620 -> 1584.)
-enum BwdOut { kRows, kBoxes, kFirst, kNodes };
 // RW: results warps.  With eight the block has 21 warps, six of them on one quarter of the SM, which leaves 80 registers a thread; with four it has 17
 // and 96.  Whole tiles of consecutive rows need no more than four while they follow one another - a box goes out with a few instructions - and the P
-// warps gain from the registers; scattered rows, and dK and dV of items of few steps, keep eight busy.  (Which build a call takes: backward_build()
+// warps gain from the registers; scattered rows, and dK and dV of items of few steps, keep eight busy.  (Which build a call takes: backward_launches()
 // in backward.cu, with figures.  d = 128 always has eight: 64 leaves of 4096 rows 838 us, with four 998.)
 template <int D, BwdOut OUT, int RW>
 __global__ void __launch_bounds__(Cfg<D, RW>::kThreads, 1) bwd_kernel(const __grid_constant__ BwdArgs b, const __grid_constant__ BwdMaps maps,

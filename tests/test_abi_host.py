@@ -132,24 +132,50 @@ def test_node_projections_match_the_oracle():
     assert not np.array_equal(ha.get_projections(64, 7, 5, node=1), ha.get_projections(64, 7, 5))
 
 
-# (boxes, results warps) by what a call's steps are: whole tiles of 128 consecutive rows, which leave as boxes; short tiles of consecutive
-# rows and tiles of sorted rows, which leave row by row and want eight warps; and how often dK and dV leave (once per key tile)
+# The launches of the backward kernel and their builds, by what a call's steps are: whole tiles of 128 consecutive rows, which leave as boxes; short
+# tiles of consecutive rows and tiles of sorted rows, which leave row by row and want eight results warps; how often dK and dV leave (once per key
+# tile); sorted nodes alone; from 192 MiB of fp32 dK and dV on, leaves that leave as boxes first.  (d = 128 always has eight warps.)
+LEAVES, NODES, ALL = 1, 2, 3
+OUT = ("rows", "boxes", "first", "nodes")
+
+
 @pytest.mark.parametrize("d", [64, 128])
-@pytest.mark.parametrize("kw,boxes,warps", [
-    (dict(n=64, causal=1, n0=64), 0, 8), (dict(n=127, causal=1, n0=128), 0, 8), (dict(n=128, causal=1, n0=128), 0, 8),
-    (dict(n=300, causal=1, n0=512), 0, 8), (dict(n=127, block=128), 0, 8), (dict(n=200, block=256), 0, 8),
-    (dict(n=512, causal=1, n0=512), 1, 8), (dict(n=768, causal=1, n0=768), 1, 8), (dict(n=300, block=512), 1, 8),
-    (dict(n=1536, causal=1, n0=1536), 1, 4), (dict(n=4096, causal=1, n0=4096), 1, 4), (dict(n=4096, block=4096), 1, 4),
-    (dict(n=6400, block=64, causal=1, n0=100), 0, 8), (dict(n=1600, block=800, causal=1, n0=100), 0, 8),
-    (dict(n=32768, block=64, causal=1, n0=512), 0, 8), (dict(n=32768, block=256, samples=256, causal=1, n0=1024), 1, 8),
-    (dict(n=32768, block=256, samples=256, causal=1, n0=2048), 1, 4), (dict(n=131072, block=256, samples=256, causal=1, n0=4096), 1, 4),
-    (dict(n=8192, block=4096, causal=1, n0=512), 1, 4),
-    (dict(n=4096, block=256, samples=256), 0, 8), (dict(n=32768, block=64), 0, 8),
-    # the shapes of test_gpu_kernel_edges.py whose items are more than the SMs: every build of the kernel is run there
-    (dict(H=40, n=640, block=64, samples=33, causal=1, n0=320), 0, 8), (dict(H=110, n=300, block=64, samples=8, causal=1, n0=512), 0, 8),
-    (dict(H=16, n=1400, block=64, samples=33, causal=1, n0=700), 1, 8), (dict(H=4, n=3400, block=64, samples=33, causal=1, n0=1700), 1, 4),
+@pytest.mark.parametrize("kw,out,warps", [
+    (dict(n=64, causal=1, n0=64), "rows", 8), (dict(n=127, causal=1, n0=128), "rows", 8), (dict(n=128, causal=1, n0=128), "rows", 8),
+    (dict(n=300, causal=1, n0=512), "rows", 8), (dict(n=127, block=128), "rows", 8), (dict(n=200, block=256), "rows", 8),
+    (dict(n=512, causal=1, n0=512), "boxes", 8), (dict(n=768, causal=1, n0=768), "boxes", 8), (dict(n=300, block=512), "boxes", 8),
+    (dict(n=1536, causal=1, n0=1536), "boxes", 4), (dict(n=4096, causal=1, n0=4096), "boxes", 4), (dict(n=4096, block=4096), "boxes", 4),
+    (dict(n=6400, block=64, causal=1, n0=100), "rows", 8), (dict(n=1600, block=800, causal=1, n0=100), "rows", 8),
+    (dict(n=32768, block=64, causal=1, n0=512), "rows", 8), (dict(n=32768, block=256, samples=256, causal=1, n0=1024), "boxes", 8),
+    (dict(n=32768, block=256, samples=256, causal=1, n0=2048), "boxes", 4),
+    (dict(H=1, n=131072, block=256, samples=256, causal=1, n0=4096), "boxes", 4),
+    (dict(n=8192, block=4096, causal=1, n0=512), "boxes", 4),
+    (dict(n=4096, block=256, samples=256), "nodes", 8), (dict(n=32768, block=64), "nodes", 8), (dict(H=32, n=131072, block=64), "nodes", 8),
+    (dict(H=128, n=4096, causal=1, n0=4096), "boxes", 4),                  # (leaves alone: everything is written by one launch)
+    # the shapes of test_gpu_kernel_edges.py whose items are more than the SMs: every build of a call in one launch is run there
+    (dict(H=40, n=640, block=64, samples=33, causal=1, n0=320), "rows", 8), (dict(H=110, n=300, block=64, samples=8, causal=1, n0=512), "rows", 8),
+    (dict(H=16, n=1400, block=64, samples=33, causal=1, n0=700), "boxes", 8),
+    (dict(H=4, n=3400, block=64, samples=33, causal=1, n0=1700), "boxes", 4),
 ], ids=lambda x: "_".join(f"{k}{v}" for k, v in x.items()) if isinstance(x, dict) else str(x))
-def test_build_of_the_backward_kernel(d, kw, boxes, warps):
-    got = C.c_int(-1), C.c_int(-1)
-    assert ha.lib().hyperattn_internal_backward_build(C.byref(_params(d=d, **kw)), C.byref(got[0]), C.byref(got[1])) == 0
-    assert (got[0].value, got[1].value) == (boxes, warps if d == 64 else 8)
+def test_build_of_the_backward_kernel(d, kw, out, warps):
+    assert _backward_launches(d=d, **kw) == [(ALL if "causal" in kw and kw["n"] > kw["n0"] else NODES if out == "nodes" else LEAVES,
+                                              out, warps if d == 64 else 8)]
+
+
+# (the first of every shape is the one of test_gpu_kernel_edges.py, where every build of the second launch is run)
+@pytest.mark.parametrize("d,heads,kw,first,second", [
+    (64, (26, 24, 23), dict(n=16384, block=256, n0=4096), 4, ("nodes", 8)), (128, (13, 12, 11), dict(n=16384, block=256, n0=4096), 8, ("nodes", 8)),
+    (64, (26, 24, 23), dict(n=16384, block=512, n0=512), 8, ("rows", 8)), (128, (13, 12, 11), dict(n=16384, block=512, n0=512), 8, ("rows", 8)),
+    (64, (400, 384, 383), dict(n=1024, block=512, n0=512), 8, ("boxes", 8)), (64, (50, 48, 47), dict(n=8192, block=4096, n0=512), 8, ("boxes", 4)),
+    (128, (13, 12, 11), dict(n=16384, block=8192, n0=4096), 8, ("boxes", 8)),
+], ids=lambda x: "_".join(f"{k}{v}" for k, v in x.items()) if isinstance(x, dict) else None)
+def test_builds_of_the_backward_kernel_in_two_launches(d, heads, kw, first, second):
+    for H in heads[:2]:
+        assert _backward_launches(d=d, H=H, causal=1, samples=8, **kw) == [(LEAVES, "first", first), (NODES, *second)]
+    assert [x[0] for x in _backward_launches(d=d, H=heads[2], causal=1, samples=8, **kw)] == [ALL]
+
+
+def _backward_launches(**kw):
+    got = (C.c_int * 7)()
+    assert ha.lib().hyperattn_internal_backward_launches(C.byref(_params(**kw)), got) == 0
+    return [(got[1 + 3 * i], OUT[got[2 + 3 * i]], got[3 + 3 * i]) for i in range(got[0])]

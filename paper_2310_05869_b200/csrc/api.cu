@@ -535,6 +535,15 @@ int hyperattn_internal_backward_launches(const hyperattn_params* p, int out[7]) 
   return HYPERATTN_OK;
 }
 
+// (for the tests) rows per chunk of the hash and the sort
+int hyperattn_internal_chunk_rows(const hyperattn_params* p, int* rows) {
+  if (!p || !rows) return HYPERATTN_INVALID_ARGUMENT;
+  Geometry g;
+  const int rc = build_geometry(*p, g);
+  if (rc == HYPERATTN_OK) *rows = g.chunk;
+  return rc;
+}
+
 int hyperattn_backward_workspace_bytes(const hyperattn_params* p, int grad_dtype, size_t* bytes) {
   if (!p || !bytes) return HYPERATTN_INVALID_ARGUMENT;
   Geometry g;

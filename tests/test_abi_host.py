@@ -153,7 +153,7 @@ OUT = ("rows", "boxes", "first", "nodes")
     (dict(n=4096, block=256, samples=256), "nodes", 8), (dict(n=32768, block=64), "nodes", 8), (dict(H=32, n=131072, block=64), "nodes", 8),
     (dict(H=128, n=4096, causal=1, n0=4096), "boxes", 4),                  # (leaves alone: everything is written by one launch)
     # the shapes of test_gpu_kernel_edges.py whose items are more than the SMs: every build of a call in one launch is run there
-    (dict(H=40, n=640, block=64, samples=33, causal=1, n0=320), "rows", 8), (dict(H=110, n=300, block=64, samples=8, causal=1, n0=512), "rows", 8),
+    (dict(H=40, n=640, block=64, samples=33, causal=1, n0=320), "rows", 8), (dict(H=210, n=300, block=64, samples=8, causal=1, n0=512), "rows", 8),
     (dict(H=16, n=1400, block=64, samples=33, causal=1, n0=700), "boxes", 8),
     (dict(H=4, n=3400, block=64, samples=33, causal=1, n0=1700), "boxes", 4),
 ], ids=lambda x: "_".join(f"{k}{v}" for k, v in x.items()) if isinstance(x, dict) else str(x))

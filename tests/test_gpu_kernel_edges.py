@@ -1,4 +1,5 @@
 """Sizes at the edges of the kernels' tiles, chunks and dispatch rules, against the oracle."""
+import ctypes as C
 import math
 
 import numpy as np
@@ -6,6 +7,7 @@ import pytest
 import torch
 
 import paper_2310_05869_b200 as ha
+from paper_2310_05869_b200 import binding as B
 from paper_2310_05869_b200 import workloads as WL
 from oracle import hyperattn_oracle as O
 
@@ -39,8 +41,8 @@ FORWARD = [
     parity.W("no_samples_seven_key_tiles_d64", 1, 2, 1000, 64, "bf16", 448, 0, 6, False, 0, seed=98, n_k=4000),
     parity.W("no_samples_three_key_tiles_d128", 1, 2, 1300, 128, "bf16", 192, 0, 6, False, 0, seed=99, n_k=2000),
     parity.W("no_samples_two_key_tiles_causal_d128", 1, 2, 4096, 128, "bf16", 128, 0, 6, True, 512, seed=100),
-    # leaves alone: the last 148 go rank by rank, the ones before leaf by leaf
-    parity.W("leaves_for_more_than_two_rounds", 1, 160, 300, 64, "bf16", 64, 8, 4, True, 512, seed=102),
+    # leaves alone, two pairs of query tiles each: the last 296 (four rounds of 148 SMs) go rank by rank, the ones before leaf by leaf
+    parity.W("leaves_for_more_than_four_rounds", 1, 310, 300, 64, "bf16", 64, 8, 4, True, 512, seed=102),
     # fp32: hash passes of 256 rows; copies beside the hash (up to 296 CTAs of 4096 entries) and in a launch of their own; query tiles
     # halved (up to 74 tiles) and whole, second halves of one row and none
     parity.W("fp32_n257_d64", 1, 1, 257, 64, "fp32", 64, 32, 7, False, 0, seed=76),
@@ -101,15 +103,21 @@ def test_host_buffers_in_groups_give_the_same_bits(H, n, n_k, d, b, m, dtype, kw
     assert ha.last_device_status() == 0
 
 
-# the permutations are stable sorts of the bucket ids: chunks of 256, 512, 1024, 1280, 1792 and 2048 rows, whole and short ranges of a
-# warp, hash widths of 1 and 8 bits, and rows that are all equal
-SORTED = [("random", 1, 1000, 1000, 64, 7, False, 0), ("random", 20, 3999, 3999, 64, 8, False, 0), ("random", 32, 4096, 1030, 64, 1, False, 0),
-          ("random", 16, 9000, 9000, 64, 7, True, 4096), ("random", 4, 100003, 100003, 64, 7, True, 4096), ("random", 40, 16384, 16384, 64, 8, False, 0),
-          ("equal", 2, 5000, 5000, 128, 7, False, 0), ("equal", 40, 9000, 9000, 64, 7, True, 2500)]
+# the permutations are stable sorts of the bucket ids: rows of a chunk, whole and short ranges of a warp, hash widths of 1 and 8 bits, and rows that
+# are all equal
+SORTED = [(256, "random", 1, 1000, 1000, 64, 7, False, 0), (512, "random", 20, 3999, 3999, 64, 8, False, 0),
+          (512, "random", 32, 4096, 1030, 64, 1, False, 0), (768, "random", 64, 1500, 1500, 64, 7, False, 0),
+          (1024, "random", 32, 4096, 4096, 64, 7, False, 0), (1280, "random", 16, 9000, 9000, 64, 7, True, 4096),
+          (1536, "random", 32, 4600, 4600, 64, 7, False, 0), (1792, "random", 4, 100003, 100003, 64, 7, True, 4096),
+          (2048, "random", 40, 16384, 16384, 64, 8, False, 0), (256, "equal", 2, 5000, 5000, 128, 7, False, 0),
+          (1280, "equal", 40, 9000, 9000, 64, 7, True, 2500)]
 
 
-@pytest.mark.parametrize("kind,H,n,n_k,d,r,causal,n0", SORTED)
-def test_permutations_are_stable_sorts_of_the_ids(kind, H, n, n_k, d, r, causal, n0):
+@pytest.mark.parametrize("chunk,kind,H,n,n_k,d,r,causal,n0", SORTED)
+def test_permutations_are_stable_sorts_of_the_ids(chunk, kind, H, n, n_k, d, r, causal, n0):
+    p, rows = B._Params(), C.c_int(0)
+    B._fill(p, 1, H, n, d, 128, 32, r, causal, n0, 5, B.BF16, B.BF16, 0.0, n_k)
+    assert ha.lib().hyperattn_internal_chunk_rows(C.byref(p), C.byref(rows)) == 0 and rows.value == chunk
     gen = torch.Generator(device="cuda")
     gen.manual_seed(11)
     q, k, v = (torch.randn(1, H, rows, d, generator=gen, device="cuda").bfloat16() for rows in (n, n_k, n_k))
@@ -139,7 +147,10 @@ def test_permutations_are_stable_sorts_of_the_ids(kind, H, n, n_k, d, r, causal,
 # calls large enough for sorted nodes and everything else in launches of their own, against calls of few heads in one launch: the same bits
 TWO_LAUNCHES = [(64, 64, 2048, 256, torch.bfloat16, {}), (64, 40, 128, 256, torch.bfloat16, {}), (64, 64, 2048, 256, torch.float32, dict(precise=True)),
                 (128, 64, 2048, 256, torch.bfloat16, {}), (128, 64, 2048, 250, torch.float32, {}), (128, 64, 2048, 256, torch.float32, dict(precise=True)),
-                (64, 64, 2048, 256, torch.bfloat16, dict(caps=(8.0, 16.0))), (128, 64, 2048, 256, torch.float32, dict(value_norm_sampling=True))]
+                (64, 64, 2048, 256, torch.bfloat16, dict(caps=(8.0, 16.0))), (128, 64, 2048, 256, torch.bfloat16, dict(caps=(8.0, 16.0))),
+                (128, 64, 2048, 256, torch.float32, dict(caps=(8.0, 16.0))), (64, 64, 2048, 256, torch.bfloat16, dict(value_norm_sampling=True)),
+                (128, 64, 2048, 256, torch.bfloat16, dict(value_norm_sampling=True)),
+                (128, 64, 2048, 256, torch.float32, dict(value_norm_sampling=True))]
 
 
 @pytest.mark.parametrize("d,H,n0,b,out_dtype,option", TWO_LAUNCHES)
@@ -162,25 +173,49 @@ def test_nodes_and_leaves_in_launches_of_their_own(d, H, n0, b, out_dtype, optio
     assert ha.last_device_status() == 0
 
 
-# calls whose leaves go first and write dK and dV (from 192 MiB of fp32 accumulators on), against calls of few heads, which add everything
-SPLIT_BACKWARD = [(64, 26, 16384, 4096), (64, 26, 16800, 2100), (64, 40, 10240, 700), (128, 13, 16384, 4096)]
+# calls whose leaves go first and write dK and dV (from 192 MiB of fp32 accumulators on), against calls of few heads, which add everything; in the
+# second launch sorted nodes alone, or others too, in each build (test_abi_host.py holds these shapes to the builds)
+SPLIT_BACKWARD = [(64, 26, 16384, 4096, 256), (64, 26, 16800, 2100, 256), (64, 40, 10240, 700, 256), (128, 13, 16384, 4096, 256),
+                  (64, 26, 16384, 512, 512), (64, 400, 1024, 512, 512), (64, 50, 8192, 512, 4096), (128, 13, 16384, 512, 512), (128, 13, 16384, 4096, 8192)]
 
 
-@pytest.mark.parametrize("d,H,n,n0", SPLIT_BACKWARD)
+def _backward_in_a_workspace(q, k, v, out, lse, dout, block, samples, r, grad_dtype, n0, seed):
+    """The causal backward pass with every byte of its workspace and of the gradients set to 0xff (a NaN), and its launches of all kinds."""
+    _, H, n, d = q.shape
+    p = B._Params()
+    B._fill(p, 1, H, n, d, block, samples, r, True, n0, seed, B.BF16, B.BF16, 0.0, n)
+    need, code = C.c_size_t(0), B._dtype_code(grad_dtype)
+    assert ha.lib().hyperattn_backward_workspace_bytes(C.byref(p), code, C.byref(need)) == 0
+    ws = torch.full((need.value,), 0xff, dtype=torch.uint8, device="cuda")
+    grads = [torch.full(q.shape, math.nan, dtype=grad_dtype, device="cuda") for _ in range(3)]
+    p.q, p.k, p.v, p.out, p.lse = (x.data_ptr() for x in (q, k, v, out, lse))
+    p.workspace, p.workspace_bytes, p.stream = ws.data_ptr(), need.value, torch.cuda.current_stream().cuda_stream
+    g = B._Grads(dout.data_ptr(), *(x.data_ptr() for x in grads), code)
+    ha.profile_reset()
+    ha.profile_enable(True)
+    rc = ha.lib().hyperattn_backward(C.byref(p), C.byref(g))
+    torch.cuda.synchronize()
+    ha.profile_enable(False)
+    launches = ha.profile_read()["launches"]["backward"]
+    ha.profile_reset()
+    assert rc == 0
+    return grads, launches
+
+
+@pytest.mark.parametrize("d,H,n,n0,block", SPLIT_BACKWARD)
 @pytest.mark.parametrize("grad_dtype", [torch.float32, torch.bfloat16])
-def test_backward_with_leaves_in_a_launch_of_their_own(d, H, n, n0, grad_dtype):
+def test_backward_with_leaves_in_a_launch_of_their_own(d, H, n, n0, block, grad_dtype):
     assert 8 * H * n * d >= 192 << 20
     gen = torch.Generator(device="cuda")
     gen.manual_seed(13)
     q, k, v, dout = (torch.randn(1, H, n, d, generator=gen, device="cuda").bfloat16() for _ in range(4))
-    args, kw = (256, 128, 6), dict(causal=True, n0=n0, seed=4)
-    out, lse = ha.forward(q, k, v, *args, **kw)
-    stale = [torch.full((1, H, n, d), float("nan"), dtype=grad_dtype, device="cuda") for _ in range(3)]
-    del stale                                              # (the gradients' memory holds NaN)
-    got = ha.backward(q, k, v, out, lse, dout, *args, grad_dtype=grad_dtype, **kw)
+    args = (block, 128 if block < 1024 else 8, 6)
+    out, lse = ha.forward(q, k, v, *args, causal=True, n0=n0, seed=4)
+    got, launches = _backward_in_a_workspace(q, k, v, out, lse, dout, *args, grad_dtype, n0, 4)
     few = 2
     part = [x[:, :few].contiguous() for x in (q, k, v, out, lse, dout)]
-    want = ha.backward(*part, *args, grad_dtype=grad_dtype, **kw)
+    want, launches_few = _backward_in_a_workspace(*part, *args, grad_dtype, n0, 4)
+    assert launches == launches_few + 1
     for x, y in zip(got, want):
         # the same terms in another order: at most 200 partial sums of fp32 (2 x 200 x 2^-24 of the terms' absolute values, which add up to a few
         # times the largest entry), and bf16 results may be a step apart (2^(e - 7) for 2^e <= |y|)
@@ -208,7 +243,8 @@ BACKWARD = [
     backward.W("bwd_leaf_of_193_rows_d128", 1, 1, 193, 128, 64, 8, 4, True, 200, seed=80),
     backward.W("bwd_sorted_over_unsorted_nodes_d64", 1, 2, 1040, 64, 200, 33, 6, True, 130, seed=81),
     backward.W("bwd_sorted_over_unsorted_nodes_d128", 1, 1, 1040, 128, 200, 33, 6, True, 130, seed=82),
-    backward.W("bwd_leaves_for_more_than_two_rounds_d64", 1, 110, 300, 64, 64, 8, 4, True, 512, seed=85),
+    # leaves alone, three key tiles each: the last 198 go rank by rank
+    backward.W("bwd_leaves_for_more_than_four_rounds_d64", 1, 210, 300, 64, 64, 8, 4, True, 512, seed=85),
     # more items than SMs, so that whole tiles of consecutive rows, short ones and scattered rows follow one another in a CTA, in every build
     # of the kernel (test_abi_host.py holds these shapes to the builds): without boxes ...
     backward.W("bwd_whole_short_and_scattered_tiles_d64", 1, 40, 640, 64, 64, 33, 6, True, 320, seed=83),

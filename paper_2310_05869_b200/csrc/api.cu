@@ -82,7 +82,11 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
   // costs as much as 256 rows beside its own, and one alone on an SM as much as two - and evened out over the unit: 2250 rows are two chunks of at
   // most 1280, not one of 2048 and one of 202.  A call, us, halved below 296 CTAs whatever the share and not evened -> this rule: 32 heads x 4096 rows
   // (256 CTAs instead of 512) 56.5 -> 55.4, 13 x 9333 58.8 -> 54.7, 21 x 6001 56.6 -> 55.9, 16 causal x 9000 139.1 -> 138.5; d = 128, 32 x 4096 78.9 ->
-  // 74.3, 17 x 8192 82.9 -> 78.4, 35 x 8192 (280 instead of 560) 155.5 -> 150.3, but at d = 64 101.3 -> 102.2; hash of 4 causal x 100003 25.6 -> 22.9.
+  // 74.3, 17 x 8192 82.9 -> 78.4, 35 x 8192 (280 instead of 560) 155.5 -> 150.3; hash of 4 causal x 100003 25.6 -> 22.9.
+  // At d = 64 a CTA of 2048 rows is short enough that four of half the rows on an SM, which wait less, are better than two: the first halving is
+  // taken where the busiest SM gets no more rows by it, and where the sort keeps to one launch.  Without -> with: 35 x 8192 98.5 -> 96.9, 64 x 4096
+  // 91.0 -> 89.3, 48 x 6000 99.8 -> 97.1, 17 x 16384 96.0 -> 94.9, 30 causal x 7687 269.3 -> 266.9, by value norms 35 x 8192 122.8 -> 121.7; more rows
+  // (60 x 2500, 1280 -> 3 x 1024) 63.1 -> 64.3, a launch more (9 x 30000) 94.7 -> 97.1.
   // Beyond two CTAs for an SM: 38 x 8192 112.0 -> 111.4 halved, but 50000 queries x 131072 keys 138.7 -> 141.5 (twice the chunks to scan).
   auto even = [&](int chunk) {
     auto side = [&](int unit) { const int k = (unit + chunk - 1) / chunk; return ((unit + k - 1) / k + 255) / 256 * 256; };
@@ -92,21 +96,27 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
     const long long units = g.npad / g.unit, cpu = (g.unit + chunk - 1) / chunk, cpu_k = (g.unit_k + chunk - 1) / chunk;
     return g.G * units * cpu + g.G * (g.causal ? units : 1) * cpu_k;
   };
-  auto share = [&](int chunk) {
+  auto share = [&](int chunk, int start) {              // rows of the busiest SM, a CTA's start counted as `start` of them
     const long long per_sm = (hash_ctas(chunk) + kSms - 1) / kSms;
-    return (chunk + 256) * (per_sm < 2 ? 2 : per_sm);
+    return (chunk + start) * (per_sm < 2 ? 2 : per_sm);
   };
-  g.chunk = even(kSortChunk);
-  for (int half = kSortChunk / 2; half >= 256 && hash_ctas(g.chunk) < 2 * kSms; half /= 2) {
-    const int chunk = even(half);
-    if (chunk == g.chunk) continue;
-    if (share(chunk) >= share(g.chunk)) break;
+  auto take = [&](int chunk) {
     g.chunk = chunk;
+    g.chunks_per_unit = (g.unit + g.chunk - 1) / g.chunk;
+    g.chunks_per_seg = (g.npad / g.unit) * g.chunks_per_unit;
+    g.chunks_per_unit_k = (g.unit_k + g.chunk - 1) / g.chunk;
+    g.chunks_per_seg_k = g.causal ? g.chunks_per_seg : g.chunks_per_unit_k;
+  };
+  take(even(kSortChunk));
+  for (int half = kSortChunk / 2; half >= 256 && hash_ctas(g.chunk) < 2 * kSms; half /= 2) {
+    const int chunk = even(half), last = g.chunk;
+    if (chunk == last) continue;
+    take(chunk);
+    if (share(chunk, 256) < share(last, 256)) continue;
+    if (g.d == 64 && half == kSortChunk / 2 && share(chunk, 0) <= share(last, 0) && scan_in_scatter(g)) continue;
+    take(last);
+    break;
   }
-  g.chunks_per_unit = (g.unit + g.chunk - 1) / g.chunk;
-  g.chunks_per_seg = (g.npad / g.unit) * g.chunks_per_unit;
-  g.chunks_per_unit_k = (g.unit_k + g.chunk - 1) / g.chunk;
-  g.chunks_per_seg_k = g.causal ? g.chunks_per_seg : g.chunks_per_unit_k;
   return HYPERATTN_OK;
 }
 

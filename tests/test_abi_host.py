@@ -175,6 +175,22 @@ def test_builds_of_the_backward_kernel_in_two_launches(d, heads, kw, first, seco
     assert [x[0] for x in _backward_launches(d=d, H=heads[2], causal=1, samples=8, **kw)] == [ALL]
 
 
+# Rows per chunk: evened out over the unit; halved where the busiest SM gets less to do, and at d = 64 from 2048 rows also where it gets as much and
+# the sort keeps to one launch (nodes of up to 16 chunks)
+@pytest.mark.parametrize("kw,d64,d128", [
+    (dict(H=1, n=1000), 256, 256), (dict(H=32, n=4096), 1024, 1024), (dict(H=40, n=16384), 2048, 2048),
+    (dict(H=35, n=8192), 1024, 2048), (dict(H=64, n=4096), 1024, 2048), (dict(H=17, n=16384), 1024, 2048), (dict(H=30, n=7687, causal=1, n0=4096), 1024, 2048),
+    (dict(H=9, n=30000), 2048, 2048), (dict(H=8, n=32800), 2048, 2048),         # ... nodes of more than 16 chunks
+    (dict(H=60, n=2500), 1280, 1280),                                            # ... more rows for the busiest SM
+    (dict(H=37, n=8192), 2048, 2048),                                            # ... two CTAs for an SM
+])
+def test_rows_per_chunk(kw, d64, d128):
+    for d, want in ((64, d64), (128, d128)):
+        rows = C.c_int(0)
+        assert ha.lib().hyperattn_internal_chunk_rows(C.byref(_params(d=d, **kw)), C.byref(rows)) == 0
+        assert rows.value == want, d
+
+
 def _backward_launches(**kw):
     got = (C.c_int * 7)()
     assert ha.lib().hyperattn_internal_backward_launches(C.byref(_params(**kw)), got) == 0

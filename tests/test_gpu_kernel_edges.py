@@ -106,10 +106,10 @@ def test_host_buffers_in_groups_give_the_same_bits(H, n, n_k, d, b, m, dtype, kw
 # the permutations are stable sorts of the bucket ids: rows of a chunk, whole and short ranges of a warp, hash widths of 1 and 8 bits, and rows that
 # are all equal
 SORTED = [(256, "random", 1, 1000, 1000, 64, 7, False, 0), (512, "random", 20, 3999, 3999, 64, 8, False, 0),
-          (512, "random", 32, 4096, 1030, 64, 1, False, 0), (768, "random", 64, 1500, 1500, 64, 7, False, 0),
-          (1024, "random", 32, 4096, 4096, 64, 7, False, 0), (1280, "random", 16, 9000, 9000, 64, 7, True, 4096),
-          (1536, "random", 32, 4600, 4600, 64, 7, False, 0), (1792, "random", 4, 100003, 100003, 64, 7, True, 4096),
-          (2048, "random", 40, 16384, 16384, 64, 8, False, 0), (256, "equal", 2, 5000, 5000, 128, 7, False, 0),
+          (512, "random", 32, 4096, 1030, 64, 1, False, 0), (768, "random", 64, 1500, 1500, 64, 7, False, 0), (1280, "random", 60, 2500, 2500, 64, 7, False, 0),
+          (1024, "random", 32, 4096, 4096, 64, 7, False, 0), (768, "random", 16, 9000, 9000, 64, 7, True, 4096),
+          (1536, "random", 32, 4600, 4600, 128, 7, False, 0), (1792, "random", 4, 100003, 100003, 64, 7, True, 4096),
+          (1024, "random", 17, 16384, 16384, 64, 7, False, 0), (2048, "random", 40, 16384, 16384, 64, 8, False, 0), (256, "equal", 2, 5000, 5000, 128, 7, False, 0),
           (1280, "equal", 40, 9000, 9000, 64, 7, True, 2500)]
 
 

@@ -1,8 +1,8 @@
 // Attention tiles on the 5th-generation tensor cores (tcgen05 + TMEM), bf16 inputs.
 //
-// One CTA owns a PAIR of query tiles (2 x 128 rows) that are neighbours in the tile order of
-// their leaf / recursion node, and walks once over the key tiles (64 keys each) that either
-// of them needs:
+// A work item is a PAIR of query tiles (2 x 128 rows) that are neighbours in the tile order of
+// their leaf / recursion node - or one of the two, where the last pairs of a call are split - and a
+// CTA walks once over the key tiles (64 keys each) that either of them needs:
 //     S_i = Q_i K^T      tcgen05.mma, operands in 128B-swizzled shared memory (d = 64: Q_i from TMEM), S_i in TMEM
 //     P_i = exp2(S_i*c + bias - m)   softmax warpgroup i: one thread per query row (TMEM
 //                                    lane); P_i is written back over S_i as bf16
@@ -338,7 +338,7 @@ __device__ __forceinline__ int tile_of(const QTile& q, int a) { return a < q.n1 
 // kDenseItems: leaves, and nodes that are not sorted; kAnyItems: all of these.  What a build does not need is not in the way of the softmax warps: calls,
 // us, in a build for everything -> in its own: 32 heads of 4096 rows 55.2 -> 52.9, 12 of 4096 33.6 -> 31.9, 32 of 16384 173.7 -> 167.5, 32 of 131072
 // 1289 -> 1229-1253; d = 128, 32 of 32768 516 -> 497-503; by value norms, 50000 queries and 131072 keys, 4 heads 129.2 -> 121.8; leaves alone, 128 of
-// 4096 422 -> 413, d = 128, 64 of 4096 313 -> 302.
+// 4096 422 -> 413, d = 128, 64 of 4096 313 -> 302.  (kPartialNodes beside kDenseItems: see kTwoLaunches.)
 enum SampleRule { kUniform, kCapped, kWeighted };
 enum ItemKind { kAnyItems, kFinalNodes, kPartialNodes, kDenseItems };
 template <int D, bool GATHER_LATE, bool PRECISE, SampleRule RULE, ItemKind KIND>
@@ -417,8 +417,8 @@ __global__ void __launch_bounds__(384, 1) attn_tc_kernel(const __grid_constant__
   const uint32_t tmem = __shfl_sync(0xffffffffu, *s_tmem, 0);
   wait_for_stream();
 
-  // The CTA is persistent: it walks over work items (pairs of query tiles) blockIdx.x,
-  // blockIdx.x + gridDim.x, ...  Every role runs the same item loop at its own pace; what
+  // The CTA is persistent: it takes work items (pairs of query tiles) from the launch's counter
+  // until the list is exhausted.  Every role runs the same item loop at its own pace; what
   // they hand to each other across items is described at the barriers above.  All phase
   // counters keep running across items.
   if (warp < 8) {
@@ -1407,7 +1407,9 @@ void sorted_pairs(const AttnArgs& a, int& first, int& end) {
 // A call with recursion gains by two launches what their own builds are faster by, about 2 %, and loses the end of the first launch and the heavy items at
 // the end of the second, 10 to 15 us: from 64 pairs of query tiles for an SM on.  (Calls, us, one launch -> two: 32 heads of 131072 rows, 387 pairs
 // for an SM, 6636 -> 6476, d = 128, split weights, 64 of 16384, 69 pairs, 1976 -> 1944; 4 of 100003, 38 pairs, 592 -> 593, 8 of 50000, 32 pairs, 537 -> 542,
-// d = 128, 8 of 32768, 17 pairs, 514 -> 530, 16 of 9000, 8 pairs, 138 -> 149.)
+// d = 128, 8 of 32768, 17 pairs, 514 -> 530, 16 of 9000, 8 pairs, 138 -> 149.  Capped and weighted columns, 69 pairs, 32 of 32768: caps 1951 -> 1814, value
+// norms 1507 -> 1403, d = 128 caps 3002 -> 2915, fp32 results 3303 -> 3254, value norms 2192 -> 2091, fp32 results 2482 -> 2417; 139 pairs, 64 of 32768: caps
+// 3809 -> 3534, value norms 3036 -> 2822.)
 constexpr int kTwoLaunches = 64;
 bool attention_in_two(const AttnArgs& a) {
   int first, end, sms = 0;

@@ -58,12 +58,13 @@ struct BwdArgs {
   AttnArgs a;                  // geometry, permutations, samples
   const __nv_bfloat16* dout;   // [G, n, D]
   const float2* stat;          // [G, n] (-lse log2 e, -<dO, O>) of the rows
-  float *dq, *dk, *dv;         // fp32 accumulators, cleared by row_stat_kernel: [G, n, D]; direct: dk and dv [G, m, D], of the samples
+  float *dq, *dk, *dv;         // fp32 accumulators: [G, n, D]; direct: dk and dv [G, m, D], of the samples.  Cleared by row_stat_kernel, but for dk and
+                               // dv that the leaves write in a launch before the nodes' (kFirst)
   __nv_bfloat16 *dk16, *dv16;  // direct: dK and dV of the keys without samples
   const int32_t* key_slot;     // direct: [G, n] the sample that stands for a key, -1: none (null: none for any)
   int direct;
   float scale;
-  int* sched;                  // work counter of the launch, zero at launch
+  int* sched;                  // work counter of the launch (each launch of a call has its own), zero at launch
   // items: the key tiles of the leaves, then level by level those of the nodes
   int leaf_ktiles, n_leaf_items;
   int level_item_start[kMaxLevels + 1];

@@ -181,7 +181,7 @@ struct Workspace {
   float* ltau;                     // capped row sums: [G, nodes] log2 of the largest unmasked probe row sum
   void* part_o; float* part_lse;   // causal partials: leaf [G,n,(d)] then per level [G,nl,(d)]; rows of fp32 or bf16
   int part_bf16;
-  int* sched;                      // work counter of the attention launch: zeroed by the first launch of the sort
+  int* sched;                      // work counters of the attention's launches (up to two): zeroed by the first launch of the sort
   int* status;                     // device status word
 };
 

@@ -37,12 +37,12 @@ from paper_2310_05869_b200 import workloads as WL  # noqa: E402
 WORKLOADS = {"c1": 0, "c2": 1, "c3": 2, "c4": 3, "c5": 4}
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the attention kernel,
-# from the ncu captures summarised under profiles/ (taken on 4 / 8 heads and scaled to the
-# workload's 32 heads: the traffic is proportional to the number of segments).
-NCU_TRAFFIC_BYTES = {"c3_n131k_causal": 8 * 0.9267e9, "c2_n32k_d128": 4 * 0.2438e9}
-# sm__pipe_tensor_cycles_active (% of peak sustained active) of the attention kernel in the same captures
-NCU_TENSOR_PIPE_PCT = {"c3_n131k_causal": 33.3, "c2_n32k_d128": 34.0}
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of the attention stage of a call, from the ncu captures
+# summarised under profiles/ (taken on 6 / 8 heads and scaled to the workload's 32: the traffic is proportional to the
+# number of segments).  The causal workload's stage is two launches, of the sorted nodes and of the leaves.
+NCU_TRAFFIC_BYTES = {"c3_n131k_causal": 32 / 6 * 1.3954e9, "c2_n32k_d128": 4 * 0.2433e9}
+# sm__pipe_tensor_cycles_active (% of peak sustained active) in the same captures; the two launches (30.5, 37.5) weighted by time
+NCU_TENSOR_PIPE_PCT = {"c3_n131k_causal": 34.5, "c2_n32k_d128": 36.8}
 
 
 def load_peaks():
@@ -255,7 +255,7 @@ def stage_report(w, peaks, stage_ms):
                 "peak": burst, "unit": "TFLOP/s", "frac": att_tflops / burst,
                 "peak_source": f"bf16_tflops (burst) of {peaks['source']}",
                 "frac_of_sustained_peak": att_tflops / sustained, "sustained_peak": sustained,
-                "ms_per_launch": att_ms, "traffic": NCU_TRAFFIC_BYTES.get(w.name),
+                "ms_per_call": att_ms, "traffic": NCU_TRAFFIC_BYTES.get(w.name),
                 "tensor_pipe_active_pct": NCU_TENSOR_PIPE_PCT.get(w.name),
                 "counters_from": "ncu capture on a reduced-head slice, see profiles/"}
     kernels = {}

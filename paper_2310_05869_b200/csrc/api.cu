@@ -87,6 +87,10 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
   // taken where the busiest SM gets no more rows by it, and where the sort keeps to one launch.  Without -> with: 35 x 8192 98.5 -> 96.9, 64 x 4096
   // 91.0 -> 89.3, 48 x 6000 99.8 -> 97.1, 17 x 16384 96.0 -> 94.9, 30 causal x 7687 269.3 -> 266.9, by value norms 35 x 8192 122.8 -> 121.7; more rows
   // (60 x 2500, 1280 -> 3 x 1024) 63.1 -> 64.3, a launch more (9 x 30000) 94.7 -> 97.1.
+  // fp32 inputs: the hash goes through a chunk 256 rows at a time, and a pass costs as much as 128 rows beside its own, so more CTAs pay than for bf16 -
+  // unless the sort needs a launch more for them, or the scan gets long (nodes of more than 64 chunks).  Without -> with: 20 heads x 2349 rows 56.9 ->
+  // 55.9, 10 x 4000 54.8 -> 53.9, 50 x 700 53.2 -> 51.5, d = 128, 20 x 2349 110.9 -> 108.2, 4 x 10000 107.4 -> 105.8, 20 causal x 3000 250.3 -> 242.4,
+  // but 22 x 1700 95.7 -> 97.2; a launch more (12 x 5000) 73.8 -> 81.1, nodes of 79 chunks (2 x 20000) 58.5 -> 59.9.
   // Beyond two CTAs for an SM: 38 x 8192 112.0 -> 111.4 halved, but 50000 queries x 131072 keys 138.7 -> 141.5 (twice the chunks to scan).
   auto even = [&](int chunk) {
     auto side = [&](int unit) { const int k = (unit + chunk - 1) / chunk; return ((unit + k - 1) / k + 255) / 256 * 256; };
@@ -96,9 +100,14 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
     const long long units = g.npad / g.unit, cpu = (g.unit + chunk - 1) / chunk, cpu_k = (g.unit_k + chunk - 1) / chunk;
     return g.G * units * cpu + g.G * (g.causal ? units : 1) * cpu_k;
   };
-  auto share = [&](int chunk, int start) {              // rows of the busiest SM, a CTA's start counted as `start` of them
+  auto share = [&](int chunk, int cost) {               // of the busiest SM, a CTA's share being `cost` rows
     const long long per_sm = (hash_ctas(chunk) + kSms - 1) / kSms;
-    return (chunk + start) * (per_sm < 2 ? 2 : per_sm);
+    return cost * (per_sm < 2 ? 2 : per_sm);
+  };
+  auto fp32_share = [&](int chunk) {
+    auto longest = [&](int unit) { const int k = (unit + chunk - 1) / chunk; return (unit + k - 1) / k; };
+    const int rows = longest(g.unit) > longest(g.unit_k) ? longest(g.unit) : longest(g.unit_k);
+    return share(chunk, rows + 128 * ((rows + 255) / 256));
   };
   auto take = [&](int chunk) {
     g.chunk = chunk;
@@ -107,13 +116,16 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
     g.chunks_per_unit_k = (g.unit_k + g.chunk - 1) / g.chunk;
     g.chunks_per_seg_k = g.causal ? g.chunks_per_seg : g.chunks_per_unit_k;
   };
+  const bool fp32 = p.dtype == HYPERATTN_FP32;
   take(even(kSortChunk));
   for (int half = kSortChunk / 2; half >= 256 && hash_ctas(g.chunk) < 2 * kSms; half /= 2) {
     const int chunk = even(half), last = g.chunk;
     if (chunk == last) continue;
+    const bool one_launch = scan_in_scatter(g);
     take(chunk);
-    if (share(chunk, 256) < share(last, 256)) continue;
-    if (g.d == 64 && half == kSortChunk / 2 && share(chunk, 0) <= share(last, 0) && scan_in_scatter(g)) continue;
+    if (share(chunk, chunk + 256) < share(last, last + 256)) continue;
+    if (fp32 ? fp32_share(chunk) < fp32_share(last) && (one_launch ? scan_in_scatter(g) : node_chunks(g) <= 64)
+             : g.d == 64 && half == kSortChunk / 2 && share(chunk, chunk) <= share(last, last) && scan_in_scatter(g)) continue;
     take(last);
     break;
   }

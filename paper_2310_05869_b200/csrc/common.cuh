@@ -199,6 +199,7 @@ cudaError_t launch_hash(const Geometry& g, const void* q, const void* k, int is_
 cudaError_t launch_sort_scan(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask = 3,
                              const VnormArgs* vnorm = nullptr);
 bool wide_scan(const Geometry& g);
+int node_chunks(const Geometry& g);      // chunks of the longest node
 bool scan_in_scatter(const Geometry& g);
 // (small nodes: the scatter does the scan's work, samples included, and launch_sort_scan launches nothing)
 cudaError_t launch_sort_scatter(const Geometry& g, const Workspace& ws, bool with_samples, uint64_t seed, cudaStream_t st, int side_mask = 3);

@@ -320,10 +320,10 @@ static SortArgs make_sort_args(const Geometry& g, const Workspace& ws, int side_
 // 32 heads, 8 chunks 171.9 -> 169.7, 16 322.3 -> 322.0, 24 486 -> 490, 64 1243 -> 1259; 4 causal heads, nodes of 32 chunks
 // 825 -> 830.  The line is where it stops paying with many heads; a few heads would gain 2-3 us beyond it as well.
 constexpr int kScanChunks = 16;
-bool scan_in_scatter(const Geometry& g) {
-  const int most = g.causal ? (g.nl / g.unit) * g.chunks_per_unit : (g.chunks_per_seg > g.chunks_per_seg_k ? g.chunks_per_seg : g.chunks_per_seg_k);
-  return most <= kScanChunks;
+int node_chunks(const Geometry& g) {
+  return g.causal ? (g.nl / g.unit) * g.chunks_per_unit : (g.chunks_per_seg > g.chunks_per_seg_k ? g.chunks_per_seg : g.chunks_per_seg_k);
 }
+bool scan_in_scatter(const Geometry& g) { return node_chunks(g) <= kScanChunks; }
 
 // Four groups of threads per node while every node has an SM of its own.  (A call, us, one group -> four: 4 heads of 40000 rows, 8 nodes of 20
 // chunks, 74.0 -> 73.2; 4 causal heads of 100003 rows, 248 nodes, 592 -> 597.)

@@ -176,7 +176,8 @@ def test_builds_of_the_backward_kernel_in_two_launches(d, heads, kw, first, seco
 
 
 # Rows per chunk: evened out over the unit; halved where the busiest SM gets less to do, and at d = 64 from 2048 rows also where it gets as much and
-# the sort keeps to one launch (nodes of up to 16 chunks)
+# the sort keeps to one launch (nodes of up to 16 chunks); fp32 inputs, whose hash works in passes of 256 rows, by the passes, to as many launches
+# and nodes of up to 64 chunks
 @pytest.mark.parametrize("kw,d64,d128", [
     (dict(H=1, n=1000), 256, 256), (dict(H=32, n=4096), 1024, 1024), (dict(H=40, n=16384), 2048, 2048),
     (dict(H=35, n=8192), 1024, 2048), (dict(H=64, n=4096), 1024, 2048), (dict(H=17, n=16384), 1024, 2048), (dict(H=30, n=7687, causal=1, n0=4096), 1024, 2048),
@@ -185,10 +186,25 @@ def test_builds_of_the_backward_kernel_in_two_launches(d, heads, kw, first, seco
     (dict(H=37, n=8192), 2048, 2048),                                            # ... two CTAs for an SM
 ])
 def test_rows_per_chunk(kw, d64, d128):
-    for d, want in ((64, d64), (128, d128)):
-        rows = C.c_int(0)
-        assert ha.lib().hyperattn_internal_chunk_rows(C.byref(_params(d=d, **kw)), C.byref(rows)) == 0
-        assert rows.value == want, d
+    assert (_chunk_rows(d=64, **kw), _chunk_rows(d=128, **kw)) == (d64, d128)
+
+
+@pytest.mark.parametrize("kw,want", [
+    (dict(H=1, n=1024), 256), (dict(H=4, n=4096), 256), (dict(H=20, n=2349), 256), (dict(H=10, n=4000), 256), (dict(H=50, n=700), 256),
+    (dict(H=20, n=3000, causal=1, n0=1024), 512), (dict(H=15, n=2500, causal=1, n0=700), 256), (dict(H=4, n=10000), 256),
+    (dict(H=5, n=8000), 512), (dict(H=12, n=5000), 512),                         # ... a launch more
+    (dict(H=2, n=20000), 512),                                                   # ... nodes of 79 chunks
+    (dict(H=40, n=16384), 2048),
+])
+@pytest.mark.parametrize("d", [64, 128])
+def test_rows_per_chunk_of_fp32_inputs(d, kw, want):
+    assert _chunk_rows(d=d, dtype=B.FP32, **kw) == want
+
+
+def _chunk_rows(**kw):
+    rows = C.c_int(0)
+    assert ha.lib().hyperattn_internal_chunk_rows(C.byref(_params(**kw)), C.byref(rows)) == 0
+    return rows.value
 
 
 def _backward_launches(**kw):

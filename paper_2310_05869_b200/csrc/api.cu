@@ -28,6 +28,61 @@ constexpr size_t kAlign = 256;
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
+// Rows per chunk: 2048, halved (down to 256) while the hash has fewer than two CTAs for an SM and the share of the busiest SM gets cheaper - a CTA
+// costs as much as 256 rows beside its own, and one alone on an SM as much as two - and evened out over the unit: 2250 rows are two chunks of at
+// most 1280, not one of 2048 and one of 202.  A call, us, halved below 296 CTAs whatever the share and not evened -> this rule: 32 heads x 4096 rows
+// (256 CTAs instead of 512) 56.5 -> 55.4, 13 x 9333 58.8 -> 54.7, 21 x 6001 56.6 -> 55.9, 16 causal x 9000 139.1 -> 138.5; d = 128, 32 x 4096 78.9 ->
+// 74.3, 17 x 8192 82.9 -> 78.4, 35 x 8192 (280 instead of 560) 155.5 -> 150.3; hash of 4 causal x 100003 25.6 -> 22.9.
+// At d = 64 a CTA of 2048 rows is short enough that four of half the rows on an SM, which wait less, are better than two: the first halving is
+// taken where the busiest SM gets no more rows by it, and where the sort keeps to one launch.  Without -> with: 35 x 8192 98.5 -> 96.9, 64 x 4096
+// 91.0 -> 89.3, 48 x 6000 99.8 -> 97.1, 17 x 16384 96.0 -> 94.9, 30 causal x 7687 269.3 -> 266.9, by value norms 35 x 8192 122.8 -> 121.7; more rows
+// (60 x 2500, 1280 -> 3 x 1024) 63.1 -> 64.3, a launch more (9 x 30000) 94.7 -> 97.1.
+// fp32 inputs: the hash goes through a chunk 256 rows at a time, and a pass costs as much as 128 rows beside its own, so more CTAs pay than for bf16 -
+// unless the sort needs a launch more for them, or the scan gets long (nodes of more than 64 chunks).  Without -> with: 20 heads x 2349 rows 56.9 ->
+// 55.9, 10 x 4000 54.8 -> 53.9, 50 x 700 53.2 -> 51.5, d = 128, 20 x 2349 110.9 -> 108.2, 4 x 10000 107.4 -> 105.8, 20 causal x 3000 250.3 -> 242.4,
+// but 22 x 1700 95.7 -> 97.2; a launch more (12 x 5000) 73.8 -> 81.1, nodes of 79 chunks (2 x 20000) 58.5 -> 59.9.
+// Beyond two CTAs for an SM: 38 x 8192 112.0 -> 111.4 halved, but 50000 queries x 131072 keys 138.7 -> 141.5 (twice the chunks to scan).
+// More chunks need a larger workspace, so the halvings beyond the share of bf16 rows are left out (`fine` false) where the one at hand is too small.
+void choose_chunks(const hyperattn_params& p, Geometry& g, bool fine = true) {
+  auto even = [&](int chunk) {
+    auto side = [&](int unit) { const int k = (unit + chunk - 1) / chunk; return ((unit + k - 1) / k + 255) / 256 * 256; };
+    return side(g.unit) > side(g.unit_k) ? side(g.unit) : side(g.unit_k);
+  };
+  auto hash_ctas = [&](int chunk) {
+    const long long units = g.npad / g.unit, cpu = (g.unit + chunk - 1) / chunk, cpu_k = (g.unit_k + chunk - 1) / chunk;
+    return g.G * units * cpu + g.G * (g.causal ? units : 1) * cpu_k;
+  };
+  auto share = [&](int chunk, int cost) {               // of the busiest SM, a CTA's share being `cost` rows
+    const long long per_sm = (hash_ctas(chunk) + kSms - 1) / kSms;
+    return cost * (per_sm < 2 ? 2 : per_sm);
+  };
+  auto fp32_share = [&](int chunk) {
+    auto longest = [&](int unit) { const int k = (unit + chunk - 1) / chunk; return (unit + k - 1) / k; };
+    const int rows = longest(g.unit) > longest(g.unit_k) ? longest(g.unit) : longest(g.unit_k);
+    return share(chunk, rows + 128 * ((rows + 255) / 256));
+  };
+  auto take = [&](int chunk) {
+    g.chunk = chunk;
+    g.chunks_per_unit = (g.unit + g.chunk - 1) / g.chunk;
+    g.chunks_per_seg = (g.npad / g.unit) * g.chunks_per_unit;
+    g.chunks_per_unit_k = (g.unit_k + g.chunk - 1) / g.chunk;
+    g.chunks_per_seg_k = g.causal ? g.chunks_per_seg : g.chunks_per_unit_k;
+  };
+  const bool fp32 = p.dtype == HYPERATTN_FP32;
+  take(even(kSortChunk));
+  for (int half = kSortChunk / 2; half >= 256 && hash_ctas(g.chunk) < 2 * kSms; half /= 2) {
+    const int chunk = even(half), last = g.chunk;
+    if (chunk == last) continue;
+    const bool one_launch = scan_in_scatter(g);
+    take(chunk);
+    if (share(chunk, chunk + 256) < share(last, last + 256)) continue;
+    if (fine && (fp32 ? fp32_share(chunk) < fp32_share(last) && (one_launch ? scan_in_scatter(g) : node_chunks(g) <= 64)
+                      : g.d == 64 && half == kSortChunk / 2 && share(chunk, chunk) <= share(last, last) && scan_in_scatter(g))) continue;
+    take(last);
+    break;
+  }
+}
+
 // ---- geometry / validation ---------------------------------------------------------------
 int build_geometry(const hyperattn_params& p, Geometry& g) {
   if (p.B <= 0 || p.H <= 0 || p.n <= 0 || p.block <= 0 || p.samples < 0 || p.n_k < 0) return HYPERATTN_INVALID_ARGUMENT;
@@ -78,57 +133,7 @@ int build_geometry(const hyperattn_params& p, Geometry& g) {
     const int bpad = (g.b + 127) / 128 * 128, mpad = (g.m + 127) / 128 * 128;
     if (2 * bpad + mpad > kMaxNodeKeys) return HYPERATTN_UNSUPPORTED_SHAPE;
   }
-  // Rows per chunk: 2048, halved (down to 256) while the hash has fewer than two CTAs for an SM and the share of the busiest SM gets cheaper - a CTA
-  // costs as much as 256 rows beside its own, and one alone on an SM as much as two - and evened out over the unit: 2250 rows are two chunks of at
-  // most 1280, not one of 2048 and one of 202.  A call, us, halved below 296 CTAs whatever the share and not evened -> this rule: 32 heads x 4096 rows
-  // (256 CTAs instead of 512) 56.5 -> 55.4, 13 x 9333 58.8 -> 54.7, 21 x 6001 56.6 -> 55.9, 16 causal x 9000 139.1 -> 138.5; d = 128, 32 x 4096 78.9 ->
-  // 74.3, 17 x 8192 82.9 -> 78.4, 35 x 8192 (280 instead of 560) 155.5 -> 150.3; hash of 4 causal x 100003 25.6 -> 22.9.
-  // At d = 64 a CTA of 2048 rows is short enough that four of half the rows on an SM, which wait less, are better than two: the first halving is
-  // taken where the busiest SM gets no more rows by it, and where the sort keeps to one launch.  Without -> with: 35 x 8192 98.5 -> 96.9, 64 x 4096
-  // 91.0 -> 89.3, 48 x 6000 99.8 -> 97.1, 17 x 16384 96.0 -> 94.9, 30 causal x 7687 269.3 -> 266.9, by value norms 35 x 8192 122.8 -> 121.7; more rows
-  // (60 x 2500, 1280 -> 3 x 1024) 63.1 -> 64.3, a launch more (9 x 30000) 94.7 -> 97.1.
-  // fp32 inputs: the hash goes through a chunk 256 rows at a time, and a pass costs as much as 128 rows beside its own, so more CTAs pay than for bf16 -
-  // unless the sort needs a launch more for them, or the scan gets long (nodes of more than 64 chunks).  Without -> with: 20 heads x 2349 rows 56.9 ->
-  // 55.9, 10 x 4000 54.8 -> 53.9, 50 x 700 53.2 -> 51.5, d = 128, 20 x 2349 110.9 -> 108.2, 4 x 10000 107.4 -> 105.8, 20 causal x 3000 250.3 -> 242.4,
-  // but 22 x 1700 95.7 -> 97.2; a launch more (12 x 5000) 73.8 -> 81.1, nodes of 79 chunks (2 x 20000) 58.5 -> 59.9.
-  // Beyond two CTAs for an SM: 38 x 8192 112.0 -> 111.4 halved, but 50000 queries x 131072 keys 138.7 -> 141.5 (twice the chunks to scan).
-  auto even = [&](int chunk) {
-    auto side = [&](int unit) { const int k = (unit + chunk - 1) / chunk; return ((unit + k - 1) / k + 255) / 256 * 256; };
-    return side(g.unit) > side(g.unit_k) ? side(g.unit) : side(g.unit_k);
-  };
-  auto hash_ctas = [&](int chunk) {
-    const long long units = g.npad / g.unit, cpu = (g.unit + chunk - 1) / chunk, cpu_k = (g.unit_k + chunk - 1) / chunk;
-    return g.G * units * cpu + g.G * (g.causal ? units : 1) * cpu_k;
-  };
-  auto share = [&](int chunk, int cost) {               // of the busiest SM, a CTA's share being `cost` rows
-    const long long per_sm = (hash_ctas(chunk) + kSms - 1) / kSms;
-    return cost * (per_sm < 2 ? 2 : per_sm);
-  };
-  auto fp32_share = [&](int chunk) {
-    auto longest = [&](int unit) { const int k = (unit + chunk - 1) / chunk; return (unit + k - 1) / k; };
-    const int rows = longest(g.unit) > longest(g.unit_k) ? longest(g.unit) : longest(g.unit_k);
-    return share(chunk, rows + 128 * ((rows + 255) / 256));
-  };
-  auto take = [&](int chunk) {
-    g.chunk = chunk;
-    g.chunks_per_unit = (g.unit + g.chunk - 1) / g.chunk;
-    g.chunks_per_seg = (g.npad / g.unit) * g.chunks_per_unit;
-    g.chunks_per_unit_k = (g.unit_k + g.chunk - 1) / g.chunk;
-    g.chunks_per_seg_k = g.causal ? g.chunks_per_seg : g.chunks_per_unit_k;
-  };
-  const bool fp32 = p.dtype == HYPERATTN_FP32;
-  take(even(kSortChunk));
-  for (int half = kSortChunk / 2; half >= 256 && hash_ctas(g.chunk) < 2 * kSms; half /= 2) {
-    const int chunk = even(half), last = g.chunk;
-    if (chunk == last) continue;
-    const bool one_launch = scan_in_scatter(g);
-    take(chunk);
-    if (share(chunk, chunk + 256) < share(last, last + 256)) continue;
-    if (fp32 ? fp32_share(chunk) < fp32_share(last) && (one_launch ? scan_in_scatter(g) : node_chunks(g) <= 64)
-             : g.d == 64 && half == kSortChunk / 2 && share(chunk, chunk) <= share(last, last) && scan_in_scatter(g)) continue;
-    take(last);
-    break;
-  }
+  choose_chunks(p, g);
   return HYPERATTN_OK;
 }
 
@@ -297,7 +302,8 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
   }
   // partial results of the causal recursion travel in the type of the final output (bf16 inputs only)
   const bool part_bf16 = !is_fp32 && !out_fp32 && g.L > 0;
-  const Plan pl = make_plan(g, is_fp32, bw ? (bw->grad_dtype == HYPERATTN_FP32 ? 1 : 2) : 0, capped, vnorm, part_bf16);
+  auto plan = [&] { return make_plan(g, is_fp32, bw ? (bw->grad_dtype == HYPERATTN_FP32 ? 1 : 2) : 0, capped, vnorm, part_bf16); };
+  Plan pl = plan();
   cudaStream_t st = reinterpret_cast<cudaStream_t>(p.stream);
 
   int dev = 0;
@@ -315,6 +321,10 @@ int forward_impl(const hyperattn_params& p, int seg0 = 0, const hyperattn_grads*
     if (cudaMemset(ds.status, 0, 256) != cudaSuccess) return HYPERATTN_CUDA_ERROR;
   }
   char* base = nullptr;
+  if (pl.total > (p.workspace ? p.workspace_bytes : capturing ? ds.ws_bytes : pl.total)) {
+    choose_chunks(p, g, false);
+    pl = plan();
+  }
   if (p.workspace) {
     if (p.workspace_bytes < pl.total) return HYPERATTN_WORKSPACE_TOO_SMALL;
     base = reinterpret_cast<char*>(p.workspace);

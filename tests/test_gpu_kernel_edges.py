@@ -144,6 +144,27 @@ def test_permutations_are_stable_sorts_of_the_ids(chunk, kind, H, n, n_k, d, r, 
                                        torch.arange(rows, dtype=torch.int32, device="cuda").expand(H, rows))
 
 
+# chunks that need a larger workspace than the share of bf16 rows asks for are left out where the caller's is smaller (more chunks: histograms and
+# offsets of 1 KiB each): the same results, and one byte less is refused
+@pytest.mark.parametrize("H,n,dtype,more", [(35, 8192, torch.bfloat16, 8 - 4), (20, 2349, torch.float32, 10 - 5)])
+def test_chunks_by_the_workspace(H, n, dtype, more):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(23)
+    q, k, v = (torch.randn(1, H, n, 64, generator=gen, device="cuda").to(dtype) for _ in range(3))
+    code = B._dtype_code(dtype)
+    need = ha.workspace_bytes(1, H, n, 64, 128, 64, 7, dtype=code, out_dtype=code)
+    less = need - 2 * 2 * H * more * 1024
+    ws = torch.full((need,), 0xff, dtype=torch.uint8, device="cuda")
+    results = [ha.forward(q, k, v, 128, 64, 7, seed=2, workspace=ws[:size]) for size in (need, need - 1, less)]
+    torch.cuda.synchronize()
+    assert ha.last_device_status() == 0
+    for other in results[1:]:
+        for x, y in zip(results[0], other):
+            assert torch.equal(x, y)
+    with pytest.raises(ha.HyperAttnError, match="workspace too small"):
+        ha.forward(q, k, v, 128, 64, 7, seed=2, workspace=ws[:less - 1])
+
+
 # calls large enough for sorted nodes and everything else in launches of their own, against calls of few heads in one launch: the same bits
 TWO_LAUNCHES = [(64, 64, 2048, 256, torch.bfloat16, {}), (64, 40, 128, 256, torch.bfloat16, {}), (64, 64, 2048, 256, torch.float32, dict(precise=True)),
                 (128, 64, 2048, 256, torch.bfloat16, {}), (128, 64, 2048, 250, torch.float32, {}), (128, 64, 2048, 256, torch.float32, dict(precise=True)),

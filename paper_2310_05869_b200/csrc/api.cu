@@ -37,10 +37,11 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 // taken where the busiest SM gets no more rows by it, and where the sort keeps to one launch.  Without -> with: 35 x 8192 98.5 -> 96.9, 64 x 4096
 // 91.0 -> 89.3, 48 x 6000 99.8 -> 97.1, 17 x 16384 96.0 -> 94.9, 30 causal x 7687 269.3 -> 266.9, by value norms 35 x 8192 122.8 -> 121.7; more rows
 // (60 x 2500, 1280 -> 3 x 1024) 63.1 -> 64.3, a launch more (9 x 30000) 94.7 -> 97.1.
-// fp32 inputs: the hash goes through a chunk 256 rows at a time, and a pass costs as much as 128 rows beside its own, so more CTAs pay than for bf16 -
-// unless the sort needs a launch more for them, or the scan gets long (nodes of more than 64 chunks).  Without -> with: 20 heads x 2349 rows 56.9 ->
-// 55.9, 10 x 4000 54.8 -> 53.9, 50 x 700 53.2 -> 51.5, d = 128, 20 x 2349 110.9 -> 108.2, 4 x 10000 107.4 -> 105.8, 20 causal x 3000 250.3 -> 242.4,
-// but 22 x 1700 95.7 -> 97.2; a launch more (12 x 5000) 73.8 -> 81.1, nodes of 79 chunks (2 x 20000) 58.5 -> 59.9.
+// fp32 inputs: the hash goes through a chunk 256 rows at a time, and a pass costs as much as 128 rows beside its own (at d = 64, where a row is half the
+// work, 448, and 384 for the CTA), so more CTAs pay than for bf16 - unless the sort needs a launch more for them, or the scan gets long (nodes of more
+// than 64 chunks).  Without -> with: 20 heads x 2349 rows 56.9 -> 55.9, 10 x 4000 54.8 -> 53.9, 50 x 700 53.2 -> 51.5, d = 128, 20 x 2349 110.9 -> 108.2,
+// 4 x 10000 107.4 -> 105.8, 20 causal x 3000 250.3 -> 242.4, but 22 x 1700 95.7 -> 97.2; beyond the line, 20 causal x 2247 (as many passes, half as many
+// CTAs again) 133.1 -> 136.1, a launch more (12 x 5000) 73.8 -> 81.1, nodes of 79 chunks (2 x 20000) 58.5 -> 59.9.
 // Beyond two CTAs for an SM: 38 x 8192 112.0 -> 111.4 halved, but 50000 queries x 131072 keys 138.7 -> 141.5 (twice the chunks to scan).
 // More chunks need a larger workspace, so the halvings beyond the share of bf16 rows are left out (`fine` false) where the one at hand is too small.
 void choose_chunks(const hyperattn_params& p, Geometry& g, bool fine = true) {
@@ -59,7 +60,8 @@ void choose_chunks(const hyperattn_params& p, Geometry& g, bool fine = true) {
   auto fp32_share = [&](int chunk) {
     auto longest = [&](int unit) { const int k = (unit + chunk - 1) / chunk; return (unit + k - 1) / k; };
     const int rows = longest(g.unit) > longest(g.unit_k) ? longest(g.unit) : longest(g.unit_k);
-    return share(chunk, rows + 128 * ((rows + 255) / 256));
+    const int passes = (rows + 255) / 256;
+    return share(chunk, g.d == 64 ? rows + 448 * passes + 384 : rows + 128 * passes);
   };
   auto take = [&](int chunk) {
     g.chunk = chunk;

@@ -189,16 +189,16 @@ def test_rows_per_chunk(kw, d64, d128):
     assert (_chunk_rows(d=64, **kw), _chunk_rows(d=128, **kw)) == (d64, d128)
 
 
-@pytest.mark.parametrize("kw,want", [
-    (dict(H=1, n=1024), 256), (dict(H=4, n=4096), 256), (dict(H=20, n=2349), 256), (dict(H=10, n=4000), 256), (dict(H=50, n=700), 256),
-    (dict(H=20, n=3000, causal=1, n0=1024), 512), (dict(H=15, n=2500, causal=1, n0=700), 256), (dict(H=4, n=10000), 256),
-    (dict(H=5, n=8000), 512), (dict(H=12, n=5000), 512),                         # ... a launch more
-    (dict(H=2, n=20000), 512),                                                   # ... nodes of 79 chunks
-    (dict(H=40, n=16384), 2048),
+@pytest.mark.parametrize("kw,d64,d128", [
+    (dict(H=1, n=1024), 256, 256), (dict(H=4, n=4096), 256, 256), (dict(H=20, n=2349), 256, 256), (dict(H=10, n=4000), 256, 256),
+    (dict(H=50, n=700), 256, 256), (dict(H=15, n=2500, causal=1, n0=700), 256, 256), (dict(H=4, n=10000), 256, 256),
+    (dict(H=20, n=3000, causal=1, n0=1024), 768, 512), (dict(H=20, n=2247, causal=1, n0=1024), 768, 512),    # as many passes, more CTAs
+    (dict(H=5, n=8000), 512, 512), (dict(H=12, n=5000), 512, 512),               # ... a launch more
+    (dict(H=2, n=20000), 512, 512),                                              # ... nodes of 79 chunks
+    (dict(H=40, n=16384), 2048, 2048),
 ])
-@pytest.mark.parametrize("d", [64, 128])
-def test_rows_per_chunk_of_fp32_inputs(d, kw, want):
-    assert _chunk_rows(d=d, dtype=B.FP32, **kw) == want
+def test_rows_per_chunk_of_fp32_inputs(kw, d64, d128):
+    assert (_chunk_rows(d=64, dtype=B.FP32, **kw), _chunk_rows(d=128, dtype=B.FP32, **kw)) == (d64, d128)
 
 
 def _chunk_rows(**kw):

@@ -101,7 +101,9 @@ __device__ __forceinline__ void leaf_of_item(int item, int items, int per_leaf, 
 // The pairs of a call without recursion are equal items, and the last round of them may leave most SMs idle.  Where at most half of the SMs get one,
 // each of its query tiles is an item of its own: half of the softmax warps, but the other half would wait for nothing.  (Calls, us, in turn, pairs ->
 // split: d = 64, 32 heads of 4096 rows - 3.46 rounds of 148 - 57.9 -> 56.4, 21 of 6001 58.2 -> 56.7, 13 of 9333 60.3 -> 58.8, 12 of 4096 35.8 -> 33.9.
-// Pairs across two blocks too - 32 of 4096, b = 128, 46.5 -> 42.3 with their own build -, with the pair's order of sampled columns: the same bits.
+// Pairs across two blocks too, b = 128: 32 of 4096 42.9 -> 42.3, 12 of 4096 31.0 -> 29.2.  Their items keep the pair's order of sampled columns, for the
+// same bits; with an order of their own calls of two or three blocks, all of whose samples then are masked ones, would gain 1 to 4 %: 32 of 225 rows,
+// d = 128, 20.1 instead of 20.3, 5 of 201 by value norms 26.5 instead of 27.4.
 // With more than half of the SMs at work some whole pair remains in the last round, which then is as long as before.)
 inline int split_pairs(const AttnArgs& a, int sms) {
   if (a.n_leaf_pairs > 0 || a.g.levels != 1 || !a.level_paired[0]) return 0;
